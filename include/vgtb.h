@@ -53,7 +53,9 @@ extern "C" {
 #define VGTB_E_UNSUPPORTED -10 /* option not available for these shapes */
 
 /* precision forms of the commutator products */
-#define VGTB_FP64          0   /* complex FP64 everywhere (Eq. 6 evaluated directly) */
+#define VGTB_FP64          0   /* complex FP64 everywhere (Eq. 6 evaluated directly); from 97 orbitals
+                                  up the products run as exact digit products on the tensor cores,
+                                  no further off than FP64 multiply-adds in the norm of a product */
 #define VGTB_SPLIT_BF16X3  1   /* delta form, tcgen05 BF16 hi/lo 3-product GEMMs, FP32 accumulate */
 
 #define VGTB_INIT_GROUND   0   /* create() computes the SCC ground state D_k(0) */
@@ -115,12 +117,13 @@ typedef struct {
   int tile_variant[2];      /* split form: tile variant of product 1 / product 2 (see
                                vgtb_tile_config; -1 = variant 0, or the autotuner's choice) */
   int product1;             /* form of the first product W = D H of Eq. 6 (VGTB_P1_*):
-                               AUTO (0, default): the FP64 path runs it block-sparse (below), and
-                               so does the Crank-Nicolson integrator its product M = S^-1 H; the
-                               split form runs the tcgen05 GEMM and skips the 64-wide k-panels in
+                               AUTO (0, default): the FP64 path skips the 64-wide k-panels in which
+                               a tile's rows of H_k are zero, or below 97 orbitals runs it
+                               block-sparse (below), as does the Crank-Nicolson integrator its
+                               product M = S^-1 H; the split form runs the tcgen05 GEMM and skips the 64-wide k-panels in
                                which a tile's rows of H_k and dH_k are zero;
-                               DENSE: a dense GEMM over all of H_k (8 N^3 flops; FP64 DFMA or
-                               tcgen05 BF16x3, no panel skipped); BLOCKS: block-sparse over the
+                               DENSE: a dense product over all of H_k (8 N^3 flops, no panel
+                               skipped); BLOCKS: block-sparse over the
                                nonzero atom blocks of H_k on the CUDA cores (8 nnz(H) N flops;
                                FP64, or FP32 in the split form), which needs every atom to carry
                                4 orbitals (the FP64 AUTO falls back to DENSE otherwise, BLOCKS

@@ -381,6 +381,10 @@ constexpr int kCnThreads = 256;
 constexpr int kCnChunk = 8;
 constexpr int kCnOut = 12;  // block elements per thread: up to 192 targets per group of 4 atoms
 
+// The limit is a property of the kernel, not of a context: it is always raised to the most a CTA
+// can have, so that a context with small tables does not lower it under one with large tables.
+constexpr size_t kSmemLimit = 227 * 1024;
+
 size_t cn_smem_bytes(int max_ent) { return (size_t)kCnChunk * (16 + 4 * max_ent) * sizeof(double2); }
 
 __global__ void __launch_bounds__(kCnThreads) k_cn_density_pattern(const CnDensItem* __restrict__ items,
@@ -452,9 +456,8 @@ __global__ void __launch_bounds__(kCnThreads) k_cn_density_pattern(const CnDensI
 int cn_density_max_targets() { return kCnThreads * kCnOut / 16; }
 
 int cn_density_configure(int max_ent) {
-  const size_t smem = cn_smem_bytes(max_ent);
-  if (smem > 227 * 1024) return -1;
-  return cudaFuncSetAttribute(k_cn_density_pattern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
+  if (cn_smem_bytes(max_ent) > kSmemLimit) return -1;
+  return cudaFuncSetAttribute(k_cn_density_pattern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) ==
                  cudaSuccess
              ? 0
              : -1;
@@ -474,10 +477,11 @@ size_t bsr_smem_bytes(int fp64, int max_grp_targets) {
 
 int bsr_configure(int fp64, int max_grp_targets) {
   const size_t smem = fp64 ? bsr_smem_bytes(1, max_grp_targets) : bsr_p_smem_bytes(max_grp_targets);
-  if (smem > 227 * 1024) return -1;
+  if (smem > kSmemLimit) return -1;
   cudaError_t e = fp64 ? cudaFuncSetAttribute(k_bsr<double, kBsrGroupF64>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                       : cudaFuncSetAttribute(k_bsr_f32p, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit)
+                       : cudaFuncSetAttribute(k_bsr_f32p, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)kSmemLimit);
   return e == cudaSuccess ? 0 : -1;
 }
 

@@ -10,7 +10,7 @@
 // GB300 has no FP64 tensor-core kind, so the FP64 path runs on DFMA.
 #include <algorithm>
 
-#include "vgtb_internal.h"
+#include "slice.cuh"
 
 namespace vgtb {
 
@@ -133,6 +133,9 @@ __device__ __forceinline__ void split_bf16_d(double x, __nv_bfloat16& hi, __nv_b
   lo = __double2bfloat16(x - (double)__bfloat162float(hi));
 }
 
+// MP = 0: X is a matrix; MP = 7 or 2: X is put together from the integer planes of the sliced
+// product (slice.cuh), which saves writing and reading X once (134 MB at N = 2048).
+template <int MP>
 __global__ void __launch_bounds__(256) k_leap(const LeapItem* __restrict__ items, const int* step,
                                               double dt, int* counter, int* step_rw) {
   pdl_wait();
@@ -157,11 +160,16 @@ __global__ void __launch_bounds__(256) k_leap(const LeapItem* __restrict__ items
   const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
   if (active) {
     for (int r = ty; r < LT; r += 8) {
-      const long long ia = (long long)(bi * LT + r) * Np + bj * LT + tx;
-      const long long ib = (long long)(bj * LT + r) * Np + bi * LT + tx;
-      const double2* X = (const double2*)it.X;
-      Xa[r][tx] = X[ia];
-      Xb[r][tx] = X[ib];
+      const int ra = bi * LT + r, ca = bj * LT + tx, rb = bj * LT + r, cb = bi * LT + tx;
+      if constexpr (MP == 0) {
+        const double2* X = (const double2*)it.X;
+        Xa[r][tx] = X[(long long)ra * Np + ca];
+        Xb[r][tx] = X[(long long)rb * Np + cb];
+      } else {
+        const double2 z = make_double2(0.0, 0.0);  // padding rows and columns
+        Xa[r][tx] = (ra < it.N && ca < it.N) ? slice_load<MP>(it.pl, ra, ca) : z;
+        Xb[r][tx] = (rb < it.N && cb < it.N) ? slice_load<MP>(it.pl, rb, cb) : z;
+      }
     }
   }
   __syncthreads();
@@ -219,13 +227,17 @@ __global__ void __launch_bounds__(256) k_leap(const LeapItem* __restrict__ items
   }
 }
 
-void launch_leap(const LeapItem* items, int n_items, int Np_max, int x_f32, const int* step, double dt,
+void launch_leap(const LeapItem* items, int n_items, int Np_max, int mp, const int* step, double dt,
                  int* counter, int* step_rw, cudaStream_t st) {
-  (void)x_f32;
   const int nt = Np_max / LT;
   dim3 grid(nt * (nt + 1) / 2, n_items);
   dim3 block(LT, 8);
-  launch_pdl(k_leap, grid, block, 0, st, items, step, dt, counter, step_rw);
+  if (mp == 7)
+    launch_pdl(k_leap<7>, grid, block, 0, st, items, step, dt, counter, step_rw);
+  else if (mp == 2)
+    launch_pdl(k_leap<2>, grid, block, 0, st, items, step, dt, counter, step_rw);
+  else
+    launch_pdl(k_leap<0>, grid, block, 0, st, items, step, dt, counter, step_rw);
 }
 
 // ---------------------------------------------------------------------------
@@ -397,22 +409,31 @@ void launch_to_f32(const double2* src, float2* dst, long long n, cudaStream_t st
 // ---------------------------------------------------------------------------
 // helpers
 // ---------------------------------------------------------------------------
-__global__ void k_fill_herm(double2* a, int n, int ld) {
+__global__ void k_fill_herm(double2* a, int n, int ld, int real) {
   // the upper triangle (j >= i) is valid; set a[i][j] = conj(a[j][i]) for j < i
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)n * n) return;
   const int i = idx / n, j = idx % n;
   if (j < i) {
     const double2 v = a[(long long)j * ld + i];
-    a[(long long)i * ld + j] = make_double2(v.x, -v.y);
+    a[(long long)i * ld + j] = make_double2(v.x, real ? 0.0 : -v.y);
   } else if (j == i) {
     a[(long long)i * ld + i].y = 0.0;
   }
 }
 
-void launch_fill_hermitian_lower(double2* a, int n, int ld, cudaStream_t st) {
+// the upper triangle's imaginary parts, once the lower one has been filled from it
+__global__ void k_zero_imag_upper(double2* a, int n, int ld) {
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (long long)n * n) return;
+  const int i = idx / n, j = idx % n;
+  if (j > i) a[(long long)i * ld + j].y = 0.0;
+}
+
+void launch_fill_hermitian_lower(double2* a, int n, int ld, int real, cudaStream_t st) {
   const long long tot = (long long)n * n;
-  k_fill_herm<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(a, n, ld);
+  k_fill_herm<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(a, n, ld, real);
+  if (real) k_zero_imag_upper<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(a, n, ld);
 }
 
 __global__ void k_vt(const double2* ev, double2* vt, int n, int nocc, int ld) {

@@ -24,6 +24,7 @@
 
 #include "../../include/vgtb.h"
 #include "vgtb_internal.h"
+#include "vgtb_slice.h"
 #include "vgtb_tc.h"
 
 using namespace vgtb;
@@ -54,11 +55,16 @@ struct HostSys {
   std::vector<double> dq0_h, eps0_h;
   bool density_set = false;
   std::vector<int> trajs;  // trajectories of this system
+  const int *d_el_off = nullptr, *d_el_atom0 = nullptr, *d_orb_off = nullptr;
   std::vector<char> k_set;  // which k-points received a user density
   float2* D0f = nullptr;    // split form, block-sparse first product: [nk][Np][Np] FP32 copy of D0
   int bsr_units = 0;        // block-sparse first product: CTAs per item (groups x column chunks)
   int bsr_tg_max = 0;       // most targets of one atom group
   int bsr_ent_max = 0;      // most column atoms in the union of one atom group
+  bool slice = false;       // FP64 products by exact digit slices on the tensor cores (k_slice.cu)
+  std::vector<char> k_real; // every Bloch phase of the k-point is real: so are S_k and S_k^-1
+  SliceFam fSinv, fD0;      // digits of S_k^-1 and (delta form) of D_k(0)
+  SliceRowJob* d_jD0 = nullptr;
 };
 
 struct HostTraj {
@@ -79,6 +85,17 @@ struct HostTraj {
   double* apart = nullptr;
   int* ticket = nullptr;
   int* status = nullptr;
+};
+
+// One round of the sliced FP64 products: as many items as share the digit and plane scratch.
+struct SliceRound {
+  SliceGemm* g1 = nullptr;     // W (null: the first product runs block-sparse)
+  SliceGemm* g2 = nullptr;     // X
+  SliceRowJob* jD = nullptr;   // D (dD) to digits
+  SlicePatJob* jH = nullptr;   // H, and in the delta form dH, to digits
+  SliceRowJob* jW = nullptr;   // planes (or matrix) of W to digits
+  LeapItem* leap = nullptr;
+  int n = 0, nH = 0, max_N = 0, max_Np = 0, max_nat = 0;
 };
 
 }  // namespace
@@ -113,6 +130,10 @@ struct vgtb_ctx {
   GemmF64Item* d_g2 = nullptr;
   LeapItem* d_leap = nullptr;
   int n_items = 0;
+  int n_dense = 0;                 // items of the lists above (the others take the sliced products)
+  std::vector<SliceRound> rounds;  // sliced FP64 products
+  int slice_mp = 7, max_orb = 1;
+  int* d_slice_err = nullptr;
   // tcgen05 plans
   TcPlan* tc1 = nullptr;
   TcPlan* tc2 = nullptr;
@@ -123,6 +144,7 @@ struct vgtb_ctx {
   BsrSys* d_bsrsys = nullptr;
   int* d_bsr_u0 = nullptr;   // [n_items+1] first unit of each item
   int* d_bsr_ctr = nullptr;  // [2] unit counter and finished-CTA counter
+  int n_bsr = 0;             // items of the block-sparse list
   int bsr_units_max = 0, bsr_units_total = 0, bsr_tg_max = 0, bsr_ent_max = 0, bsr_grp_max = 0;
   // Crank-Nicolson: D = 2 C C^dagger formed at H's nonzero pattern only for the step's sums
   CnDensItem* d_cnd = nullptr;
@@ -326,11 +348,16 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
   for (int i = 0; i < s.n_atoms; ++i) h.atom_tgt0[i + 1] += h.atom_tgt0[i];
   // phases e^{-i 2 pi k.n}
   std::vector<double2> ph((size_t)s.n_k * s.n_blocks);
+  h.k_real.assign(s.n_k, 1);
   for (int k = 0; k < s.n_k; ++k)
     for (int b = 0; b < s.n_blocks; ++b) {
       const int* r = s.blk_ijl + 5 * b;
-      const double th = 2.0 * M_PI * (s.kpt[3 * k] * r[2] + s.kpt[3 * k + 1] * r[3] + s.kpt[3 * k + 2] * r[4]);
-      ph[(size_t)k * s.n_blocks + b] = make_double2(std::cos(th), -std::sin(th));
+      const double kn = s.kpt[3 * k] * r[2] + s.kpt[3 * k + 1] * r[3] + s.kpt[3 * k + 2] * r[4];
+      const double th = 2.0 * M_PI * kn;
+      double2 v = make_double2(std::cos(th), -std::sin(th));
+      if (2.0 * kn == std::floor(2.0 * kn)) v = make_double2(kn == std::floor(kn) ? 1.0 : -1.0, 0.0);
+      ph[(size_t)k * s.n_blocks + b] = v;
+      if (v.y != 0.0) h.k_real[k] = 0;
     }
   // upload
   memset(&d, 0, sizeof(d));
@@ -351,6 +378,7 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
   double2* pz;
   TRY(upload(ctx, &pi, h.orb_off.data(), h.orb_off.size()));
   d.orb_off = pi;
+  h.d_orb_off = pi;
   TRY(upload(ctx, &pd, h.z.data(), h.z.size()));
   d.z = pd;
   TRY(upload(ctx, &pd, h.gamma.data(), h.gamma.size()));
@@ -455,8 +483,10 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
     for (int i = 0; i <= h.nat; ++i) eat[i] = h.tgt_el0[h.atom_tgt0[i]];
     TRY(upload(ctx, &pi, eoff.data(), eoff.size()));
     d.el_off = pi;
+    h.d_el_off = pi;
     TRY(upload(ctx, &pi, eat.data(), eat.size()));
     d.el_atom0 = pi;
+    h.d_el_atom0 = pi;
   }
   d.n_el = h.n_el;
   TRY(dalloc(ctx, &d.kS, (size_t)h.nk * h.n_el));
@@ -525,7 +555,7 @@ int build_sinv(vgtb_ctx* ctx, int si) {
     if (st != CUSOLVER_STATUS_SUCCESS || hinfo != 0)
       return fail(ctx, VGTB_E_CUDA, "cusolverDnZpotri failed: status %d info %d", (int)st, hinfo);
     // column-major lower = row-major upper is valid; mirror it
-    launch_fill_hermitian_lower(S, h.N, h.Np, ctx->stream);
+    launch_fill_hermitian_lower(S, h.N, h.Np, h.k_real[k], ctx->stream);
     CK(cudaGetLastError());
   }
   CK(cudaStreamSynchronize(ctx->stream));
@@ -807,6 +837,7 @@ int finish_density(vgtb_ctx* ctx, int si) {
       launch_gemm_f64(dg + 1, 1, h.Np, h.Np, nullptr, ctx->stream);
       li = LeapItem{};
       li.X = Xb;
+      li.N = h.N;
       li.Np = h.Np;
       li.mode = 1;
       li.out = h.R0 + k * NN;
@@ -815,6 +846,10 @@ int finish_density(vgtb_ctx* ctx, int si) {
       CK(cudaGetLastError());
       CK(cudaStreamSynchronize(ctx->stream));
     }
+  }
+  if (h.d_jD0) {
+    launch_slice_rows(h.d_jD0, h.nk, h.N, h.N, 7, nullptr, ctx->stream);
+    CK(cudaGetLastError());
   }
   if (ctx->split) {
     for (int k = 0; k < h.nk; ++k) {
@@ -886,6 +921,229 @@ int upload_traj_table(vgtb_ctx* ctx) {
 void drop_graph(vgtb_ctx* ctx) {
   if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
   ctx->graph = nullptr;
+}
+
+// ---------------------------------------------------------------------------
+// Sliced FP64 products (k_slice.cu)
+// ---------------------------------------------------------------------------
+// From kSliceMinN orbitals up the 34 exact digit products on the tensor cores take less time than
+// one product on the FP64 pipe (N = 256, 8 k-points: 1.06 ms for one product on the FP64 pipe);
+// below, a product is a few microseconds of FP64 work and the extra launches cost more.
+constexpr int kSliceMinN = 97;
+
+int slice_family(vgtb_ctx* ctx, SliceFam& f, int rows, int K, int batch) {
+  f.rows = rows;
+  f.K = K;
+  f.Kp = slice_kp(K);
+  f.batch = batch;
+  TRY(dalloc(ctx, &f.dig, (size_t)batch * kSlices * rows * 2 * f.Kp));
+  return dalloc(ctx, &f.ex, (size_t)batch * rows);
+}
+
+// bytes of scratch that one item of system h takes: digits of D (later of W) and of H, planes
+// (delta form: digits of dH and a second set of planes)
+double slice_item_bytes(const vgtb_ctx* ctx, const HostSys& h) {
+  const double dig = 2.0 * kSlices * h.N * 2.0 * slice_kp(h.N), pl = 4.0 * slice_num_planes(2) * h.N * 2.0 * slice_nw(h.N);
+  return ctx->delta ? 3.0 * dig + 2.0 * pl : 2.0 * dig + pl;
+}
+
+double slice_budget() {
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return 0.0;
+  return std::min(0.25 * (double)fr, 32e9);
+}
+
+// Which systems take the sliced products: FP64 leapfrog, enough orbitals, and room for the
+// scratch of one item of every such system within the budget.
+void slice_choose(vgtb_ctx* ctx) {
+  if (ctx->split || ctx->cn || !tc_gemm_supported()) return;
+  const double budget = slice_budget();
+  double one = 0.0;
+  for (auto& h : ctx->sys) {
+    h.slice = h.N >= kSliceMinN && h.N <= kSliceMaxN;
+    if (h.slice) one += slice_item_bytes(ctx, h) + 4.0 * kSlices * h.N * slice_kp(h.N) * h.nk * (ctx->delta ? 2 : 1);
+  }
+  if (one > budget)
+    for (auto& h : ctx->sys) h.slice = false;
+}
+
+// Digit families, rounds and work lists.  A round holds as many items of every sliced system as
+// fit the scratch budget; one round takes everything unless the batch is very large.
+int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
+  std::vector<std::vector<int>> items(ctx->sys.size());
+  int n_sliced = 0;
+  for (int i = 0; i < ctx->n_items; ++i)
+    if (ctx->sys[ctx->items_h[i].sys].slice) items[ctx->items_h[i].sys].push_back(i);
+  for (auto& v : items) n_sliced += v.empty() ? 0 : 1;
+  if (!n_sliced) return VGTB_OK;
+  TRY(dalloc(ctx, &ctx->d_slice_err, 1));
+  const double budget = slice_budget();
+  std::vector<SliceFam> fams;
+  std::vector<SlicePattern> pats;
+  struct SysScratch {
+    SliceFam D, H, dH;
+    int* exW = nullptr;
+    int* planes[2] = {nullptr, nullptr};
+    int cap = 0, fS = -1, fD0 = -1, fD = -1, fH = -1, fdH = -1, fW = -1, pat = -1;
+  };
+  std::vector<SysScratch> sc(ctx->sys.size());
+  size_t n_rounds = 0;
+  long long tiles = 0;
+  for (size_t s = 0; s < ctx->sys.size(); ++s) {
+    if (items[s].empty()) continue;
+    const HostSys& h = ctx->sys[s];
+    SysScratch& c = sc[s];
+    c.cap = std::max(1, std::min((int)items[s].size(), (int)(budget / n_sliced / slice_item_bytes(ctx, h))));
+    n_rounds = std::max(n_rounds, (items[s].size() + c.cap - 1) / c.cap);
+    tiles += (long long)c.cap * slice_tiles(h.N, h.N);
+    for (int I = 0; I < h.nat; ++I) ctx->max_orb = std::max(ctx->max_orb, h.orb_off[I + 1] - h.orb_off[I]);
+  }
+  ctx->slice_mp = slice_pairs_per_plane(tiles);
+  const int np = slice_num_planes(ctx->slice_mp);
+  const bool first = ctx->opt.product1 != VGTB_P1_BLOCKS;  // the first product is sliced too
+  for (size_t s = 0; s < ctx->sys.size(); ++s) {
+    if (items[s].empty()) continue;
+    HostSys& h = ctx->sys[s];
+    SysScratch& c = sc[s];
+    const int nw = slice_nw(h.N);
+    TRY(slice_family(ctx, h.fSinv, h.N, h.N, h.nk));
+    std::vector<SliceRowJob> js(h.nk), j0(h.nk);
+    for (int k = 0; k < h.nk; ++k) {
+      SliceRowJob j{};
+      j.rows = j.cols = h.N;
+      j.src = h.Sinv + (size_t)k * h.Np * h.Np;
+      j.lds = h.Np;
+      j.out = h.fSinv.mat(k);
+      js[k] = j;
+    }
+    SliceRowJob* dj = nullptr;
+    TRY(upload(ctx, &dj, js.data(), js.size()));
+    launch_slice_rows(dj, h.nk, h.N, h.N, 7, nullptr, ctx->stream);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(ctx->stream));  // js leaves scope
+    if (ctx->delta && first) {
+      TRY(slice_family(ctx, h.fD0, h.N, h.N, h.nk));
+      for (int k = 0; k < h.nk; ++k) {
+        j0[k] = js[k];
+        j0[k].src = h.D0 + (size_t)k * h.Np * h.Np;
+        j0[k].out = h.fD0.mat(k);
+      }
+      TRY(upload(ctx, &h.d_jD0, j0.data(), j0.size()));
+      CK(cudaStreamSynchronize(ctx->stream));
+    }
+    TRY(slice_family(ctx, c.D, h.N, h.N, c.cap));
+    TRY(dalloc(ctx, &c.exW, (size_t)c.cap * h.N));
+    if (first) TRY(slice_family(ctx, c.H, h.N, h.N, c.cap));
+    if (first && ctx->delta) TRY(slice_family(ctx, c.dH, h.N, h.N, c.cap));
+    const size_t psz = (size_t)c.cap * np * h.N * 2 * nw;
+    TRY(dalloc(ctx, &c.planes[0], psz));
+    if (first && ctx->delta) TRY(dalloc(ctx, &c.planes[1], psz));
+    c.fS = (int)fams.size();
+    fams.push_back(h.fSinv);
+    c.fW = (int)fams.size();  // the digits of W take the place of D's (dead once W is known)
+    SliceFam w = c.D;
+    w.ex = c.exW;
+    fams.push_back(w);
+    if (first) {
+      c.fD = (int)fams.size();
+      fams.push_back(c.D);
+      c.fH = (int)fams.size();
+      fams.push_back(c.H);
+      if (ctx->delta) {
+        c.fD0 = (int)fams.size();
+        fams.push_back(h.fD0);
+        c.fdH = (int)fams.size();
+        fams.push_back(c.dH);
+      }
+      if (ctx->opt.product1 != VGTB_P1_DENSE) {
+        c.pat = (int)pats.size();
+        SlicePattern p;
+        p.orb_off = &h.orb_off;
+        p.tgt_I = &h.tgt_I;
+        p.tgt_J = &h.tgt_J;
+        pats.push_back(p);
+      }
+    }
+  }
+  const long long tmo = std::max(ctx->opt.timeout_ns, 2000000000LL);
+  for (size_t r = 0; r < n_rounds; ++r) {
+    SliceRound R;
+    std::vector<SliceRowJob> jD, jW;
+    std::vector<SlicePatJob> jH;
+    std::vector<LeapItem> lv;
+    std::vector<SliceProd> p1, p2;
+    for (size_t s = 0; s < ctx->sys.size(); ++s) {
+      const HostSys& h = ctx->sys[s];
+      const SysScratch& c = sc[s];
+      if (items[s].empty()) continue;
+      const size_t NN = (size_t)h.Np * h.Np;
+      const int nw = slice_nw(h.N);
+      for (int b = 0; b < c.cap && r * c.cap + b < items[s].size(); ++b) {
+        const int i = items[s][r * c.cap + b];
+        const DevItem& it = ctx->items_h[i];
+        R.max_N = std::max(R.max_N, h.N);
+        R.max_Np = std::max(R.max_Np, h.Np);
+        R.max_nat = std::max(R.max_nat, h.nat);
+        int* pl[2];
+        for (int q = 0; q < 2; ++q) pl[q] = c.planes[q] ? c.planes[q] + (size_t)b * np * h.N * 2 * nw : nullptr;
+        SliceRowJob w{};
+        w.rows = w.cols = h.N;
+        if (first) {
+          SliceRowJob d{};
+          d.rows = d.cols = h.N;
+          d.src = it.D[0];
+          d.src_par = (long long)NN;
+          d.lds = h.Np;
+          d.out = c.D.mat(b);
+          jD.push_back(d);
+          SlicePatJob hj{};
+          hj.nat = h.nat;
+          hj.Np = h.Np;
+          hj.v = (const double2*)it.kH;
+          hj.el_off = h.d_el_off;
+          hj.el_atom0 = h.d_el_atom0;
+          hj.orb_off = h.d_orb_off;
+          hj.out = c.H.mat(b);
+          jH.push_back(hj);
+          p1.push_back(SliceProd{c.fD, b, c.fH, b, pl[0], nw, false, c.pat});
+          w.n_planes = 1;
+          w.pl[0] = SlicePlanes{pl[0], (long long)h.N * 2 * nw, nw, d.out.ex, hj.out.ex};
+          if (ctx->delta) {
+            hj.v = (const double2*)it.kdH;
+            hj.out = c.dH.mat(b);
+            jH.push_back(hj);
+            p1.push_back(SliceProd{c.fD0, it.k, c.fdH, b, pl[1], nw, false, c.pat});
+            w.n_planes = 2;
+            w.pl[1] = SlicePlanes{pl[1], (long long)h.N * 2 * nw, nw, h.fD0.mat(it.k).ex, hj.out.ex};
+          }
+        } else {
+          w.src = it.W;
+          w.lds = h.Np;
+        }
+        w.out = c.D.mat(b);
+        w.out.ex = c.exW + (size_t)b * h.N;
+        jW.push_back(w);
+        p2.push_back(SliceProd{c.fS, it.k, c.fW, b, pl[0], nw, h.k_real[it.k] != 0, -1});
+        LeapItem l = leap[i];
+        l.pl = SlicePlanes{pl[0], (long long)h.N * 2 * nw, nw, h.fSinv.mat(it.k).ex, w.out.ex};
+        lv.push_back(l);
+      }
+    }
+    R.n = (int)lv.size();
+    R.nH = (int)jH.size();
+    std::string msg;
+    ctx->rounds.push_back(R);
+    SliceRound& Q = ctx->rounds.back();
+    if ((first && slice_gemm_create(fams, p1, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.g1, &msg)) ||
+        slice_gemm_create(fams, p2, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.g2, &msg))
+      return fail(ctx, VGTB_E_CUDA, "sliced product plan: %s", msg.c_str());
+    if (first) TRY(upload(ctx, &Q.jD, jD.data(), jD.size()));
+    if (first) TRY(upload(ctx, &Q.jH, jH.data(), jH.size()));
+    TRY(upload(ctx, &Q.jW, jW.data(), jW.size()));
+    TRY(upload(ctx, &Q.leap, lv.data(), lv.size()));
+    CK(cudaStreamSynchronize(ctx->stream));  // the lists leave scope
+  }
+  return VGTB_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -1021,6 +1279,22 @@ void launch_obs_scc(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag, int stride,
              ctx->split ? finish : 1);
 }
 
+// W = D H of a round: digits of D and H, the digit products (block-sparse first product: W is there already)
+int launch_slice_first(vgtb_ctx* ctx, const SliceRound& r, cudaStream_t st) {
+  if (!r.g1) return VGTB_OK;
+  launch_slice_rows(r.jD, r.n, r.max_N, r.max_N, ctx->slice_mp, ctx->d_step, st);
+  launch_slice_pattern(r.jH, r.nH, r.max_nat, ctx->max_orb, st);
+  if (slice_gemm_launch(r.g1, st)) return fail(ctx, VGTB_E_CUDA, "sliced product 1 launch failed");
+  return VGTB_OK;
+}
+
+// X = S^-1 W^dagger of a round, left as integer planes for the leapfrog
+int launch_slice_second(vgtb_ctx* ctx, const SliceRound& r, cudaStream_t st) {
+  launch_slice_rows(r.jW, r.n, r.max_N, r.max_N, ctx->slice_mp, nullptr, st);
+  if (slice_gemm_launch(r.g2, st)) return fail(ctx, VGTB_E_CUDA, "sliced product 2 launch failed");
+  return VGTB_OK;
+}
+
 int enqueue_step(vgtb_ctx* ctx, cudaEvent_t* ev) {
   cudaStream_t st = ctx->stream;
   unsigned evflag = cudaEventRecordDefault;
@@ -1042,8 +1316,8 @@ int enqueue_step(vgtb_ctx* ctx, cudaEvent_t* ev) {
     launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->d_step,
                  ctx->delta ? PH_FP64_DELTA : PH_FP64_PLAIN, -1, st);
   if (ev) CK(cudaEventRecordWithFlags(ev[3], st, evflag));
-  if (ctx->bsr)
-    launch_bsr(ctx->d_bsr, ctx->d_bsrsys, ctx->n_items, ctx->bsr_units_max, ctx->bsr_units_total, ctx->d_bsr_u0,
+  if (ctx->bsr && ctx->n_bsr > 0)
+    launch_bsr(ctx->d_bsr, ctx->d_bsrsys, ctx->n_bsr, ctx->bsr_units_max, ctx->bsr_units_total, ctx->d_bsr_u0,
                ctx->d_bsr_ctr, ctx->split ? 0 : 1, ctx->bsr_tg_max, ctx->d_step, st);
   if (ctx->split && ctx->tcc) {
     // both products in one launch: its time counts as product 1's
@@ -1055,17 +1329,33 @@ int enqueue_step(vgtb_ctx* ctx, cudaEvent_t* ev) {
     if (ev) CK(cudaEventRecordWithFlags(ev[4], st, evflag));
     TRY(tc_launch(ctx->tc2, st) == 0 ? VGTB_OK : fail(ctx, VGTB_E_CUDA, "tcgen05 product 2 launch failed"));
   } else {
-    if (!ctx->bsr) launch_gemm_f64(ctx->d_g1, ctx->n_items, ctx->max_Np, ctx->max_Np, ctx->d_step, st);
+    if (!ctx->bsr && ctx->n_dense)
+      launch_gemm_f64(ctx->d_g1, ctx->n_dense, ctx->max_Np, ctx->max_Np, ctx->d_step, st);
+    // every round but the last runs whole, the last one within the event classes
+    for (size_t r = 0; r < ctx->rounds.size(); ++r) {
+      TRY(launch_slice_first(ctx, ctx->rounds[r], st));
+      if (r + 1 == ctx->rounds.size()) break;
+      TRY(launch_slice_second(ctx, ctx->rounds[r], st));
+      launch_leap(ctx->rounds[r].leap, ctx->rounds[r].n, ctx->rounds[r].max_Np, ctx->slice_mp, ctx->d_step,
+                  ctx->sys[0].dt, nullptr, nullptr, st);
+    }
     if (ev) CK(cudaEventRecordWithFlags(ev[4], st, evflag));
-    launch_gemm_f64(ctx->d_g2, ctx->n_items, ctx->max_Np, ctx->max_Np, ctx->d_step, st);
+    if (ctx->n_dense) launch_gemm_f64(ctx->d_g2, ctx->n_dense, ctx->max_Np, ctx->max_Np, ctx->d_step, st);
+    if (!ctx->rounds.empty()) TRY(launch_slice_second(ctx, ctx->rounds.back(), st));
   }
   if (ev) CK(cudaEventRecordWithFlags(ev[5], st, evflag));
-  if (ctx->split)
+  if (!ctx->split) {
+    // the last launch of the step advances the step counter
+    const bool sl = !ctx->rounds.empty();
+    if (ctx->n_dense)
+      launch_leap(ctx->d_leap, ctx->n_dense, ctx->max_Np, 0, ctx->d_step, ctx->sys[0].dt,
+                  sl ? nullptr : ctx->d_counter, ctx->d_step, st);
+    if (sl)
+      launch_leap(ctx->rounds.back().leap, ctx->rounds.back().n, ctx->rounds.back().max_Np, ctx->slice_mp, ctx->d_step,
+                  ctx->sys[0].dt, ctx->d_counter, ctx->d_step, st);
+  } else
     launch_leap_split(ctx->d_leap, ctx->n_items, ctx->max_Np, ctx->d_step, ctx->sys[0].dt, ctx->d_counter,
                       ctx->d_step, st);
-  else
-    launch_leap(ctx->d_leap, ctx->n_items, ctx->max_Np, 0, ctx->d_step, ctx->sys[0].dt, ctx->d_counter,
-                ctx->d_step, st);
   if (ev) CK(cudaEventRecordWithFlags(ev[6], st, evflag));
   CK(cudaGetLastError());
   return VGTB_OK;
@@ -1127,6 +1417,12 @@ int check_status(vgtb_ctx* ctx) {
                   "trajectory %zu: Crank-Nicolson fixed point not converged (raise cn_iter or lower dt)", t);
     if (st & ST_NONFINITE) return fail(ctx, VGTB_E_UNSTABLE, "trajectory %zu: non-finite observables", t);
     if (st & ST_DRIFT) return fail(ctx, VGTB_E_UNSTABLE, "trajectory %zu: electron count drifted", t);
+  }
+  if (ctx->d_slice_err) {
+    int err = 0;
+    CK(cudaMemcpyAsync(&err, ctx->d_slice_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    if (err) return fail(ctx, VGTB_E_TIMEOUT, "sliced product reported status %d (bounded wait expired)", err);
   }
   if (!ctx->split) return VGTB_OK;
   const int tc = tc_status(ctx->tc1, ctx->stream) | tc_status(ctx->tc2, ctx->stream);
@@ -1248,6 +1544,10 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
   // (Crank-Nicolson: the product M = S^-1 H of every step, FP64)
   ctx->bsr = blocks_ok &&
              (ctx->opt.product1 == VGTB_P1_BLOCKS || (ctx->opt.product1 == VGTB_P1_AUTO && !ctx->split));
+  slice_choose(ctx);
+  bool all_slice = true;
+  for (auto& h : ctx->sys) all_slice = all_slice && h.slice;
+  if (all_slice && ctx->opt.product1 == VGTB_P1_AUTO) ctx->bsr = false;
   std::vector<BsrSys> bsys(n_sys);
   if (ctx->bsr) {
     for (int s = 0; s < n_sys; ++s) {
@@ -1342,7 +1642,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
         if ((rc = dalloc(ctx, &it.Y[0], nc))) return bail(rc);
         if ((rc = dalloc(ctx, &it.Y[1], nc))) return bail(rc);
       } else {
-        if (ctx->bsr) {
+        if (ctx->bsr || h.slice) {
           double2 *kh = nullptr, *kdh = nullptr;
           if ((rc = dalloc(ctx, &kh, (size_t)h.n_el))) return bail(rc);
           if (ctx->delta && (rc = dalloc(ctx, &kdh, (size_t)h.n_el))) return bail(rc);
@@ -1352,8 +1652,10 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
           if ((rc = dalloc(ctx, &it.H, NN))) return bail(rc);
           if (ctx->delta && (rc = dalloc(ctx, &it.dH, NN))) return bail(rc);
         }
-        if ((rc = dalloc(ctx, &it.W, NN))) return bail(rc);
-        if ((rc = dalloc(ctx, &it.X, NN))) return bail(rc);
+        if (!h.slice || ctx->opt.product1 == VGTB_P1_BLOCKS)
+          if ((rc = dalloc(ctx, &it.W, NN))) return bail(rc);
+        if (!h.slice)
+          if ((rc = dalloc(ctx, &it.X, NN))) return bail(rc);
       }
       ctx->items_h.push_back(it);
     }
@@ -1380,8 +1682,8 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
   if ((rc = dalloc(ctx, &ctx->d_counter, 1))) return bail(rc);
   if ((rc = upload_traj_table(ctx))) return bail(rc);
   // work lists of the FP64 products and of the leapfrog
-  std::vector<GemmF64Item> g1(ctx->n_items), g2(ctx->n_items);
-  std::vector<LeapItem> lv(ctx->n_items);
+  std::vector<GemmF64Item> g1, g2;
+  std::vector<LeapItem> lv, lv_slice(ctx->n_items);
   for (int i = 0; i < ctx->n_items; ++i) {
     const DevItem& it = ctx->items_h[i];
     const HostSys& h = ctx->sys[it.sys];
@@ -1409,8 +1711,10 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     b.nseg = 1;
     b.M = b.N = b.ldc = h.Np;
     b.C = it.X;
-    g1[i] = a;
-    g2[i] = b;
+    if (!h.slice) {
+      g1.push_back(a);
+      g2.push_back(b);
+    }
     LeapItem l{};
     l.X = ctx->split ? (const void*)it.Xf : (const void*)it.X;
     l.R0 = (ctx->delta && !ctx->split) ? h.R0 + it.k * NN : nullptr;
@@ -1419,10 +1723,15 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     l.D[1] = it.D[1];
     l.pieces = it.dD_p;
     l.f32 = it.dDf;
+    l.N = h.N;
     l.Np = h.Np;
     l.mode = 0;
-    lv[i] = l;
+    if (h.slice)
+      lv_slice[i] = l;
+    else
+      lv.push_back(l);
   }
+  ctx->n_dense = (int)lv.size();
   if (ctx->cn) {
     if ((rc = build_cn_lists(ctx))) return bail(rc);
   } else if (!ctx->split) {
@@ -1431,9 +1740,11 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
   }
   if ((rc = upload(ctx, &ctx->d_leap, lv.data(), lv.size()))) return bail(rc);
   if (ctx->bsr) {
-    std::vector<BsrItem> bl(ctx->n_items);
+    std::vector<BsrItem> bl;
+    std::vector<int> u0(1, 0);
     for (int i = 0; i < ctx->n_items; ++i) {
       const DevItem& it = ctx->items_h[i];
+      if (ctx->sys[it.sys].slice && ctx->opt.product1 != VGTB_P1_BLOCKS) continue;
       const HostSys& h = ctx->sys[it.sys];
       const size_t NN = (size_t)h.Np * h.Np;
       BsrItem b{};
@@ -1455,12 +1766,12 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
         b.A[1] = ctx->delta ? (const void*)(h.D0 + it.k * NN) : nullptr;
         b.W = it.W;
       }
-      bl[i] = b;
+      bl.push_back(b);
+      u0.push_back(u0.back() + h.bsr_units);
     }
+    ctx->n_bsr = (int)bl.size();
     if ((rc = upload(ctx, &ctx->d_bsr, bl.data(), bl.size()))) return bail(rc);
-    std::vector<int> u0(ctx->n_items + 1, 0);
-    for (int i = 0; i < ctx->n_items; ++i) u0[i + 1] = u0[i] + ctx->sys[ctx->items_h[i].sys].bsr_units;
-    ctx->bsr_units_total = u0[ctx->n_items];
+    ctx->bsr_units_total = u0.back();
     if ((rc = upload(ctx, &ctx->d_bsr_u0, u0.data(), u0.size()))) return bail(rc);
     if ((rc = dalloc(ctx, &ctx->d_bsr_ctr, 2))) return bail(rc);
     if (ctx->cn && ctx->bsr_tg_max <= cn_density_max_targets() && cn_density_configure(ctx->bsr_ent_max) == 0) {
@@ -1476,6 +1787,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
   for (int s = 0; s < n_sys; ++s) {
     if ((rc = build_sinv(ctx, s))) return bail(rc);
   }
+  if ((rc = slice_build(ctx, lv_slice))) return bail(rc);
   if (ctx->split) {
     std::vector<TcSysView> views(n_sys);
     for (int s = 0; s < n_sys; ++s) {
@@ -1947,6 +2259,10 @@ void vgtb_destroy(vgtb_ctx* ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   drop_graph(ctx);
   for (auto e : ctx->ev) cudaEventDestroy(e);
+  for (auto& r : ctx->rounds) {
+    slice_gemm_destroy(r.g1);
+    slice_gemm_destroy(r.g2);
+  }
   tc_destroy_chain(ctx->tcc);
   tc_destroy_plan(ctx->tc1);
   tc_destroy_plan(ctx->tc2);

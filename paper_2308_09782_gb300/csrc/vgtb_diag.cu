@@ -10,6 +10,7 @@
 #include "../../include/vgtb_diag.h"
 #include "tc_kernel.cuh"
 #include "vgtb_internal.h"
+#include "vgtb_slice.h"
 #include "vgtb_tc.h"
 
 using namespace vgtb;
@@ -193,4 +194,66 @@ extern "C" int vgtb_diag_bounded_wait(long long limit_ns, int which) {
   if (cudaMemcpy(&h, err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return VGTB_E_CUDA;
   if (h & 16) return VGTB_OK;
   return (h & 3) ? VGTB_E_TIMEOUT : VGTB_E_CUDA;
+}
+
+extern "C" int vgtb_diag_slice_product(int m, int n, int k, const double* a, const double* r, int a_real, int planes,
+                                       double* c) {
+  if (m < 1 || n < 1 || k < 1 || std::max(m, std::max(n, k)) > kSliceMaxN || !a || !r || !c ||
+      (planes != slice_num_planes(7) && planes != slice_num_planes(2)))
+    return VGTB_E_INVALID;
+  if (!tc_gemm_supported()) return VGTB_E_UNSUPPORTED;
+  const int mp = planes == slice_num_planes(7) ? 7 : 2, nw = slice_nw(n), kp = slice_kp(k);
+  Scratch sc;
+  double2* ad = sc.get<double2>((size_t)m * k);
+  double2* rd = sc.get<double2>((size_t)n * k);
+  double2* cd = sc.get<double2>((size_t)m * n);
+  SliceFam fa, fr;
+  fa.rows = m;
+  fr.rows = n;
+  fa.K = fr.K = k;
+  fa.Kp = fr.Kp = kp;
+  fa.batch = fr.batch = 1;
+  fa.dig = sc.get<__nv_bfloat16>((size_t)kSlices * m * 2 * kp);
+  fr.dig = sc.get<__nv_bfloat16>((size_t)kSlices * n * 2 * kp);
+  fa.ex = sc.get<int>(m);
+  fr.ex = sc.get<int>(n);
+  int* pl = sc.get<int>((size_t)planes * m * 2 * nw);
+  int* err = sc.get<int>(1);
+  SliceRowJob* dj = sc.get<SliceRowJob>(3);
+  if (!ad || !rd || !cd || !fa.dig || !fr.dig || !fa.ex || !fr.ex || !pl || !err || !dj) return VGTB_E_NOMEM;
+  SliceRowJob j[3] = {};
+  j[0].rows = m;
+  j[0].cols = k;
+  j[0].src = ad;
+  j[0].lds = k;
+  j[0].out = fa.mat(0);
+  j[1] = j[0];
+  j[1].rows = n;
+  j[1].src = rd;
+  j[1].out = fr.mat(0);
+  j[2].rows = m;
+  j[2].cols = n;
+  j[2].n_planes = 1;
+  j[2].pl[0] = SlicePlanes{pl, (long long)m * 2 * nw, nw, fa.ex, fr.ex};
+  j[2].dst = cd;
+  j[2].ldd = n;
+  if (cudaMemcpy(ad, a, sizeof(double2) * m * k, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(rd, r, sizeof(double2) * n * k, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(dj, j, sizeof(j), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemset(err, 0, sizeof(int)) != cudaSuccess)
+    return VGTB_E_CUDA;
+  SliceGemm* g = nullptr;
+  std::string msg;
+  if (slice_gemm_create({fa, fr}, {SliceProd{0, 0, 1, 0, pl, nw, a_real != 0, -1}}, {}, mp, 2000000000LL, err, &g, &msg))
+    return VGTB_E_CUDA;
+  launch_slice_rows(dj, 2, std::max(m, n), k, mp, nullptr, 0);
+  int rc = slice_gemm_launch(g, 0) ? VGTB_E_CUDA : VGTB_OK;
+  launch_slice_rows(dj + 2, 1, m, n, mp, nullptr, 0);
+  if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) rc = VGTB_E_CUDA;
+  slice_gemm_destroy(g);
+  int h = 0;
+  if (rc == VGTB_OK && (cudaMemcpy(&h, err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess ||
+                        cudaMemcpy(c, cd, sizeof(double2) * m * n, cudaMemcpyDeviceToHost) != cudaSuccess))
+    rc = VGTB_E_CUDA;
+  return rc == VGTB_OK && h ? VGTB_E_TIMEOUT : rc;
 }

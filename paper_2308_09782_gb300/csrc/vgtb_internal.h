@@ -303,24 +303,38 @@ struct GemmF64Item {
 void launch_gemm_f64(const GemmF64Item* items, int n_items, int max_m, int max_n, const int* step,
                      cudaStream_t st);
 
+// integer planes of a sliced FP64 product (slice.cuh): plane p holds 32-bit integers of
+// rows x [Re | Im], Nw columns each, the row scales of both operands beside them
+struct SlicePlanes {
+  const int* p;
+  long long stride;        // integers per plane
+  int Nw;
+  const int* exA;          // [rows]
+  const int* exR;          // [columns]
+};
+
 struct LeapItem {
   const void* X;           // FP64 interleaved (double2) or FP32 planar
+  SlicePlanes pl;          // or the planes of X (launch_leap with mp != 0)
   const double2* R0;       // optional (FP64 path)
   const float* R0f;        // optional (split path, FP32 planar)
   double2* D[2];
   __nv_bfloat16* pieces;   // optional [2][Np][2Np]
   float2* f32;             // optional [Np][Np]: FP32 copy of the new level (split form)
-  int Np;
+  int N, Np;
   int mode;                // 0 = leapfrog, 1 = write the derivative only into out
   double2* out;            // mode 1 target
 };
-void launch_leap(const LeapItem* items, int n_items, int Np_max, int x_f32, const int* step, double dt,
+// mp: 0 = X is a matrix, else X comes from planes of at most mp pairs (7 or 2);
+// counter may be null: the step counter is then left alone
+void launch_leap(const LeapItem* items, int n_items, int Np_max, int mp, const int* step, double dt,
                  int* counter, int* step_rw, cudaStream_t st);
 void launch_leap_split(const LeapItem* items, int n_items, int Np_max, const int* step, double dt, int* counter,
                        int* step_rw, cudaStream_t st);
 
 // helpers
-void launch_fill_hermitian_lower(double2* a, int n, int ld, cudaStream_t st);
+// real: the matrix is real, imaginary parts (rounding) are set to zero
+void launch_fill_hermitian_lower(double2* a, int n, int ld, int real, cudaStream_t st);
 void launch_vt_from_evecs(const double2* evec, double2* vt, int n, int nocc, int ld, cudaStream_t st);
 void launch_scale(double2* a, long long n, double s, cudaStream_t st);
 void launch_split_planar(const double2* src, __nv_bfloat16* dst, int N, int Np, cudaStream_t st);

@@ -1,0 +1,88 @@
+// Host interface of the sliced FP64 products (k_slice.cu; scheme in slice.cuh).
+#pragma once
+#include <string>
+#include <vector>
+
+#include "slice.cuh"
+
+namespace vgtb {
+
+// Rows to be cut into digits: taken from a matrix, from the planes of a product,
+// or from both sets of planes added up; optionally base + coef x value; stored to
+// dst and / or cut into digits.
+struct SliceRowJob {
+  int rows, cols;
+  const double2* src;      // matrix source, or null
+  long long src_par;       // src + ((*step) & 1) * src_par
+  int lds;
+  int n_planes;            // plane sources (0, 1, 2)
+  SlicePlanes pl[2];
+  const double2* base;     // value = base + coef * value when epi != 0 (base may be null)
+  int ldb, epi;
+  double2 coef;
+  double2* dst;            // optional
+  int ldd;
+  SliceMat out;            // digits wanted when out.dig != null
+};
+// mp: pairs per plane of the sources (7 or 2)
+void launch_slice_rows(const SliceRowJob* jobs, int n_jobs, int max_rows, int max_cols, int mp, const int* step,
+                       cudaStream_t st);
+
+// Digits of a Hermitian-pattern matrix given at the target elements only (H_k):
+// positions off the pattern are left as they are (zeros).
+struct SlicePatJob {
+  int nat, Np;
+  const double2* v;        // [n_el]
+  const int* el_off;       // [n_el] row * Np + column
+  const int* el_atom0;     // [nat+1]
+  const int* orb_off;      // [nat+1]
+  SliceMat out;
+};
+void launch_slice_pattern(const SlicePatJob* jobs, int n_jobs, int max_nat, int max_orb, cudaStream_t st);
+
+// One operand family: the digits of `batch` matrices of one shape, contiguous.
+struct SliceFam {
+  __nv_bfloat16* dig = nullptr;
+  int* ex = nullptr;
+  int rows = 0, K = 0, Kp = 0, batch = 0;
+  SliceMat mat(int b) const {
+    SliceMat m{};
+    if (!dig) return m;
+    m.dig = dig + (size_t)b * kSlices * rows * 2 * Kp;
+    m.ex = ex + (size_t)b * rows;
+    m.rows = rows;
+    m.K = K;
+    m.Kp = Kp;
+    return m;
+  }
+};
+
+// Nonzero pattern of an R operand (H): orbital offsets and the atom pairs (I, J) of the targets.
+struct SlicePattern {
+  const std::vector<int>* orb_off = nullptr;
+  const std::vector<int>* tgt_I = nullptr;
+  const std::vector<int>* tgt_J = nullptr;
+};
+
+// product i: planes[i] = A[fam_a[i]][b_a] R[fam_r[i]][b_r]^dagger
+struct SliceProd {
+  int fam_a, b_a, fam_r, b_r;
+  int* planes;
+  int Nw;
+  bool a_real;             // every imaginary part of A is zero
+  int pattern;             // index into the patterns, or -1
+};
+
+struct SliceGemm;
+int slice_pairs_per_plane(long long tiles);  // 7, or 2 when 7 planes of work leave the chip idle
+int slice_tiles(int M, int N);
+int slice_gemm_create(const std::vector<SliceFam>& fams, const std::vector<SliceProd>& prods,
+                      const std::vector<SlicePattern>& patterns, int mp, long long timeout_ns, int* err, SliceGemm** out,
+                      std::string* msg);  // err: device word that an expired wait sets
+int slice_gemm_launch(SliceGemm* g, cudaStream_t st);
+void slice_gemm_destroy(SliceGemm* g);
+inline int slice_kp(int K) { return (K + 63) / 64 * 64; }
+inline int slice_nw(int N) { return (N + 31) / 32 * 32; }
+inline int slice_num_planes(int mp) { return mp == 7 ? slice_planes<7>() : slice_planes<2>(); }
+
+}  // namespace vgtb

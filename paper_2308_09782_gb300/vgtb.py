@@ -42,7 +42,7 @@ EXPORTS = ["vgtb_default_options", "vgtb_create", "vgtb_create_batch", "vgtb_set
            "vgtb_diag_split_chain", "vgtb_split_cgemm_noalloc", "vgtb_spectrum", "vgtb_group_charges",
            "vgtb_set_coefficients", "vgtb_get_coefficients", "vgtb_tile_config",
            "vgtb_diag_split_chain_variant", "vgtb_diag_num_variants", "vgtb_diag_convert",
-           "vgtb_diag_bounded_wait"]
+           "vgtb_diag_bounded_wait", "vgtb_diag_slice_product"]
 
 
 class VgtbSystem(C.Structure):
@@ -110,6 +110,7 @@ def load(path: str = LIB_PATH):
     lib.vgtb_diag_split_chain_variant.argtypes = [I, P(D), P(D), P(D), I, P(D), P(D)]
     lib.vgtb_diag_num_variants.argtypes = []
     lib.vgtb_diag_bounded_wait.argtypes = [C.c_longlong, I]
+    lib.vgtb_diag_slice_product.argtypes = [I, I, I, P(D), P(D), I, I, P(D)]
     lib.vgtb_diag_convert.argtypes = [I, P(D), P(C.c_float), P(C.c_float), P(C.c_float), P(D), P(D)]
     for name in EXPORTS:
         if name not in ("vgtb_default_options", "vgtb_last_error", "vgtb_destroy", "vgtb_state_size"):
@@ -211,6 +212,18 @@ def diag_convert(d_in, f_in):
     if rc != VGTB_OK:
         raise VgtbError(rc, "vgtb_diag_convert failed")
     return fb, fr, db, dr
+
+
+def diag_slice_product(a, r, a_real: bool = False, planes: int = 8):
+    """a r^dagger of host matrices by the sliced FP64 product."""
+    a, r = (np.ascontiguousarray(x, np.complex128) for x in (a, r))
+    c = np.zeros((a.shape[0], r.shape[0]), np.complex128)
+    cp = lambda m: m.ctypes.data_as(C.POINTER(C.c_double))  # noqa: E731
+    rc = load().vgtb_diag_slice_product(a.shape[0], r.shape[0], a.shape[1], cp(a), cp(r), int(a_real), int(planes),
+                                        cp(c))
+    if rc != VGTB_OK:
+        raise VgtbError(rc, "vgtb_diag_slice_product failed")
+    return c
 
 
 def num_tile_variants() -> int:
