@@ -560,7 +560,7 @@ void launch_cn_check(const CnCheckItem* items, int n_items, int max_elems, const
   k_cn_check<<<dim3(blocks > 0 ? blocks : 1, n_items), 256, 0, st>>>(items, trj, tol);
 }
 
-__global__ void k_conj_t(const double2* src, int lds, double2* dst, int ldd, int rows, int cols) {
+__device__ __forceinline__ void conj_t_tile(const double2* src, int lds, double2* dst, int ldd, int rows, int cols) {
   __shared__ double2 tile[32][33];
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   for (int y = threadIdx.y; y < 32; y += 8) {
@@ -575,6 +575,21 @@ __global__ void k_conj_t(const double2* src, int lds, double2* dst, int ldd, int
       dst[(long long)dr * ldd + dc] = make_double2(v.x, -v.y);
     }
   }
+}
+
+__global__ void k_conj_t(const double2* src, int lds, double2* dst, int ldd, int rows, int cols) {
+  conj_t_tile(src, lds, dst, ldd, rows, cols);
+}
+
+__global__ void k_conj_t_items(const ConjTItem* __restrict__ items) {
+  pdl_wait();
+  pdl_trigger();
+  const ConjTItem& it = items[blockIdx.z];
+  conj_t_tile(it.src, it.lds, it.dst, it.ldd, it.rows, it.cols);
+}
+
+void launch_conj_transpose_items(const ConjTItem* items, int n_items, int max_rows, int max_cols, cudaStream_t st) {
+  launch_pdl(k_conj_t_items, dim3((max_cols + 31) / 32, (max_rows + 31) / 32, n_items), dim3(32, 8), 0, st, items);
 }
 
 void launch_conj_transpose(const double2* src, int lds, double2* dst, int ldd, int rows, int cols, cudaStream_t st) {

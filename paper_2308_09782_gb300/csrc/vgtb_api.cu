@@ -96,6 +96,12 @@ struct SliceRound {
   SliceRowJob* jW = nullptr;   // planes (or matrix) of W to digits
   LeapItem* leap = nullptr;
   int n = 0, nH = 0, max_N = 0, max_Np = 0, max_nat = 0;
+  // Crank-Nicolson: D = 2 C C^dagger, M = S^-1 H (g2), the sweeps Y^dagger M^dagger (g1)
+  SliceGemm* gD = nullptr;
+  ConjTItem* tC = nullptr;     // C from C^dagger
+  SliceRowJob *jC = nullptr, *jDout = nullptr, *jM = nullptr, *jC0 = nullptr;
+  SliceRowJob* jS[4] = {nullptr, nullptr, nullptr, nullptr};  // sweep epilogues: digits only, + Y[0], + Y[1], last
+  int max_nocc = 0;
 };
 
 }  // namespace
@@ -943,8 +949,9 @@ int slice_family(vgtb_ctx* ctx, SliceFam& f, int rows, int K, int batch) {
 // bytes of scratch that one item of system h takes: digits of D (later of W) and of H, planes
 // (delta form: digits of dH and a second set of planes)
 double slice_item_bytes(const vgtb_ctx* ctx, const HostSys& h) {
+  // (Crank-Nicolson: digits of C, C^dagger or Y, H and M take no more than four full matrices)
   const double dig = 2.0 * kSlices * h.N * 2.0 * slice_kp(h.N), pl = 4.0 * slice_num_planes(2) * h.N * 2.0 * slice_nw(h.N);
-  return ctx->delta ? 3.0 * dig + 2.0 * pl : 2.0 * dig + pl;
+  return ctx->cn ? 4.0 * dig + pl : (ctx->delta ? 3.0 * dig + 2.0 * pl : 2.0 * dig + pl);
 }
 
 double slice_budget() {
@@ -956,7 +963,8 @@ double slice_budget() {
 // Which systems take the sliced products: FP64 leapfrog, enough orbitals, and room for the
 // scratch of one item of every such system within the budget.
 void slice_choose(vgtb_ctx* ctx) {
-  if (ctx->split || ctx->cn || !tc_gemm_supported()) return;
+  // an explicit block-sparse product keeps its kernel (Crank-Nicolson: and all that goes with it)
+  if (ctx->split || !tc_gemm_supported() || (ctx->cn && ctx->opt.product1 == VGTB_P1_BLOCKS)) return;
   const double budget = slice_budget();
   double one = 0.0;
   for (auto& h : ctx->sys) {
@@ -965,6 +973,37 @@ void slice_choose(vgtb_ctx* ctx) {
   }
   if (one > budget)
     for (auto& h : ctx->sys) h.slice = false;
+}
+
+SliceRowJob slice_row_job(const double2* src, int lds, int rows, int cols, const SliceMat& out) {
+  SliceRowJob j{};
+  j.rows = rows;
+  j.cols = cols;
+  j.src = src;
+  j.lds = lds;
+  j.out = out;
+  return j;
+}
+
+// digits of S_k^-1
+int slice_sinv(vgtb_ctx* ctx, HostSys& h) {
+  TRY(slice_family(ctx, h.fSinv, h.N, h.N, h.nk));
+  std::vector<SliceRowJob> js(h.nk);
+  for (int k = 0; k < h.nk; ++k) js[k] = slice_row_job(h.Sinv + (size_t)k * h.Np * h.Np, h.Np, h.N, h.N, h.fSinv.mat(k));
+  SliceRowJob* dj = nullptr;
+  TRY(upload(ctx, &dj, js.data(), js.size()));
+  launch_slice_rows(dj, h.nk, h.N, h.N, 7, nullptr, ctx->stream);
+  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(ctx->stream));  // js leaves scope
+  return VGTB_OK;
+}
+
+SlicePattern slice_pattern(const HostSys& h) {
+  SlicePattern p;
+  p.orb_off = &h.orb_off;
+  p.tgt_I = &h.tgt_I;
+  p.tgt_J = &h.tgt_J;
+  return p;
 }
 
 // Digit families, rounds and work lists.  A round holds as many items of every sliced system as
@@ -1006,28 +1045,11 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
     HostSys& h = ctx->sys[s];
     SysScratch& c = sc[s];
     const int nw = slice_nw(h.N);
-    TRY(slice_family(ctx, h.fSinv, h.N, h.N, h.nk));
-    std::vector<SliceRowJob> js(h.nk), j0(h.nk);
-    for (int k = 0; k < h.nk; ++k) {
-      SliceRowJob j{};
-      j.rows = j.cols = h.N;
-      j.src = h.Sinv + (size_t)k * h.Np * h.Np;
-      j.lds = h.Np;
-      j.out = h.fSinv.mat(k);
-      js[k] = j;
-    }
-    SliceRowJob* dj = nullptr;
-    TRY(upload(ctx, &dj, js.data(), js.size()));
-    launch_slice_rows(dj, h.nk, h.N, h.N, 7, nullptr, ctx->stream);
-    CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(ctx->stream));  // js leaves scope
+    TRY(slice_sinv(ctx, h));
     if (ctx->delta && first) {
       TRY(slice_family(ctx, h.fD0, h.N, h.N, h.nk));
-      for (int k = 0; k < h.nk; ++k) {
-        j0[k] = js[k];
-        j0[k].src = h.D0 + (size_t)k * h.Np * h.Np;
-        j0[k].out = h.fD0.mat(k);
-      }
+      std::vector<SliceRowJob> j0(h.nk);
+      for (int k = 0; k < h.nk; ++k) j0[k] = slice_row_job(h.D0 + (size_t)k * h.Np * h.Np, h.Np, h.N, h.N, h.fD0.mat(k));
       TRY(upload(ctx, &h.d_jD0, j0.data(), j0.size()));
       CK(cudaStreamSynchronize(ctx->stream));
     }
@@ -1057,11 +1079,7 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
       }
       if (ctx->opt.product1 != VGTB_P1_DENSE) {
         c.pat = (int)pats.size();
-        SlicePattern p;
-        p.orb_off = &h.orb_off;
-        p.tgt_I = &h.tgt_I;
-        p.tgt_J = &h.tgt_J;
-        pats.push_back(p);
+        pats.push_back(slice_pattern(h));
       }
     }
   }
@@ -1089,12 +1107,8 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
         SliceRowJob w{};
         w.rows = w.cols = h.N;
         if (first) {
-          SliceRowJob d{};
-          d.rows = d.cols = h.N;
-          d.src = it.D[0];
+          SliceRowJob d = slice_row_job(it.D[0], h.Np, h.N, h.N, c.D.mat(b));
           d.src_par = (long long)NN;
-          d.lds = h.Np;
-          d.out = c.D.mat(b);
           jD.push_back(d);
           SlicePatJob hj{};
           hj.nat = h.nat;
@@ -1146,6 +1160,158 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
   return VGTB_OK;
 }
 
+// The Crank-Nicolson counterpart: per round the density product C C^dagger, M = S^-1 H and the
+// sweeps.  The digits of C (N rows of nocc) and of C^dagger or Y^dagger (nocc rows of N) are never
+// needed at the same time and share their place.
+int slice_build_cn(vgtb_ctx* ctx) {
+  std::vector<std::vector<int>> items(ctx->sys.size());
+  int n_sliced = 0;
+  for (int i = 0; i < ctx->n_items; ++i)
+    if (ctx->sys[ctx->items_h[i].sys].slice) items[ctx->items_h[i].sys].push_back(i);
+  for (auto& v : items) n_sliced += v.empty() ? 0 : 1;
+  if (!n_sliced) return VGTB_OK;
+  TRY(dalloc(ctx, &ctx->d_slice_err, 1));
+  const double budget = slice_budget();
+  const double theta = 0.5 * ctx->sys[0].dt;
+  std::vector<SliceFam> fams;
+  std::vector<SlicePattern> pats;
+  struct SysScratch {
+    SliceFam C, Y, H, M;
+    int* planes = nullptr;
+    int cap = 0, fS = -1, fC = -1, fY = -1, fH = -1, fM = -1, pat = -1;
+  };
+  std::vector<SysScratch> sc(ctx->sys.size());
+  size_t n_rounds = 0;
+  long long tiles = 0;
+  for (size_t s = 0; s < ctx->sys.size(); ++s) {
+    if (items[s].empty()) continue;
+    const HostSys& h = ctx->sys[s];
+    SysScratch& c = sc[s];
+    c.cap = std::max(1, std::min((int)items[s].size(), (int)(budget / n_sliced / slice_item_bytes(ctx, h))));
+    n_rounds = std::max(n_rounds, (items[s].size() + c.cap - 1) / c.cap);
+    tiles += (long long)c.cap * slice_tiles(h.nocc, h.N);
+    for (int I = 0; I < h.nat; ++I) ctx->max_orb = std::max(ctx->max_orb, h.orb_off[I + 1] - h.orb_off[I]);
+  }
+  ctx->slice_mp = slice_pairs_per_plane(tiles);
+  const int np = slice_num_planes(ctx->slice_mp);
+  for (size_t s = 0; s < ctx->sys.size(); ++s) {
+    if (items[s].empty()) continue;
+    HostSys& h = ctx->sys[s];
+    SysScratch& c = sc[s];
+    TRY(slice_sinv(ctx, h));
+    // one place for the digits of C and of Y, each with its own row scales
+    const size_t szC = (size_t)h.N * slice_kp(h.nocc), szY = (size_t)h.nocc * slice_kp(h.N);
+    __nv_bfloat16* dig = nullptr;
+    TRY(dalloc(ctx, &dig, 2 * kSlices * c.cap * std::max(szC, szY)));
+    c.C.dig = c.Y.dig = dig;
+    c.C.rows = c.Y.K = h.N;
+    c.C.K = c.Y.rows = h.nocc;
+    c.C.Kp = slice_kp(h.nocc);
+    c.Y.Kp = slice_kp(h.N);
+    c.C.batch = c.Y.batch = c.cap;
+    TRY(dalloc(ctx, &c.C.ex, (size_t)c.cap * h.N));
+    TRY(dalloc(ctx, &c.Y.ex, (size_t)c.cap * h.nocc));
+    TRY(slice_family(ctx, c.H, h.N, h.N, c.cap));
+    TRY(slice_family(ctx, c.M, h.N, h.N, c.cap));
+    TRY(dalloc(ctx, &c.planes, (size_t)c.cap * np * h.N * 2 * slice_nw(h.N)));
+    for (auto p : {std::make_pair(&c.fS, &h.fSinv), std::make_pair(&c.fC, &c.C), std::make_pair(&c.fY, &c.Y),
+                   std::make_pair(&c.fH, &c.H), std::make_pair(&c.fM, &c.M)}) {
+      *p.first = (int)fams.size();
+      fams.push_back(*p.second);
+    }
+    if (ctx->opt.product1 != VGTB_P1_DENSE) {
+      c.pat = (int)pats.size();
+      pats.push_back(slice_pattern(h));
+    }
+  }
+  const long long tmo = std::max(ctx->opt.timeout_ns, 2000000000LL);
+  for (size_t r = 0; r < n_rounds; ++r) {
+    SliceRound R;
+    std::vector<ConjTItem> tC;
+    std::vector<SliceRowJob> jC, jD, jM, jC0, jS[4];
+    std::vector<SlicePatJob> jH;
+    std::vector<SliceProd> pD, pM, pS;
+    for (size_t s = 0; s < ctx->sys.size(); ++s) {
+      const HostSys& h = ctx->sys[s];
+      const SysScratch& c = sc[s];
+      if (items[s].empty()) continue;
+      const int nw = slice_nw(h.N);
+      for (int b = 0; b < c.cap && r * c.cap + b < items[s].size(); ++b) {
+        const DevItem& it = ctx->items_h[items[s][r * c.cap + b]];
+        R.max_N = std::max(R.max_N, h.N);
+        R.max_nocc = std::max(R.max_nocc, h.nocc);
+        R.max_nat = std::max(R.max_nat, h.nat);
+        int* pl = c.planes + (size_t)b * np * h.N * 2 * nw;
+        // C = (C^dagger)^dagger into the first iterate's buffer (N x nocc fits nocc x Np)
+        tC.push_back(ConjTItem{it.Cd, h.Np, it.Y[0], h.nocc, h.N, h.nocc});
+        jC.push_back(slice_row_job(it.Y[0], h.nocc, h.N, h.nocc, c.C.mat(b)));
+        pD.push_back(SliceProd{c.fC, b, c.fC, b, pl, nw, false, -1});
+        SliceRowJob d{};
+        d.rows = d.cols = h.N;
+        d.n_planes = 1;
+        d.pl[0] = SlicePlanes{pl, (long long)h.N * 2 * nw, nw, c.C.mat(b).ex, c.C.mat(b).ex};
+        d.epi = 1;
+        d.coef = make_double2(2.0, 0.0);
+        d.dst = it.D[0];
+        d.ldd = h.Np;
+        jD.push_back(d);
+        SlicePatJob hj{};
+        hj.nat = h.nat;
+        hj.Np = h.Np;
+        hj.v = (const double2*)it.kH;
+        hj.el_off = h.d_el_off;
+        hj.el_atom0 = h.d_el_atom0;
+        hj.orb_off = h.d_orb_off;
+        hj.out = c.H.mat(b);
+        jH.push_back(hj);
+        pM.push_back(SliceProd{c.fS, it.k, c.fH, b, pl, nw, h.k_real[it.k] != 0, c.pat});
+        SliceRowJob mj{};
+        mj.rows = mj.cols = h.N;
+        mj.n_planes = 1;
+        mj.pl[0] = SlicePlanes{pl, (long long)h.N * 2 * nw, nw, h.fSinv.mat(it.k).ex, hj.out.ex};
+        mj.out = c.M.mat(b);
+        jM.push_back(mj);
+        jC0.push_back(slice_row_job(it.Cd, h.Np, h.nocc, h.N, c.Y.mat(b)));
+        pS.push_back(SliceProd{c.fY, b, c.fM, b, pl, nw, false, -1});
+        for (int q = 0; q < 4; ++q) {
+          SliceRowJob y{};
+          y.rows = h.nocc;
+          y.cols = h.N;
+          y.n_planes = 1;
+          y.pl[0] = SlicePlanes{pl, (long long)h.nocc * 2 * nw, nw, c.Y.mat(b).ex, c.M.mat(b).ex};
+          y.base = it.Cd;
+          y.ldb = h.Np;
+          y.epi = 1;
+          y.coef = make_double2(0.0, q == 3 ? 2.0 * theta : theta);
+          if (q != 3) y.out = c.Y.mat(b);
+          if (q != 0) {
+            y.dst = q == 3 ? it.Cd : it.Y[q - 1];
+            y.ldd = h.Np;
+          }
+          jS[q].push_back(y);
+        }
+      }
+    }
+    R.n = R.nH = (int)jC.size();
+    std::string msg;
+    ctx->rounds.push_back(R);
+    SliceRound& Q = ctx->rounds.back();
+    if (slice_gemm_create(fams, pD, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.gD, &msg) ||
+        slice_gemm_create(fams, pM, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.g2, &msg) ||
+        slice_gemm_create(fams, pS, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.g1, &msg))
+      return fail(ctx, VGTB_E_CUDA, "sliced product plan: %s", msg.c_str());
+    TRY(upload(ctx, &Q.tC, tC.data(), tC.size()));
+    TRY(upload(ctx, &Q.jC, jC.data(), jC.size()));
+    TRY(upload(ctx, &Q.jDout, jD.data(), jD.size()));
+    TRY(upload(ctx, &Q.jH, jH.data(), jH.size()));
+    TRY(upload(ctx, &Q.jM, jM.data(), jM.size()));
+    TRY(upload(ctx, &Q.jC0, jC0.data(), jC0.size()));
+    for (int q = 0; q < 4; ++q) TRY(upload(ctx, &Q.jS[q], jS[q].data(), jS[q].size()));
+    CK(cudaStreamSynchronize(ctx->stream));  // the lists leave scope
+  }
+  return VGTB_OK;
+}
+
 // ---------------------------------------------------------------------------
 // one step for every trajectory; ev != nullptr records 7 timing events (as
 // external event nodes when the stream is being captured into a graph)
@@ -1156,12 +1322,21 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
 int build_cn_lists(vgtb_ctx* ctx) {
   const int m = ctx->opt.cn_iter, n = ctx->n_items;
   const double theta = 0.5 * ctx->sys[0].dt;
-  std::vector<GemmF64Item> gD(n), gM(n);
-  std::vector<std::vector<GemmF64Item>> gs(m, std::vector<GemmF64Item>(n));
-  std::vector<CnCheckItem> ck(n);
+  std::vector<GemmF64Item> gD, gM;
+  std::vector<std::vector<GemmF64Item>> gs(m);
+  std::vector<CnCheckItem> ck;
   for (int i = 0; i < n; ++i) {
     const DevItem& it = ctx->items_h[i];
     const HostSys& h = ctx->sys[it.sys];
+    CnCheckItem c{};
+    c.a = it.Y[(m - 1) & 1];
+    c.b = it.Y[(m - 2) & 1];
+    c.rows = h.nocc;
+    c.cols = h.N;
+    c.ld = h.Np;
+    c.traj = it.traj;
+    ck.push_back(c);
+    if (h.slice) continue;  // the products below are the sliced ones (slice_build_cn)
     const size_t NN = (size_t)h.Np * h.Np;
     GemmF64Item d{};  // D = 2 C C^dagger: both operands are read as conj-transposed rows of C^dagger
     d.A[0] = it.Cd;
@@ -1174,7 +1349,7 @@ int build_cn_lists(vgtb_ctx* ctx) {
     d.C = it.D[0];
     d.epi = 1;
     d.coef = make_double2(2.0, 0.0);
-    gD[i] = d;
+    gD.push_back(d);
     GemmF64Item mm{};  // M = S^-1 H = S^-1 (H^dagger)
     mm.A[0] = h.Sinv + it.k * NN;
     mm.R[0] = it.H;
@@ -1183,7 +1358,7 @@ int build_cn_lists(vgtb_ctx* ctx) {
     mm.nseg = 1;
     mm.M = mm.N = mm.ldc = h.Np;
     mm.C = it.W;
-    gM[i] = mm;
+    gM.push_back(mm);
     for (int j = 1; j <= m; ++j) {
       GemmF64Item s{};  // out = C^dagger + coef (Y^dagger M^dagger)
       s.A[0] = (j == 1) ? it.Cd : it.Y[(j - 1) & 1];
@@ -1199,17 +1374,10 @@ int build_cn_lists(vgtb_ctx* ctx) {
       s.ldb = h.Np;
       s.coef = make_double2(0.0, j == m ? 2.0 * theta : theta);
       s.C = (j == m) ? it.Cd : it.Y[j & 1];
-      gs[j - 1][i] = s;
+      gs[j - 1].push_back(s);
     }
-    CnCheckItem c{};
-    c.a = it.Y[(m - 1) & 1];
-    c.b = it.Y[(m - 2) & 1];
-    c.rows = h.nocc;
-    c.cols = h.N;
-    c.ld = h.Np;
-    c.traj = it.traj;
-    ck[i] = c;
   }
+  ctx->n_dense = (int)gD.size();
   TRY(upload(ctx, &ctx->d_gD, gD.data(), gD.size()));
   TRY(upload(ctx, &ctx->d_gM, gM.data(), gM.size()));
   ctx->sweep.assign(m, nullptr);
@@ -1229,10 +1397,39 @@ int build_cn_lists(vgtb_ctx* ctx) {
 // D_k = 2 C_k C_k^dagger for the charge, current and energy sums: at H's nonzero
 // pattern only when the sampled kernel is set up, else the dense product
 void launch_cn_density(vgtb_ctx* ctx, cudaStream_t st) {
-  if (ctx->d_cnd)
-    launch_cn_density_pattern(ctx->d_cnd, ctx->d_bsrsys, ctx->n_items, ctx->bsr_grp_max, ctx->bsr_ent_max, st);
-  else
-    launch_gemm_f64(ctx->d_gD, ctx->n_items, ctx->max_Np, ctx->max_Np, nullptr, st);
+  if (ctx->n_dense == 0) {
+  } else if (ctx->d_cnd) {
+    launch_cn_density_pattern(ctx->d_cnd, ctx->d_bsrsys, ctx->n_dense, ctx->bsr_grp_max, ctx->bsr_ent_max, st);
+  } else {
+    launch_gemm_f64(ctx->d_gD, ctx->n_dense, ctx->max_Np, ctx->max_Np, nullptr, st);
+  }
+  // sliced systems: the whole D
+  for (const SliceRound& r : ctx->rounds) {
+    launch_conj_transpose_items(r.tC, r.n, r.max_N, r.max_nocc, st);
+    launch_slice_rows(r.jC, r.n, r.max_N, r.max_nocc, ctx->slice_mp, nullptr, st);
+    slice_gemm_launch(r.gD, st);
+    launch_slice_rows(r.jDout, r.n, r.max_N, r.max_N, ctx->slice_mp, nullptr, st);
+  }
+}
+
+// M = S^-1 H of a round's items, as digits
+void launch_cn_m(vgtb_ctx* ctx, const SliceRound& r, cudaStream_t st) {
+  launch_slice_pattern(r.jH, r.nH, r.max_nat, ctx->max_orb, st);
+  slice_gemm_launch(r.g2, st);
+  launch_slice_rows(r.jM, r.n, r.max_N, r.max_N, ctx->slice_mp, nullptr, st);
+}
+
+// the fixed-point sweeps of a round: sweep j's epilogue forms C^dagger + coef Y^dagger M^dagger,
+// cuts it into the digits of the next sweep and stores it where the convergence check or the
+// next step reads it (the last two iterates, C^dagger(t_{n+1}))
+void launch_cn_sweeps(vgtb_ctx* ctx, const SliceRound& r, cudaStream_t st) {
+  const int m = ctx->opt.cn_iter;
+  launch_slice_rows(r.jC0, r.n, r.max_nocc, r.max_N, ctx->slice_mp, nullptr, st);
+  for (int j = 1; j <= m; ++j) {
+    slice_gemm_launch(r.g1, st);
+    launch_slice_rows(r.jS[j == m ? 3 : (j >= m - 2 ? 1 + (j & 1) : 0)], r.n, r.max_nocc, r.max_N, ctx->slice_mp,
+                      nullptr, st);
+  }
 }
 
 int enqueue_step_cn(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag) {
@@ -1247,13 +1444,22 @@ int enqueue_step_cn(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag) {
   launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->d_step, PH_FP64_CN, -1,
                st);
   if (ev) CK(cudaEventRecordWithFlags(ev[3], st, evflag));
-  if (ctx->bsr)
-    launch_bsr(ctx->d_bsr, ctx->d_bsrsys, ctx->n_items, ctx->bsr_units_max, ctx->bsr_units_total, ctx->d_bsr_u0,
+  if (ctx->n_dense == 0) {
+  } else if (ctx->bsr) {
+    launch_bsr(ctx->d_bsr, ctx->d_bsrsys, ctx->n_bsr, ctx->bsr_units_max, ctx->bsr_units_total, ctx->d_bsr_u0,
                ctx->d_bsr_ctr, 1, ctx->bsr_tg_max, nullptr, st);
-  else
-    launch_gemm_f64(ctx->d_gM, ctx->n_items, ctx->max_Np, ctx->max_Np, nullptr, st);
+  } else {
+    launch_gemm_f64(ctx->d_gM, ctx->n_dense, ctx->max_Np, ctx->max_Np, nullptr, st);
+  }
+  // every round but the last runs whole, the last one within the event classes
+  for (size_t r = 0; r < ctx->rounds.size(); ++r) {
+    launch_cn_m(ctx, ctx->rounds[r], st);
+    if (r + 1 < ctx->rounds.size()) launch_cn_sweeps(ctx, ctx->rounds[r], st);
+  }
   if (ev) CK(cudaEventRecordWithFlags(ev[4], st, evflag));
-  for (GemmF64Item* g : ctx->sweep) launch_gemm_f64(g, ctx->n_items, ctx->max_nocc, ctx->max_Np, nullptr, st);
+  if (ctx->n_dense)
+    for (GemmF64Item* g : ctx->sweep) launch_gemm_f64(g, ctx->n_dense, ctx->max_nocc, ctx->max_Np, nullptr, st);
+  if (!ctx->rounds.empty()) launch_cn_sweeps(ctx, ctx->rounds.back(), st);
   if (ev) CK(cudaEventRecordWithFlags(ev[5], st, evflag));
   if (ctx->d_cnchk)
     launch_cn_check(ctx->d_cnchk, ctx->n_items, ctx->max_nocc * ctx->max_Np, ctx->d_trj, ctx->opt.cn_tol, st);
@@ -1630,14 +1836,15 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
         it.Xf = fam[T.sys].Xf + 2 * NN * li;
       } else if (ctx->cn) {
         const size_t nc = (size_t)h.nocc * h.Np;
-        if (ctx->bsr) {
+        if (ctx->bsr || h.slice) {
           double2* kh = nullptr;
           if ((rc = dalloc(ctx, &kh, (size_t)h.n_el))) return bail(rc);
           it.kH = kh;
         } else if ((rc = dalloc(ctx, &it.H, NN))) {
           return bail(rc);
         }
-        if ((rc = dalloc(ctx, &it.W, NN))) return bail(rc);
+        if (!h.slice)
+          if ((rc = dalloc(ctx, &it.W, NN))) return bail(rc);
         if ((rc = dalloc(ctx, &it.Cd, nc))) return bail(rc);
         if ((rc = dalloc(ctx, &it.Y[0], nc))) return bail(rc);
         if ((rc = dalloc(ctx, &it.Y[1], nc))) return bail(rc);
@@ -1733,7 +1940,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
   }
   ctx->n_dense = (int)lv.size();
   if (ctx->cn) {
-    if ((rc = build_cn_lists(ctx))) return bail(rc);
+    if ((rc = build_cn_lists(ctx))) return bail(rc);  // sets n_dense
   } else if (!ctx->split) {
     if ((rc = upload(ctx, &ctx->d_g1, g1.data(), g1.size()))) return bail(rc);
     if ((rc = upload(ctx, &ctx->d_g2, g2.data(), g2.size()))) return bail(rc);
@@ -1744,7 +1951,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     std::vector<int> u0(1, 0);
     for (int i = 0; i < ctx->n_items; ++i) {
       const DevItem& it = ctx->items_h[i];
-      if (ctx->sys[it.sys].slice && ctx->opt.product1 != VGTB_P1_BLOCKS) continue;
+      if (ctx->sys[it.sys].slice && (ctx->cn || ctx->opt.product1 != VGTB_P1_BLOCKS)) continue;
       const HostSys& h = ctx->sys[it.sys];
       const size_t NN = (size_t)h.Np * h.Np;
       BsrItem b{};
@@ -1775,10 +1982,10 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     if ((rc = upload(ctx, &ctx->d_bsr_u0, u0.data(), u0.size()))) return bail(rc);
     if ((rc = dalloc(ctx, &ctx->d_bsr_ctr, 2))) return bail(rc);
     if (ctx->cn && ctx->bsr_tg_max <= cn_density_max_targets() && cn_density_configure(ctx->bsr_ent_max) == 0) {
-      std::vector<CnDensItem> cd(ctx->n_items);
+      std::vector<CnDensItem> cd;
       for (int i = 0; i < ctx->n_items; ++i) {
         const DevItem& it = ctx->items_h[i];
-        cd[i] = CnDensItem{it.sys, it.Cd, it.D[0], ctx->sys[it.sys].nocc};
+        if (!ctx->sys[it.sys].slice) cd.push_back(CnDensItem{it.sys, it.Cd, it.D[0], ctx->sys[it.sys].nocc});
       }
       if ((rc = upload(ctx, &ctx->d_cnd, cd.data(), cd.size()))) return bail(rc);
     }
@@ -1787,7 +1994,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
   for (int s = 0; s < n_sys; ++s) {
     if ((rc = build_sinv(ctx, s))) return bail(rc);
   }
-  if ((rc = slice_build(ctx, lv_slice))) return bail(rc);
+  if ((rc = ctx->cn ? slice_build_cn(ctx) : slice_build(ctx, lv_slice))) return bail(rc);
   if (ctx->split) {
     std::vector<TcSysView> views(n_sys);
     for (int s = 0; s < n_sys; ++s) {
@@ -2051,7 +2258,9 @@ int vgtb_get_density(vgtb_ctx* ctx, int t, int k, double* d_out) {
   const size_t NN = (size_t)h.Np * h.Np;
   const int cur = ctx->n_done & 1;
   // Crank-Nicolson steps form D only at H's nonzero pattern: the whole D = 2 C C^dagger now
-  if (ctx->cn && ctx->d_cnd) launch_gemm_f64(ctx->d_gD, ctx->n_items, ctx->max_Np, ctx->max_Np, nullptr, ctx->stream);
+  // (sliced systems form the whole D at every level)
+  if (ctx->cn && ctx->d_cnd && ctx->n_dense)
+    launch_gemm_f64(ctx->d_gD, ctx->n_dense, ctx->max_Np, ctx->max_Np, nullptr, ctx->stream);
   std::vector<double2> a(NN), b;
   CK(cudaMemcpyAsync(a.data(), it.D[cur], NN * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream));
   if (ctx->delta) {
@@ -2262,6 +2471,7 @@ void vgtb_destroy(vgtb_ctx* ctx) {
   for (auto& r : ctx->rounds) {
     slice_gemm_destroy(r.g1);
     slice_gemm_destroy(r.g2);
+    slice_gemm_destroy(r.gD);
   }
   tc_destroy_chain(ctx->tcc);
   tc_destroy_plan(ctx->tc1);

@@ -252,6 +252,15 @@ void launch_cn_check(const CnCheckItem* items, int n_items, int max_elems, const
 // dst[r][c] = conj(src[c][r]) for r < rows, c < cols (dst row stride ldd, src row stride lds)
 void launch_conj_transpose(const double2* src, int lds, double2* dst, int ldd, int rows, int cols, cudaStream_t st);
 
+// the same for a list (grid over max_rows x max_cols of dst)
+struct ConjTItem {
+  const double2* src;
+  int lds;
+  double2* dst;
+  int ldd, rows, cols;
+};
+void launch_conj_transpose_items(const ConjTItem* items, int n_items, int max_rows, int max_cols, cudaStream_t st);
+
 // What the phase-build kernel writes.
 enum PhaseMode : int {
   PH_FP64_PLAIN = 0,   // H = H0 + (alpha + (eps_I+eps_J)/2) S + (i/c) A.dS  -> item.H
