@@ -619,7 +619,9 @@ __global__ void __launch_bounds__(256) k_phase(const DevSys* __restrict__ sysv, 
   const double ebar = 0.5 * (eI + eJ);
   const double beta = (mode == PH_FP64_PLAIN) ? alpha + ebar : ebar;
   const double dbeta = (mode == PH_FP64_PLAIN) ? 0.0 : 0.5 * ((T.eps[I] - S.eps0[I]) + (T.eps[J] - S.eps0[J]));
-  for (int k = 0; k < S.nk; ++k) {
+  // one k-point per grid row: a few atoms at many k-points would otherwise leave most SMs idle and
+  // walk k-points x images one after the other (8 atoms, 8 k-points: 37 us)
+  for (int k = blockIdx.y; k < S.nk; k += gridDim.y) {
     const DevItem& it = items[T.item0 + k];
     for (int e = lane; e < nel; e += 16) {
       const int a = e / nj, b = e - a * nj;
@@ -651,10 +653,11 @@ __global__ void __launch_bounds__(256) k_phase(const DevSys* __restrict__ sysv, 
 }
 
 void launch_phase(const DevSys* sys, const DevTraj* trj, const DevItem* items, const int* warp_prefix,
-                  int n_traj, int total_units, const int* step, int mode, int fixed_step, cudaStream_t st) {
-  const int threads = 256;
+                  int n_traj, int total_units, int max_nk, const int* step, int mode, int fixed_step,
+                  cudaStream_t st) {
+  const int threads = 128;
   const int blocks = (total_units * 16 + threads - 1) / threads;
-  launch_pdl(k_phase, blocks, threads, 0, st, sys, trj, items, warp_prefix, n_traj, total_units, step, mode,
+  launch_pdl(k_phase, dim3(blocks, max_nk), threads, 0, st, sys, trj, items, warp_prefix, n_traj, total_units, step, mode,
              fixed_step);
 }
 

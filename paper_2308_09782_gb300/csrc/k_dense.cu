@@ -110,8 +110,99 @@ __global__ void __launch_bounds__(256) k_gemm_f64(const GemmF64Item* __restrict_
   }
 }
 
+// Small products (the sliced tensor-core products take over from kSliceMinN orbitals): 8 x 8 output
+// tile per CTA of 64 threads, one output each, so that even 32 orbitals at 8 k-points give 128
+// CTAs; an SM issues an FP64 warp instruction about every 18 clocks, so what counts is how many SMs
+// take part.  K tiles of 32, the next one loaded into registers while the current one is used.  The
+// sums run over k in the order of k_gemm_f64.  32 orbitals x 8 k-points: 531 us with the 64 x 64
+// tiles over the 128 padded orbitals (32 CTAs).
+constexpr int GS = 8, GSK = 32;
+
+__global__ void __launch_bounds__(GS* GS) k_gemm_f64_small(const GemmF64Item* __restrict__ items,
+                                                           const int* __restrict__ step) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ double2 As[GSK][GS + 1];
+  __shared__ double2 Rs[GSK][GS + 1];
+  const GemmF64Item& it = items[blockIdx.z];
+  const int m0 = blockIdx.y * GS, n0 = blockIdx.x * GS;
+  const int M = it.M, N = it.N;
+  if (m0 >= M || n0 >= N) return;
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int par = step ? (*step & 1) : 0;
+  const bool ta = it.conj_t & 1, tr = (it.conj_t >> 1) & 1;
+  double cr = 0.0, ci = 0.0;
+  for (int sg = 0; sg < it.nseg; ++sg) {
+    const double2* A = it.A[sg] + par * it.a_par[sg];
+    const double2* R = it.R[sg];
+    const int K = it.K[sg], lda = it.lda[sg], ldr = it.ldr[sg];
+    double2 av[4], rv[4];
+    // element p of this thread: row idx / 32, k idx % 32 (a conjugate-transposed operand: idx % 8, idx / 8)
+    auto load = [&](const double2* X, int ld, int x0, int lim, bool t, int k0, double2(&v)[4]) {
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const int idx = tid + 64 * p;
+        const int r = x0 + (t ? idx & 7 : idx >> 5), k = k0 + (t ? idx >> 3 : idx & 31);
+        v[p] = make_double2(0.0, 0.0);
+        if (r < lim && k < K) {
+          v[p] = t ? X[(long long)k * ld + r] : X[(long long)r * ld + k];
+          if (t) v[p].y = -v[p].y;
+        }
+      }
+    };
+    load(A, lda, m0, M, ta, 0, av);
+    load(R, ldr, n0, N, tr, 0, rv);
+    for (int k0 = 0; k0 < K; k0 += GSK) {
+      __syncthreads();  // the previous tile's readers are done
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const int idx = tid + 64 * p;
+        if (ta)
+          As[idx >> 3][idx & 7] = av[p];
+        else
+          As[idx & 31][idx >> 5] = av[p];
+        if (tr)
+          Rs[idx >> 3][idx & 7] = rv[p];
+        else
+          Rs[idx & 31][idx >> 5] = rv[p];
+      }
+      __syncthreads();
+      if (k0 + GSK < K) {
+        load(A, lda, m0, M, ta, k0 + GSK, av);
+        load(R, ldr, n0, N, tr, k0 + GSK, rv);
+      }
+#pragma unroll 8
+      for (int kk = 0; kk < GSK; ++kk) {
+        const double2 a = As[kk][ty], b = Rs[kk][tx];
+        cr = fma(a.x, b.x, cr);
+        cr = fma(a.y, b.y, cr);
+        ci = fma(a.y, b.x, ci);
+        ci = fma(-a.x, b.y, ci);
+      }
+    }
+  }
+  const int gm = m0 + ty, gn = n0 + tx;
+  if (gm >= M || gn >= N) return;
+  double2 v = make_double2(cr, ci);
+  if (it.epi == 1) {
+    const double2 c = it.coef;
+    v = make_double2(c.x * v.x - c.y * v.y, c.x * v.y + c.y * v.x);
+    if (it.base) {
+      const double2 b = it.base[(long long)gm * it.ldb + gn];
+      v.x += b.x;
+      v.y += b.y;
+    }
+  }
+  it.C[(long long)gm * it.ldc + gn] = v;
+}
+
 void launch_gemm_f64(const GemmF64Item* items, int n_items, int max_m, int max_n, const int* step,
                      cudaStream_t st) {
+  if (std::max(max_m, max_n) <= kGemmSmall) {
+    launch_pdl(k_gemm_f64_small, dim3((max_n + GS - 1) / GS, (max_m + GS - 1) / GS, n_items), GS * GS, 0, st, items,
+               step);
+    return;
+  }
   dim3 grid((max_n + GT - 1) / GT, (max_m + GT - 1) / GT, n_items);
   launch_pdl(k_gemm_f64, grid, 256, 0, st, items, step);
 }

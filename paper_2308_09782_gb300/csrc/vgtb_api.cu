@@ -137,6 +137,7 @@ struct vgtb_ctx {
   LeapItem* d_leap = nullptr;
   int n_items = 0;
   int n_dense = 0;                 // items of the lists above (the others take the sliced products)
+  int max_dense = 0, max_dense_occ = 0;  // their largest matrix size and count of occupied states
   std::vector<SliceRound> rounds;  // sliced FP64 products
   int slice_mp = 7, max_orb = 1;
   int* d_slice_err = nullptr;
@@ -1345,7 +1346,8 @@ int build_cn_lists(vgtb_ctx* ctx) {
     d.lda[0] = d.ldr[0] = h.Np;
     d.nseg = 1;
     d.conj_t = 3;
-    d.M = d.N = d.ldc = h.Np;
+    d.M = d.N = h.N;
+    d.ldc = h.Np;
     d.C = it.D[0];
     d.epi = 1;
     d.coef = make_double2(2.0, 0.0);
@@ -1353,21 +1355,22 @@ int build_cn_lists(vgtb_ctx* ctx) {
     GemmF64Item mm{};  // M = S^-1 H = S^-1 (H^dagger)
     mm.A[0] = h.Sinv + it.k * NN;
     mm.R[0] = it.H;
-    mm.K[0] = h.Np;
+    mm.K[0] = h.N;
     mm.lda[0] = mm.ldr[0] = h.Np;
     mm.nseg = 1;
-    mm.M = mm.N = mm.ldc = h.Np;
+    mm.M = mm.N = h.N;
+    mm.ldc = h.Np;
     mm.C = it.W;
     gM.push_back(mm);
     for (int j = 1; j <= m; ++j) {
       GemmF64Item s{};  // out = C^dagger + coef (Y^dagger M^dagger)
       s.A[0] = (j == 1) ? it.Cd : it.Y[(j - 1) & 1];
       s.R[0] = it.W;
-      s.K[0] = h.Np;
+      s.K[0] = h.N;
       s.lda[0] = s.ldr[0] = h.Np;
       s.nseg = 1;
       s.M = h.nocc;
-      s.N = h.Np;
+      s.N = h.N;
       s.ldc = h.Np;
       s.epi = 1;
       s.base = it.Cd;
@@ -1401,7 +1404,7 @@ void launch_cn_density(vgtb_ctx* ctx, cudaStream_t st) {
   } else if (ctx->d_cnd) {
     launch_cn_density_pattern(ctx->d_cnd, ctx->d_bsrsys, ctx->n_dense, ctx->bsr_grp_max, ctx->bsr_ent_max, st);
   } else {
-    launch_gemm_f64(ctx->d_gD, ctx->n_dense, ctx->max_Np, ctx->max_Np, nullptr, st);
+    launch_gemm_f64(ctx->d_gD, ctx->n_dense, ctx->max_dense, ctx->max_dense, nullptr, st);
   }
   // sliced systems: the whole D
   for (const SliceRound& r : ctx->rounds) {
@@ -1441,15 +1444,15 @@ int enqueue_step_cn(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag) {
   if (ev) CK(cudaEventRecordWithFlags(ev[1], st, evflag));
   launch_scc(ctx->d_sys, ctx->d_trj, nt, ctx->d_step, stride, -1, 1, ctx->max_nat, 0, st);
   if (ev) CK(cudaEventRecordWithFlags(ev[2], st, evflag));
-  launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->d_step, PH_FP64_CN, -1,
-               st);
+  launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk, ctx->d_step,
+               PH_FP64_CN, -1, st);
   if (ev) CK(cudaEventRecordWithFlags(ev[3], st, evflag));
   if (ctx->n_dense == 0) {
   } else if (ctx->bsr) {
     launch_bsr(ctx->d_bsr, ctx->d_bsrsys, ctx->n_bsr, ctx->bsr_units_max, ctx->bsr_units_total, ctx->d_bsr_u0,
                ctx->d_bsr_ctr, 1, ctx->bsr_tg_max, nullptr, st);
   } else {
-    launch_gemm_f64(ctx->d_gM, ctx->n_dense, ctx->max_Np, ctx->max_Np, nullptr, st);
+    launch_gemm_f64(ctx->d_gM, ctx->n_dense, ctx->max_dense, ctx->max_dense, nullptr, st);
   }
   // every round but the last runs whole, the last one within the event classes
   for (size_t r = 0; r < ctx->rounds.size(); ++r) {
@@ -1458,7 +1461,7 @@ int enqueue_step_cn(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag) {
   }
   if (ev) CK(cudaEventRecordWithFlags(ev[4], st, evflag));
   if (ctx->n_dense)
-    for (GemmF64Item* g : ctx->sweep) launch_gemm_f64(g, ctx->n_dense, ctx->max_nocc, ctx->max_Np, nullptr, st);
+    for (GemmF64Item* g : ctx->sweep) launch_gemm_f64(g, ctx->n_dense, ctx->max_dense_occ, ctx->max_dense, nullptr, st);
   if (!ctx->rounds.empty()) launch_cn_sweeps(ctx, ctx->rounds.back(), st);
   if (ev) CK(cudaEventRecordWithFlags(ev[5], st, evflag));
   if (ctx->d_cnchk)
@@ -1519,7 +1522,7 @@ int enqueue_step(vgtb_ctx* ctx, cudaEvent_t* ev) {
     launch_phase_split(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk,
                        ctx->d_step, 1, st);
   else
-    launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->d_step,
+    launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk, ctx->d_step,
                  ctx->delta ? PH_FP64_DELTA : PH_FP64_PLAIN, -1, st);
   if (ev) CK(cudaEventRecordWithFlags(ev[3], st, evflag));
   if (ctx->bsr && ctx->n_bsr > 0)
@@ -1536,7 +1539,7 @@ int enqueue_step(vgtb_ctx* ctx, cudaEvent_t* ev) {
     TRY(tc_launch(ctx->tc2, st) == 0 ? VGTB_OK : fail(ctx, VGTB_E_CUDA, "tcgen05 product 2 launch failed"));
   } else {
     if (!ctx->bsr && ctx->n_dense)
-      launch_gemm_f64(ctx->d_g1, ctx->n_dense, ctx->max_Np, ctx->max_Np, ctx->d_step, st);
+      launch_gemm_f64(ctx->d_g1, ctx->n_dense, ctx->max_dense, ctx->max_dense, ctx->d_step, st);
     // every round but the last runs whole, the last one within the event classes
     for (size_t r = 0; r < ctx->rounds.size(); ++r) {
       TRY(launch_slice_first(ctx, ctx->rounds[r], st));
@@ -1546,7 +1549,7 @@ int enqueue_step(vgtb_ctx* ctx, cudaEvent_t* ev) {
                   ctx->sys[0].dt, nullptr, nullptr, st);
     }
     if (ev) CK(cudaEventRecordWithFlags(ev[4], st, evflag));
-    if (ctx->n_dense) launch_gemm_f64(ctx->d_g2, ctx->n_dense, ctx->max_Np, ctx->max_Np, ctx->d_step, st);
+    if (ctx->n_dense) launch_gemm_f64(ctx->d_g2, ctx->n_dense, ctx->max_dense, ctx->max_dense, ctx->d_step, st);
     if (!ctx->rounds.empty()) TRY(launch_slice_second(ctx, ctx->rounds.back(), st));
   }
   if (ev) CK(cudaEventRecordWithFlags(ev[5], st, evflag));
@@ -1751,9 +1754,11 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
   ctx->bsr = blocks_ok &&
              (ctx->opt.product1 == VGTB_P1_BLOCKS || (ctx->opt.product1 == VGTB_P1_AUTO && !ctx->split));
   slice_choose(ctx);
-  bool all_slice = true;
-  for (auto& h : ctx->sys) all_slice = all_slice && h.slice;
-  if (all_slice && ctx->opt.product1 == VGTB_P1_AUTO) ctx->bsr = false;
+  // the block-sparse kernel is left for explicit requests and for systems that take neither the
+  // sliced products nor the small dense ones (64 orbitals: dense 8 us, block-sparse 79 us)
+  bool other = false;
+  for (auto& h : ctx->sys) other = other || !(h.slice || h.N <= kGemmSmall);
+  if (!other && !ctx->split && ctx->opt.product1 == VGTB_P1_AUTO) ctx->bsr = false;
   std::vector<BsrSys> bsys(n_sys);
   if (ctx->bsr) {
     for (int s = 0; s < n_sys; ++s) {
@@ -1899,26 +1904,30 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     a.A[0] = it.D[0];
     a.a_par[0] = (long long)NN;
     a.R[0] = it.H;
-    a.K[0] = h.Np;
+    a.K[0] = h.N;  // padding rows and columns are zero and stay so
     a.lda[0] = a.ldr[0] = h.Np;
     a.nseg = 1;
     if (ctx->delta) {
       a.A[1] = h.D0 + it.k * NN;
       a.R[1] = it.dH;
-      a.K[1] = h.Np;
+      a.K[1] = h.N;
       a.lda[1] = a.ldr[1] = h.Np;
       a.nseg = 2;
     }
-    a.M = a.N = a.ldc = h.Np;
+    a.M = a.N = h.N;
+    a.ldc = h.Np;
     a.C = it.W;
     b.A[0] = h.Sinv + it.k * NN;
     b.R[0] = it.W;
-    b.K[0] = h.Np;
+    b.K[0] = h.N;
     b.lda[0] = b.ldr[0] = h.Np;
     b.nseg = 1;
-    b.M = b.N = b.ldc = h.Np;
+    b.M = b.N = h.N;
+    b.ldc = h.Np;
     b.C = it.X;
     if (!h.slice) {
+      ctx->max_dense = std::max(ctx->max_dense, h.N);
+      ctx->max_dense_occ = std::max(ctx->max_dense_occ, h.nocc);
       g1.push_back(a);
       g2.push_back(b);
     }
@@ -2260,7 +2269,7 @@ int vgtb_get_density(vgtb_ctx* ctx, int t, int k, double* d_out) {
   // Crank-Nicolson steps form D only at H's nonzero pattern: the whole D = 2 C C^dagger now
   // (sliced systems form the whole D at every level)
   if (ctx->cn && ctx->d_cnd && ctx->n_dense)
-    launch_gemm_f64(ctx->d_gD, ctx->n_dense, ctx->max_Np, ctx->max_Np, nullptr, ctx->stream);
+    launch_gemm_f64(ctx->d_gD, ctx->n_dense, ctx->max_dense, ctx->max_dense, nullptr, ctx->stream);
   std::vector<double2> a(NN), b;
   CK(cudaMemcpyAsync(a.data(), it.D[cur], NN * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream));
   if (ctx->delta) {

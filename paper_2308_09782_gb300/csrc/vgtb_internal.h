@@ -285,8 +285,9 @@ void launch_obs_atoms_split(const DevSys* sys, DevTraj* trj, const DevItem* item
 void launch_phase_split(const DevSys* sys, DevTraj* trj, const DevItem* items, const int* warp_prefix,
                         int n_traj, int total_units, int max_nk, const int* step, int finish, cudaStream_t st);
 void launch_to_planar_f32(const double2* src, float* dst, int Np, cudaStream_t st);
+// grid rows = max_nk, as launch_phase_split
 void launch_phase(const DevSys* sys, const DevTraj* trj, const DevItem* items, const int* warp_prefix,
-                  int n_traj, int total_warps, const int* step, int mode, int fixed_step, cudaStream_t st);
+                  int n_traj, int total_warps, int max_nk, const int* step, int mode, int fixed_step, cudaStream_t st);
 int scc_configure(int max_nat);
 void launch_kblocks(const DevSys* sys, int s_idx, int n_tgt, int k, cudaStream_t st);
 void launch_obs0(const DevSys* sys, int s_idx, int n_tgt, int nat, int split, cudaStream_t st);
@@ -309,6 +310,7 @@ struct GemmF64Item {
   const double2* base;     // may alias C (element-wise read-before-write by one thread)
   int ldb;
 };
+constexpr int kGemmSmall = 96;  // products up to this size take 8 x 8 tiles instead of 64 x 64
 void launch_gemm_f64(const GemmF64Item* items, int n_items, int max_m, int max_n, const int* step,
                      cudaStream_t st);
 
