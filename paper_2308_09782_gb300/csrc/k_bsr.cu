@@ -477,11 +477,11 @@ size_t bsr_smem_bytes(int fp64, int max_grp_targets) {
 
 int bsr_configure(int fp64, int max_grp_targets) {
   const size_t smem = fp64 ? bsr_smem_bytes(1, max_grp_targets) : bsr_p_smem_bytes(max_grp_targets);
-  if (smem > kSmemLimit) return -1;
+  if (smem > kSmemLimit - (fp64 ? 0 : 128)) return -1;
   cudaError_t e = fp64 ? cudaFuncSetAttribute(k_bsr<double, kBsrGroupF64>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit)
                        : cudaFuncSetAttribute(k_bsr_f32p, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)kSmemLimit);
+                                              (int)kSmemLimit - 128);  // it holds a static word beside
   return e == cudaSuccess ? 0 : -1;
 }
 
