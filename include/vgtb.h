@@ -268,7 +268,7 @@ int vgtb_kernel_stats(vgtb_ctx* ctx, long long* launches, double* ms, int n);
  * create (variant 0, or the autotuner's fastest).  cfg[4] = {tile width,
  * pipeline stages, schedule (0 classic, 1 stream-K, 2 whole waves classic and
  * stream-K over the rest; + 4: the k-panels skipped in which the tile's rows
- * of H_k and dH_k are zero, product 1 only; + 8: classic over column tiles of
+ * of H_k and dH_k are zero (product 1), or the imaginary half of a real S_k^-1 (product 2); + 8: classic over column tiles of
  * planned widths, multiples of 16, the tile width being the widest; + 16: both
  * products run as one launch, VGTB_CHAIN_*), 1 if the tile spans a 2-SM CTA pair}.  When the first product runs block-sparse
  * (VGTB_P1_BLOCKS), product 1 reports {atoms per group, output rows per CTA, 3, 0}.

@@ -266,13 +266,14 @@ static std::vector<int> even_split(int total, int n) {
 // of G workers when all its tiles (n_items x tiles_m row tiles) are assigned
 // longest first.  With the zero k-panels skipped a tile's k-iterations are its
 // panel count.
-static std::vector<int> plan_columns(const TcSysView& v, bool skip, int nseg, int tiles_m, int G, int mode) {
+// `full`: k-iterations of a tile whose panels are not skipped.
+static std::vector<int> plan_columns(const TcSysView& v, bool skip, int nseg, int full, int tiles_m, int G, int mode) {
   const int total = 2 * v.Np, n0 = (total + 255) / 256;
   std::vector<std::pair<double, int>> score;
   for (int n = n0; n <= std::max(total / 96, n0); ++n) {
     const std::vector<int> st = even_split(total, n);
     if (mode == 2 && n > n0 && st[n] - st[n - 1] < 192) continue;
-    std::vector<int> kt(n, nseg * total / BK);
+    std::vector<int> kt(n, full);
     if (skip) {
       std::vector<int> kofs;
       std::vector<short> kidx;
@@ -314,12 +315,17 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
   bool skip = epi == 0;
   const bool uniform = var.streamk != 0;
   for (const TcSysView& v : sys) skip = skip && v.orb_off && v.tgt_I && v.tgt_J;
+  // product 2 at a k-point with a real S_k^-1: the imaginary half of its k-panels is zero
+  auto k_real = [&](const TcSysView& v, int k) { return v.k_real && (*v.k_real)[k] != 0; };
+  int n_real = 0;
+  for (const DevItem& it : items) n_real += k_real(sys[it.sys], it.k) ? 1 : 0;
   // column tiles of every system
   std::vector<std::vector<int>> starts(sys.size());
   int wmax = 0;
   for (size_t s = 0; s < sys.size(); ++s) {
     const int tiles_m = (sys[s].Np + tm_rows - 1) / tm_rows;
-    starts[s] = var.widths ? plan_columns(sys[s], skip, nseg, tiles_m, G_full, var.widths)
+    const int full = nseg * 2 * sys[s].Np / BK / (epi == 1 && n_real == (int)items.size() ? 2 : 1);
+    starts[s] = var.widths ? plan_columns(sys[s], skip, nseg, full, tiles_m, G_full, var.widths)
                            : even_split(2 * sys[s].Np, 2 * sys[s].Np / BNv);
     for (size_t i = 0; i + 1 < starts[s].size(); ++i) wmax = std::max(wmax, starts[s][i + 1] - starts[s][i]);
   }
@@ -342,11 +348,18 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
   std::vector<int> sys_kofs0(sys.size(), 0), sys_kidx0(sys.size(), 0), sys_cofs0(sys.size(), 0), all_kofs, all_cofs;
   std::vector<short> all_kidx;
   std::vector<std::vector<int>> sys_cnt(sys.size());
-  if (skip) {
+  if (skip || (epi == 1 && n_real)) {
     for (size_t s = 0; s < sys.size(); ++s) {
-      std::vector<int> kofs;
+      std::vector<int> kofs(1, 0);
       std::vector<short> kidx;
-      zero_panel_lists(sys[s], starts[s], uniform, kofs, kidx);
+      if (skip) {
+        zero_panel_lists(sys[s], starts[s], uniform, kofs, kidx);
+      } else {
+        for (size_t i = 0; i + 1 < starts[s].size(); ++i) {
+          for (int k = 0; k < sys[s].Np / BK; ++k) kidx.push_back((short)k);
+          kofs.push_back((int)kidx.size());
+        }
+      }
       sys_kofs0[s] = (int)all_kofs.size();
       sys_kidx0[s] = (int)all_kidx.size();
       for (size_t i = 0; i + 1 < kofs.size(); ++i) sys_cnt[s].push_back(kofs[i + 1] - kofs[i]);
@@ -394,6 +407,7 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
       pr.a_b[1] = it.k;
       pr.b_b[1] = li;
       pr.out = it.Wemb_p;
+      pr.w_half = k_real(v, it.k) ? 1 : 0;
     } else {
       pr.a_b[0] = it.k;
       pr.b_b[0] = li;
@@ -401,7 +415,8 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
     }
     pr.kt = nseg * (2 * v.Np) / BK;
     pr.iter0 = (int)iters;
-    if (skip) {
+    const bool listed = skip || (epi == 1 && k_real(v, it.k));
+    if (listed) {
       pr.kofs = plan->d_kofs + sys_kofs0[it.sys];
       pr.kidx = plan->d_kidx + sys_kidx0[it.sys];
       pr.kt = nseg * sys_cnt[it.sys][0];  // every segment takes the panel list (uniform lists: one length)
@@ -409,7 +424,7 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
     if (var.widths) pr.cofs = plan->d_cofs + sys_cofs0[it.sys];
     for (int nt = 0; nt < pr.tiles_n; ++nt)
       for (int mt = 0; mt < pr.tiles_m; ++mt)
-        tile_cost.push_back(tile_model(st[nt + 1] - st[nt], skip ? nseg * sys_cnt[it.sys][nt] : pr.kt));
+        tile_cost.push_back(tile_model(st[nt + 1] - st[nt], listed ? nseg * sys_cnt[it.sys][nt] : pr.kt));
     tiles += pr.tiles_m * pr.tiles_n;
     iters += (long long)pr.tiles_m * pr.tiles_n * pr.kt;
     probs.push_back(pr);
@@ -433,7 +448,8 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
   plan->grid = std::min(tiles, nsm);
   plan->smem = variant_smem(variant);
   if (pair) plan->grid = 2 * std::min(tiles, nsm / 2);
-  if (!var.streamk && ((skip && !uniform) || var.widths)) {
+  const bool mixed = epi == 1 && n_real > 0 && n_real < (int)items.size();
+  if (!var.streamk && ((skip && !uniform) || var.widths || mixed)) {
     // tiles of unequal cost: longest first, each to the least loaded worker
     const std::vector<int> tord = lpt_order(tile_cost, pair ? plan->grid / 2 : plan->grid, nullptr);
     if (cudaMalloc(&plan->d_tord, sizeof(int) * tord.size()) != cudaSuccess) {

@@ -49,8 +49,10 @@ struct TcProb {
   // classic schedule with zero panels skipped (null = every panel): the
   // 64-wide k-panels of one segment in which the B rows of column tile nt have
   // a nonzero are kidx[kofs[nt] .. kofs[nt+1]-1]; every segment uses the list
+  // (product 2 of a real S_k^-1: the panels of its real half)
   const int* kofs;
   const short* kidx;
+  int w_half;          // product 1: product 2 reads only the left half [Re W; -Im W] of the embedded W
   // 2-SM pair kernel, classic schedule: first B row of each column tile
   // (tiles_n + 1 entries, the last 2 Np; widths multiples of 16 up to 256, so
   // that the tiles can be balanced over the workers); null = tiles of 256
@@ -366,8 +368,9 @@ __device__ __forceinline__ uint4 pack8_bf16(const float (&x)[16], int h, float s
 // embedded BF16 pieces of W that product 2 reads as its B operand: top row m =
 // [Re W | Im W], bottom row Np + m = [-Im W | Re W], hi at 0 and lo at 4 Np^2.
 // (nh = 1: only the first 16 accumulator columns are the tile's, 8 W columns).
+// half: only [Re W] of the top and [-Im W] of the bottom row (w_half).
 __device__ __forceinline__ void store_w_pieces(__nv_bfloat16* W, int Np, int row, int gn, const uint32_t (&r)[32],
-                                               int nh) {
+                                               int nh, int half) {
   const long long ld = 2LL * Np, P1 = 4LL * Np * Np;
   const int j0 = gn >> 1;
   float re[16], im[16], rel[16], iml[16];
@@ -392,10 +395,11 @@ __device__ __forceinline__ void store_w_pieces(__nv_bfloat16* W, int Np, int row
     if (h >= nh) break;
     reinterpret_cast<uint4*>(W + top)[h] = pack8_bf16(re, h, 1.f);
     reinterpret_cast<uint4*>(W + P1 + top)[h] = pack8_bf16(rel, h, 1.f);
-    reinterpret_cast<uint4*>(W + top + Np)[h] = pack8_bf16(im, h, 1.f);
-    reinterpret_cast<uint4*>(W + P1 + top + Np)[h] = pack8_bf16(iml, h, 1.f);
     reinterpret_cast<uint4*>(W + bot)[h] = pack8_bf16(im, h, -1.f);
     reinterpret_cast<uint4*>(W + P1 + bot)[h] = pack8_bf16(iml, h, -1.f);
+    if (half) continue;
+    reinterpret_cast<uint4*>(W + top + Np)[h] = pack8_bf16(im, h, 1.f);
+    reinterpret_cast<uint4*>(W + P1 + top + Np)[h] = pack8_bf16(iml, h, 1.f);
     reinterpret_cast<uint4*>(W + bot + Np)[h] = pack8_bf16(re, h, 1.f);
     reinterpret_cast<uint4*>(W + P1 + bot + Np)[h] = pack8_bf16(rel, h, 1.f);
   }
@@ -596,7 +600,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcPa
                 make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]),
                             __uint_as_float(r[4 * v + 3]));
         } else {
-          store_w_pieces(reinterpret_cast<__nv_bfloat16*>(pr.out), Np, row, gn, r, 2);
+          store_w_pieces(reinterpret_cast<__nv_bfloat16*>(pr.out), Np, row, gn, r, 2, pr.w_half);
         }
       }
       tc_fence_before();
@@ -911,7 +915,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
                   make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
                               __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
         } else {
-          store_w_pieces(reinterpret_cast<__nv_bfloat16*>(pr.out), Np, row, gn, r, nv >> 4);
+          store_w_pieces(reinterpret_cast<__nv_bfloat16*>(pr.out), Np, row, gn, r, nv >> 4, pr.w_half);
         }
       }
       tc_fence_before();

@@ -2016,6 +2016,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
       views[s].Hemb_p = fam[s].Hemb;
       views[s].dHemb_p = fam[s].dHemb;
       views[s].Wemb_p = fam[s].Wemb;
+      views[s].k_real = &ctx->sys[s].k_real;
       if (ctx->opt.product1 != VGTB_P1_DENSE) {  // nonzero pattern: zero k-panels of product 1 are skipped
         views[s].orb_off = &ctx->sys[s].orb_off;
         views[s].tgt_I = &ctx->sys[s].tgt_I;

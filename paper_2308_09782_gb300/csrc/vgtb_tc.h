@@ -26,6 +26,9 @@ struct TcSysView {
   const std::vector<int>* orb_off = nullptr;
   const std::vector<int>* tgt_I = nullptr;
   const std::vector<int>* tgt_J = nullptr;
+  // k-points whose S_k^-1 is real (host data, may be null): product 2 takes only
+  // the real half of its k-panels there, and product 1 stores only what that reads
+  const std::vector<char>* k_real = nullptr;
 };
 
 // Plans for the two products of the split form, over every item:
