@@ -519,7 +519,8 @@ __global__ void __launch_bounds__(kSccThreads) k_scc_eps(const DevSys* __restric
       if (T.eps_lv) T.eps_lv[(long long)(n & 1) * S.nat + I] = eh;
       if (T.epsf) {
         T.epsf[I] = (float)eh;
-        T.depsf[I] = (float)(eh - S.eps0[I]);
+        const float d = (float)(0.5 * (eh - S.eps0[I]));
+        for (int o = S.orb_off[I]; o < S.orb_off[I + 1]; ++o) T.deh[o] = d;
       }
       // this atom's shares of T_x, T_y, T_z, the band energy, dq.eps and the electron count
       const double* a = T.apart + 4LL * I;
@@ -662,7 +663,7 @@ void launch_phase(const DevSys* sys, const DevTraj* trj, const DevItem* items, c
 }
 
 // ---------------------------------------------------------------------------
-// Phase build, split form: the delta-form H and dH summed in FP32 and stored
+// Phase build, split form: the delta-form H (without the |A|^2 term) summed in FP32 and stored
 // either at the target elements in FP32 (block-sparse first product) or as the
 // embedded real matrix [[Re, Im], [-Im, Re]] in BF16 hi/lo pieces (the B
 // operand of the tcgen05 first product), whose rows the first product takes
@@ -772,7 +773,6 @@ __global__ void __launch_bounds__(256, 4) k_phase_split(const DevSys* __restrict
   const bool vec = (t1.z >> 16) != 0;
   const int nel = ni * nj;
   const float beta = 0.5f * (T.epsf[I] + T.epsf[J]);
-  const float dbeta = 0.5f * (T.depsf[I] + T.depsf[J]);
   const long long dss = S.ds_stride;
   // one k-point per grid row (blockIdx.y): the k-points of a target run in parallel
   for (int k = blockIdx.y; k < S.nk; k += gridDim.y) {
@@ -780,7 +780,6 @@ __global__ void __launch_bounds__(256, 4) k_phase_split(const DevSys* __restrict
     if (vec) {
       for (int r = sub; r < ni; r += 4) {
         float hr[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
-        float dr[4] = {0.f, 0.f, 0.f, 0.f}, di[4] = {0.f, 0.f, 0.f, 0.f};
         for (int g = g0; g < g1; ++g) {
           const long long off = S.img_off[g] + 4LL * r;
           const float4 sv = *reinterpret_cast<const float4*>(S.sf + off);
@@ -798,9 +797,6 @@ __global__ void __launch_bounds__(256, 4) k_phase_split(const DevSys* __restrict
             const float vr = h4[j] + beta * s4[j];
             hr[j] += ph.x * vr - ph.y * adS;
             hi[j] += ph.x * adS + ph.y * vr;
-            const float wr = dbeta * s4[j];
-            dr[j] += ph.x * wr - ph.y * adS;
-            di[j] += ph.x * adS + ph.y * wr;
           }
         }
         if (it.kH) {
@@ -808,20 +804,16 @@ __global__ void __launch_bounds__(256, 4) k_phase_split(const DevSys* __restrict
           // atom has 4 orbitals there, so the element index is a multiple of 4)
           const long long ce = S.tgt_el0[U.tg] + 4LL * r;
           float4* h4 = reinterpret_cast<float4*>(reinterpret_cast<float2*>(it.kH) + ce);
-          float4* d4 = reinterpret_cast<float4*>(reinterpret_cast<float2*>(it.kdH) + ce);
           h4[0] = make_float4(hr[0], hi[0], hr[1], hi[1]);
           h4[1] = make_float4(hr[2], hi[2], hr[3], hi[3]);
-          d4[0] = make_float4(dr[0], di[0], dr[1], di[1]);
-          d4[1] = make_float4(dr[2], di[2], dr[3], di[3]);
         } else {
           store_emb_f4(it.Hemb_p, S.Np, oi + r, oj, hr, hi);
-          store_emb_f4(it.dHemb_p, S.Np, oi + r, oj, dr, di);
         }
       }
     } else {
       for (int e = sub; e < nel; e += 4) {
         const int a = e / nj, b = e - a * nj;
-        float hr = 0.f, hi = 0.f, dr = 0.f, di = 0.f;
+        float hr = 0.f, hi = 0.f;
         for (int g = g0; g < g1; ++g) {
           const long long off = S.img_off[g] + e;
           const float sv = S.sf[off], hv = S.h0f[off];
@@ -830,17 +822,12 @@ __global__ void __launch_bounds__(256, 4) k_phase_split(const DevSys* __restrict
           const float vr = hv + beta * sv;
           hr += ph.x * vr - ph.y * adS;
           hi += ph.x * adS + ph.y * vr;
-          const float wr = dbeta * sv;
-          dr += ph.x * wr - ph.y * adS;
-          di += ph.x * adS + ph.y * wr;
         }
         if (it.kH) {
           const long long ce = S.tgt_el0[U.tg] + e;
           reinterpret_cast<float2*>(it.kH)[ce] = make_float2(hr, hi);
-          reinterpret_cast<float2*>(it.kdH)[ce] = make_float2(dr, di);
         } else {
           store_emb_f(it.Hemb_p, S.Np, oi + a, oj + b, hr, hi);
-          store_emb_f(it.dHemb_p, S.Np, oi + a, oj + b, dr, di);
         }
       }
     }

@@ -3,7 +3,7 @@
 //   W = sum_seg A_seg R_seg^dagger
 //
 // FP64 path: W = D H (one segment; D at the level of the step's parity) or, in
-// the delta form, W = dD H + D0 dH.  Split form: W = dD H + D0 dH in FP32 with
+// the delta form, W = dD H + D0 dH.  Split form: W = dD H + G diag(e) in FP32 with
 // the output stored as the embedded BF16 hi/lo pieces that the tcgen05 second
 // product (X = S^-1 W^dagger) reads.
 //
@@ -213,9 +213,8 @@ __global__ void __launch_bounds__(kBsrThreads) k_bsr(const BsrItem* __restrict__
 // 8 x 4 complex accumulators of the group's atoms.  Each thread stages its own
 // four A values of an entry through a ring of kBsrStages shared-memory slots
 // with cp.async (no other thread reads them, so no CTA barrier is needed per
-// entry), so kBsrStages - 1 entries are in flight while one is applied; the
-// ring runs on across the segment boundary.  The R blocks of the group's current
-// segment sit in shared memory.  The last CTA to run out of units resets the
+// entry), so kBsrStages - 1 entries are in flight while one is applied.  The R
+// blocks of the group sit in shared memory; the D0 term G_ij e_j is added at the end.  The last CTA to run out of units resets the
 // counters for the next launch.
 // ---------------------------------------------------------------------------
 constexpr int kBsrPThreads = 128;
@@ -260,18 +259,15 @@ __global__ void __launch_bounds__(kBsrPThreads, 3) k_bsr_f32p(const BsrItem* __r
     const int i = ch * kBsrPThreads + tid;
     const int t0 = S.grp_t0[g], nt = S.grp_t0[g + 1] - t0;
     const int e0 = S.grp_e0[g], ne = S.grp_e0[g + 1] - e0;
-    auto stage_r = [&](int sg) {
-      const float4* R = reinterpret_cast<const float4*>(reinterpret_cast<const float2*>(it.R[sg]) + 16LL * t0);
+    {
+      const float4* R = reinterpret_cast<const float4*>(reinterpret_cast<const float2*>(it.R[0]) + 16LL * t0);
       for (int x = tid; x < 8 * nt; x += kBsrPThreads) sR[x] = R[x];
-    };
-    stage_r(0);
+    }
     __syncthreads();
-    const int nsteps = it.nseg * ne;  // entries of segment 0, then of segment 1
     auto issue = [&](int st) {
-      if (st < nsteps) {
-        const int sg = st >= ne ? 1 : 0;
-        const int e = e0 + st - sg * ne;
-        const float2* p = reinterpret_cast<const float2*>(it.A[sg]) + (long long)(4 * __ldg(S.ent_K + e)) * Np + i;
+      if (st < ne) {
+        const int e = e0 + st;
+        const float2* p = reinterpret_cast<const float2*>(it.A[0]) + (long long)(4 * __ldg(S.ent_K + e)) * Np + i;
         const uint32_t d = sA_u32 + (uint32_t)(((st % kBsrStages) * 4 * kBsrPThreads + tid) * 8);
 #pragma unroll
         for (int r = 0; r < 4; ++r) cp_async8(d + r * kBsrPThreads * 8, p + (long long)r * Np);
@@ -285,16 +281,10 @@ __global__ void __launch_bounds__(kBsrPThreads, 3) k_bsr_f32p(const BsrItem* __r
     for (int j = 0; j < kBsrGroupF32; ++j)
 #pragma unroll
       for (int c = 0; c < 4; ++c) ar[j][c] = ai[j][c] = 0.f;
-    for (int st = 0; st < nsteps; ++st) {
-      if (st == ne) {  // segment 1 begins: its R blocks replace segment 0's
-        __syncthreads();
-        stage_r(1);
-        __syncthreads();
-      }
+    for (int st = 0; st < ne; ++st) {
       issue(st + kBsrStages - 1);
       cp_async_wait<kBsrStages - 1>();
-      const int sg = st >= ne ? 1 : 0;
-      const int e = e0 + st - sg * ne;
+      const int e = e0 + st;
       const float2* a_s = sA + (st % kBsrStages) * 4 * kBsrPThreads + tid;
       const float2 a0 = a_s[0], a1 = a_s[kBsrPThreads], a2 = a_s[2 * kBsrPThreads], a3 = a_s[3 * kBsrPThreads];
       const Slots<kBsrGroupF32> sl = load_slots<kBsrGroupF32>(S.ent_slot + (long long)kBsrGroupF32 * e);
@@ -325,6 +315,7 @@ __global__ void __launch_bounds__(kBsrPThreads, 3) k_bsr_f32p(const BsrItem* __r
     const int cnt = min(kBsrGroupF32, S.nat - J0);
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(it.W);
     const long long P1 = 4LL * Np * Np, ld = 2LL * Np;
+    const float* G = it.G + (long long)i * ld + 4 * J0;
     const long long top = (long long)i * ld + 4 * J0, bot = (long long)(Np + i) * ld + 4 * J0;
 #pragma unroll
     for (int j = 0; j < kBsrGroupF32; ++j) {
@@ -332,9 +323,11 @@ __global__ void __launch_bounds__(kBsrPThreads, 3) k_bsr_f32p(const BsrItem* __r
         float wr[4], wi[4], nwi[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          wr[c] = ar[j][c];
-          wi[c] = -ai[j][c];
-          nwi[c] = ai[j][c];
+          // the D0 term of W: G_ij e_j
+          const float e = it.ge[4 * (J0 + j) + c];
+          wr[c] = fmaf(G[4 * j + c], e, ar[j][c]);
+          wi[c] = fmaf(G[Np + 4 * j + c], e, -ai[j][c]);
+          nwi[c] = -wi[c];
         }
         uint2 rh, rl, ih, il, nh, nl;
         split4(wr, rh, rl);

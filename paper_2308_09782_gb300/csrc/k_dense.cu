@@ -332,117 +332,165 @@ void launch_leap(const LeapItem* items, int n_items, int Np_max, int mp, const i
 }
 
 // ---------------------------------------------------------------------------
-// Leapfrog of the split form: X (FP32 planar) and R0 (FP32 planar) give
-// dD/dt in FP32 with the same mirror-exact operations as k_leap; only the
+// Leapfrog of the split form.  With dH = (E S + S E)/2 + sum_a (A_a/c) P_a,
+// E = eps - eps0 per orbital, the D0 part of Eq. 6 needs no product per step:
+//   S^-1 dH D0 = S^-1 [E S D0 / 2] + E D0 / 2 + sum_a (A_a/c) S^-1 P_a D0.
+// The bracket is added to W by product 1, so that X holds S^-1 [H dD + E S D0 / 2]; here
+//   dD/dt = R0 + sum_a (A_a/c) K_a - (i/2) [E, D0] - i (X - X^dagger)
+// with constant Hermitian K_a = -i (S^-1 P_a D0 - h.c.), all read as FP32 (K_a only where
+// A_a is nonzero).  This replaces a second operand pair [D0 | dH] of product 1 (as many
+// k-panels again: 512 atoms, products 207 -> 153 us) by 34 MB per term read here.
+// dD/dt is formed in FP32 with mirror-exact operations as in k_leap; only the
 // master update dD_{n+1} = dD_{n-1} + 2 dt dD/dt is FP64 (GB300's FP64 rate is
 // low, so FP64 is kept to the accumulation that needs it).  The operand of the
 // next first product is written from the new level's FP32 rounding: its FP32
 // copy (block-sparse product) and/or its BF16 hi/lo pieces (dense tcgen05
 // product).
 // ---------------------------------------------------------------------------
-// Thread layout: 16 x 16 threads, each owns two adjacent columns (2 tx, 2 tx + 1)
-// of rows ty and ty + 16 of a 32 x 32 tile, so R0 is read and the BF16 pieces
-// written two columns per instruction; X is staged as separate real and
-// imaginary tiles, whose transposed reads (X_ji) hit distinct banks.
-__global__ void __launch_bounds__(256, 4) k_leap_split(const LeapItem* __restrict__ items, const int* step, double dt,
+// One CTA per tile pair (bi, bj), bi <= bj.  D, R0, K_a and D0 are Hermitian bit for bit, so only
+// the elements of tile (bi, bj) are formed, from X of both tiles; the mirror tile is written as
+// their conjugates through shared memory.  That halves the reads of all of these (512 atoms, one
+// nonzero A_a: 218 MB instead of 302 MB a step) and the FP64 updates.  Memory bound: %MEAS%
+// Thread layout: 16 x 16 threads, each owns two adjacent columns (2 tx, 2 tx + 1) of rows ty and
+// ty + 16 of a 32 x 32 tile, so the constants are read and the BF16 pieces written two columns per
+// instruction; X is staged as separate real and imaginary tiles, whose transposed reads (X_ji) hit
+// distinct banks.  The constants and D_{n-1} are in flight while X is staged.
+__device__ __forceinline__ void store_pieces2(__nv_bfloat16* p, long long pr, int Np, const float (&fr)[2],
+                                              const float (&fi)[2]) {
+  const long long P = 2LL * Np * Np;
+  __nv_bfloat162 rh, rl, ih, il;
+  rh.x = __float2bfloat16_rn(fr[0]);
+  rh.y = __float2bfloat16_rn(fr[1]);
+  ih.x = __float2bfloat16_rn(fi[0]);
+  ih.y = __float2bfloat16_rn(fi[1]);
+  rl.x = __float2bfloat16_rn(fr[0] - __bfloat162float(rh.x));
+  rl.y = __float2bfloat16_rn(fr[1] - __bfloat162float(rh.y));
+  il.x = __float2bfloat16_rn(fi[0] - __bfloat162float(ih.x));
+  il.y = __float2bfloat16_rn(fi[1] - __bfloat162float(ih.y));
+  *reinterpret_cast<__nv_bfloat162*>(p + pr) = rh;
+  *reinterpret_cast<__nv_bfloat162*>(p + P + pr) = rl;
+  *reinterpret_cast<__nv_bfloat162*>(p + pr + Np) = ih;
+  *reinterpret_cast<__nv_bfloat162*>(p + P + pr + Np) = il;
+}
+
+__global__ void __launch_bounds__(256, 3) k_leap_split(const LeapItem* __restrict__ items, const int* step, double dt,
                                                     int* counter, int* step_rw) {
   pdl_wait();
   pdl_trigger();
   __shared__ float Xre[2][LT][LT + 1];  // [0] tile (bi, bj), [1] tile (bj, bi)
   __shared__ float Xim[2][LT][LT + 1];
+  __shared__ double2 V[LT][LT + 1];     // the new level at tile (bi, bj)
   const LeapItem& it = items[blockIdx.y];
   const int Np = it.Np;
   const int nt = Np / LT;
   const int n = *step;
   int p = blockIdx.x, bi = 0;
   const int npairs = nt * (nt + 1) / 2;
-  const bool active = p < npairs;
+  const bool active = p < npairs;  // the same for the whole CTA
   if (active) {
     while (p >= nt - bi) {
       p -= nt - bi;
       ++bi;
     }
-  }
-  const int bj = bi + p;
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 16 x 16
-  const int c0 = 2 * tx;
-  const float* X = (const float*)it.X;
-  if (active) {
+    const int bj = bi + p;
+    const int tx = threadIdx.x, ty = threadIdx.y;  // 16 x 16
+    const int c0 = 2 * tx;
+    const float* X = (const float*)it.X;
+    const int nxt = (n & 1) ^ 1;
+    const bool euler = (n == 0);
+    const double coef = euler ? dt : 2.0 * dt;
+    const double2* base = euler ? it.D[n & 1] : it.D[nxt];
+    const float av[3] = {it.af[0], it.af[1], it.af[2]};
+    float2 xa[2][2], xb[2][2], cr[2], ci[2], zr[2], zi[2];
+    double2 b[2][2];
+    float di[2];
+    const float2 dj = *reinterpret_cast<const float2*>(it.deh + bj * LT + c0);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = ty + 16 * h;
       const long long ra = (long long)(bi * LT + r) * 2 * Np + bj * LT + c0;
       const long long rb = (long long)(bj * LT + r) * 2 * Np + bi * LT + c0;
-      const float2 ar = *reinterpret_cast<const float2*>(X + ra), ai = *reinterpret_cast<const float2*>(X + ra + Np);
-      const float2 br = *reinterpret_cast<const float2*>(X + rb), bim = *reinterpret_cast<const float2*>(X + rb + Np);
-      Xre[0][r][c0] = ar.x;
-      Xre[0][r][c0 + 1] = ar.y;
-      Xim[0][r][c0] = ai.x;
-      Xim[0][r][c0 + 1] = ai.y;
-      Xre[1][r][c0] = br.x;
-      Xre[1][r][c0 + 1] = br.y;
-      Xim[1][r][c0] = bim.x;
-      Xim[1][r][c0 + 1] = bim.y;
+      const long long idx = (long long)(bi * LT + r) * Np + bj * LT + c0;
+      xa[h][0] = *reinterpret_cast<const float2*>(X + ra);
+      xa[h][1] = *reinterpret_cast<const float2*>(X + ra + Np);
+      xb[h][0] = *reinterpret_cast<const float2*>(X + rb);
+      xb[h][1] = *reinterpret_cast<const float2*>(X + rb + Np);
+      cr[h] = *reinterpret_cast<const float2*>(it.R0f + ra);
+      ci[h] = *reinterpret_cast<const float2*>(it.R0f + ra + Np);
+      zr[h] = *reinterpret_cast<const float2*>(it.D0f + ra);
+      zi[h] = *reinterpret_cast<const float2*>(it.D0f + ra + Np);
+      b[h][0] = base[idx];
+      b[h][1] = base[idx + 1];
+      di[h] = it.deh[bi * LT + r];
     }
-  }
-  __syncthreads();
-  if (active) {
-    const int cur = n & 1, nxt = cur ^ 1;
-    const bool euler = (n == 0);
-    const double coef = euler ? dt : 2.0 * dt;
-    const double2* base = euler ? it.D[cur] : it.D[nxt];
-    const long long P = 2LL * Np * Np;
-    for (int half = 0; half < (bi == bj ? 1 : 2); ++half) {
-      const int gi0 = half == 0 ? bi : bj, gj0 = half == 0 ? bj : bi;
-      const int A = half, B = half ^ 1;  // tile of (i, j) and of its mirror (j, i)
-      // all loads of the thread's elements first (D_{n-1} is overwritten in place,
-      // element by element, by the same thread), then the updates and stores
-      float2 r0r[2], r0i[2];
-      double2 b[2][2];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int r = ty + 16 * h;
-        const long long idx = (long long)(gi0 * LT + r) * Np + gj0 * LT + c0;
-        const long long pr = (long long)(gi0 * LT + r) * 2 * Np + gj0 * LT + c0;
-        r0r[h] = it.R0f ? *reinterpret_cast<const float2*>(it.R0f + pr) : make_float2(0.f, 0.f);
-        r0i[h] = it.R0f ? *reinterpret_cast<const float2*>(it.R0f + pr + Np) : make_float2(0.f, 0.f);
-        b[h][0] = base[idx];
-        b[h][1] = base[idx + 1];
+    for (int a = 0; a < 3; ++a)
+      if (av[a] != 0.f) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const long long ra = (long long)(bi * LT + ty + 16 * h) * 2 * Np + bj * LT + c0;
+          const float2 kr = *reinterpret_cast<const float2*>(it.Kf + a * it.k_stride + ra);
+          const float2 ki = *reinterpret_cast<const float2*>(it.Kf + a * it.k_stride + ra + Np);
+          cr[h].x = fmaf(av[a], kr.x, cr[h].x);
+          cr[h].y = fmaf(av[a], kr.y, cr[h].y);
+          ci[h].x = fmaf(av[a], ki.x, ci[h].x);
+          ci[h].y = fmaf(av[a], ki.y, ci[h].y);
+        }
       }
 #pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = ty + 16 * h;
+      Xre[0][r][c0] = xa[h][0].x;
+      Xre[0][r][c0 + 1] = xa[h][0].y;
+      Xim[0][r][c0] = xa[h][1].x;
+      Xim[0][r][c0 + 1] = xa[h][1].y;
+      Xre[1][r][c0] = xb[h][0].x;
+      Xre[1][r][c0 + 1] = xb[h][0].y;
+      Xim[1][r][c0] = xb[h][1].x;
+      Xim[1][r][c0 + 1] = xb[h][1].y;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = ty + 16 * h;
+      const long long idx = (long long)(bi * LT + r) * Np + bj * LT + c0;
+      const long long pr = (long long)(bi * LT + r) * 2 * Np + bj * LT + c0;
+      float fr[2], fi[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int c = c0 + e;
+        // -(i/2) [E, D0]: d (D0_i, -D0_r) with d = (E_i - E_j) / 2
+        const float d = di[h] - (e ? dj.y : dj.x);
+        const float kr = fmaf(d, e ? zi[h].y : zi[h].x, e ? cr[h].y : cr[h].x);
+        const float ki = fmaf(-d, e ? zr[h].y : zr[h].x, e ? ci[h].y : ci[h].x);
+        const float dr = kr + (Xim[0][r][c] + Xim[1][c][r]);
+        const float dd = ki + (-(Xre[0][r][c] - Xre[1][c][r]));
+        const double2 v = make_double2(fma(coef, f2d_bits(dr), b[h][e].x), fma(coef, f2d_bits(dd), b[h][e].y));
+        it.D[nxt][idx + e] = v;
+        V[r][c] = v;
+        fr[e] = d2f_bits(v.x);
+        fi[e] = d2f_bits(v.y);
+      }
+      if (it.f32) *reinterpret_cast<float4*>(it.f32 + idx) = make_float4(fr[0], fi[0], fr[1], fi[1]);
+      if (it.pieces) store_pieces2(it.pieces, pr, Np, fr, fi);
+    }
+    if (bi != bj) {
+      __syncthreads();
+#pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int r = ty + 16 * h;
-        const long long idx = (long long)(gi0 * LT + r) * Np + gj0 * LT + c0;
-        const long long pr = (long long)(gi0 * LT + r) * 2 * Np + gj0 * LT + c0;
+        const long long idx = (long long)(bj * LT + r) * Np + bi * LT + c0;
+        const long long pr = (long long)(bj * LT + r) * 2 * Np + bi * LT + c0;
         float fr[2], fi[2];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-          const int c = c0 + e;
-          const float xij_re = Xre[A][r][c], xij_im = Xim[A][r][c];
-          const float xji_re = Xre[B][c][r], xji_im = Xim[B][c][r];
-          const float dr = (e ? r0r[h].y : r0r[h].x) + (xij_im + xji_im);
-          const float di = (e ? r0i[h].y : r0i[h].x) + (-(xij_re - xji_re));
-          const double2 v = make_double2(fma(coef, f2d_bits(dr), b[h][e].x), fma(coef, f2d_bits(di), b[h][e].y));
-          it.D[nxt][idx + e] = v;
+          const double2 v = V[c0 + e][r];
+          it.D[nxt][idx + e] = make_double2(v.x, -v.y);
           fr[e] = d2f_bits(v.x);
-          fi[e] = d2f_bits(v.y);
+          fi[e] = d2f_bits(-v.y);
         }
         if (it.f32) *reinterpret_cast<float4*>(it.f32 + idx) = make_float4(fr[0], fi[0], fr[1], fi[1]);
-        if (it.pieces) {
-          __nv_bfloat162 rh, rl, ih, il;
-          rh.x = __float2bfloat16_rn(fr[0]);
-          rh.y = __float2bfloat16_rn(fr[1]);
-          ih.x = __float2bfloat16_rn(fi[0]);
-          ih.y = __float2bfloat16_rn(fi[1]);
-          rl.x = __float2bfloat16_rn(fr[0] - __bfloat162float(rh.x));
-          rl.y = __float2bfloat16_rn(fr[1] - __bfloat162float(rh.y));
-          il.x = __float2bfloat16_rn(fi[0] - __bfloat162float(ih.x));
-          il.y = __float2bfloat16_rn(fi[1] - __bfloat162float(ih.y));
-          *reinterpret_cast<__nv_bfloat162*>(it.pieces + pr) = rh;
-          *reinterpret_cast<__nv_bfloat162*>(it.pieces + P + pr) = rl;
-          *reinterpret_cast<__nv_bfloat162*>(it.pieces + pr + Np) = ih;
-          *reinterpret_cast<__nv_bfloat162*>(it.pieces + P + pr + Np) = il;
-        }
+        if (it.pieces) store_pieces2(it.pieces, pr, Np, fr, fi);
       }
     }
   }
@@ -500,6 +548,16 @@ void launch_to_f32(const double2* src, float2* dst, long long n, cudaStream_t st
 // ---------------------------------------------------------------------------
 // helpers
 // ---------------------------------------------------------------------------
+// values at the nonzero pattern to their places in a zeroed Np x Np matrix
+__global__ void k_scatter(const double2* v, const int* off, int n, double2* out) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < n) out[off[e]] = v[e];
+}
+
+void launch_scatter(const double2* v, const int* off, int n, double2* out, cudaStream_t st) {
+  k_scatter<<<(n + 255) / 256, 256, 0, st>>>(v, off, n, out);
+}
+
 __global__ void k_fill_herm(double2* a, int n, int ld, int real) {
   // the upper triangle (j >= i) is valid; set a[i][j] = conj(a[j][i]) for j < i
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;

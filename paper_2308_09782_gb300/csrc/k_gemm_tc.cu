@@ -162,10 +162,10 @@ int tc_gemm_supported() {
 // Nonzero k-panels of each B column tile of product 1 for system v (tile nt =
 // B rows starts[nt] .. starts[nt+1]-1 of the embedded [[Re H, Im H], [-Im H, Re H]],
 // rows interleaved in blocks of four: B row n' holds H row 4 (n' / 8) + n' % 4): a panel kt covers
-// the 64 columns k' = 64 kt .. 64 kt + 63 of a segment, i.e. H columns k' (real
+// the 64 columns k' = 64 kt .. 64 kt + 63, i.e. H columns k' (real
 // half) or k' - Np (imaginary half); it is nonzero for the tile when some H row
 // of the tile belongs to an atom I with a target (I, J) whose columns meet the
-// panel.  H and dH share the pattern.
+// panel.
 // uniform = true pads every tile's list with panels of zeros (in increasing
 // order) to the longest list, so that all tiles take the same number of
 // k-iterations, as the stream-K schedules need.
@@ -267,7 +267,7 @@ static std::vector<int> even_split(int total, int n) {
 // longest first.  With the zero k-panels skipped a tile's k-iterations are its
 // panel count.
 // `full`: k-iterations of a tile whose panels are not skipped.
-static std::vector<int> plan_columns(const TcSysView& v, bool skip, int nseg, int full, int tiles_m, int G, int mode) {
+static std::vector<int> plan_columns(const TcSysView& v, bool skip, int full, int tiles_m, int G, int mode) {
   const int total = 2 * v.Np, n0 = (total + 255) / 256;
   std::vector<std::pair<double, int>> score;
   for (int n = n0; n <= std::max(total / 96, n0); ++n) {
@@ -278,7 +278,7 @@ static std::vector<int> plan_columns(const TcSysView& v, bool skip, int nseg, in
       std::vector<int> kofs;
       std::vector<short> kidx;
       zero_panel_lists(v, st, false, kofs, kidx);
-      for (int i = 0; i < n; ++i) kt[i] = nseg * (kofs[i + 1] - kofs[i]);
+      for (int i = 0; i < n; ++i) kt[i] = kofs[i + 1] - kofs[i];
     }
     std::vector<double> cost;
     for (int it = 0; it < v.n_items; ++it)
@@ -298,7 +298,6 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
   const int BNv = var.bn;
   const bool pair = var.pair != 0;
   const int tm_rows = pair ? 2 * BM : BM;  // output rows of one tile
-  const int nseg = epi == 0 ? 2 : 1;
   memset(&plan->P, 0, sizeof(plan->P));
   plan->epi = epi;
   plan->variant = variant;
@@ -324,8 +323,8 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
   int wmax = 0;
   for (size_t s = 0; s < sys.size(); ++s) {
     const int tiles_m = (sys[s].Np + tm_rows - 1) / tm_rows;
-    const int full = nseg * 2 * sys[s].Np / BK / (epi == 1 && n_real == (int)items.size() ? 2 : 1);
-    starts[s] = var.widths ? plan_columns(sys[s], skip, nseg, full, tiles_m, G_full, var.widths)
+    const int full = 2 * sys[s].Np / BK / (epi == 1 && n_real == (int)items.size() ? 2 : 1);
+    starts[s] = var.widths ? plan_columns(sys[s], skip, full, tiles_m, G_full, var.widths)
                            : even_split(2 * sys[s].Np, 2 * sys[s].Np / BNv);
     for (size_t i = 0; i + 1 < starts[s].size(); ++i) wmax = std::max(wmax, starts[s][i + 1] - starts[s][i]);
   }
@@ -336,13 +335,11 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
     const TcSysView& v = sys[s];
     const int Np = v.Np;
     if (epi == 0) {
-      if (!encode_map(&plan->P.mA[s][0], v.dD_p, 2 * Np, Np, v.n_items, BM, msg, var.kh)) return -1;
-      if (!encode_map(&plan->P.mA[s][1], v.D0_p, 2 * Np, Np, v.nk, BM, msg, var.kh)) return -1;
-      if (!encode_map(&plan->P.mB[s][0], v.Hemb_p, 2 * Np, 2 * Np, v.n_items, bbox, msg, var.kh)) return -1;
-      if (!encode_map(&plan->P.mB[s][1], v.dHemb_p, 2 * Np, 2 * Np, v.n_items, bbox, msg, var.kh)) return -1;
+      if (!encode_map(&plan->P.mA[s], v.dD_p, 2 * Np, Np, v.n_items, BM, msg, var.kh)) return -1;
+      if (!encode_map(&plan->P.mB[s], v.Hemb_p, 2 * Np, 2 * Np, v.n_items, bbox, msg, var.kh)) return -1;
     } else {
-      if (!encode_map(&plan->P.mA[s][0], v.Sinv_p, 2 * Np, Np, v.nk, BM, msg, var.kh)) return -1;
-      if (!encode_map(&plan->P.mB[s][0], v.Wemb_p, 2 * Np, 2 * Np, v.n_items, bbox, msg, var.kh)) return -1;
+      if (!encode_map(&plan->P.mA[s], v.Sinv_p, 2 * Np, Np, v.nk, BM, msg, var.kh)) return -1;
+      if (!encode_map(&plan->P.mB[s], v.Wemb_p, 2 * Np, 2 * Np, v.n_items, bbox, msg, var.kh)) return -1;
     }
   }
   std::vector<int> sys_kofs0(sys.size(), 0), sys_kidx0(sys.size(), 0), sys_cofs0(sys.size(), 0), all_kofs, all_cofs;
@@ -402,29 +399,29 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
     pr.tiles_n = (int)st.size() - 1;
     pr.tile0 = tiles;
     if (epi == 0) {
-      pr.a_b[0] = li;
-      pr.b_b[0] = li;
-      pr.a_b[1] = it.k;
-      pr.b_b[1] = li;
+      pr.a_b = li;
+      pr.b_b = li;
+      pr.G = it.Gf;
+      pr.ge = it.ge;
       pr.out = it.Wemb_p;
       pr.w_half = k_real(v, it.k) ? 1 : 0;
     } else {
-      pr.a_b[0] = it.k;
-      pr.b_b[0] = li;
+      pr.a_b = it.k;
+      pr.b_b = li;
       pr.out = it.Xf;
     }
-    pr.kt = nseg * (2 * v.Np) / BK;
+    pr.kt = (2 * v.Np) / BK;
     pr.iter0 = (int)iters;
     const bool listed = skip || (epi == 1 && k_real(v, it.k));
     if (listed) {
       pr.kofs = plan->d_kofs + sys_kofs0[it.sys];
       pr.kidx = plan->d_kidx + sys_kidx0[it.sys];
-      pr.kt = nseg * sys_cnt[it.sys][0];  // every segment takes the panel list (uniform lists: one length)
+      pr.kt = sys_cnt[it.sys][0];  // uniform lists: one length
     }
     if (var.widths) pr.cofs = plan->d_cofs + sys_cofs0[it.sys];
     for (int nt = 0; nt < pr.tiles_n; ++nt)
       for (int mt = 0; mt < pr.tiles_m; ++mt)
-        tile_cost.push_back(tile_model(st[nt + 1] - st[nt], listed ? nseg * sys_cnt[it.sys][nt] : pr.kt));
+        tile_cost.push_back(tile_model(st[nt + 1] - st[nt], listed ? sys_cnt[it.sys][nt] : pr.kt));
     tiles += pr.tiles_m * pr.tiles_n;
     iters += (long long)pr.tiles_m * pr.tiles_n * pr.kt;
     probs.push_back(pr);
@@ -442,7 +439,6 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
   plan->P.probs = plan->d_probs;
   plan->P.n_prob = (int)probs.size();
   plan->P.total_tiles = tiles;
-  plan->P.nseg = nseg;
   plan->P.err = plan->d_err;
   plan->P.timeout_ns = timeout_ns;
   plan->grid = std::min(tiles, nsm);

@@ -168,12 +168,11 @@ __global__ void __launch_bounds__(192, 1)
         }
         const uint32_t stage_tx = 2 * A_BYTES + 2 * (uint32_t)(Q.b_rows ? Q.b_rows : BNP / 2) * BK * 2;
         const int arow = mt * (2 * BM) + rank * BM, brow = cb + rank * (w / 2);
-        const int KT = tile_kt(Q, pr, t);
+        const int KT = tile_kt(pr, t);
         for (int kk = 0; kk < KT; ++kk, ++it) {
-          int sg, kt;
-          tile_panel(pr, t, kk, sg, kt);
-          const CUtensorMap* ma = &Q.mA[pr.sys][sg];
-          const CUtensorMap* mb = &Q.mB[pr.sys][sg];
+          const int kt = tile_panel(pr, t, kk);
+          const CUtensorMap* ma = &Q.mA[pr.sys];
+          const CUtensorMap* mb = &Q.mB[pr.sys];
           const int s = it % ST, r = it / ST;
           if (!mbar_wait(empty0 + 8 * s, (r & 1) ^ 1, limit, abort_flag, err)) {
             ok = false;
@@ -182,10 +181,10 @@ __global__ void __launch_bounds__(192, 1)
           const uint32_t base = smem_u32(sm + s * STAGE);
           if (leader_cta) mbar_expect_tx(full0 + 8 * s, 2 * stage_tx);
           const uint32_t fb = full_l + 8 * s;
-          tma_load_4d_pair(base, ma, kt * BK, arow, 0, pr.a_b[sg], fb);
-          tma_load_4d_pair(base + A_BYTES, ma, kt * BK, arow, 1, pr.a_b[sg], fb);
-          tma_load_4d_pair(base + 2 * A_BYTES, mb, kt * BK, brow, 0, pr.b_b[sg], fb);
-          tma_load_4d_pair(base + 2 * A_BYTES + B_BYTES, mb, kt * BK, brow, 1, pr.b_b[sg], fb);
+          tma_load_4d_pair(base, ma, kt * BK, arow, 0, pr.a_b, fb);
+          tma_load_4d_pair(base + A_BYTES, ma, kt * BK, arow, 1, pr.a_b, fb);
+          tma_load_4d_pair(base + 2 * A_BYTES, mb, kt * BK, brow, 0, pr.b_b, fb);
+          tma_load_4d_pair(base + 2 * A_BYTES + B_BYTES, mb, kt * BK, brow, 1, pr.b_b, fb);
         }
       }
       if (!ok) {
@@ -218,7 +217,7 @@ __global__ void __launch_bounds__(192, 1)
         int cb, w;
         col_tile(pr, (t - pr.tile0) / pr.tiles_m, cb, w);
         const uint32_t idesc = idesc_bf16(2 * BM, w);
-        const int KT = tile_kt(Q, pr, t);
+        const int KT = tile_kt(pr, t);
         for (int kk = 0; kk < KT; ++kk, ++it) {
           const int s = it % ST, r = it / ST;
           if (!mbar_wait(full0 + 8 * s, r & 1, limit, abort_flag, err)) {
@@ -290,7 +289,7 @@ __global__ void __launch_bounds__(192, 1)
                   make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
                               __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
         } else {
-          store_w_pieces(reinterpret_cast<__nv_bfloat16*>(pr.out), Np, row, gn, r, nv >> 4, pr.w_half);
+          store_w_pieces(pr, row, gn, r, nv >> 4);
         }
       }
       tc_fence_before();

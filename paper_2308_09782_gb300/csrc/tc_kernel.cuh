@@ -14,7 +14,6 @@
 // or Im W(m, 4b+q-4).  Product 2 (EPI 1) keeps the halves [Re | Im] above.
 // Each operand is held as BF16 pieces x = x_hi + x_lo; the GEMM accumulates
 // x_hi y_hi + x_hi y_lo + x_lo y_hi in FP32 in tensor memory (3 MMAs per slice).
-// Segments concatenate along k (product 1 has two: [dD | D0] [H | dH]^dagger).
 //
 // Kernel: persistent CTAs over 128 x BN output tiles (2-SM pair: 256 x w, with
 // the column tiles either all 256 wide or of planned widths w, multiples of 16,
@@ -41,17 +40,21 @@ constexpr long long kDrainNs = 200000000LL;  // 0.2 s for in-flight work after a
 
 struct TcProb {
   int sys;
-  int a_b[2], b_b[2];  // batch coordinate of each segment's A / B operand
+  int a_b, b_b;        // batch coordinates of the A and B operands
   int tiles_m, tiles_n, tile0, Np;
   void* out;
   int kt;              // k-iterations per tile (stream-K schedule)
   int iter0;           // first global k-iteration of the problem (stream-K schedule)
   // classic schedule with zero panels skipped (null = every panel): the
-  // 64-wide k-panels of one segment in which the B rows of column tile nt have
-  // a nonzero are kidx[kofs[nt] .. kofs[nt+1]-1]; every segment uses the list
+  // 64-wide k-panels in which the B rows of column tile nt have a nonzero are
+  // kidx[kofs[nt] .. kofs[nt+1]-1]
   // (product 2 of a real S_k^-1: the panels of its real half)
   const int* kofs;
   const short* kidx;
+  // product 1: added to W in the epilogue: W_mj += G_mj e_j with G planar FP32
+  // [Np][2 Np] and one factor per orbital (null: nothing)
+  const float* G;
+  const float* ge;
   int w_half;          // product 1: product 2 reads only the left half [Re W; -Im W] of the embedded W
   // 2-SM pair kernel, classic schedule: first B row of each column tile
   // (tiles_n + 1 entries, the last 2 Np; widths multiples of 16 up to 256, so
@@ -60,10 +63,10 @@ struct TcProb {
 };
 
 struct TcParams {
-  CUtensorMap mA[kMaxSys][2];
-  CUtensorMap mB[kMaxSys][2];
+  CUtensorMap mA[kMaxSys];
+  CUtensorMap mB[kMaxSys];
   const TcProb* probs;
-  int n_prob, total_tiles, nseg;
+  int n_prob, total_tiles;
   int* err;
   long long timeout_ns;
   const int* tord;     // classic schedule: worker c takes tiles tord[c], tord[c + G], ... (null = 0, 1, ...;
@@ -240,24 +243,16 @@ __device__ __forceinline__ int find_prob_any(const TcProb* probs, int n, int t) 
 }
 
 // k-iterations of tile t of problem pr (classic schedule)
-__device__ __forceinline__ int tile_kt(const TcParams& P, const TcProb& pr, int t) {
-  if (!pr.kofs) return P.nseg * (2 * pr.Np) / BK;
+__device__ __forceinline__ int tile_kt(const TcProb& pr, int t) {
+  if (!pr.kofs) return (2 * pr.Np) / BK;
   const int nt = (t - pr.tile0) / pr.tiles_m;
-  return P.nseg * (pr.kofs[nt + 1] - pr.kofs[nt]);
+  return pr.kofs[nt + 1] - pr.kofs[nt];
 }
 
-// segment and k-panel of k-iteration kk of tile t
-__device__ __forceinline__ void tile_panel(const TcProb& pr, int t, int kk, int& sg, int& kt) {
-  if (!pr.kofs) {
-    const int kts = (2 * pr.Np) / BK;
-    sg = kk / kts;
-    kt = kk - sg * kts;
-    return;
-  }
-  const int nt = (t - pr.tile0) / pr.tiles_m;
-  const int k0 = pr.kofs[nt], cnt = pr.kofs[nt + 1] - k0;
-  sg = kk / cnt;
-  kt = pr.kidx[k0 + kk - sg * cnt];
+// k-panel of k-iteration kk of tile t
+__device__ __forceinline__ int tile_panel(const TcProb& pr, int t, int kk) {
+  if (!pr.kofs) return kk;
+  return pr.kidx[pr.kofs[(t - pr.tile0) / pr.tiles_m] + kk];
 }
 
 // first B row and width of column tile nt of the 2-SM pair kernel
@@ -300,7 +295,7 @@ __device__ __forceinline__ bool cursor_next(const TcParams& P, UnitCursor& u, in
     if (t < 0) return false;
     u.t_next += G;
     u.p = P.tord ? find_prob_any(P.probs, P.n_prob, t) : find_prob(P.probs, P.n_prob, t, u.p);
-    KT = tile_kt(P, P.probs[u.p], t);
+    KT = tile_kt(P.probs[u.p], t);
     kb = 0;
     ke = KT;
     return true;
@@ -368,9 +363,11 @@ __device__ __forceinline__ uint4 pack8_bf16(const float (&x)[16], int h, float s
 // embedded BF16 pieces of W that product 2 reads as its B operand: top row m =
 // [Re W | Im W], bottom row Np + m = [-Im W | Re W], hi at 0 and lo at 4 Np^2.
 // (nh = 1: only the first 16 accumulator columns are the tile's, 8 W columns).
-// half: only [Re W] of the top and [-Im W] of the bottom row (w_half).
-__device__ __forceinline__ void store_w_pieces(__nv_bfloat16* W, int Np, int row, int gn, const uint32_t (&r)[32],
-                                               int nh, int half) {
+// half: only [Re W] of the top and [-Im W] of the bottom row (w_half).  The term
+// G_mj e_j is added first, in FP32.
+__device__ __forceinline__ void store_w_pieces(const TcProb& pr, int row, int gn, const uint32_t (&r)[32], int nh) {
+  __nv_bfloat16* W = reinterpret_cast<__nv_bfloat16*>(pr.out);
+  const int Np = pr.Np, half = pr.w_half;
   const long long ld = 2LL * Np, P1 = 4LL * Np * Np;
   const int j0 = gn >> 1;
   float re[16], im[16], rel[16], iml[16];
@@ -381,6 +378,23 @@ __device__ __forceinline__ void store_w_pieces(__nv_bfloat16* W, int Np, int row
       re[4 * b + q] = __uint_as_float(r[8 * b + q]);
       im[4 * b + q] = __uint_as_float(r[8 * b + 4 + q]);
     }
+  if (pr.G) {
+    const float4* g = reinterpret_cast<const float4*>(pr.G + (long long)row * ld + j0);
+    const float4* e = reinterpret_cast<const float4*>(pr.ge + j0);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      if (b >= 2 * nh) break;
+      const float4 gr = g[b], gi = g[b + Np / 4], f = e[b];
+      re[4 * b] = fmaf(gr.x, f.x, re[4 * b]);
+      re[4 * b + 1] = fmaf(gr.y, f.y, re[4 * b + 1]);
+      re[4 * b + 2] = fmaf(gr.z, f.z, re[4 * b + 2]);
+      re[4 * b + 3] = fmaf(gr.w, f.w, re[4 * b + 3]);
+      im[4 * b] = fmaf(gi.x, f.x, im[4 * b]);
+      im[4 * b + 1] = fmaf(gi.y, f.y, im[4 * b + 1]);
+      im[4 * b + 2] = fmaf(gi.z, f.z, im[4 * b + 2]);
+      im[4 * b + 3] = fmaf(gi.w, f.w, im[4 * b + 3]);
+    }
+  }
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const float rh = __bfloat162float(__float2bfloat16_rn(re[i])), ih = __bfloat162float(__float2bfloat16_rn(im[i]));
@@ -465,10 +479,9 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcPa
         const int local = t - pr.tile0;
         const int mt = local % pr.tiles_m, nt = local / pr.tiles_m;
         for (int kk = kb; kk < ke; ++kk, ++it) {
-          int sg, kt;
-          tile_panel(pr, t, kk, sg, kt);
-          const CUtensorMap* ma = &P.mA[pr.sys][sg];
-          const CUtensorMap* mb = &P.mB[pr.sys][sg];
+          const int kt = tile_panel(pr, t, kk);
+          const CUtensorMap* ma = &P.mA[pr.sys];
+          const CUtensorMap* mb = &P.mB[pr.sys];
           const int s = it % ST, r = it / ST;
           if (!mbar_wait(empty0 + 8 * s, (r & 1) ^ 1, P.timeout_ns, abort_flag, P.err)) {
             ok = false;
@@ -476,10 +489,10 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcPa
           }
           const uint32_t base = smem_u32(sm + s * STAGE);
           mbar_expect_tx(full0 + 8 * s, STAGE);
-          tma_load_4d(base, ma, kt * BK, mt * BM, 0, pr.a_b[sg], full0 + 8 * s);
-          tma_load_4d(base + A_BYTES, ma, kt * BK, mt * BM, 1, pr.a_b[sg], full0 + 8 * s);
-          tma_load_4d(base + 2 * A_BYTES, mb, kt * BK, nt * BN, 0, pr.b_b[sg], full0 + 8 * s);
-          tma_load_4d(base + 2 * A_BYTES + B_BYTES, mb, kt * BK, nt * BN, 1, pr.b_b[sg], full0 + 8 * s);
+          tma_load_4d(base, ma, kt * BK, mt * BM, 0, pr.a_b, full0 + 8 * s);
+          tma_load_4d(base + A_BYTES, ma, kt * BK, mt * BM, 1, pr.a_b, full0 + 8 * s);
+          tma_load_4d(base + 2 * A_BYTES, mb, kt * BK, nt * BN, 0, pr.b_b, full0 + 8 * s);
+          tma_load_4d(base + 2 * A_BYTES + B_BYTES, mb, kt * BK, nt * BN, 1, pr.b_b, full0 + 8 * s);
         }
       }
       if (!ok) {
@@ -600,7 +613,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcPa
                 make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]),
                             __uint_as_float(r[4 * v + 3]));
         } else {
-          store_w_pieces(reinterpret_cast<__nv_bfloat16*>(pr.out), Np, row, gn, r, 2, pr.w_half);
+          store_w_pieces(pr, row, gn, r, 2);
         }
       }
       tc_fence_before();
@@ -755,10 +768,9 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
         col_tile(pr, nt, cb, w);
         const int arow = mt * (2 * BM) + rank * BM, brow = cb + rank * (w / 2);
         for (int kk = kb; ok && kk < ke; ++kk) {
-          int sg, kt;
-          tile_panel(pr, t, kk, sg, kt);
-          const CUtensorMap* ma = &P.mA[pr.sys][sg];
-          const CUtensorMap* mb = &P.mB[pr.sys][sg];
+          const int kt = tile_panel(pr, t, kk);
+          const CUtensorMap* ma = &P.mA[pr.sys];
+          const CUtensorMap* mb = &P.mB[pr.sys];
 #pragma unroll 1
           for (int h = 0; h < KH; ++h, ++it) {
             const int s = it % ST, r = it / ST;
@@ -770,10 +782,10 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
             if (leader_cta) mbar_expect_tx(full0 + 8 * s, 2 * stage_tx);
             const uint32_t fb = full_l + 8 * s;
             const int x = kt * BK + h * BKS;
-            tma_load_4d_pair(base, ma, x, arow, 0, pr.a_b[sg], fb);
-            tma_load_4d_pair(base + A_BYTES, ma, x, arow, 1, pr.a_b[sg], fb);
-            tma_load_4d_pair(base + 2 * A_BYTES, mb, x, brow, 0, pr.b_b[sg], fb);
-            tma_load_4d_pair(base + 2 * A_BYTES + B_BYTES, mb, x, brow, 1, pr.b_b[sg], fb);
+            tma_load_4d_pair(base, ma, x, arow, 0, pr.a_b, fb);
+            tma_load_4d_pair(base + A_BYTES, ma, x, arow, 1, pr.a_b, fb);
+            tma_load_4d_pair(base + 2 * A_BYTES, mb, x, brow, 0, pr.b_b, fb);
+            tma_load_4d_pair(base + 2 * A_BYTES + B_BYTES, mb, x, brow, 1, pr.b_b, fb);
           }
         }
       }
@@ -915,7 +927,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
                   make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
                               __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
         } else {
-          store_w_pieces(reinterpret_cast<__nv_bfloat16*>(pr.out), Np, row, gn, r, nv >> 4, pr.w_half);
+          store_w_pieces(pr, row, gn, r, nv >> 4);
         }
       }
       tc_fence_before();

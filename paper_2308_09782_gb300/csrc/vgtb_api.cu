@@ -33,6 +33,12 @@ namespace {
 
 thread_local std::string g_create_error;
 
+// From kSliceMinN orbitals up the 34 exact digit products on the tensor cores take less time than
+// one product on the FP64 pipe (N = 256, 8 k-points: 1.06 ms for one product on the FP64 pipe);
+// below, a product is a few microseconds of FP64 work and the extra launches cost more.
+constexpr int kSliceMinN = 97;
+static_assert(kSliceMinN == kGemmSmall + 1, "every FP64 size has its kernel");
+
 struct HostSys {
   int N = 0, Np = 0, nat = 0, nk = 0, n_blk = 0, n_tgt = 0, nocc = 0;
   double omega = 0, nel = 0, dt = 0;
@@ -49,15 +55,16 @@ struct HostSys {
   double* dq0 = nullptr;
   double* eps0 = nullptr;
   __nv_bfloat16* Sinv_p = nullptr;
-  __nv_bfloat16* D0_p = nullptr;
   float* R0f = nullptr;
   double2* C0d = nullptr;   // Crank-Nicolson: [nk][nocc][Np] initial states as rows (C^dagger)
   std::vector<double> dq0_h, eps0_h;
   bool density_set = false;
   std::vector<int> trajs;  // trajectories of this system
+  const double2 *d_kS = nullptr, *d_kP = nullptr;
   const int *d_el_off = nullptr, *d_el_atom0 = nullptr, *d_orb_off = nullptr;
   std::vector<char> k_set;  // which k-points received a user density
-  float2* D0f = nullptr;    // split form, block-sparse first product: [nk][Np][Np] FP32 copy of D0
+  // split form, FP32 planar [nk][Np][2Np] each (Kf: [3][nk]): D0 S, D0, -i (S^-1 P_a D0 - h.c.)
+  float *Gf = nullptr, *D0f = nullptr, *Kf = nullptr;
   int bsr_units = 0;        // block-sparse first product: CTAs per item (groups x column chunks)
   int bsr_tg_max = 0;       // most targets of one atom group
   int bsr_ent_max = 0;      // most column atoms in the union of one atom group
@@ -78,7 +85,7 @@ struct HostTraj {
   double* eps = nullptr;
   double* eps_lv = nullptr;
   float* epsf = nullptr;
-  float* depsf = nullptr;
+  float* deh = nullptr;
   float* af = nullptr;
   double* part = nullptr;
   double* cpart = nullptr;
@@ -499,6 +506,8 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
   TRY(dalloc(ctx, &d.kS, (size_t)h.nk * h.n_el));
   TRY(dalloc(ctx, &d.kH0, (size_t)h.nk * h.n_el));
   TRY(dalloc(ctx, &d.kP, 3 * (size_t)h.nk * h.n_el));
+  h.d_kS = d.kS;
+  h.d_kP = d.kP;
   TRY(dalloc(ctx, &d.obs0, 5 * (size_t)h.n_tgt));
   if (ctx->split) TRY(dalloc(ctx, &d.obs0a, 5 * (size_t)h.nat));
   const size_t NN = (size_t)h.Np * h.Np;
@@ -510,7 +519,9 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
   if (ctx->cn) TRY(dalloc(ctx, &h.C0d, (size_t)h.nk * h.nocc * h.Np));
   if (ctx->split) {
     TRY(dalloc(ctx, &h.Sinv_p, 4 * NN * h.nk));
-    TRY(dalloc(ctx, &h.D0_p, 4 * NN * h.nk));
+    TRY(dalloc(ctx, &h.Gf, 2 * NN * h.nk));
+    TRY(dalloc(ctx, &h.D0f, 2 * NN * h.nk));
+    TRY(dalloc(ctx, &h.Kf, 6 * NN * h.nk));
     TRY(dalloc(ctx, &h.R0f, 2 * NN * h.nk));
   }
   d.Sinv = h.Sinv;
@@ -519,7 +530,6 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
   d.dq0 = h.dq0;
   d.eps0 = h.eps0;
   d.Sinv_p = h.Sinv_p;
-  d.D0_p = h.D0_p;
   d.R0f = h.R0f;
   return VGTB_OK;
 }
@@ -796,6 +806,107 @@ int ground_state(vgtb_ctx* ctx, int si) {
   return fail(ctx, VGTB_E_NO_CONVERGE, "system %d: SCC ground state not converged in %d iterations", si, max_it);
 }
 
+// FP64 products C = A R^dagger of the set-up (N x N, row stride Np): the sliced products from
+// kSliceMinN orbitals up (58 ms -> 2 ms each at N = 2048), else the FP64 pipe.  Owns its scratch.
+class SetupProducts {
+ public:
+  SetupProducts(vgtb_ctx* c, const HostSys& hs) : ctx(c), h(hs) {}
+  ~SetupProducts() {
+    cudaStreamSynchronize(ctx->stream);
+    slice_gemm_destroy(g);
+    for (void* p : mem) cudaFree(p);
+  }
+  template <class T>
+  int alloc(T** p, size_t n) {
+    void* q = nullptr;
+    *p = nullptr;
+    if (cudaMalloc(&q, n * sizeof(T)) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(ctx, VGTB_E_NOMEM, "cudaMalloc of %zu bytes failed", n * sizeof(T));
+    }
+    mem.push_back(q);
+    CK(cudaMemsetAsync(q, 0, n * sizeof(T), ctx->stream));
+    *p = (T*)q;
+    return VGTB_OK;
+  }
+  int init() {
+    TRY(alloc(&dg, 1));
+    if (h.N < kSliceMinN || h.N > kSliceMaxN || !tc_gemm_supported()) return VGTB_OK;
+    const size_t held = mem.size();
+    fa.rows = fa.K = h.N;
+    fa.Kp = slice_kp(h.N);
+    fa.batch = 1;
+    fr = fa;
+    const size_t dig = (size_t)kSlices * h.N * 2 * fa.Kp;
+    mp = slice_pairs_per_plane(slice_tiles(h.N, h.N));
+    nw = slice_nw(h.N);
+    std::string msg;
+    if (alloc(&fa.dig, dig) || alloc(&fr.dig, dig) || alloc(&fa.ex, h.N) || alloc(&fr.ex, h.N) ||
+        alloc(&planes, (size_t)slice_num_planes(mp) * h.N * 2 * nw) || alloc(&dj, 3) || alloc(&err, 1) ||
+        slice_gemm_create({fa, fr}, {SliceProd{0, 0, 1, 0, planes, nw, false, -1}}, {}, mp, 2000000000LL, err, &g,
+                          &msg)) {
+      // no room for the digits: the FP64 pipe
+      slice_gemm_destroy(g);
+      g = nullptr;
+      cudaStreamSynchronize(ctx->stream);
+      while (mem.size() > held) {
+        cudaFree(mem.back());
+        mem.pop_back();
+      }
+      cudaGetLastError();
+    }
+    return VGTB_OK;
+  }
+  int run(const double2* A, const double2* R, double2* C) {
+    if (g) {
+      SliceRowJob j[3] = {};
+      for (int q = 0; q < 2; ++q) {
+        j[q].rows = j[q].cols = h.N;
+        j[q].src = q ? R : A;
+        j[q].lds = h.Np;
+        j[q].out = q ? fr.mat(0) : fa.mat(0);
+      }
+      j[2].rows = j[2].cols = h.N;
+      j[2].n_planes = 1;
+      j[2].pl[0] = SlicePlanes{planes, (long long)h.N * 2 * nw, nw, fa.ex, fr.ex};
+      j[2].dst = C;
+      j[2].ldd = h.Np;
+      CK(cudaMemcpyAsync(dj, j, sizeof(j), cudaMemcpyHostToDevice, ctx->stream));
+      launch_slice_rows(dj, 2, h.N, h.N, mp, nullptr, ctx->stream);
+      if (slice_gemm_launch(g, ctx->stream)) return fail(ctx, VGTB_E_CUDA, "sliced set-up product launch failed");
+      launch_slice_rows(dj + 2, 1, h.N, h.N, mp, nullptr, ctx->stream);
+    } else {
+      GemmF64Item t{};
+      t.A[0] = A;
+      t.R[0] = R;
+      t.K[0] = t.M = t.N = h.N;
+      t.lda[0] = t.ldr[0] = t.ldc = h.Np;
+      t.nseg = 1;
+      t.C = C;
+      CK(cudaMemcpyAsync(dg, &t, sizeof(t), cudaMemcpyHostToDevice, ctx->stream));
+      launch_gemm_f64(dg, 1, h.N, h.N, nullptr, ctx->stream);
+    }
+    CK(cudaGetLastError());
+    return VGTB_OK;
+  }
+  int finish() {
+    int e = 0;
+    if (g) CK(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    return e ? fail(ctx, VGTB_E_TIMEOUT, "sliced set-up product reported status %d", e) : VGTB_OK;
+  }
+
+ private:
+  vgtb_ctx* ctx;
+  const HostSys& h;
+  SliceFam fa, fr;
+  int *planes = nullptr, *err = nullptr, mp = 7, nw = 0;
+  SliceRowJob* dj = nullptr;
+  GemmF64Item* dg = nullptr;
+  SliceGemm* g = nullptr;
+  std::vector<void*> mem;
+};
+
 // After D0 is set: charges of D0, eps0, R0 (delta forms), split pieces, and
 // every trajectory of the system back to step 0.
 int finish_density(vgtb_ctx* ctx, int si) {
@@ -812,59 +923,54 @@ int finish_density(vgtb_ctx* ctx, int si) {
   CK(cudaMemcpyAsync(h.dq0, h.dq0_h.data(), sizeof(double) * h.nat, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(h.eps0, h.eps0_h.data(), sizeof(double) * h.nat, cudaMemcpyHostToDevice, ctx->stream));
   if (ctx->delta) {
-    // R0 = -i(S^-1 H_ref D0 - h.c.) with H_ref = H(A = 0, eps0), all in FP64
-    double2 *Hb = nullptr, *Wb = nullptr, *Xb = nullptr;
-    TRY(dalloc(ctx, &Hb, NN));
-    TRY(dalloc(ctx, &Wb, NN));
-    TRY(dalloc(ctx, &Xb, NN));
-    double* eps_d = h.eps0;
-    GemmF64Item g[2] = {};
-    GemmF64Item* dg = nullptr;
-    LeapItem li{};
+    // constant terms of the delta form, all in FP64: R0 = -i(S^-1 H_ref D0 - h.c.) with
+    // H_ref = H(A = 0, eps0); split form: D0 S and K_a = -i(S^-1 P_a D0 - h.c.)
+    SetupProducts sp(ctx, h);
+    TRY(sp.init());
+    double2 *Hb = nullptr, *Wb = nullptr, *Xb = nullptr, *Kb = nullptr;
     LeapItem* dl = nullptr;
-    TRY(dalloc(ctx, &dg, 2));
-    TRY(dalloc(ctx, &dl, 1));
-    for (int k = 0; k < h.nk; ++k) {
-      CK(cudaMemsetAsync(Hb, 0, NN * sizeof(double2), ctx->stream));
-      launch_bloch_setup(ctx->d_sys, si, h.n_tgt, k, 1, eps_d, Hb, ctx->stream);
-      g[0] = GemmF64Item{};
-      g[0].A[0] = h.D0 + k * NN;
-      g[0].R[0] = Hb;
-      g[0].K[0] = h.Np;
-      g[0].lda[0] = g[0].ldr[0] = h.Np;
-      g[0].nseg = 1;
-      g[0].M = g[0].N = g[0].ldc = h.Np;
-      g[0].C = Wb;
-      g[1] = g[0];
-      g[1].A[0] = h.Sinv + k * NN;
-      g[1].R[0] = Wb;
-      g[1].C = Xb;
-      CK(cudaMemcpyAsync(dg, g, sizeof(g), cudaMemcpyHostToDevice, ctx->stream));
-      launch_gemm_f64(dg, 1, h.Np, h.Np, nullptr, ctx->stream);
-      launch_gemm_f64(dg + 1, 1, h.Np, h.Np, nullptr, ctx->stream);
-      li = LeapItem{};
+    TRY(sp.alloc(&Hb, NN));
+    TRY(sp.alloc(&Wb, NN));
+    TRY(sp.alloc(&Xb, NN));
+    TRY(sp.alloc(&Kb, NN));
+    TRY(sp.alloc(&dl, 1));
+    // out = -i(S^-1 B D0 - h.c.) for the Hermitian B in Hb
+    auto derivative = [&](int k, double2* out) -> int {
+      TRY(sp.run(h.D0 + k * NN, Hb, Wb));
+      TRY(sp.run(h.Sinv + k * NN, Wb, Xb));
+      LeapItem li{};
       li.X = Xb;
       li.N = h.N;
       li.Np = h.Np;
       li.mode = 1;
-      li.out = h.R0 + k * NN;
+      li.out = out;
       CK(cudaMemcpyAsync(dl, &li, sizeof(li), cudaMemcpyHostToDevice, ctx->stream));
       launch_leap(dl, 1, h.Np, 0, nullptr, 0.0, nullptr, nullptr, ctx->stream);
       CK(cudaGetLastError());
-      CK(cudaStreamSynchronize(ctx->stream));
+      return VGTB_OK;
+    };
+    for (int k = 0; k < h.nk; ++k) {
+      CK(cudaMemsetAsync(Hb, 0, NN * sizeof(double2), ctx->stream));
+      launch_bloch_setup(ctx->d_sys, si, h.n_tgt, k, 1, h.eps0, Hb, ctx->stream);
+      TRY(derivative(k, h.R0 + k * NN));
+      if (!ctx->split) continue;
+      launch_to_planar_f32(h.R0 + k * NN, h.R0f + 2 * NN * k, h.Np, ctx->stream);
+      launch_to_planar_f32(h.D0 + k * NN, h.D0f + 2 * NN * k, h.Np, ctx->stream);
+      launch_split_planar(h.Sinv + k * NN, h.Sinv_p + 4 * NN * k, h.N, h.Np, ctx->stream);
+      launch_scatter(h.d_kS + (size_t)k * h.n_el, h.d_el_off, h.n_el, Hb, ctx->stream);
+      TRY(sp.run(h.D0 + k * NN, Hb, Wb));
+      launch_to_planar_f32(Wb, h.Gf + 2 * NN * k, h.Np, ctx->stream);
+      for (int a = 0; a < 3; ++a) {
+        launch_scatter(h.d_kP + ((size_t)a * h.nk + k) * h.n_el, h.d_el_off, h.n_el, Hb, ctx->stream);
+        TRY(derivative(k, Kb));
+        launch_to_planar_f32(Kb, h.Kf + ((size_t)a * h.nk + k) * 2 * NN, h.Np, ctx->stream);
+      }
     }
+    CK(cudaGetLastError());
+    TRY(sp.finish());
   }
   if (h.d_jD0) {
     launch_slice_rows(h.d_jD0, h.nk, h.N, h.N, 7, nullptr, ctx->stream);
-    CK(cudaGetLastError());
-  }
-  if (ctx->split) {
-    for (int k = 0; k < h.nk; ++k) {
-      if (h.D0f) launch_to_f32(h.D0 + k * NN, h.D0f + k * NN, (long long)NN, ctx->stream);
-      if (h.D0_p) launch_split_planar(h.D0 + k * NN, h.D0_p + 4 * NN * k, h.N, h.Np, ctx->stream);
-      launch_split_planar(h.Sinv + k * NN, h.Sinv_p + 4 * NN * k, h.N, h.Np, ctx->stream);
-      launch_to_planar_f32(h.R0 + k * NN, h.R0f + 2 * NN * k, h.Np, ctx->stream);
-    }
     CK(cudaGetLastError());
   }
   h.density_set = true;
@@ -912,7 +1018,7 @@ int upload_traj_table(vgtb_ctx* ctx) {
     d.eps = h.eps;
     d.eps_lv = h.eps_lv;
     d.epsf = h.epsf;
-    d.depsf = h.depsf;
+    d.deh = h.deh;
     d.af = h.af;
     d.part = h.part;
     d.cpart = h.cpart;
@@ -933,10 +1039,6 @@ void drop_graph(vgtb_ctx* ctx) {
 // ---------------------------------------------------------------------------
 // Sliced FP64 products (k_slice.cu)
 // ---------------------------------------------------------------------------
-// From kSliceMinN orbitals up the 34 exact digit products on the tensor cores take less time than
-// one product on the FP64 pipe (N = 256, 8 k-points: 1.06 ms for one product on the FP64 pipe);
-// below, a product is a few microseconds of FP64 work and the extra launches cost more.
-constexpr int kSliceMinN = 97;
 
 int slice_family(vgtb_ctx* ctx, SliceFam& f, int rows, int K, int batch) {
   f.rows = rows;
@@ -1772,12 +1874,6 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
       return bail(fail(ctx, VGTB_E_UNSUPPORTED, "block-sparse product: %d targets per atom group exceed shared memory",
                        ctx->bsr_tg_max));
     if ((rc = upload(ctx, &ctx->d_bsrsys, bsys.data(), bsys.size()))) return bail(rc);
-    if (ctx->split)
-      for (int s = 0; s < n_sys; ++s) {
-        HostSys& h = ctx->sys[s];
-        if ((rc = dalloc(ctx, &h.D0f, (size_t)h.nk * h.Np * h.Np))) return bail(rc);
-        dsys[s].D0f = h.D0f;
-      }
   }
   if ((rc = upload(ctx, &ctx->d_sys, dsys.data(), dsys.size()))) return bail(rc);
   // trajectories and items; the split form keeps each operand family of a
@@ -1787,7 +1883,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
   std::vector<int> sys_items(n_sys, 0), sys_next(n_sys, 0);
   for (int t = 0; t < n_traj; ++t) sys_items[traj_sys[t]] += ctx->sys[traj_sys[t]].nk;
   struct Fam {
-    __nv_bfloat16 *dD = nullptr, *Hemb = nullptr, *dHemb = nullptr, *Wemb = nullptr;
+    __nv_bfloat16 *dD = nullptr, *Hemb = nullptr, *Wemb = nullptr;
     float* Xf = nullptr;
   };
   std::vector<Fam> fam(n_sys);
@@ -1798,7 +1894,6 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
       if (!ctx->bsr) {
         if ((rc = dalloc(ctx, &fam[s].dD, 4 * NN * ni))) return bail(rc);
         if ((rc = dalloc(ctx, &fam[s].Hemb, 8 * NN * ni))) return bail(rc);
-        if ((rc = dalloc(ctx, &fam[s].dHemb, 8 * NN * ni))) return bail(rc);
       }
       if ((rc = dalloc(ctx, &fam[s].Wemb, 8 * NN * ni))) return bail(rc);
       if ((rc = dalloc(ctx, &fam[s].Xf, 2 * NN * ni))) return bail(rc);
@@ -1826,19 +1921,17 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
       if (ctx->split) {
         const size_t li = sys_next[T.sys]++;
         if (ctx->bsr) {
-          float2 *kh = nullptr, *kdh = nullptr;
+          float2* kh = nullptr;
           if ((rc = dalloc(ctx, &it.dDf, NN))) return bail(rc);
           if ((rc = dalloc(ctx, &kh, (size_t)h.n_el))) return bail(rc);
-          if ((rc = dalloc(ctx, &kdh, (size_t)h.n_el))) return bail(rc);
           it.kH = kh;
-          it.kdH = kdh;
         } else {
           it.dD_p = fam[T.sys].dD + 4 * NN * li;
           it.Hemb_p = fam[T.sys].Hemb + 8 * NN * li;
-          it.dHemb_p = fam[T.sys].dHemb + 8 * NN * li;
         }
         it.Wemb_p = fam[T.sys].Wemb + 8 * NN * li;
         it.Xf = fam[T.sys].Xf + 2 * NN * li;
+        it.Gf = h.Gf + 2 * NN * k;
       } else if (ctx->cn) {
         const size_t nc = (size_t)h.nocc * h.Np;
         if (ctx->bsr || h.slice) {
@@ -1876,7 +1969,8 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     if (ctx->cn && (rc = dalloc(ctx, &T.eps_lv, 2 * (size_t)h.nat))) return bail(rc);
     if (ctx->split) {
       if ((rc = dalloc(ctx, &T.epsf, h.nat))) return bail(rc);
-      if ((rc = dalloc(ctx, &T.depsf, h.nat))) return bail(rc);
+      if ((rc = dalloc(ctx, &T.deh, h.Np))) return bail(rc);
+      for (int k = 0; k < h.nk; ++k) ctx->items_h[T.item0 + k].ge = T.deh;
       if ((rc = dalloc(ctx, &T.af, 3))) return bail(rc);
     }
     if ((rc = dalloc(ctx, &T.part, 5 * (size_t)h.n_tgt))) return bail(rc);
@@ -1934,7 +2028,14 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     LeapItem l{};
     l.X = ctx->split ? (const void*)it.Xf : (const void*)it.X;
     l.R0 = (ctx->delta && !ctx->split) ? h.R0 + it.k * NN : nullptr;
-    l.R0f = ctx->split ? h.R0f + 2 * NN * it.k : nullptr;
+    if (ctx->split) {
+      l.R0f = h.R0f + 2 * NN * it.k;
+      l.Kf = h.Kf + 2 * NN * it.k;
+      l.k_stride = (long long)(2 * NN * h.nk);
+      l.D0f = h.D0f + 2 * NN * it.k;
+      l.af = ctx->trj[it.traj].af;
+      l.deh = it.ge;
+    }
     l.D[0] = it.D[0];
     l.D[1] = it.D[1];
     l.pieces = it.dD_p;
@@ -1965,7 +2066,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
       const size_t NN = (size_t)h.Np * h.Np;
       BsrItem b{};
       b.sys = it.sys;
-      b.nseg = ctx->delta ? 2 : 1;
+      b.nseg = ctx->delta && !ctx->split ? 2 : 1;
       b.R[0] = it.kH;
       b.R[1] = it.kdH;
       if (ctx->cn) {
@@ -1974,7 +2075,8 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
         b.W = it.W;
       } else if (ctx->split) {
         b.A[0] = it.dDf;                       // FP32 copy of the current dD level
-        b.A[1] = h.D0f + it.k * NN;
+        b.G = it.Gf;
+        b.ge = it.ge;
         b.W = it.Wemb_p;
       } else {
         b.A[0] = it.D[0];                      // level of the step's parity
@@ -2011,10 +2113,8 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
       views[s].nk = ctx->sys[s].nk;
       views[s].n_items = sys_items[s];
       views[s].Sinv_p = ctx->sys[s].Sinv_p;
-      views[s].D0_p = ctx->sys[s].D0_p;
       views[s].dD_p = fam[s].dD;
       views[s].Hemb_p = fam[s].Hemb;
-      views[s].dHemb_p = fam[s].dHemb;
       views[s].Wemb_p = fam[s].Wemb;
       views[s].k_real = &ctx->sys[s].k_real;
       if (ctx->opt.product1 != VGTB_P1_DENSE) {  // nonzero pattern: zero k-panels of product 1 are skipped

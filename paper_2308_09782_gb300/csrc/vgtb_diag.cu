@@ -55,13 +55,11 @@ extern "C" int vgtb_diag_split_chain_variant(int n, const double* a, const doubl
   Scratch m;
   double2* dsrc = m.get<double2>(NN);
   __nv_bfloat16* a_p = m.get<__nv_bfloat16>(4 * NN);
-  __nv_bfloat16* d0_p = m.get<__nv_bfloat16>(4 * NN);
   __nv_bfloat16* s_p = m.get<__nv_bfloat16>(4 * NN);
   __nv_bfloat16* r_e = m.get<__nv_bfloat16>(8 * NN);
-  __nv_bfloat16* z_e = m.get<__nv_bfloat16>(8 * NN);
   __nv_bfloat16* w_e = m.get<__nv_bfloat16>(8 * NN);
   float* xf = m.get<float>(2 * NN);
-  if (!dsrc || !a_p || !d0_p || !s_p || !r_e || !z_e || !w_e || !xf) return VGTB_E_NOMEM;
+  if (!dsrc || !a_p || !s_p || !r_e || !w_e || !xf) return VGTB_E_NOMEM;
   cudaStream_t st = 0;
   std::vector<double2> h;
   to_padded(a, h, n, Np);
@@ -81,10 +79,8 @@ extern "C" int vgtb_diag_split_chain_variant(int n, const double* a, const doubl
   views[0].nk = 1;
   views[0].n_items = 1;
   views[0].Sinv_p = s_p;
-  views[0].D0_p = d0_p;
   views[0].dD_p = a_p;
   views[0].Hemb_p = r_e;
-  views[0].dHemb_p = z_e;
   views[0].Wemb_p = w_e;
   std::vector<DevItem> items(1);
   memset(&items[0], 0, sizeof(DevItem));

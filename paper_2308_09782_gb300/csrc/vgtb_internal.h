@@ -130,14 +130,12 @@ struct DevSys {
   double* dq0;             // [nat] charges of D(0)
   double* eps0;            // [nat] shift of D(0)
   __nv_bfloat16* Sinv_p;   // [nk][2][Np][2Np] split pieces (split form)
-  __nv_bfloat16* D0_p;     // [nk][2][Np][2Np]
   // split form only: FP32 copies for the phase build and the leapfrog derivative
   const float* h0f;        // values as float
   const float* sf;
   const float* dsf;        // [3][ds_stride]
   const float2* phasef;    // [nk][n_blk]
   float* R0f;              // [nk][Np][2Np] planar
-  float2* D0f;             // [nk][Np][Np] FP32 copy of D0 (split form, block-sparse first product)
   // split-form phase build: per target {I, J, first image, end image} and
   // {o_I, o_J, n_I | vec << 16, n_J}; the FP32 phase of every (k, image)
   const int4* tgt_p0;      // [n_tgt]
@@ -160,7 +158,7 @@ struct DevTraj {
   double* eps_lv;          // [2][nat] eps of the two latest levels by parity (Crank-Nicolson), or null
   // split form: FP32 operands of the phase build, written by k_scc_eps at level n
   float* epsf;             // [nat] eps_I
-  float* depsf;            // [nat] eps_I - eps0_I
+  float* deh;              // [Np] (eps_I - eps0_I) / 2 of every orbital (padding 0): D0 terms of W and dD/dt
   float* af;               // [3] A(t_n) / c
   double* part;            // [n_tgt][5] per-target partial sums
   double* cpart;           // [ceil(nat / kSccRowsPerCta)][6] per-CTA partial sums of k_scc_eps
@@ -178,13 +176,14 @@ struct DevItem {
   double2* X;              // FP64 second product
   __nv_bfloat16* dD_p;     // split form: [2][Np][2Np] pieces of dD
   __nv_bfloat16* Hemb_p;   // split form: [2][2Np][2Np] embedded H
-  __nv_bfloat16* dHemb_p;  // split form: [2][2Np][2Np] embedded dH
   __nv_bfloat16* Wemb_p;   // split form: [2][2Np][2Np] embedded W
+  const float* Gf;         // split form: D0 S of the item's k-point, planar FP32 [Np][2Np]
+  const float* ge;         // split form: (eps_I - eps0_I) / 2 of every orbital [Np]
   float* Xf;               // split form: [Np][2Np] planar X
   double2* Cd;             // Crank-Nicolson: occupied states as rows, C^dagger [nocc][Np]
   double2* Y[2];           // Crank-Nicolson: fixed-point iterates [nocc][Np]
   // block-sparse first product: H_k(t) and dH_k(t) at the target elements only
-  // ([n_el], complex; double2 on the FP64 path, float2 in the split form), and in
+  // ([n_el], complex; double2 on the FP64 path, float2 in the split form, which has no kdH), and in
   // the split form the FP32 copy of the current dD level ([Np][Np] float2)
   void* kH;
   void* kdH;
@@ -215,6 +214,8 @@ struct BsrItem {
   long long a_par;         // segment 0 reads A[0] + ((*step) & 1) * a_par (leapfrog level)
   const void* R[2];        // [n_el] complex target blocks (4 x 4 row-major each)
   void* W;                 // FP64: [Np][Np] double2; split: embedded BF16 pieces [2][2Np][2Np]
+  const float* G;          // split: W_ij += G_ij ge_j (planar FP32 [Np][2Np], one factor per orbital)
+  const float* ge;
 };
 int bsr_group(int fp64);
 size_t bsr_smem_bytes(int fp64, int max_grp_targets);
@@ -329,6 +330,12 @@ struct LeapItem {
   SlicePlanes pl;          // or the planes of X (launch_leap with mp != 0)
   const double2* R0;       // optional (FP64 path)
   const float* R0f;        // optional (split path, FP32 planar)
+  // split path, the terms of the derivative that are linear in A and in the shift:
+  const float* Kf;         // [3] planes, stride k_stride: K_a = -i (S^-1 P_a D0 - h.c.), FP32 planar
+  long long k_stride;
+  const float* D0f;        // D0, FP32 planar
+  const float* af;         // A(t_n) / c
+  const float* deh;        // (eps_I - eps0_I) / 2 per orbital
   double2* D[2];
   __nv_bfloat16* pieces;   // optional [2][Np][2Np]
   float2* f32;             // optional [Np][Np]: FP32 copy of the new level (split form)
@@ -347,6 +354,7 @@ void launch_leap_split(const LeapItem* items, int n_items, int Np_max, const int
 // real: the matrix is real, imaginary parts (rounding) are set to zero
 void launch_fill_hermitian_lower(double2* a, int n, int ld, int real, cudaStream_t st);
 void launch_vt_from_evecs(const double2* evec, double2* vt, int n, int nocc, int ld, cudaStream_t st);
+void launch_scatter(const double2* v, const int* off, int n, double2* out, cudaStream_t st);
 void launch_scale(double2* a, long long n, double s, cudaStream_t st);
 void launch_split_planar(const double2* src, __nv_bfloat16* dst, int N, int Np, cudaStream_t st);
 void launch_increment(int* step, cudaStream_t st);

@@ -99,8 +99,8 @@ __global__ void k_na_embedded(const double2* __restrict__ r, int n, int Np, __nv
 __global__ void k_na_prob(TcProb* prob, int* err, int Np, float* out) {
   TcProb p;
   p.sys = 0;
-  p.a_b[0] = p.a_b[1] = 0;
-  p.b_b[0] = p.b_b[1] = 0;
+  p.a_b = 0;
+  p.b_b = 0;
   p.tiles_m = Np / BM;
   p.tiles_n = 2 * Np / 256;
   p.tile0 = 0;
@@ -110,6 +110,8 @@ __global__ void k_na_prob(TcProb* prob, int* err, int Np, float* out) {
   p.iter0 = 0;
   p.kofs = nullptr;  // every k-panel
   p.kidx = nullptr;
+  p.G = nullptr;
+  p.ge = nullptr;
   p.w_half = 0;
   p.cofs = nullptr;  // column tiles of 256
   *prob = p;
@@ -199,12 +201,11 @@ extern "C" int vgtb_split_cgemm_noalloc(int n, const double* a, const double* r,
   k_na_prob<<<1, 1, 0, st>>>(prob, err, Np, xo);
   TcParams P;
   memset(&P, 0, sizeof(P));
-  if (!na_map(&P.mA[0][0], ap, 2 * Np, Np, BM) || !na_map(&P.mB[0][0], rp, 2 * Np, 2 * Np, 256))
+  if (!na_map(&P.mA[0], ap, 2 * Np, Np, BM) || !na_map(&P.mB[0], rp, 2 * Np, 2 * Np, 256))
     return VGTB_E_CUDA;
   P.probs = prob;
   P.n_prob = 1;
   P.total_tiles = (Np / BM) * (2 * Np / 256);
-  P.nseg = 1;
   P.err = err;
   P.timeout_ns = 2000000000LL;
   const int smem = 2 * (2 * BM * BK * 2 + 2 * 256 * BK * 2) + 1024 + 256;

@@ -14,15 +14,12 @@ struct TcPlan;  // tensor maps, problem table and launch shape of one product
 struct TcSysView {
   int Np, nk, n_items;
   __nv_bfloat16* Sinv_p;   // [nk][2][Np][2Np]
-  __nv_bfloat16* D0_p;     // [nk][2][Np][2Np]
   __nv_bfloat16* dD_p;     // [n_items][2][Np][2Np]
   __nv_bfloat16* Hemb_p;   // [n_items][2][2Np][2Np]
-  __nv_bfloat16* dHemb_p;  // [n_items][2][2Np][2Np]
   __nv_bfloat16* Wemb_p;   // [n_items][2][2Np][2Np]
   // nonzero pattern of H_k (host data, may be null): orbital offsets of the
   // atoms and the atom pairs (I, J) of the targets.  With it, the classic
-  // schedules of product 1 skip the k-panels in which a tile's rows of H and dH
-  // are zero.
+  // schedules of product 1 skip the k-panels in which a tile's rows of H are zero.
   const std::vector<int>* orb_off = nullptr;
   const std::vector<int>* tgt_I = nullptr;
   const std::vector<int>* tgt_J = nullptr;
@@ -32,7 +29,7 @@ struct TcSysView {
 };
 
 // Plans for the two products of the split form, over every item:
-//   product 1: W = [dD | D0] [H | dH]^dagger  -> embedded BF16 hi/lo pieces of W
+//   product 1: W = dD H^dagger + G diag(e)     -> embedded BF16 hi/lo pieces of W
 //   product 2: X = S^-1 W^dagger               -> FP32 planar X
 // force_variant[p] >= 0 uses that tile variant for product p+1; otherwise variant
 // 0, or with autotune the fastest candidate (median of 9 timed launches).
