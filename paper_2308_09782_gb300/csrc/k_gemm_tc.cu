@@ -63,18 +63,18 @@ struct Variant {
 // near-equal widths, multiples of 16, with the shortest modelled time of the
 // longest worker, see plan_columns; 2: the same among splits into tiles at
 // least 192 wide, which re-read the A operand less often), k-slices per 64-wide
-// panel (1: stages of 64 columns; 2: stages of 32 columns, 7 of them, for the
+// panel (1: stages of 64 columns; 2: stages of 32 columns, 6 of them, for the
 // pair kernel).  Variant 0 is the default; all are
 // autotune candidates.
 constexpr Variant kVariants[] = {{256, 3, 0, 1, 0, 1}, {256, 3, 1, 1, 0, 1}, {256, 3, 2, 1, 0, 1},
                                  {256, 2, 0, 0, 0, 1}, {256, 2, 1, 0, 0, 1}, {128, 3, 0, 0, 0, 1},
                                  {128, 3, 1, 0, 0, 1}, {256, 3, 0, 1, 1, 1}, {256, 3, 0, 1, 2, 1},
-                                 {256, 7, 0, 1, 0, 2}, {256, 7, 0, 1, 1, 2}, {256, 7, 1, 1, 0, 2}};
+                                 {256, 6, 0, 1, 0, 2}, {256, 6, 0, 1, 1, 2}, {256, 6, 1, 1, 0, 2}};
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
 template <int BN, int ST, int EPI>
 int smem_bytes() {
-  return ST * (2 * BM * BK * 2 + 2 * BN * BK * 2) + 1024 + 256;
+  return ST * (2 * BM * BK * 2 + 2 * BN * BK * 2) + 256 + 4 * kEpiStage + 1024;
 }
 
 template <int BN, int ST, int EPI>
@@ -84,7 +84,7 @@ cudaError_t launch_t(const TcPlan* p, cudaStream_t st) {
 
 template <int ST, int KH>
 int smem_pair() {
-  return ST * (2 * BM * (BK / KH) * 2 + 2 * 128 * (BK / KH) * 2) + 1024 + 256;
+  return ST * (2 * BM * (BK / KH) * 2 + 2 * 128 * (BK / KH) * 2) + 256 + 4 * kEpiStage + 1024;
 }
 
 template <int ST, int EPI, int KH>
@@ -115,7 +115,7 @@ cudaError_t configure_t() {
 cudaError_t launch_variant(const TcPlan* p, cudaStream_t st) {
   if (kVariants[p->variant].pair) {
     if (kVariants[p->variant].kh == 2)
-      return p->epi == 0 ? launch_pair<7, 0, 2>(p, st) : launch_pair<7, 1, 2>(p, st);
+      return p->epi == 0 ? launch_pair<6, 0, 2>(p, st) : launch_pair<6, 1, 2>(p, st);
     return p->epi == 0 ? launch_pair<3, 0, 1>(p, st) : launch_pair<3, 1, 1>(p, st);
   }
   const bool wide = kVariants[p->variant].bn == 256;
@@ -124,7 +124,7 @@ cudaError_t launch_variant(const TcPlan* p, cudaStream_t st) {
 }
 
 int variant_smem(int v) {
-  if (kVariants[v].pair) return kVariants[v].kh == 2 ? smem_pair<7, 2>() : smem_pair<3, 1>();
+  if (kVariants[v].pair) return kVariants[v].kh == 2 ? smem_pair<6, 2>() : smem_pair<3, 1>();
   return kVariants[v].bn == 256 ? smem_bytes<256, 2, 0>() : smem_bytes<128, 3, 0>();
 }
 
@@ -140,11 +140,11 @@ cudaError_t configure_all() {
   if ((e = cudaFuncSetAttribute(k_tc_gemm2<3, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 smem_pair<3, 1>())) != cudaSuccess)
     return e;
-  if ((e = cudaFuncSetAttribute(k_tc_gemm2<7, 0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                smem_pair<7, 2>())) != cudaSuccess)
+  if ((e = cudaFuncSetAttribute(k_tc_gemm2<6, 0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                smem_pair<6, 2>())) != cudaSuccess)
     return e;
-  if ((e = cudaFuncSetAttribute(k_tc_gemm2<7, 1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                smem_pair<7, 2>())) != cudaSuccess)
+  if ((e = cudaFuncSetAttribute(k_tc_gemm2<6, 1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                smem_pair<6, 2>())) != cudaSuccess)
     return e;
   return cudaFuncSetAttribute(k_tc_chain<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_pair<3, 1>());
 }
@@ -321,11 +321,24 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
   // column tiles of every system
   std::vector<std::vector<int>> starts(sys.size());
   int wmax = 0;
+  // 2-SM pairs with equal column tiles: halve the width (down to 32) as long as the tiles do not
+  // fill half of the pairs.  Few tiles leave most pairs idle, and what a tile costs beyond its
+  // k-iterations (the epilogue) shrinks with its width; above that, wider tiles read A less often.
+  int bw = BNv;
+  if (pair && !var.widths && !var.streamk) {
+    auto count = [&](int w) {
+      long long n = 0;
+      for (const DevItem& it : items) n += (long long)((sys[it.sys].Np + tm_rows - 1) / tm_rows) * (2 * sys[it.sys].Np / w);
+      return n;
+    };
+    while (bw > 32 && 2 * count(bw) <= G_full) bw /= 2;
+  }
+  const bool narrow = bw != BNv;
   for (size_t s = 0; s < sys.size(); ++s) {
     const int tiles_m = (sys[s].Np + tm_rows - 1) / tm_rows;
     const int full = 2 * sys[s].Np / BK / (epi == 1 && n_real == (int)items.size() ? 2 : 1);
     starts[s] = var.widths ? plan_columns(sys[s], skip, full, tiles_m, G_full, var.widths)
-                           : even_split(2 * sys[s].Np, 2 * sys[s].Np / BNv);
+                           : even_split(2 * sys[s].Np, 2 * sys[s].Np / bw);
     for (size_t i = 0; i + 1 < starts[s].size(); ++i) wmax = std::max(wmax, starts[s][i + 1] - starts[s][i]);
   }
   const int bbox = pair ? wmax / 2 : BNv;  // B rows loaded by one CTA
@@ -372,7 +385,7 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
     cudaMemcpy(plan->d_kidx, all_kidx.data(), sizeof(short) * all_kidx.size(), cudaMemcpyHostToDevice);
     plan->skip = true;
   }
-  if (var.widths) {
+  if (var.widths || narrow) {
     for (size_t s = 0; s < sys.size(); ++s) {
       sys_cofs0[s] = (int)all_cofs.size();
       all_cofs.insert(all_cofs.end(), starts[s].begin(), starts[s].end());
@@ -418,7 +431,7 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
       pr.kidx = plan->d_kidx + sys_kidx0[it.sys];
       pr.kt = sys_cnt[it.sys][0];  // uniform lists: one length
     }
-    if (var.widths) pr.cofs = plan->d_cofs + sys_cofs0[it.sys];
+    if (var.widths || narrow) pr.cofs = plan->d_cofs + sys_cofs0[it.sys];
     for (int nt = 0; nt < pr.tiles_n; ++nt)
       for (int mt = 0; mt < pr.tiles_m; ++mt)
         tile_cost.push_back(tile_model(st[nt + 1] - st[nt], listed ? sys_cnt[it.sys][nt] : pr.kt));
@@ -631,10 +644,8 @@ void tc_clear_error(TcPlan* p) {
 int tc_plan_info(const TcPlan* p, int* out4) {
   if (!p || tc_variant_info(p->variant, out4)) return -1;
   if (p->skip) out4[2] += 4;  // 4, 5, 6: the schedule with zero k-panels skipped
-  if (kVariants[p->variant].widths) {
-    out4[0] = p->wmax;        // the widest column tile
-    out4[2] += 8;             // 8, 12: classic over planned column widths
-  }
+  if (kVariants[p->variant].pair) out4[0] = p->wmax;  // the widest column tile
+  if (kVariants[p->variant].widths) out4[2] += 8;       // 8, 12: classic over planned column widths
   return 0;
 }
 

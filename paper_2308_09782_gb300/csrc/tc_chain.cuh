@@ -169,10 +169,14 @@ __global__ void __launch_bounds__(192, 1)
         const uint32_t stage_tx = 2 * A_BYTES + 2 * (uint32_t)(Q.b_rows ? Q.b_rows : BNP / 2) * BK * 2;
         const int arow = mt * (2 * BM) + rank * BM, brow = cb + rank * (w / 2);
         const int KT = tile_kt(pr, t);
+        const CUtensorMap* ma = &Q.mA[pr.sys];
+        const CUtensorMap* mb = &Q.mB[pr.sys];
+        const int a_b = pr.a_b, b_b = pr.b_b;
+        const short* kidx = pr.kofs ? pr.kidx + pr.kofs[nt] : nullptr;
+        int ktn = kidx ? kidx[0] : 0;  // the next panel's number is read a panel ahead
         for (int kk = 0; kk < KT; ++kk, ++it) {
-          const int kt = tile_panel(pr, t, kk);
-          const CUtensorMap* ma = &Q.mA[pr.sys];
-          const CUtensorMap* mb = &Q.mB[pr.sys];
+          const int kt = ktn;
+          if (kk + 1 < KT) ktn = kidx ? kidx[kk + 1] : kk + 1;
           const int s = it % ST, r = it / ST;
           if (!mbar_wait(empty0 + 8 * s, (r & 1) ^ 1, limit, abort_flag, err)) {
             ok = false;
@@ -181,10 +185,10 @@ __global__ void __launch_bounds__(192, 1)
           const uint32_t base = smem_u32(sm + s * STAGE);
           if (leader_cta) mbar_expect_tx(full0 + 8 * s, 2 * stage_tx);
           const uint32_t fb = full_l + 8 * s;
-          tma_load_4d_pair(base, ma, kt * BK, arow, 0, pr.a_b, fb);
-          tma_load_4d_pair(base + A_BYTES, ma, kt * BK, arow, 1, pr.a_b, fb);
-          tma_load_4d_pair(base + 2 * A_BYTES, mb, kt * BK, brow, 0, pr.b_b, fb);
-          tma_load_4d_pair(base + 2 * A_BYTES + B_BYTES, mb, kt * BK, brow, 1, pr.b_b, fb);
+          tma_load_4d_pair(base, ma, kt * BK, arow, 0, a_b, fb);
+          tma_load_4d_pair(base + A_BYTES, ma, kt * BK, arow, 1, a_b, fb);
+          tma_load_4d_pair(base + 2 * A_BYTES, mb, kt * BK, brow, 0, b_b, fb);
+          tma_load_4d_pair(base + 2 * A_BYTES + B_BYTES, mb, kt * BK, brow, 1, b_b, fb);
         }
       }
       if (!ok) {
@@ -251,6 +255,7 @@ __global__ void __launch_bounds__(192, 1)
     // ---------------- epilogue (warps 2..5 of both CTAs) ----------------
     const int q = warp & 3;
     const bool leader = threadIdx.x == 64;
+    uint4* stg = reinterpret_cast<uint4*>(sm + ST * STAGE + 256 + (warp - 2) * kEpiStage);
     int i = 0, j = 0, e, t;
     for (; chain_next(X, pair, G2, j, e, t); ++i) {
       const TcParams& Q = e ? P2 : P1;
@@ -259,37 +264,35 @@ __global__ void __launch_bounds__(192, 1)
       const int local = t - pr.tile0;
       const int mt = local % pr.tiles_m, nt = local / pr.tiles_m;
       const int ab = i & 1, u = i >> 1;
+      const int rt = q * 32 + lane;
+      const int row = mt * (2 * BM) + rank * BM + rt;
+      int cb, w;
+      col_tile(pr, nt, cb, w);
+      GChunk g;
+      if (!e) load_g(pr, row, cb, w < 32 ? 1 : 2, g);  // in flight during the wait
       if (leader) {
         s_epi_ok[i & 1] = mbar_wait(accf0 + 8 * ab, u & 1, limit, abort_flag, err) ? 1 : 0;
       }
       epi_bar();
       if (!s_epi_ok[i & 1]) break;
       tc_fence_after();
-      const int Np = pr.Np;
-      const long long ld = 2LL * Np;
-      const int rt = q * 32 + lane;
-      const int row = mt * (2 * BM) + rank * BM + rt;
-      int cb, w;
-      col_tile(pr, nt, cb, w);
 #pragma unroll 1
       for (int c0 = 0; c0 < w; c0 += 32) {
         uint32_t r[32];
+        const GChunk gc = g;
+        if (!e && c0 + 32 < w) load_g(pr, row, cb + c0 + 32, w - c0 - 32 < 32 ? 1 : 2, g);
         const uint32_t taddr = tmem + ab * BNP + c0 + ((uint32_t)(q * 32) << 16);
         TMEM_LD32(taddr, r);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         const int gn = cb + c0;
         const int nv = w - c0 < 32 ? w - c0 : 32;
-        if (row >= Np) continue;
         if (e) {
-          float* Xo = reinterpret_cast<float*>(pr.out) + row * ld + gn;
-#pragma unroll
-          for (int v = 0; v < 8; ++v)
-            if (4 * v < nv)
-              reinterpret_cast<float4*>(Xo)[v] =
-                  make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
-                              __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
+          store_x(pr, stg, row - lane, lane, gn, r, nv);
         } else {
-          store_w_pieces(pr, row, gn, r, nv >> 4);
+          const int slot = (c0 >> 5) & 1;
+          stage_w(pr, stg, row, lane, gc, r, nv >> 4, slot);
+          if (slot || c0 + 32 >= w)
+            flush_w(pr, stg, row - lane, lane, (gn - 32 * slot) >> 1, 2 * slot + (nv >> 4));
         }
       }
       tc_fence_before();

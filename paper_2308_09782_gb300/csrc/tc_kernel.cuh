@@ -146,7 +146,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long lo
   long long t0 = 0;
   for (int it = 0;; ++it) {
     if (mbar_try(bar, parity)) return true;
-    if ((it & 31) == 31) {
+    if ((it & 3) == 0) {
       if (check_abort && *abort_flag) return false;
       const long long now = gtime();
       if (t0 == 0) {
@@ -352,24 +352,43 @@ __device__ __forceinline__ float4* ws_slot(const TcParams& P, int c, int bn) {
 
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
-__device__ __forceinline__ uint4 pack8_bf16(const float (&x)[16], int h, float sgn) {
-  return make_uint4(pack_bf16(sgn * x[8 * h], sgn * x[8 * h + 1]), pack_bf16(sgn * x[8 * h + 2], sgn * x[8 * h + 3]),
-                    pack_bf16(sgn * x[8 * h + 4], sgn * x[8 * h + 5]), pack_bf16(sgn * x[8 * h + 6], sgn * x[8 * h + 7]));
+// Epilogue staging: every epilogue warp has 8 KB of shared memory in which it turns the rows that
+// its threads hold (one accumulator row each) into runs of 64 bytes (W) or 128 bytes (X) per row, so
+// that a store instruction touches 8 or 4 lines instead of 32.  With direct stores an epilogue of a
+// 256-wide tile spent 16 thousand clocks (W) or 8 thousand (X) in the load/store unit.
+constexpr int kEpiStage = 8192;  // bytes per epilogue warp
+
+__device__ __forceinline__ uint4 pack8_bf16(const float (&x)[16], int h) {
+  return make_uint4(pack_bf16(x[8 * h], x[8 * h + 1]), pack_bf16(x[8 * h + 2], x[8 * h + 3]),
+                    pack_bf16(x[8 * h + 4], x[8 * h + 5]), pack_bf16(x[8 * h + 6], x[8 * h + 7]));
 }
 
 // Product 1 epilogue: 32 accumulator columns gn .. gn + 31 of output row `row`
-// (gn a multiple of 32) in the interleaved order (4 Re, 4 Im per block of four W
-// columns) become 16 consecutive W columns j0 = gn / 2 .. j0 + 15, stored as the
-// embedded BF16 pieces of W that product 2 reads as its B operand: top row m =
-// [Re W | Im W], bottom row Np + m = [-Im W | Re W], hi at 0 and lo at 4 Np^2.
+// (gn a multiple of 16) in the interleaved order (4 Re, 4 Im per block of four W
+// columns) become 16 consecutive W columns j0 = gn / 2 .. j0 + 15.  The term
+// G_mj e_j is added first, in FP32; the hi and lo pieces of Re and Im go to slot
+// `slot` (0 or 1) of the staging area [piece][row][64 bytes].
 // (nh = 1: only the first 16 accumulator columns are the tile's, 8 W columns).
-// half: only [Re W] of the top and [-Im W] of the bottom row (w_half).  The term
-// G_mj e_j is added first, in FP32.
-__device__ __forceinline__ void store_w_pieces(const TcProb& pr, int row, int gn, const uint32_t (&r)[32], int nh) {
-  __nv_bfloat16* W = reinterpret_cast<__nv_bfloat16*>(pr.out);
-  const int Np = pr.Np, half = pr.w_half;
-  const long long ld = 2LL * Np, P1 = 4LL * Np * Np;
-  const int j0 = gn >> 1;
+// The D0 term's operands for 32 accumulator columns, read a chunk ahead of their use.
+struct GChunk {
+  float4 re[4], im[4], e[4];
+};
+
+__device__ __forceinline__ void load_g(const TcProb& pr, int row, int gn, int nh, GChunk& c) {
+  if (!pr.G || row >= pr.Np) return;
+  const float4* g = reinterpret_cast<const float4*>(pr.G + (long long)row * 2 * pr.Np + (gn >> 1));
+  const float4* e = reinterpret_cast<const float4*>(pr.ge + (gn >> 1));
+#pragma unroll
+  for (int b = 0; b < 4; ++b)
+    if (b < 2 * nh) {
+      c.re[b] = g[b];
+      c.im[b] = g[b + pr.Np / 4];
+      c.e[b] = e[b];
+    }
+}
+
+__device__ __forceinline__ void stage_w(const TcProb& pr, uint4* stg, int row, int lane, const GChunk& g,
+                                        const uint32_t (&r)[32], int nh, int slot) {
   float re[16], im[16], rel[16], iml[16];
 #pragma unroll
   for (int b = 0; b < 4; ++b)
@@ -378,13 +397,11 @@ __device__ __forceinline__ void store_w_pieces(const TcProb& pr, int row, int gn
       re[4 * b + q] = __uint_as_float(r[8 * b + q]);
       im[4 * b + q] = __uint_as_float(r[8 * b + 4 + q]);
     }
-  if (pr.G) {
-    const float4* g = reinterpret_cast<const float4*>(pr.G + (long long)row * ld + j0);
-    const float4* e = reinterpret_cast<const float4*>(pr.ge + j0);
+  if (pr.G && row < pr.Np) {
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       if (b >= 2 * nh) break;
-      const float4 gr = g[b], gi = g[b + Np / 4], f = e[b];
+      const float4 gr = g.re[b], gi = g.im[b], f = g.e[b];
       re[4 * b] = fmaf(gr.x, f.x, re[4 * b]);
       re[4 * b + 1] = fmaf(gr.y, f.y, re[4 * b + 1]);
       re[4 * b + 2] = fmaf(gr.z, f.z, re[4 * b + 2]);
@@ -403,20 +420,65 @@ __device__ __forceinline__ void store_w_pieces(const TcProb& pr, int row, int gn
     re[i] = rh;
     im[i] = ih;
   }
-  const long long top = (long long)row * ld + j0, bot = (long long)(Np + row) * ld + j0;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    if (h >= nh) break;
-    reinterpret_cast<uint4*>(W + top)[h] = pack8_bf16(re, h, 1.f);
-    reinterpret_cast<uint4*>(W + P1 + top)[h] = pack8_bf16(rel, h, 1.f);
-    reinterpret_cast<uint4*>(W + bot)[h] = pack8_bf16(im, h, -1.f);
-    reinterpret_cast<uint4*>(W + P1 + bot)[h] = pack8_bf16(iml, h, -1.f);
-    if (half) continue;
-    reinterpret_cast<uint4*>(W + top + Np)[h] = pack8_bf16(im, h, 1.f);
-    reinterpret_cast<uint4*>(W + P1 + top + Np)[h] = pack8_bf16(iml, h, 1.f);
-    reinterpret_cast<uint4*>(W + bot + Np)[h] = pack8_bf16(re, h, 1.f);
-    reinterpret_cast<uint4*>(W + P1 + bot + Np)[h] = pack8_bf16(rel, h, 1.f);
+    uint4* s = stg + lane * 4 + ((2 * slot + h) ^ ((lane >> 1) & 3));
+    s[0] = pack8_bf16(re, h);
+    s[128] = pack8_bf16(rel, h);
+    s[256] = pack8_bf16(im, h);
+    s[384] = pack8_bf16(iml, h);
   }
+}
+
+// The staged pieces of the warp's 32 rows (from row0) and 8 nu W columns (from j0) to the embedded
+// matrix that product 2 reads as its B operand: top row m = [Re W | Im W], bottom row Np + m =
+// [-Im W | Re W], hi at 0 and lo at 4 Np^2; w_half: the left half only.
+__device__ __forceinline__ void flush_w(const TcProb& pr, const uint4* stg, int row0, int lane, int j0, int nu) {
+  __nv_bfloat16* W = reinterpret_cast<__nv_bfloat16*>(pr.out);
+  const int Np = pr.Np, u = lane & 3;
+  const long long ld = 2LL * Np, P1 = 4LL * Np * Np;
+  __syncwarp();
+  if (u < nu) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int r = 8 * t + (lane >> 2), row = row0 + r;
+      if (row >= Np) break;  // rows grow with t
+      const uint4* s = stg + r * 4 + (u ^ ((r >> 1) & 3));
+      const long long top = (long long)row * ld + j0 + 8 * u, bot = top + Np * ld;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const uint4 a = s[128 * q], b = s[256 + 128 * q];
+        __nv_bfloat16* w = W + q * P1;
+        *reinterpret_cast<uint4*>(w + top) = a;
+        *reinterpret_cast<uint4*>(w + bot) =
+            make_uint4(b.x ^ 0x80008000u, b.y ^ 0x80008000u, b.z ^ 0x80008000u, b.w ^ 0x80008000u);
+        if (!pr.w_half) {
+          *reinterpret_cast<uint4*>(w + top + Np) = b;
+          *reinterpret_cast<uint4*>(w + bot + Np) = a;
+        }
+      }
+    }
+  }
+  __syncwarp();
+}
+
+// Product 2 epilogue: 32 accumulator columns of the warp's 32 rows to FP32 planar X (nv of them are
+// the tile's).
+__device__ __forceinline__ void store_x(const TcProb& pr, uint4* stg, int row0, int lane, int gn,
+                                        const uint32_t (&r)[32], int nv) {
+#pragma unroll
+  for (int v = 0; v < 8; ++v)
+    stg[lane * 8 + (v ^ (lane & 7))] = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+  __syncwarp();
+  float* X = reinterpret_cast<float*>(pr.out);
+  const int c = lane & 7;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const int q = 4 * t + (lane >> 3), row = row0 + q;
+    if (row < pr.Np && 4 * c < nv)
+      *reinterpret_cast<uint4*>(X + (long long)row * 2 * pr.Np + gn + 4 * c) = stg[q * 8 + (c ^ (q & 7))];
+  }
+  __syncwarp();
 }
 
 // ----------------------------------------------------------------------------
@@ -552,6 +614,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcPa
     // shared memory before a group barrier, so the four warps always agree.
     const int q = warp & 3;
     const bool leader = threadIdx.x == 64;
+    uint4* stg = reinterpret_cast<uint4*>(sm + ST * STAGE + 256 + (warp - 2) * kEpiStage);
     int i = 0, t, kb, ke, KT;
     UnitCursor cur;
     cursor_init(P, cur, blockIdx.x, gridDim.x);
@@ -573,13 +636,13 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcPa
       epi_bar();
       if (!s_epi_ok[i & 1]) break;
       tc_fence_after();
-      const int Np = pr.Np;
-      const long long ld = 2LL * Np;
       const int rt = q * 32 + lane;  // row within the tile
       const int row = mt * BM + rt;
 #pragma unroll 1
       for (int c0 = 0; c0 < BN; c0 += 32) {
         uint32_t r[32];
+        GChunk g;
+        if (EPI == 0) load_g(pr, row, nt * BN + c0, 2, g);
         const uint32_t taddr = tmem + ab * BN + c0 + ((uint32_t)(q * 32) << 16);
         TMEM_LD32(taddr, r);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -606,14 +669,11 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcPa
         }
         const int gn = nt * BN + c0;
         if (EPI == 1) {
-          float* X = reinterpret_cast<float*>(pr.out) + row * ld + gn;
-#pragma unroll
-          for (int v = 0; v < 8; ++v)
-            reinterpret_cast<float4*>(X)[v] =
-                make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]),
-                            __uint_as_float(r[4 * v + 3]));
+          store_x(pr, stg, row - lane, lane, gn, r, 32);
         } else {
-          store_w_pieces(pr, row, gn, r, 2);
+          const int slot = (c0 >> 5) & 1;
+          stage_w(pr, stg, row, lane, g, r, 2, slot);
+          if (slot) flush_w(pr, stg, row - lane, lane, (gn - 32) >> 1, 4);
         }
       }
       tc_fence_before();
@@ -767,10 +827,14 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
         int cb, w;
         col_tile(pr, nt, cb, w);
         const int arow = mt * (2 * BM) + rank * BM, brow = cb + rank * (w / 2);
+        const CUtensorMap* ma = &P.mA[pr.sys];
+        const CUtensorMap* mb = &P.mB[pr.sys];
+        const int a_b = pr.a_b, b_b = pr.b_b;
+        const short* kidx = pr.kofs ? pr.kidx + pr.kofs[nt] : nullptr;
+        int ktn = kidx ? kidx[kb] : kb;  // the next panel's number is read a panel ahead
         for (int kk = kb; ok && kk < ke; ++kk) {
-          const int kt = tile_panel(pr, t, kk);
-          const CUtensorMap* ma = &P.mA[pr.sys];
-          const CUtensorMap* mb = &P.mB[pr.sys];
+          const int kt = ktn;
+          if (kk + 1 < ke) ktn = kidx ? kidx[kk + 1] : kk + 1;
 #pragma unroll 1
           for (int h = 0; h < KH; ++h, ++it) {
             const int s = it % ST, r = it / ST;
@@ -782,10 +846,10 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
             if (leader_cta) mbar_expect_tx(full0 + 8 * s, 2 * stage_tx);
             const uint32_t fb = full_l + 8 * s;
             const int x = kt * BK + h * BKS;
-            tma_load_4d_pair(base, ma, x, arow, 0, pr.a_b, fb);
-            tma_load_4d_pair(base + A_BYTES, ma, x, arow, 1, pr.a_b, fb);
-            tma_load_4d_pair(base + 2 * A_BYTES, mb, x, brow, 0, pr.b_b, fb);
-            tma_load_4d_pair(base + 2 * A_BYTES + B_BYTES, mb, x, brow, 1, pr.b_b, fb);
+            tma_load_4d_pair(base, ma, x, arow, 0, a_b, fb);
+            tma_load_4d_pair(base + A_BYTES, ma, x, arow, 1, a_b, fb);
+            tma_load_4d_pair(base + 2 * A_BYTES, mb, x, brow, 0, b_b, fb);
+            tma_load_4d_pair(base + 2 * A_BYTES + B_BYTES, mb, x, brow, 1, b_b, fb);
           }
         }
       }
@@ -861,6 +925,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
     const int q = warp & 3;
     const bool leader = threadIdx.x == 64;
     const int me = 2 * pair + (int)rank;
+    uint4* stg = reinterpret_cast<uint4*>(sm + ST * STAGE + 256 + (warp - 2) * kEpiStage);
     int i = 0, t, kb, ke, KT;
     UnitCursor cur;
     cursor_init(P, cur, pair, G2);
@@ -872,6 +937,12 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
       const bool contrib = P.streamk && kb > 0;
       const bool finish = P.streamk && kb == 0 && ke < KT;
       const int p_last = finish ? sk_last_worker(P, pr, local, KT, pair, G2) : pair;
+      const int rt = q * 32 + lane;
+      const int row = mt * (2 * BM) + rank * BM + rt;
+      int cb, w;
+      col_tile(pr, nt, cb, w);
+      GChunk g;
+      if (EPI == 0 && !contrib) load_g(pr, row, cb, w < 32 ? 1 : 2, g);  // in flight during the wait
       if (leader) {
         int ok = mbar_wait(accf0 + 8 * ab, u & 1, P.timeout_ns, abort_flag, P.err) ? 1 : 0;
         for (int p2 = pair + 1; ok && finish && p2 <= p_last; ++p2)
@@ -882,15 +953,11 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
       epi_bar();
       if (!s_epi_ok[i & 1]) break;
       tc_fence_after();
-      const int Np = pr.Np;
-      const long long ld = 2LL * Np;
-      const int rt = q * 32 + lane;
-      const int row = mt * (2 * BM) + rank * BM + rt;
-      int cb, w;
-      col_tile(pr, nt, cb, w);
 #pragma unroll 1
       for (int c0 = 0; c0 < w; c0 += 32) {
         uint32_t r[32];
+        const GChunk gc = g;
+        if (EPI == 0 && !contrib && c0 + 32 < w) load_g(pr, row, cb + c0 + 32, w - c0 - 32 < 32 ? 1 : 2, g);
         const uint32_t taddr = tmem + ab * BNP + c0 + ((uint32_t)(q * 32) << 16);
         TMEM_LD32(taddr, r);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -917,17 +984,14 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
         }
         const int gn = cb + c0;
         const int nv = w - c0 < 32 ? w - c0 : 32;  // 16 in the last chunk of a width 32 m + 16
-        if (row >= Np) continue;  // last row tile of an Np that is not a multiple of 256
+        // (the last row tile of an Np that is not a multiple of 256 has rows past the matrix)
         if (EPI == 1) {
-          float* X = reinterpret_cast<float*>(pr.out) + row * ld + gn;
-#pragma unroll
-          for (int v = 0; v < 8; ++v)
-            if (4 * v < nv)
-              reinterpret_cast<float4*>(X)[v] =
-                  make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
-                              __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
+          store_x(pr, stg, row - lane, lane, gn, r, nv);
         } else {
-          store_w_pieces(pr, row, gn, r, nv >> 4);
+          const int slot = (c0 >> 5) & 1;
+          stage_w(pr, stg, row, lane, gc, r, nv >> 4, slot);
+          if (slot || c0 + 32 >= w)
+            flush_w(pr, stg, row - lane, lane, (gn - 32 * slot) >> 1, 2 * slot + (nv >> 4));
         }
       }
       tc_fence_before();

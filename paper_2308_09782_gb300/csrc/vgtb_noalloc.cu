@@ -37,6 +37,7 @@ constexpr size_t kNaScratchBytes = kOffErr + 256;                   // 2 MiB + 5
 static __device__ __align__(256) unsigned char g_na_scratch[kNaScratchBytes];
 
 constexpr int kMaxDevices = 64;
+constexpr int kNaSmem = 2 * (2 * BM * BK * 2 + 2 * 256 * BK * 2) + 256 + 4 * kEpiStage + 1024;
 
 // Per-device set-up state, read and written under g_na_mu only.
 struct NaDevice {
@@ -155,7 +156,7 @@ int na_setup(int dev, unsigned char** addr) {
   cudaError_t e = cudaGetSymbolAddress(&p, g_na_scratch);
   if (e != cudaSuccess || !p) return VGTB_E_CUDA;
   e = cudaFuncSetAttribute(k_tc_gemm<256, 2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           2 * (2 * BM * BK * 2 + 2 * 256 * BK * 2) + 1024 + 256);
+                           kNaSmem);
   if (e != cudaSuccess) return VGTB_E_CUDA;
   d.addr = static_cast<unsigned char*>(p);
   d.ctx_id = id;
@@ -208,7 +209,7 @@ extern "C" int vgtb_split_cgemm_noalloc(int n, const double* a, const double* r,
   P.total_tiles = (Np / BM) * (2 * Np / 256);
   P.err = err;
   P.timeout_ns = 2000000000LL;
-  const int smem = 2 * (2 * BM * BK * 2 + 2 * 256 * BK * 2) + 1024 + 256;
+  const int smem = kNaSmem;
   k_tc_gemm<256, 2, 1><<<P.total_tiles, 192, smem, st>>>(P);
   k_na_out<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, st>>>(xo, n, Np, err, reinterpret_cast<double2*>(c));
   cudaError_t e = cudaGetLastError();
