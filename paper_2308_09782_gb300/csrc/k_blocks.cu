@@ -1,7 +1,6 @@
 // Block-sparse kernels of one propagation step:
-//   k_obs         - Mulliken, current and energy partial sums from D_k(t_n) (Eqs. 10, 14)
-//   k_scc_atoms,
-//   k_scc_eps     - dq, eps = gamma dq, J, E per trajectory (Eq. 10, Eq. 14)
+//   k_obs_atoms   - Mulliken, current and energy sums per atom from D_k(t_n) (Eqs. 10, 14)
+//   k_scc_eps     - eps = gamma dq, J, E per trajectory (Eq. 10, Eq. 14)
 //   k_phase       - Bloch sum of H_k(t_n) with the vector potential (Eqs. 7-12), FP64
 //   k_phase_split - the same sum in FP32, written as embedded BF16 hi/lo pieces
 // A half-warp (16 lanes) handles one target (I, J) of one trajectory: it walks the
@@ -52,91 +51,6 @@ __device__ __forceinline__ Unit unit_of(const int* wpre, int n_traj, int total) 
   return r;
 }
 
-// ---------------------------------------------------------------------------
-// Partial sums per target, summed over k with weights w_k, from the
-// time-independent k-space blocks S_k, P_k^a, H0_k (Bloch-summed at setup):
-//   s_S = sum Re(D conj(S_k)),  s_a = sum Re(D conj(P^a_k)),  s_H = sum Re(D conj(H0_k))
-//   q = s_S                                          (Eq. 10: [D S]_{mu mu})
-//   T_a = s_a + (A_a/c) s_S                          (Eq. 14: Tr[D Pi^a], Pi = P + (A/c) S)
-//   E_band = s_H + (A/c).(s_x, s_y, s_z) + |A|^2/(2c^2) s_S
-// In the delta forms D = D0 + dD and the D0 part of every sum is a constant
-// computed once (obs0), so only dD is read.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_obs(const DevSys* __restrict__ sysv, const DevTraj* __restrict__ trj,
-                                             const DevItem* __restrict__ items, const int* __restrict__ wpre,
-                                             int n_traj, int total, const int* __restrict__ step, int delta,
-                                             int fixed_step) {
-  pdl_wait();
-  pdl_trigger();
-  const Unit U = unit_of(wpre, n_traj, total);
-  const int lane = threadIdx.x & 15;
-  double sS = 0.0, sx = 0.0, sy = 0.0, sz = 0.0, sH = 0.0;
-  const DevTraj& T = trj[U.t];
-  const DevSys& S = sysv[T.sys];
-  int n = 0;
-  if (U.active) {
-    n = fixed_step >= 0 ? fixed_step : *step;
-    const int par = n & 1;
-    const int I = S.tgt_I[U.tg], J = S.tgt_J[U.tg];
-    const int oi = S.orb_off[I];
-    const int oj = S.orb_off[J], nj = S.orb_off[J + 1] - oj;
-    const int el0 = S.tgt_el0[U.tg], nel = S.tgt_el0[U.tg + 1] - el0;
-    for (int k = 0; k < S.nk; ++k) {
-      const double2* Dk = items[T.item0 + k].D[par];
-      const long long kb = (long long)k * S.n_el + el0;
-      const long long pstride = (long long)S.nk * S.n_el;
-      double lS = 0.0, lx = 0.0, ly = 0.0, lz = 0.0, lH = 0.0;
-      for (int e = lane; e < nel; e += 16) {
-        const int a = e / nj, b = e - a * nj;
-        const double2 d = Dk[(long long)(oi + a) * S.Np + (oj + b)];
-        const double2 cs = S.kS[kb + e], ch = S.kH0[kb + e];
-        const double2 px = S.kP[kb + e], py = S.kP[pstride + kb + e], pz = S.kP[2 * pstride + kb + e];
-        lS += d.x * cs.x + d.y * cs.y;
-        lx += d.x * px.x + d.y * px.y;
-        ly += d.x * py.x + d.y * py.y;
-        lz += d.x * pz.x + d.y * pz.y;
-        lH += d.x * ch.x + d.y * ch.y;
-      }
-      const double wk = S.wk[k];
-      sS += wk * lS;
-      sx += wk * lx;
-      sy += wk * ly;
-      sz += wk * lz;
-      sH += wk * lH;
-    }
-  }
-  sS = half_sum(sS);
-  sx = half_sum(sx);
-  sy = half_sum(sy);
-  sz = half_sum(sz);
-  sH = half_sum(sH);
-  if (U.active && lane == 0) {
-    if (delta) {
-      const double* o = S.obs0 + 5LL * U.tg;
-      sS += o[0];
-      sx += o[1];
-      sy += o[2];
-      sz += o[3];
-      sH += o[4];
-    }
-    double A0 = 0.0, A1 = 0.0, A2 = 0.0;
-    if (T.A) {
-      A0 = T.A[3 * n];
-      A1 = T.A[3 * n + 1];
-      A2 = T.A[3 * n + 2];
-    }
-    constexpr double ic = 1.0 / kLight;
-    const double a0 = A0 * ic, a1 = A1 * ic, a2 = A2 * ic;
-    const double alpha = 0.5 * (a0 * a0 + a1 * a1 + a2 * a2);
-    double* p = T.part + 5LL * U.tg;
-    p[0] = sS;
-    p[1] = sx + a0 * sS;
-    p[2] = sy + a1 * sS;
-    p[3] = sz + a2 * sS;
-    p[4] = sH + (a0 * sx + a1 * sy + a2 * sz) + alpha * sS;
-  }
-}
-
 // Setup: the k-space blocks of one system at one k (half-warp per target).
 __global__ void k_kblocks(const DevSys* __restrict__ sysv, int s_idx, int k) {
   const int tg = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
@@ -178,7 +92,7 @@ void launch_kblocks(const DevSys* sys, int s_idx, int n_tgt, int k, cudaStream_t
   k_kblocks<<<blocks, threads, 0, st>>>(sys, s_idx, k);
 }
 
-// Setup (delta forms): obs0[tg] = the k_obs sums of the target evaluated with D0.
+// Setup (delta forms): obs0[tg] = the target's part of the observable sums evaluated with D0.
 __global__ void k_obs0(const DevSys* __restrict__ sysv, int s_idx) {
   const int tg = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
   const int lane = threadIdx.x & 15;
@@ -212,7 +126,7 @@ __global__ void k_obs0(const DevSys* __restrict__ sysv, int s_idx) {
     for (int i = 0; i < 5; ++i) S.obs0[5LL * tg + i] = v[i];
 }
 
-// Setup (split form): obs0a[I] = obs0 summed over the targets of row atom I, in target order.
+// Setup (delta forms): obs0a[I] = obs0 summed over the targets of row atom I, in target order.
 __global__ void k_obs0_atoms(const DevSys* __restrict__ sysv, int s_idx) {
   const DevSys& S = sysv[s_idx];
   const int I = blockIdx.x * blockDim.x + threadIdx.x;
@@ -223,11 +137,11 @@ __global__ void k_obs0_atoms(const DevSys* __restrict__ sysv, int s_idx) {
   for (int i = 0; i < 5; ++i) S.obs0a[5LL * I + i] = v[i];
 }
 
-void launch_obs0(const DevSys* sys, int s_idx, int n_tgt, int nat, int split, cudaStream_t st) {
+void launch_obs0(const DevSys* sys, int s_idx, int n_tgt, int nat, cudaStream_t st) {
   const int threads = 256;
   const int blocks = (n_tgt * 16 + threads - 1) / threads;
   k_obs0<<<blocks, threads, 0, st>>>(sys, s_idx);
-  if (split) k_obs0_atoms<<<(nat + 127) / 128, 128, 0, st>>>(sys, s_idx);
+  k_obs0_atoms<<<(nat + 127) / 128, 128, 0, st>>>(sys, s_idx);
 }
 
 __device__ __forceinline__ float half_sum_f(float v) {
@@ -237,21 +151,28 @@ __device__ __forceinline__ float half_sum_f(float v) {
 }
 
 // ---------------------------------------------------------------------------
-// k_obs_atoms_split: the split form's observables and per-atom sums in one
-// launch.  One CTA of 4 warps per (trajectory, atom I); its threads take the
-// nonzeros of the atom's rows (all targets (I, J), ~490 for an sp3 atom, so at
-// most a few per thread, whose loads are issued together) and form the dD
-// sums in FP64 from the FP64 master dD and the FP64 k-space blocks (S_k, P_k,
-// H0_k), so charges, current and energy keep the precision of the master copy.
-// Each warp reduces its five sums with one reduce-scatter (nine FP64 additions
-// per lane: GB300 issues FP64 warp instructions at a small fraction of the FP32
-// rate whatever the number of active lanes), thread 0 adds the warps, the
-// constant D0 part (obs0a) and the A terms (both linear in the sums) and writes
-// dq_I, q_I and the atom's shares of T and of the band energy, as k_scc_atoms
-// does for the FP64 paths.
+// k_obs_atoms: charges, current and energy sums of one level, per atom, from the
+// time-independent k-space blocks S_k, P_k^a, H0_k (Bloch-summed at setup):
+//   s_S = sum Re(D conj(S_k)),  s_a = sum Re(D conj(P^a_k)),  s_H = sum Re(D conj(H0_k))
+//   q = s_S                                          (Eq. 10: [D S]_{mu mu})
+//   T_a = s_a + (A_a/c) s_S                          (Eq. 14: Tr[D Pi^a], Pi = P + (A/c) S)
+//   E_band = s_H + (A/c).(s_x, s_y, s_z) + |A|^2/(2c^2) s_S
+// summed over k with weights w_k.  In the delta forms D = D0 + dD and the D0 part of
+// every sum is a constant computed once (obs0a), so only dD is read.
+// One CTA per (trajectory, atom I): groups of 128 threads take the k-points in turn
+// (up to 4 groups), the threads of a group the nonzeros of the atom's rows (all
+// targets (I, J), ~490 for an sp3 atom, so at most a few per thread, whose loads
+// are issued together); FP64 throughout.  Each warp reduces its five sums with one
+// reduce-scatter (nine FP64 additions per lane: GB300 issues FP64 warp instructions
+// at a small fraction of the FP32 rate whatever the number of active lanes).
+// Latency bound: the offsets are read before the wait for the kernel that writes D.  With the
+// k-points one after the other in 128 threads, FP64 instructions issued for empty slots, and two
+// kernels for the FP64 paths (per target, per atom), a step took 55 us instead of 44 (8 atoms x 8 k,
+// split), 202 instead of 191 (batch of 64 atoms x 8 k and 216 atoms), 60 instead of 46 (8 atoms, FP64).
 // ---------------------------------------------------------------------------
-constexpr int kObsThreads = 128;
-constexpr int kObsChunk = 4;  // nonzeros per thread whose loads are issued together
+constexpr int kObsThreads = 128;  // threads per k-point group
+constexpr int kObsGroups = 4;     // most groups
+constexpr int kObsChunk = 4;      // nonzeros per thread whose loads are issued together
 
 // Reduce-scatter of eight per-lane values over a warp: afterwards lane l holds
 // the warp total of value (l >> 2) & 7 (every lane of a group of four holds the
@@ -287,48 +208,58 @@ __device__ __forceinline__ double warp_reduce_scatter8(double (&v)[8], int lane)
   return v[0];
 }
 
-__global__ void __launch_bounds__(kObsThreads, 4) k_obs_atoms_split(const DevSys* __restrict__ sysv, DevTraj* trj,
-                                                               const DevItem* __restrict__ items, int n_traj,
-                                                               int max_nat, const int* __restrict__ step, int stride,
-                                                               int fixed_step, int record) {
-  pdl_wait();
-  pdl_trigger();
-  constexpr int NW = kObsThreads / 32;
-  __shared__ double s_tot[NW][5];
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// G: k-point groups (1: every system has one k-point; the registers then hold more loads in flight)
+template <int G>
+__global__ void __launch_bounds__(kObsThreads* G, G == 1 ? 4 : 2)
+    k_obs_atoms(const DevSys* __restrict__ sysv, DevTraj* trj, const DevItem* __restrict__ items, int n_traj,
+                int max_nat, const int* __restrict__ step, int stride, int delta) {
+  __shared__ double s_tot[kObsThreads * G / 32][5];
   const int t = blockIdx.x / max_nat, I = blockIdx.x % max_nat;
-  if (t >= n_traj) return;
   DevTraj& T = trj[t];
   const DevSys& S = sysv[T.sys];
-  if (I >= S.nat) return;
-  const int n = fixed_step >= 0 ? fixed_step : *step;
-  const int par = n & 1;
+  const bool live = I < S.nat;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // S, P_x, P_y, P_z, H0 sums (3 slots unused)
+  const int grp = threadIdx.x / kObsThreads, tg = threadIdx.x % kObsThreads;
   // the atom's nonzeros are contiguous (targets sorted by row atom); el_off gives
   // each one's offset in the Np x Np matrix
-  const int e0 = S.el_atom0[I], e1 = S.el_atom0[I + 1];
+  const int e0 = live ? S.el_atom0[I] : 0, e1 = live ? S.el_atom0[I + 1] : 0;
   const long long ps = (long long)S.nk * S.n_el;
-  for (int k = 0; k < S.nk; ++k) {
+  const double2 *kS = S.kS, *kP = S.kP, *kH0 = S.kH0;
+  int off0[kObsChunk];
+#pragma unroll
+  for (int u = 0; u < kObsChunk; ++u) {
+    const int e = e0 + tg + kObsThreads * u;
+    off0[u] = 0;
+    if (e < e1) off0[u] = S.el_off[e];
+  }
+  pdl_wait();
+  pdl_trigger();
+  if (!live) return;
+  const int n = *step;
+  const int par = n & 1;
+  double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // S, P_x, P_y, P_z, H0 sums (3 slots unused)
+  for (int k = grp; k < S.nk; k += G) {
     const double2* Dk = items[T.item0 + k].D[par];
     const long long kb = (long long)k * S.n_el;
     double c[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     for (int eb = e0; eb < e1; eb += kObsThreads * kObsChunk) {
       int ee[kObsChunk];
-      bool ok[kObsChunk];
       double2 d[kObsChunk];
 #pragma unroll
       for (int u = 0; u < kObsChunk; ++u) {
-        const int e = eb + threadIdx.x + kObsThreads * u;
-        ok[u] = e < e1;
-        ee[u] = ok[u] ? e : e0;
+        const int e = eb + tg + kObsThreads * u;
+        ee[u] = e < e1 ? e : e0;
+        d[u] = e < e1 ? Dk[eb == e0 ? off0[u] : S.el_off[e]] : make_double2(0.0, 0.0);
       }
 #pragma unroll
-      for (int u = 0; u < kObsChunk; ++u) d[u] = ok[u] ? Dk[S.el_off[ee[u]]] : make_double2(0.0, 0.0);
-#pragma unroll
       for (int u = 0; u < kObsChunk; ++u) {
+        // a warp past the end issues no FP64 instruction (8 atoms: a fourth of the slots are in use)
+        if (eb + (tg & ~31) + kObsThreads * u >= e1) break;
         const long long x = kb + ee[u];
-        const double2 bs = S.kS[x], bx = S.kP[x], by = S.kP[ps + x], bz = S.kP[2 * ps + x], bh = S.kH0[x];
-        // Re(dD conj(X)) for X = S_k, P_k^x, P_k^y, P_k^z, H0_k
+        const double2 bs = kS[x], bx = kP[x], by = kP[ps + x], bz = kP[2 * ps + x], bh = kH0[x];
+        // Re(D conj(X)) for X = S_k, P_k^x, P_k^y, P_k^z, H0_k
         c[0] = fma(d[u].x, bs.x, fma(d[u].y, bs.y, c[0]));
         c[1] = fma(d[u].x, bx.x, fma(d[u].y, bx.y, c[1]));
         c[2] = fma(d[u].x, by.x, fma(d[u].y, by.y, c[2]));
@@ -344,14 +275,18 @@ __global__ void __launch_bounds__(kObsThreads, 4) k_obs_atoms_split(const DevSys
   const int slot = (lane >> 2) & 7;
   if ((lane & 3) == 0 && slot < 5) s_tot[warp][slot] = tot;
   __syncthreads();
-  if (threadIdx.x != 0) return;
+  if (warp != 0) return;
+  // lane i (< 5) adds the warps' sums of value i in order, then lane 0 has them all
+  constexpr int n_warp = kObsThreads * G / 32;
+  double a = 0.0;
+  if (lane < 5) {
+    if (delta) a = S.obs0a[5LL * I + lane];
+    for (int w2 = 0; w2 < n_warp; ++w2) a += s_tot[w2][lane];
+  }
   double r[5];
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    double a = S.obs0a[5LL * I + i];
-    for (int w2 = 0; w2 < NW; ++w2) a += s_tot[w2][i];
-    r[i] = a;
-  }
+  for (int i = 0; i < 5; ++i) r[i] = __shfl_sync(0xffffffffu, a, i);
+  if (lane != 0) return;
   double A0 = 0.0, A1 = 0.0, A2 = 0.0;
   if (T.A) {
     A0 = T.A[3 * n];
@@ -362,7 +297,7 @@ __global__ void __launch_bounds__(kObsThreads, 4) k_obs_atoms_split(const DevSys
   const double a0 = A0 * ic, a1 = A1 * ic, a2 = A2 * ic;
   const double alpha = 0.5 * (a0 * a0 + a1 * a1 + a2 * a2);
   T.dq[I] = r[0] - S.z[I];
-  if (record && T.q && n % stride == 0) T.q[(long long)(n / stride) * S.nat + I] = r[0];
+  if (T.q && n % stride == 0) T.q[(long long)(n / stride) * S.nat + I] = r[0];
   double* ap = T.apart + 4LL * I;
   ap[0] = r[1] + a0 * r[0];
   ap[1] = r[2] + a1 * r[0];
@@ -370,25 +305,18 @@ __global__ void __launch_bounds__(kObsThreads, 4) k_obs_atoms_split(const DevSys
   ap[3] = r[4] + (a0 * r[1] + a1 * r[2] + a2 * r[3]) + alpha * r[0];
 }
 
-void launch_obs_atoms_split(const DevSys* sys, DevTraj* trj, const DevItem* items, int n_traj, int max_nat,
-                            const int* step, int stride, int fixed_step, int record, cudaStream_t st) {
-  launch_pdl(k_obs_atoms_split, n_traj * max_nat, kObsThreads, 0, st, sys, trj, items, n_traj, max_nat, step, stride,
-             fixed_step, record);
-}
-
-void launch_obs(const DevSys* sys, const DevTraj* trj, const DevItem* items, const int* warp_prefix,
-                int n_traj, int total_units, const int* step, int delta, int fixed_step, cudaStream_t st) {
-  const int threads = 256;
-  const int blocks = (total_units * 16 + threads - 1) / threads;
-  launch_pdl(k_obs, blocks, threads, 0, st, sys, trj, items, warp_prefix, n_traj, total_units, step, delta,
-             fixed_step);
+void launch_obs_atoms(const DevSys* sys, DevTraj* trj, const DevItem* items, int n_traj, int max_nat, int max_nk,
+                      const int* step, int stride, int delta, cudaStream_t st) {
+  if (max_nk == 1)
+    launch_pdl(k_obs_atoms<1>, n_traj * max_nat, kObsThreads, 0, st, sys, trj, items, n_traj, max_nat, step, stride,
+               delta);
+  else
+    launch_pdl(k_obs_atoms<kObsGroups>, n_traj * max_nat, kObsThreads * kObsGroups, 0, st, sys, trj, items, n_traj,
+               max_nat, step, stride, delta);
 }
 
 // ---------------------------------------------------------------------------
-// SCC reduction in two launches per step (all trajectories at once):
-//   k_scc_atoms: one warp per atom sums the partials of the atom's targets
-//                (targets are sorted by row atom): q_I, dq_I, and the atom's
-//                share of T_a and of the band energy;
+// SCC reduction (all trajectories at once), after k_obs_atoms:
 //   k_scc_eps:   kSccRows rows of eps = gamma dq per CTA, one per warp (Eq. 10), and one
 //                partial of J, the band energy, dq.eps/2 and the electron count per CTA;
 //                scc_finish adds the partials in a fixed order (J of Eq. 14, the energy,
@@ -397,45 +325,13 @@ void launch_obs(const DevSys* sys, const DevTraj* trj, const DevItem* items, con
 // ---------------------------------------------------------------------------
 constexpr int kSccThreads = 32 * kSccRowsPerCta;
 constexpr int kSccRows = kSccRowsPerCta;
-constexpr int kAtomsPerCta = kSccThreads / 32;
-
-__global__ void __launch_bounds__(kSccThreads) k_scc_atoms(const DevSys* __restrict__ sysv, DevTraj* trj, int n_traj,
-                                                          int nblk, const int* __restrict__ step, int stride,
-                                                          int fixed_step, int record) {
-  pdl_wait();
-  pdl_trigger();
-  const int t = blockIdx.x / nblk, b = blockIdx.x % nblk;
-  if (t >= n_traj) return;
-  DevTraj& T = trj[t];
-  const DevSys& S = sysv[T.sys];
-  const int I = b * kAtomsPerCta + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (I >= S.nat) return;
-  const int n = fixed_step >= 0 ? fixed_step : *step;
-  double v[5] = {0, 0, 0, 0, 0};
-  for (int tg = S.atom_tgt0[I] + lane; tg < S.atom_tgt0[I + 1]; tg += 32) {
-    const double* p = T.part + 5LL * tg;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) v[i] += p[i];
-  }
-#pragma unroll
-  for (int i = 0; i < 5; ++i) v[i] = warp_sum(v[i]);
-  if (lane == 0) {
-    T.dq[I] = v[0] - S.z[I];
-    if (record && T.q && n % stride == 0) T.q[(long long)(n / stride) * S.nat + I] = v[0];
-    double* a = T.apart + 4LL * I;
-    a[0] = v[1];
-    a[1] = v[2];
-    a[2] = v[3];
-    a[3] = v[4];
-  }
-}
 
 // The trajectory's totals at level n from the per-CTA partials of k_scc_eps, in a
 // fixed order (lane-strided sums, then a butterfly): J (Eq. 14), the energy, and
 // the checks of the level.  Run by one warp: the last CTA of k_scc_eps, or a
 // finisher CTA of k_phase_split (the split form's step, where the phase build
 // does not wait for these totals).
-__device__ void scc_finish(DevTraj& T, const DevSys& S, int n, int record, int lane) {
+__device__ void scc_finish(DevTraj& T, const DevSys& S, int n, int lane) {
   const int myblk = (S.nat + kSccRows - 1) / kSccRows;
   double v[6] = {0, 0, 0, 0, 0, 0};  // Tx, Ty, Tz, E_band, dq.eps, electron count
   for (int c = lane; c < myblk; c += 32) {
@@ -448,12 +344,10 @@ __device__ void scc_finish(DevTraj& T, const DevSys& S, int n, int record, int l
   if (lane == 0) {
     const double J0 = -v[0] * S.inv_omega, J1 = -v[1] * S.inv_omega, J2 = -v[2] * S.inv_omega;
     const double E = v[3] + 0.5 * v[4];
-    if (record) {
-      T.J[3LL * n] = J0;
-      T.J[3LL * n + 1] = J1;
-      T.J[3LL * n + 2] = J2;
-      T.E[n] = E;
-    }
+    T.J[3LL * n] = J0;
+    T.J[3LL * n + 1] = J1;
+    T.J[3LL * n + 2] = J2;
+    T.E[n] = E;
     int st = 0;
     if (!isfinite(J0) || !isfinite(J1) || !isfinite(J2) || !isfinite(E) || !isfinite(v[5])) st |= ST_NONFINITE;
     if (fabs(v[5] - S.nel) > 1e-6 * fmax(1.0, S.nel)) st |= ST_DRIFT;
@@ -464,22 +358,25 @@ __device__ void scc_finish(DevTraj& T, const DevSys& S, int n, int record, int l
 // finish = 1: the last CTA of each trajectory runs scc_finish; finish = 0: the
 // CTAs only store their partials (the step's k_phase_split finishes them).
 __global__ void __launch_bounds__(kSccThreads) k_scc_eps(const DevSys* __restrict__ sysv, DevTraj* trj, int n_traj,
-                                                        int nblk, const int* __restrict__ step, int fixed_step,
-                                                        int record, int finish) {
-  pdl_wait();
-  pdl_trigger();
+                                                        int nblk, const int* __restrict__ step, int finish) {
   constexpr int NW = kSccThreads / 32;
   __shared__ double red[NW][6];
   __shared__ int s_last;
   const int t = blockIdx.x / nblk, b = blockIdx.x % nblk;
-  if (t >= n_traj) return;
   DevTraj& T = trj[t];
   const DevSys& S = sysv[T.sys];
   const int myblk = (S.nat + kSccRows - 1) / kSccRows;
-  if (b >= myblk) return;
-  const int n = fixed_step >= 0 ? fixed_step : *step;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int I = b * kSccRows + warp;  // one warp per row of gamma
+  // the first 512 columns of the row, constant data, are read before the wait for dq
+  const double* g = S.gamma + (long long)I * S.nat;
+  double gv[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) gv[j] = (I < S.nat && lane + 32 * j < S.nat) ? g[lane + 32 * j] : 0.0;
+  pdl_wait();
+  pdl_trigger();
+  if (b >= myblk) return;
+  const int n = *step;
   if (tid == 0 && b == 0 && T.af) {
     // A(t_n)/c in FP32 for the phase build
     constexpr double inv_c = 1.0 / kLight;
@@ -489,17 +386,16 @@ __global__ void __launch_bounds__(kSccThreads) k_scc_eps(const DevSys* __restric
 #pragma unroll
     for (int i = 0; i < 6; ++i) red[warp][i] = 0.0;
   if (I < S.nat) {
-    const double* g = S.gamma + (long long)I * S.nat;
     const double* dq = T.dq;
     // chunks of 512 columns: all 16 loads of a lane are issued before the first
     // FMA, so a chunk costs one memory latency; four partial sums
     double e0 = 0.0, e1 = 0.0, e2 = 0.0, e3 = 0.0;
     for (int base = 0; base < S.nat; base += 512) {
-      double gv[16], qv[16];
+      double qv[16];
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const int K = base + lane + 32 * j;
-        gv[j] = K < S.nat ? g[K] : 0.0;
+        if (base > 0) gv[j] = K < S.nat ? g[K] : 0.0;
         qv[j] = K < S.nat ? dq[K] : 0.0;
       }
 #pragma unroll
@@ -551,18 +447,14 @@ __global__ void __launch_bounds__(kSccThreads) k_scc_eps(const DevSys* __restric
   __syncthreads();
   if (!s_last || warp != 0) return;
   __threadfence();
-  scc_finish(T, S, n, record, lane);
+  scc_finish(T, S, n, lane);
   if (lane == 0) *T.ticket = 0;
 }
 
-void launch_scc(const DevSys* sys, DevTraj* trj, int n_traj, const int* step, int stride, int fixed_step,
-                int record, int max_nat, int atoms_done, cudaStream_t st, int finish) {
-  const int nblk_a = (max_nat + kAtomsPerCta - 1) / kAtomsPerCta;
-  if (!atoms_done)
-    launch_pdl(k_scc_atoms, n_traj * nblk_a, kSccThreads, 0, st, sys, trj, n_traj, nblk_a, step, stride, fixed_step,
-               record);
+void launch_scc(const DevSys* sys, DevTraj* trj, int n_traj, const int* step, int max_nat, cudaStream_t st,
+                int finish) {
   const int nblk = (max_nat + kSccRows - 1) / kSccRows;
-  launch_pdl(k_scc_eps, n_traj * nblk, kSccThreads, 0, st, sys, trj, n_traj, nblk, step, fixed_step, record, finish);
+  launch_pdl(k_scc_eps, n_traj * nblk, kSccThreads, 0, st, sys, trj, n_traj, nblk, step, finish);
 }
 
 int scc_configure(int max_nat) {
@@ -750,24 +642,43 @@ __global__ void __launch_bounds__(256, 4) k_phase_split(const DevSys* __restrict
                                                      const DevItem* __restrict__ items,
                                                      const int* __restrict__ wpre, int n_traj, int total,
                                                      int fin0, const int* __restrict__ step) {
+  // the target's constants and the block values of its first image are on their way before the
+  // wait for the shifts
+  const bool fin = fin0 >= 0 && (int)blockIdx.x >= fin0;
+  Unit U;
+  U.active = false;
+  U.t = U.tg = 0;
+  if (!fin) U = unit_of_q(wpre, n_traj, total);
+  const int sub = threadIdx.x & 3;
+  int4 t0 = make_int4(0, 0, 0, 0), t1 = t0;
+  if (U.active) {
+    const DevSys& S = sysv[trj[U.t].sys];
+    t0 = S.tgt_p0[U.tg];
+    t1 = S.tgt_p1[U.tg];
+    if ((t1.z >> 16) != 0 && sub < (t1.z & 0xffff)) {
+      const long long off = S.img_off[t0.z] + 4LL * sub;
+      prefetch_l2(S.sf + off);
+      prefetch_l2(S.h0f + off);
+      prefetch_l2(S.dsf + off);
+      prefetch_l2(S.dsf + S.ds_stride + off);
+      prefetch_l2(S.dsf + 2 * S.ds_stride + off);
+    }
+  }
   pdl_wait();
   pdl_trigger();
   if (fin0 >= 0 && (int)blockIdx.x >= fin0) {
     const int t = (int)blockIdx.x - fin0;
     if (blockIdx.y != 0 || t >= n_traj || threadIdx.x >= 32) return;
-    scc_finish(trj[t], sysv[trj[t].sys], *step, 1, threadIdx.x);
+    scc_finish(trj[t], sysv[trj[t].sys], *step, threadIdx.x);
     return;
   }
-  const Unit U = unit_of_q(wpre, n_traj, total);
   if (!U.active) return;
-  const int sub = threadIdx.x & 3;
   const DevTraj& T = trj[U.t];
   const DevSys& S = sysv[T.sys];
   // A(t_n)/c and the shifts as FP32, prepared once per step by k_scc_eps: the
   // kernel issues no FP64 instruction (each costs a warp many FP32 issue slots)
   const float a0 = T.af[0], a1 = T.af[1], a2 = T.af[2];
   // the target's constants in two 16-byte records (one load each, no lookups)
-  const int4 t0 = S.tgt_p0[U.tg], t1 = S.tgt_p1[U.tg];
   const int I = t0.x, J = t0.y, g0 = t0.z, g1 = t0.w;
   const int oi = t1.x, oj = t1.y, ni = t1.z & 0xffff, nj = t1.w & 0xffff;
   const bool vec = (t1.z >> 16) != 0;

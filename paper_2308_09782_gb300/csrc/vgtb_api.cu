@@ -87,7 +87,6 @@ struct HostTraj {
   float* epsf = nullptr;
   float* deh = nullptr;
   float* af = nullptr;
-  double* part = nullptr;
   double* cpart = nullptr;
   double* apart = nullptr;
   int* ticket = nullptr;
@@ -509,7 +508,7 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
   h.d_kS = d.kS;
   h.d_kP = d.kP;
   TRY(dalloc(ctx, &d.obs0, 5 * (size_t)h.n_tgt));
-  if (ctx->split) TRY(dalloc(ctx, &d.obs0a, 5 * (size_t)h.nat));
+  if (ctx->delta) TRY(dalloc(ctx, &d.obs0a, 5 * (size_t)h.nat));
   const size_t NN = (size_t)h.Np * h.Np;
   TRY(dalloc(ctx, &h.Sinv, NN * h.nk));
   TRY(dalloc(ctx, &h.D0, NN * h.nk));
@@ -913,7 +912,7 @@ int finish_density(vgtb_ctx* ctx, int si) {
   HostSys& h = ctx->sys[si];
   const size_t NN = (size_t)h.Np * h.Np;
   for (int k = 0; k < h.nk; ++k) launch_hermitize(h.D0 + k * NN, h.N, h.Np, ctx->stream);
-  if (ctx->delta) launch_obs0(ctx->d_sys, si, h.n_tgt, h.nat, ctx->split ? 1 : 0, ctx->stream);
+  if (ctx->delta) launch_obs0(ctx->d_sys, si, h.n_tgt, h.nat, ctx->stream);
   CK(cudaGetLastError());
   std::vector<double> q;
   TRY(host_charges(ctx, si, h.D0, q));
@@ -1020,7 +1019,6 @@ int upload_traj_table(vgtb_ctx* ctx) {
     d.epsf = h.epsf;
     d.deh = h.deh;
     d.af = h.af;
-    d.part = h.part;
     d.cpart = h.cpart;
     d.apart = h.apart;
     d.ticket = h.ticket;
@@ -1542,9 +1540,9 @@ int enqueue_step_cn(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag) {
   const int nt = (int)ctx->trj.size();
   const int stride = ctx->opt.obs_stride > 0 ? ctx->opt.obs_stride : 1;
   launch_cn_density(ctx, st);
-  launch_obs(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->d_step, 0, -1, st);
+  launch_obs_atoms(ctx->d_sys, ctx->d_trj, ctx->d_items, nt, ctx->max_nat, ctx->max_nk, ctx->d_step, stride, 0, st);
   if (ev) CK(cudaEventRecordWithFlags(ev[1], st, evflag));
-  launch_scc(ctx->d_sys, ctx->d_trj, nt, ctx->d_step, stride, -1, 1, ctx->max_nat, 0, st);
+  launch_scc(ctx->d_sys, ctx->d_trj, nt, ctx->d_step, ctx->max_nat, st);
   if (ev) CK(cudaEventRecordWithFlags(ev[2], st, evflag));
   launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk, ctx->d_step,
                PH_FP64_CN, -1, st);
@@ -1574,20 +1572,15 @@ int enqueue_step_cn(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag) {
   return VGTB_OK;
 }
 
-// observables and SCC of the current level: split form k_obs_atoms_split + k_scc_eps,
-// FP64 paths k_obs + k_scc_atoms + k_scc_eps
+// observables and SCC of the current level
 // finish = 0 (split step): the phase build's finisher CTAs add up J, E and the checks
 void launch_obs_scc(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag, int stride, int finish = 1) {
   cudaStream_t st = ctx->stream;
   const int nt = (int)ctx->trj.size();
-  if (ctx->split)
-    launch_obs_atoms_split(ctx->d_sys, ctx->d_trj, ctx->d_items, nt, ctx->max_nat, ctx->d_step, stride, -1, 1, st);
-  else
-    launch_obs(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->d_step,
-               ctx->delta ? 1 : 0, -1, st);
+  launch_obs_atoms(ctx->d_sys, ctx->d_trj, ctx->d_items, nt, ctx->max_nat, ctx->max_nk, ctx->d_step, stride,
+                   ctx->delta ? 1 : 0, st);
   if (ev) cudaEventRecordWithFlags(ev[1], st, evflag);
-  launch_scc(ctx->d_sys, ctx->d_trj, nt, ctx->d_step, stride, -1, 1, ctx->max_nat, ctx->split ? 1 : 0, st,
-             ctx->split ? finish : 1);
+  launch_scc(ctx->d_sys, ctx->d_trj, nt, ctx->d_step, ctx->max_nat, st, ctx->split ? finish : 1);
 }
 
 // W = D H of a round: digits of D and H, the digit products (block-sparse first product: W is there already)
@@ -1973,7 +1966,6 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
       for (int k = 0; k < h.nk; ++k) ctx->items_h[T.item0 + k].ge = T.deh;
       if ((rc = dalloc(ctx, &T.af, 3))) return bail(rc);
     }
-    if ((rc = dalloc(ctx, &T.part, 5 * (size_t)h.n_tgt))) return bail(rc);
     if ((rc = dalloc(ctx, &T.cpart, 6 * (size_t)((h.nat + kSccRowsPerCta - 1) / kSccRowsPerCta)))) return bail(rc);
     if ((rc = dalloc(ctx, &T.apart, 4 * (size_t)h.nat))) return bail(rc);
     if ((rc = dalloc(ctx, &T.ticket, 1))) return bail(rc);
@@ -2325,15 +2317,8 @@ int vgtb_propagate(vgtb_ctx* ctx, int nsteps) {
     left -= chunk;
   }
   // observables of the final level
-  const int nt = (int)ctx->trj.size();
   if (ctx->cn) launch_cn_density(ctx, ctx->stream);
-  if (ctx->cn) {
-    launch_obs(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->d_step, 0, -1,
-               ctx->stream);
-    launch_scc(ctx->d_sys, ctx->d_trj, nt, ctx->d_step, ctx->opt.obs_stride, -1, 1, ctx->max_nat, 0, ctx->stream);
-  } else {
-    launch_obs_scc(ctx, nullptr, 0, ctx->opt.obs_stride);
-  }
+  launch_obs_scc(ctx, nullptr, 0, ctx->opt.obs_stride);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(ctx->stream));
   ctx->n_done += nsteps;

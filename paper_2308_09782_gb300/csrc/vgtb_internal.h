@@ -122,8 +122,8 @@ struct DevSys {
   double2* kS;             // [nk][n_el] Bloch-summed S_k at the target elements (Eq. 7)
   double2* kP;             // [3][nk][n_el] momentum P_k = sum e^{-ik.L} i dS/dR_J (Eq. 12)
   double2* kH0;            // [nk][n_el] H0_k
-  double* obs0;            // [n_tgt][5] delta forms: the D0 part of the k_obs sums
-  double* obs0a;           // [nat][5] split form: obs0 summed over the targets of each row atom
+  double* obs0;            // [n_tgt][5] delta forms: the D0 part of the observable sums per target
+  double* obs0a;           // [nat][5] delta forms: obs0 summed over the targets of each row atom
   double2* Sinv;           // [nk][Np*Np]
   double2* D0;             // [nk][Np*Np]
   double2* R0;             // [nk][Np*Np] (delta forms), else null
@@ -160,7 +160,6 @@ struct DevTraj {
   float* epsf;             // [nat] eps_I
   float* deh;              // [Np] (eps_I - eps0_I) / 2 of every orbital (padding 0): D0 terms of W and dD/dt
   float* af;               // [3] A(t_n) / c
-  double* part;            // [n_tgt][5] per-target partial sums
   double* cpart;           // [ceil(nat / kSccRowsPerCta)][6] per-CTA partial sums of k_scc_eps
   double* apart;           // [nat][4] per-atom shares of T_x, T_y, T_z and the band energy
   int* ticket;             // [1] CTA arrival counter of k_scc (reset by the last CTA)
@@ -270,16 +269,13 @@ enum PhaseMode : int {
 };
 
 // Launchers (all enqueue on `st`)
-// delta: 0 = D itself (FP64), 1 = dD with the D0 part from obs0 (FP64)
-void launch_obs(const DevSys* sys, const DevTraj* trj, const DevItem* items, const int* warp_prefix,
-                int n_traj, int total_warps, const int* step, int delta, int fixed_step, cudaStream_t st);
-// atoms_done = 1: the per-atom sums were made by k_obs_atoms_split (split form);
+// delta: 0 = D itself, 1 = dD with the D0 part from obs0a
+void launch_obs_atoms(const DevSys* sys, DevTraj* trj, const DevItem* items, int n_traj, int max_nat, int max_nk,
+                      const int* step, int stride, int delta, cudaStream_t st);
 // finish = 0: J, E and the checks of the level are left to launch_phase_split's
 // finisher CTAs (the split form's step), else the last CTA of k_scc_eps does them
-void launch_scc(const DevSys* sys, DevTraj* trj, int n_traj, const int* step, int stride,
-                int fixed_step, int record, int max_nat, int atoms_done, cudaStream_t st, int finish = 1);
-void launch_obs_atoms_split(const DevSys* sys, DevTraj* trj, const DevItem* items, int n_traj, int max_nat,
-                            const int* step, int stride, int fixed_step, int record, cudaStream_t st);
+void launch_scc(const DevSys* sys, DevTraj* trj, int n_traj, const int* step, int max_nat, cudaStream_t st,
+                int finish = 1);
 // grid rows = max_nk: row y builds k-points y, y + max_nk, ... of every target;
 // finish = 1 adds one CTA per trajectory that finishes the level's J, E and
 // checks from k_scc_eps's partials (launched with finish = 0)
@@ -291,7 +287,7 @@ void launch_phase(const DevSys* sys, const DevTraj* trj, const DevItem* items, c
                   int n_traj, int total_warps, int max_nk, const int* step, int mode, int fixed_step, cudaStream_t st);
 int scc_configure(int max_nat);
 void launch_kblocks(const DevSys* sys, int s_idx, int n_tgt, int k, cudaStream_t st);
-void launch_obs0(const DevSys* sys, int s_idx, int n_tgt, int nat, int split, cudaStream_t st);
+void launch_obs0(const DevSys* sys, int s_idx, int n_tgt, int nat, cudaStream_t st);
 void launch_bloch_setup(const DevSys* sys, int s_idx, int n_tgt, int k, int mode, const double* eps,
                         double2* out, cudaStream_t st);
 void launch_mulliken_setup(const DevSys* sys, int s_idx, int n_tgt, const double2* D, double* part,
