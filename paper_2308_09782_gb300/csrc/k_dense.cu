@@ -549,6 +549,22 @@ void launch_to_f32(const double2* src, float2* dst, long long n, cudaStream_t st
 // ---------------------------------------------------------------------------
 // helpers
 // ---------------------------------------------------------------------------
+// rows r0 .. r0 + rows - 1 of D0 + dD without the padding columns, n x n row-major
+__global__ void k_sum_rows(const double2* a, const double2* b, int ld, int n, int r0, int rows, double2* out) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (long long)rows * n) return;
+  const int r = (int)(i / n), c = (int)(i - (long long)r * n);
+  const long long s = (long long)(r0 + r) * ld + c;
+  const double2 x = a[s], y = b[s];
+  out[i] = make_double2(x.x + y.x, x.y + y.y);
+}
+
+void launch_sum_rows(const double2* a, const double2* b, int ld, int n, int r0, int rows, double2* out,
+                     cudaStream_t st) {
+  const long long tot = (long long)rows * n;
+  k_sum_rows<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(a, b, ld, n, r0, rows, out);
+}
+
 // values at the nonzero pattern to their places in a zeroed Np x Np matrix
 __global__ void k_scatter(const double2* v, const int* off, int n, double2* out) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;

@@ -29,24 +29,56 @@ __global__ void __launch_bounds__(kSpecThreads) k_conductivity(const double* __r
                                                                double e0, double tau0,
                                                                const double* __restrict__ omega, double* sigma,
                                                                double* eps) {
+  // Level m = n - n0 = 256 a + b: e^{iwt} e^{-t/tau0} is the product of a factor of b, kept by thread
+  // b, and one of a, made for 256 rows at a time, so a level costs four multiplications instead of a
+  // sincos and an exp on the FP64 pipe, which bound this kernel (1201 levels: 5 + 5 calls a thread,
+  // now 2 + 2; 5001 levels: 20 + 20, now 2 + 2).
   __shared__ double sh[kSpecThreads];
+  __shared__ double2 sf[kSpecThreads];
   const double w = omega[blockIdx.x];
-  double acc[6] = {0, 0, 0, 0, 0, 0};  // (re, im) for x, y, z
-  for (int n = n0 + threadIdx.x; n <= n1; n += kSpecThreads) {
-    const double t = (n - n0) * dt;
-    const double wt = (n == n0 || n == n1) ? 0.5 * dt : dt;
-    const double f = wt * exp(-t / tau0);
+  auto factor = [&](double t) {
     double s, c;
     sincos(w * t, &s, &c);
+    const double f = exp(-t / tau0);
+    return make_double2(f * c, f * s);
+  };
+  const double2 fb = factor(threadIdx.x * dt);
+  double acc[6] = {0, 0, 0, 0, 0, 0};  // (re, im) for x, y, z
+  const int rows = (n1 - n0) / kSpecThreads + 1;
+  for (int m = threadIdx.x, a = 0; a < rows; m += kSpecThreads, ++a) {
+    if (a % kSpecThreads == 0) {
+      __syncthreads();
+      if (a + threadIdx.x < rows) sf[threadIdx.x] = factor((double)(a + threadIdx.x) * kSpecThreads * dt);
+      __syncthreads();
+    }
+    const int n = n0 + m;
+    if (n > n1) continue;
+    const double2 fa = sf[a % kSpecThreads];
+    const double wt = (n == n0 || n == n1) ? 0.5 * dt : dt;
+    const double c = wt * (fa.x * fb.x - fa.y * fb.y), s = wt * (fa.x * fb.y + fa.y * fb.x);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const double j = f * J[3LL * n + a];
-      acc[2 * a] += c * j;
-      acc[2 * a + 1] += s * j;
+    for (int x = 0; x < 3; ++x) {
+      const double j = J[3LL * n + x];
+      acc[2 * x] += c * j;
+      acc[2 * x + 1] += s * j;
     }
   }
-  for (int i = 0; i < 6; ++i) acc[i] = block_sum(acc[i], sh);
+  // warp butterflies, then thread 0 adds the warps in order
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+    if ((threadIdx.x & 31) == 0) sh[i * 8 + (threadIdx.x >> 5)] = acc[i];
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    double v = sh[8 * threadIdx.x];
+    for (int q = 1; q < kSpecThreads / 32; ++q) v += sh[8 * threadIdx.x + q];
+    sh[64 + threadIdx.x] = v;
+  }
+  __syncwarp();
   if (threadIdx.x == 0) {
+    for (int i = 0; i < 6; ++i) acc[i] = sh[64 + i];
     const double k = 4.0 * M_PI / w;
     for (int a = 0; a < 3; ++a) {
       const double sr = acc[2 * a] / e0, si = acc[2 * a + 1] / e0;

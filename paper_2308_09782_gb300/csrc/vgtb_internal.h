@@ -350,6 +350,8 @@ void launch_leap_split(const LeapItem* items, int n_items, int Np_max, const int
 // real: the matrix is real, imaginary parts (rounding) are set to zero
 void launch_fill_hermitian_lower(double2* a, int n, int ld, int real, cudaStream_t st);
 void launch_vt_from_evecs(const double2* evec, double2* vt, int n, int nocc, int ld, cudaStream_t st);
+void launch_sum_rows(const double2* a, const double2* b, int ld, int n, int r0, int rows, double2* out,
+                     cudaStream_t st);
 void launch_scatter(const double2* v, const int* off, int n, double2* out, cudaStream_t st);
 void launch_scale(double2* a, long long n, double s, cudaStream_t st);
 void launch_split_planar(const double2* src, __nv_bfloat16* dst, int N, int Np, cudaStream_t st);

@@ -59,3 +59,58 @@ def test_slice_product_real_operand_planes_and_nonfinite_rows():
     want[[3, 7]] = True
     want[:, 9] = True
     assert np.array_equal(bad, want)
+
+
+def _mixed_system(kgrid):
+    """64 diamond sites, 24 of them with a single s orbital: N = 184, uneven blocks, no block-sparse kernel."""
+    from paper_2308_09782_gb300 import inputs
+    sysd = inputs.diamond_si(2, 0.05, seed=64, kgrid=kgrid)
+    light = np.zeros(64, bool)
+    light[np.random.default_rng(2).permutation(64)[:24]] = True
+    norb = np.where(light, 1, 4)
+    ijl = sysd["blk_ijl"]
+    a = np.arange(4)
+    keep = ((a[None, :, None] < norb[ijl[:, 0]][:, None, None]) & (a[None, None, :] < norb[ijl[:, 1]][:, None, None])).ravel()
+    z = np.where(light, 1.0, 4.0)
+    return {**sysd, "orb_offset": np.concatenate([[0], np.cumsum(norb)]).astype(np.int32), "h0": sysd["h0"][keep],
+            "s": sysd["s"][keep], "ds": np.ascontiguousarray(sysd["ds"][:, keep]), "z_ref": z,
+            "n_electrons": float(z.sum())}
+
+
+@pytest.mark.parametrize("kgrid", ["gamma", "mp2"])
+@pytest.mark.parametrize("form", ["fp64", "fp64_delta", "cn", "split", "split_batch"])
+def test_uneven_orbitals_match_oracle(form, kgrid):
+    """Every product route with uneven atom blocks and an N off every tile size, at a real and at
+    complex S_k, over graph-free steps: the FP64 bounds of the parity tests (J 1e-8, D 1e-10), the
+    split form's J bound of 1e-4."""
+    import oracle as O
+    from oracle import crank_nicolson as ocn
+    from paper_2308_09782_gb300 import inputs
+    sysd = _mixed_system(kgrid)
+    n = 6
+    A = inputs.pulse_field(n, sysd["dt"], 0.01, 0.1, pol=(1.0, 0.5, 0.2), duration=40.0)
+    cx = O.setup(sysd)
+    nocc = int(sysd["n_electrons"]) // 2
+    C = [O.occupied_states(H, S, nocc)[0] for H, S in zip(cx["H0"], cx["S"])]
+    D = [2.0 * (c @ c.conj().T) for c in C]
+    cn = form == "cn"
+    ref = ocn.propagate_cn(sysd, A, n, C, ctx=cx) if cn else O.propagate(sysd, A, n, D, ctx=cx)
+    split = form.startswith("split")
+    traj = [0, 0] if form == "split_batch" else [0]
+    with vgtb.Context([sysd], traj_sys=traj, init=vgtb.INIT_USER, delta_form=int(form == "fp64_delta"),
+                      precision=vgtb.SPLIT_BF16X3 if split else vgtb.FP64,
+                      integrator=vgtb.CRANK_NICOLSON if cn else vgtb.LEAPFROG) as c:
+        for k in range(len(C)):
+            (c.set_coefficients if cn else c.set_density)(0, k, C[k] if cn else D[k])
+        for t in range(len(traj)):
+            c.set_field(t, A)
+        c.propagate(n)
+        for t in range(len(traj)):
+            J, E, q = c.observables(t)
+            err = np.linalg.norm(J - ref["J"]) / np.linalg.norm(ref["J"])
+            assert err <= (1e-4 if split else 1e-8), err
+            assert np.max(np.abs(q - ref["q"])) <= (1e-5 if split else 1e-9)
+            if not cn:
+                X = np.stack([c.get_density(t, k) for k in range(len(C))])
+                R = np.stack(ref["D"])
+                assert np.linalg.norm(X - R) / np.linalg.norm(R) <= (1e-4 if split else 1e-10)
