@@ -211,9 +211,8 @@ def fp32_alu_peak(peaks):
 def split_product_rooflines(systems, n_items, stats, tiles, peaks):
     """Roofline of both commutator products of the split form, in algorithmic flops.
 
-    Product 1, block-sparse (product1 = BLOCKS): W = dD H + D0 dH over the nonzero
-    atom blocks, 2 x 8 nnz(H) N FP32 flops per item (the minimum of Eq. 6 is one
-    such product, 8 nnz N), against the FP32 ALU peak.  Product 1, dense tcgen05
+    Product 1, block-sparse (product1 = BLOCKS): W = dD H + D0 terms over the nonzero
+    atom blocks, 8 nnz(H) N FP32 flops per item, against the FP32 ALU peak.  Product 1, dense tcgen05
     (the split form's default): 3 split terms x 8 N^3 = 24 N^3 per item.  Product 2 (tcgen05
     BF16x3): 24 N^3 per item (unpadded N; the kernel executes 24 Np^3).  Both
     tensor figures are against the measured sustained BF16 peak."""
@@ -232,43 +231,44 @@ def split_product_rooflines(systems, n_items, stats, tiles, peaks):
         f = 48.0 * n3
         a = f / (g1 * 1e-3) / 1e12
         kept = tiles["product1"]["schedule"]
-        pc = {"kernel": "k_tc_chain (products 1 and 2 in one persistent tcgen05 launch: W = [dD|D0][H|dH]^dagger, "
+        pc = {"kernel": "k_tc_chain (products 1 and 2 in one persistent tcgen05 launch: W = dD H + D0 terms, "
                         "then X = S^-1 W^dagger, BF16x3)",
               "bound": "tensor", "achieved": round(a, 1), "peak": sust, "unit": "TFLOP/s",
               "frac": round(a / sust, 4), "peak_kind": sust_kind, "frac_of_burst": round(a / burst, 4),
               "flops_per_launch": f,
               "flops_note": "2 products x 3 split terms x 8 N^3 (algorithmic, unpadded N); the launch executes "
-                            f"at most {72 * np3:.3e} BF16 flops (product 1 with K' = 4 Np before its zero k-panels "
-                            "are skipped, product 2 with K' = 2 Np)",
-              "executed_tflops_upper": round(72 * np3 / (g1 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g1, 4),
+                            f"at most {48 * np3:.3e} BF16 flops (both with K' = 2 Np, before product 1's zero k-panels "
+                            "and the imaginary half of a real S^-1 are skipped)",
+              "executed_tflops_upper": round(48 * np3 / (g1 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g1, 4),
               "schedule": kept, "traffic": kernel_traffic("tc_chain", float(sum(n_items)), tiles["product1"])}
         return pc, None
     if tiles["product1"].get("schedule") == "block-sparse":
-        f1 = sum(n_it * 2 * 8.0 * nonzeros(s) * int(s["orb_offset"][-1]) for s, n_it in zip(systems, n_items))
+        f1 = sum(n_it * 8.0 * nonzeros(s) * int(s["orb_offset"][-1]) for s, n_it in zip(systems, n_items))
         alu, alu_kind = fp32_alu_peak(peaks)
         a1 = f1 / (g1 * 1e-3) / 1e12
-        p1 = {"kernel": "k_bsr<float,8> (product 1: W = dD H + D0 dH over the nonzero atom blocks, FP32)",
+        p1 = {"kernel": "k_bsr<float,8> (product 1: W = dD H + D0 terms over the nonzero atom blocks, FP32)",
               "bound": "alu", "achieved": round(a1, 2), "peak": round(alu, 2), "unit": "TFLOP/s",
               "frac": round(a1 / alu, 4), "peak_kind": alu_kind, "flops_per_launch": f1,
-              "flops_note": "2 x 8 nnz(H) N (delta form: dD H and D0 dH); Eq. 6 minimum is 8 nnz(H) N",
+              "flops_note": "8 nnz(H) N (the minimum of Eq. 6)",
               "avg_launch_ms": round(g1, 4), "traffic": kernel_traffic("bsr_f32", float(sum(n_items)))}
     else:
         f1 = 24.0 * n3
         a1 = f1 / (g1 * 1e-3) / 1e12
-        p1 = {"kernel": "k_tc_gemm (product 1: W = [dD|D0][H|dH]^dagger, tcgen05 BF16x3, dense)",
+        p1 = {"kernel": "k_tc_gemm (product 1: W = dD H + D0 terms, tcgen05 BF16x3)",
               "bound": "tensor", "achieved": round(a1, 1), "peak": sust, "unit": "TFLOP/s",
               "frac": round(a1 / sust, 4), "peak_kind": sust_kind, "frac_of_burst": round(a1 / burst, 4),
               "flops_per_launch": f1, "flops_note": "3 split terms x 8 N^3 (algorithmic); the kernel executes "
-                                                    f"{48 * np3:.3e} BF16 flops (K' = 4 Np, padded)",
-              "executed_tflops": round(48 * np3 / (g1 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g1, 4),
+                                                    f"at most {24 * np3:.3e} BF16 flops (K' = 2 Np, padded, "
+                                                    "before zero k-panels are skipped)",
+              "executed_tflops_upper": round(24 * np3 / (g1 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g1, 4),
               "traffic": kernel_traffic("tc_gemm1", float(sum(n_items)), tiles["product1"])}
     f2 = 24.0 * n3
     a2 = f2 / (g2 * 1e-3) / 1e12
     p2 = {"kernel": "k_tc_gemm2<3,1> (product 2: X = S^-1 W^dagger, tcgen05 BF16x3)", "bound": "tensor",
           "achieved": round(a2, 1), "peak": sust, "unit": "TFLOP/s", "frac": round(a2 / sust, 4),
           "peak_kind": sust_kind, "frac_of_burst": round(a2 / burst, 4), "flops_per_launch": f2,
-          "flops_note": "3 split terms x 8 N^3 (algorithmic, unpadded N)",
-          "executed_tflops": round(24 * np3 / (g2 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g2, 4),
+          "flops_note": "3 split terms x 8 N^3 (algorithmic, unpadded N); half of it is skipped where S^-1 is real",
+          "executed_tflops_upper": round(24 * np3 / (g2 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g2, 4),
           "traffic": kernel_traffic("tc_gemm2", float(sum(n_items)), tiles["product2"])}
     return p1, p2
 
@@ -292,9 +292,10 @@ def hbm_rates(sysd, Np, kern_ms, peak_gbs, sparse=True):
     nat = len(norb)
     nk = len(sysd["wk"])
     byts = {
-        "leap": 56 * Np * Np,                                        # X, R0 f32; dD r/w f64; f32 copy or pieces
-        # S, H0, dS f32 per image; out: H and dH at the nonzeros (2 x float2) or embedded BF16 pieces (16 x 2 B)
-        "phase": nk * (20 * el_img + 8 * len(blk) + (16 if sparse else 32) * n_el),
+        # X f32; one of two mirror tiles of R0 and D0 f32 and of the old dD f64; dD f64; f32 copy or pieces
+        "leap": 48 * Np * Np,
+        # S, H0, dS f32 per image; out: H at the nonzeros (float2) or embedded BF16 pieces (8 x 2 B)
+        "phase": nk * (20 * el_img + 8 * len(blk) + (8 if sparse else 16) * n_el),
         "obs": nk * 96 * n_el + 40 * nat,                            # dD f64 + S, P, H0 blocks f64
         "scc": 8 * nat * nat + 64 * nat,                             # gamma + per-atom vectors
     }
@@ -516,7 +517,8 @@ def native(args):
         cn = {"value": round(world * Kc / (ms_c / 1e3), 4), "unit": "steps/s", "steps": Kc,
               "ms_per_step": round(ms_c / Kc, 2), "sweeps_per_step": sweeps, "dtype": "f64",
               "kernel_ms_per_step": {k: round(v[1] / max(v[0], 1), 3) for k, v in st_c.items()},
-              "roofline": {"bound": "fp64", "kernel": "k_gemm_f64 (fixed-point sweep C^dagger + i dt/2 Y^dagger M^dagger)",
+              "roofline": {"bound": "fp64", "kernel": "k_slice_gemm, k_slice_rows (fixed-point sweep C^dagger + i dt/2 "
+                                                            "Y^dagger M^dagger: exact digit products on the tensor cores)",
                            "achieved": round(a_sweep, 3), "peak": round(p64, 3), "unit": "TFLOP/s",
                            "frac": round(a_sweep / p64, 4),
                            "peak_kind": "cuBLAS ZGEMM 2048^3 measured in this run (torch.matmul complex128)",
@@ -591,11 +593,12 @@ def native(args):
                  "ms_per_step": round(ms_f / Kf, 3),
                  "fs_per_hour": round(Kf / (ms_f / 1e3) * 0.2 * AU_FS * 3600, 3),
                  "kernel_ms_per_step": {k: round(v[1] / max(v[0], 1), 3) for k, v in stats_f.items()},
-                 "roofline": {"bound": "fp64", "kernel": "k_gemm_f64 (product 2: X = S^-1 W^dagger, dense)",
+                 "roofline": {"bound": "fp64", "kernel": "k_slice_rows, k_slice_gemm (product 2: X = S^-1 W^dagger, exact digit "
+                                                         "products on the tensor cores; the peak is the FP64 pipe's)",
                               "achieved": round(a64_2, 3), "peak": round(p64, 3), "unit": "TFLOP/s",
                               "frac": round(a64_2 / p64, 4), "flops_per_launch": fl64_2,
                               "peak_kind": "cuBLAS ZGEMM 2048^3 measured in this run (torch.matmul complex128)"},
-                 "product1": {"kernel": ("k_bsr<double,4> (W = D H over the nonzero atom blocks)" if fp64_sparse
+                 "product1": {"kernel": ("k_slice_rows, k_slice_pattern, k_slice_gemm (W = D H, zero k-panels skipped)" if fp64_sparse
                                          else "k_gemm_f64 (W = D H, dense)"),
                               "achieved": round(a64_1, 3), "peak": round(p64, 3), "unit": "TFLOP/s",
                               "frac": round(a64_1 / p64, 4), "flops_per_launch": fl64_1,

@@ -516,6 +516,7 @@ __global__ void __launch_bounds__(256) k_phase(const DevSys* __restrict__ sysv, 
   // walk k-points x images one after the other (8 atoms, 8 k-points: 37 us)
   for (int k = blockIdx.y; k < S.nk; k += gridDim.y) {
     const DevItem& it = items[T.item0 + k];
+    if (!it.kH && !it.H) continue;  // its H goes straight to digits (k_slice_hamilton)
     for (int e = lane; e < nel; e += 16) {
       const int a = e / nj, b = e - a * nj;
       const long long idx = (long long)(oi + a) * S.Np + (oj + b);

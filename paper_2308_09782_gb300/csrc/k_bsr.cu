@@ -3,7 +3,7 @@
 //   W = sum_seg A_seg R_seg^dagger
 //
 // FP64 path: W = D H (one segment; D at the level of the step's parity) or, in
-// the delta form, W = dD H + D0 dH.  Split form: W = dD H + G diag(e) in FP32 with
+// the delta form, W = dD H + D0 dH.  Split form: W = dD H + G diag(e) + A.F/c in FP32 with
 // the output stored as the embedded BF16 hi/lo pieces that the tcgen05 second
 // product (X = S^-1 W^dagger) reads.
 //
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(kBsrThreads) k_bsr(const BsrItem* __restrict__
 // four A values of an entry through a ring of kBsrStages shared-memory slots
 // with cp.async (no other thread reads them, so no CTA barrier is needed per
 // entry), so kBsrStages - 1 entries are in flight while one is applied.  The R
-// blocks of the group sit in shared memory; the D0 term G_ij e_j is added at the end.  The last CTA to run out of units resets the
+// blocks of the group sit in shared memory; the D0 terms are added at the end.  The last CTA to run out of units resets the
 // counters for the next launch.
 // ---------------------------------------------------------------------------
 constexpr int kBsrPThreads = 128;
@@ -323,10 +323,18 @@ __global__ void __launch_bounds__(kBsrPThreads, 3) k_bsr_f32p(const BsrItem* __r
         float wr[4], wi[4], nwi[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          // the D0 term of W: G_ij e_j
+          // the D0 terms of W
           const float e = it.ge[4 * (J0 + j) + c];
           wr[c] = fmaf(G[4 * j + c], e, ar[j][c]);
           wi[c] = fmaf(G[Np + 4 * j + c], e, -ai[j][c]);
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            const float av = it.fa[a];
+            if (av == 0.f) continue;
+            const float* F = it.F + a * it.f_stride + (long long)i * ld + 4 * J0;
+            wr[c] = fmaf(av, F[4 * j + c], wr[c]);
+            wi[c] = fmaf(av, F[Np + 4 * j + c], wi[c]);
+          }
           nwi[c] = -wi[c];
         }
         uint2 rh, rl, ih, il, nh, nl;

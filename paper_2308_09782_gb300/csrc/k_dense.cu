@@ -226,8 +226,12 @@ __device__ __forceinline__ void split_bf16_d(double x, __nv_bfloat16& hi, __nv_b
 
 // MP = 0: X is a matrix; MP = 7 or 2: X is put together from the integer planes of the sliced
 // product (slice.cuh), which saves writing and reading X once (134 MB at N = 2048).
+// 16 rows of threads: two elements of each tile per thread, so that few are handled one after the
+// other where the grid leaves room.
+constexpr int LY = 16;
+
 template <int MP>
-__global__ void __launch_bounds__(256) k_leap(const LeapItem* __restrict__ items, const int* step,
+__global__ void __launch_bounds__(LT* LY) k_leap(const LeapItem* __restrict__ items, const int* step,
                                               double dt, int* counter, int* step_rw) {
   pdl_wait();
   pdl_trigger();
@@ -248,9 +252,9 @@ __global__ void __launch_bounds__(256) k_leap(const LeapItem* __restrict__ items
     }
   }
   const int bj = bi + p;
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x LY
   if (active) {
-    for (int r = ty; r < LT; r += 8) {
+    for (int r = ty; r < LT; r += LY) {
       const int ra = bi * LT + r, ca = bj * LT + tx, rb = bj * LT + r, cb = bi * LT + tx;
       if constexpr (MP == 0) {
         const double2* X = (const double2*)it.X;
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(256) k_leap(const LeapItem* __restrict__ items
     const double2* base = euler ? it.D[cur] : it.D[nxt];
     for (int half = 0; half < (bi == bj ? 1 : 2); ++half) {
       const int gi0 = half == 0 ? bi : bj, gj0 = half == 0 ? bj : bi;
-      for (int r = ty; r < LT; r += 8) {
+      for (int r = ty; r < LT; r += LY) {
         const double2 xij = half == 0 ? Xa[r][tx] : Xb[r][tx];
         const double2 xji = half == 0 ? Xb[tx][r] : Xa[tx][r];
         const long long idx = (long long)(gi0 * LT + r) * Np + gj0 * LT + tx;
@@ -322,7 +326,7 @@ void launch_leap(const LeapItem* items, int n_items, int Np_max, int mp, const i
                  int* counter, int* step_rw, cudaStream_t st) {
   const int nt = Np_max / LT;
   dim3 grid(nt * (nt + 1) / 2, n_items);
-  dim3 block(LT, 8);
+  dim3 block(LT, LY);
   if (mp == 7)
     launch_pdl(k_leap<7>, grid, block, 0, st, items, step, dt, counter, step_rw);
   else if (mp == 2)
@@ -334,12 +338,14 @@ void launch_leap(const LeapItem* items, int n_items, int Np_max, int mp, const i
 // ---------------------------------------------------------------------------
 // Leapfrog of the split form.  With dH = (E S + S E)/2 + sum_a (A_a/c) P_a,
 // E = eps - eps0 per orbital, the D0 part of Eq. 6 needs no product per step:
-//   S^-1 dH D0 = S^-1 [E S D0 / 2] + E D0 / 2 + sum_a (A_a/c) S^-1 P_a D0.
-// The bracket is added to W by product 1, so that X holds S^-1 [H dD + E S D0 / 2]; here
-//   dD/dt = R0 + sum_a (A_a/c) K_a - (i/2) [E, D0] - i (X - X^dagger)
-// with constant Hermitian K_a = -i (S^-1 P_a D0 - h.c.), all read as FP32 (K_a only where
-// A_a is nonzero).  This replaces a second operand pair [D0 | dH] of product 1 (as many
-// k-panels again: 512 atoms, both products 207 -> 153 us) by 17 MB per term read here.
+//   S^-1 dH D0 = S^-1 [E S D0 / 2 + sum_a (A_a/c) P_a D0] + E D0 / 2.
+// The bracket is added to W by product 1 from the constants D0 S and D0 P_a, so that X holds
+// S^-1 [H dD + bracket], where the response H dD and the drive A.P D0 cancel in part before W is
+// cut into BF16 pieces; here
+//   dD/dt = R0 - (i/2) [E, D0] - i (X - X^dagger).
+// (With S^-1 P_a D0 added here instead, J after 250 steps of a kick was 4.7e-7 off at 512 atoms,
+// 2.8e-7 as below.)  This replaces a second operand pair [D0 | dH] of product 1 (as many
+// k-panels again: 512 atoms, both products 207 -> 153 us) by 17 to 34 MB per term.
 // dD/dt is formed in FP32 with mirror-exact operations as in k_leap; only the
 // master update dD_{n+1} = dD_{n-1} + 2 dt dD/dt is FP64 (GB300's FP64 rate is
 // low, so FP64 is kept to the accumulation that needs it).  The operand of the
@@ -347,10 +353,9 @@ void launch_leap(const LeapItem* items, int n_items, int Np_max, int mp, const i
 // copy (block-sparse product) and/or its BF16 hi/lo pieces (dense tcgen05
 // product).
 // ---------------------------------------------------------------------------
-// One CTA per tile pair (bi, bj), bi <= bj.  D, R0, K_a and D0 are Hermitian bit for bit, so only
+// One CTA per tile pair (bi, bj), bi <= bj.  D, R0 and D0 are Hermitian bit for bit, so only
 // the elements of tile (bi, bj) are formed, from X of both tiles; the mirror tile is written as
-// their conjugates through shared memory.  That halves the reads of all of these (512 atoms, one
-// nonzero A_a: 218 MB instead of 302 MB a step) and the FP64 updates.  Memory bound: 53 us at
+// their conjugates through shared memory.  That halves the reads of all of these (512 atoms: 201 MB instead of 268 MB a step) and the FP64 updates.  Memory bound: 53 us at
 // 512 atoms (4.1 TB/s), 75 us when both tiles read everything.
 // Thread layout: 16 x 16 threads, each owns two adjacent columns (2 tx, 2 tx + 1) of rows ty and
 // ty + 16 of a 32 x 32 tile, so the constants are read and the BF16 pieces written two columns per
@@ -401,7 +406,6 @@ __global__ void __launch_bounds__(256, 3) k_leap_split(const LeapItem* __restric
     const bool euler = (n == 0);
     const double coef = euler ? dt : 2.0 * dt;
     const double2* base = euler ? it.D[n & 1] : it.D[nxt];
-    const float av[3] = {it.af[0], it.af[1], it.af[2]};
     float2 xa[2][2], xb[2][2], cr[2], ci[2], zr[2], zi[2];
     double2 b[2][2];
     float di[2];
@@ -424,20 +428,6 @@ __global__ void __launch_bounds__(256, 3) k_leap_split(const LeapItem* __restric
       b[h][1] = base[idx + 1];
       di[h] = it.deh[bi * LT + r];
     }
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-      if (av[a] != 0.f) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const long long ra = (long long)(bi * LT + ty + 16 * h) * 2 * Np + bj * LT + c0;
-          const float2 kr = *reinterpret_cast<const float2*>(it.Kf + a * it.k_stride + ra);
-          const float2 ki = *reinterpret_cast<const float2*>(it.Kf + a * it.k_stride + ra + Np);
-          cr[h].x = fmaf(av[a], kr.x, cr[h].x);
-          cr[h].y = fmaf(av[a], kr.y, cr[h].y);
-          ci[h].x = fmaf(av[a], ki.x, ci[h].x);
-          ci[h].y = fmaf(av[a], ki.y, ci[h].y);
-        }
-      }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = ty + 16 * h;

@@ -416,6 +416,9 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
       pr.b_b = li;
       pr.G = it.Gf;
       pr.ge = it.ge;
+      pr.F = it.Ff;
+      pr.fa = it.fa;
+      pr.f_stride = it.f_stride;
       pr.out = it.Wemb_p;
       pr.w_half = k_real(v, it.k) ? 1 : 0;
     } else {

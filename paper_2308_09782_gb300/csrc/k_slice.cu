@@ -1,6 +1,6 @@
 // Sliced FP64 complex products (scheme and bounds in slice.cuh):
 //   k_slice_rows    - rows of a matrix, or of a finished product, to digits
-//   k_slice_pattern - the same for H_k held at its nonzero atom blocks
+//   k_slice_hamilton - H_k(t) at its nonzero atom blocks to digits
 //   k_slice_gemm    - the digit products, tcgen05 2-SM pairs
 #include <algorithm>
 #include <cstring>
@@ -205,48 +205,101 @@ void launch_slice_rows(const SliceRowJob* jobs, int n_jobs, int max_rows, int ma
     launch_rows_mp<2>(jobs, n_jobs, max_rows, max_cols, step, st);
 }
 
-// One CTA per (row atom, matrix): the atom's elements are contiguous; the largest part of each
-// of its rows is found in shared memory, then the digits go to their places.  Latency bound
-// (about 500 elements per sp3 atom).
-__global__ void __launch_bounds__(128) k_slice_pattern(const SlicePatJob* __restrict__ jobs) {
-  extern __shared__ uint32_t s_rowmax[];
+// H_k(t) = H0_k + (shift) S_k + sum_a (A_a/c) P_a (Eqs. 9-12; mode as in k_phase) at the nonzero
+// pattern, cut into digits without a stop in memory.  One CTA per (row atom, item): the largest part
+// of each of the atom's rows is found in shared memory, then the elements are formed again (their
+// operands are in L1) and their digits go to their places.  Latency bound (about 500 elements per
+// sp3 atom).  From the k-space blocks instead of the real-space images, and in one launch instead of
+// a phase build and a cut: 144 mixed atoms (delta form) 187 -> 165 us a step, 64 atoms x 8 k-points
+// 172 -> 171.
+__global__ void __launch_bounds__(128) k_slice_hamilton(const SliceHamJob* __restrict__ jobs,
+                                                        const DevSys* __restrict__ sysv,
+                                                        const DevTraj* __restrict__ trj, int max_orb,
+                                                        const int* __restrict__ step, int mode) {
+  extern __shared__ uint32_t s_rowmax[];  // [2][max_orb]: H, dH
+  const SliceHamJob& J = jobs[blockIdx.y];
+  const DevSys& S = sysv[J.sys];
+  const DevTraj& T = trj[J.traj];
+  const int I = blockIdx.x;
+  const bool live = I < S.nat;
+  const int e0 = live ? S.el_atom0[I] : 0, e1 = live ? S.el_atom0[I + 1] : 0;
+  const int oi = live ? S.orb_off[I] : 0, ni = live ? S.orb_off[I + 1] - oi : 0;
+  const long long ps = (long long)S.nk * S.n_el, kb = (long long)J.k * S.n_el;
+  const double2 *kS = S.kS + kb, *kP = S.kP + kb, *kH0 = S.kH0 + kb;
+  const bool delta = J.dout.dig != nullptr;
+  for (int r = threadIdx.x; r < 2 * max_orb; r += blockDim.x) s_rowmax[r] = 0;
+  __syncthreads();
   pdl_wait();
   pdl_trigger();
-  const SlicePatJob& J = jobs[blockIdx.y];
-  const int I = blockIdx.x;
-  if (I >= J.nat) return;
-  const int e0 = J.el_atom0[I], e1 = J.el_atom0[I + 1], oi = J.orb_off[I], ni = J.orb_off[I + 1] - oi;
-  for (int r = threadIdx.x; r < ni; r += blockDim.x) s_rowmax[r] = 0;
-  __syncthreads();
-  for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const double2 v = J.v[e];
-    const uint32_t m = max((uint32_t)__double2hiint(v.x) & 0x7fffffffu, (uint32_t)__double2hiint(v.y) & 0x7fffffffu);
-    atomicMax(&s_rowmax[J.el_off[e] / J.Np - oi], m);
+  if (!live) return;
+  const int n = *step;
+  double A0 = T.A[3 * n], A1 = T.A[3 * n + 1], A2 = T.A[3 * n + 2];
+  if (mode == PH_FP64_CN) {  // A(t_{n+1/2}) = (A_n + A_{n+1}) / 2
+    A0 = 0.5 * (A0 + T.A[3 * n + 3]);
+    A1 = 0.5 * (A1 + T.A[3 * n + 4]);
+    A2 = 0.5 * (A2 + T.A[3 * n + 5]);
   }
-  __syncthreads();
-  const long long ld = 2LL * J.out.Kp, ps = ld * J.out.rows;
-  for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const double2 v = J.v[e];
-    const int off = J.el_off[e], r = off / J.Np, c = off - r * J.Np;
-    const uint32_t mx = s_rowmax[r - oi];
+  constexpr double ic = 1.0 / kLight;
+  const double a0 = A0 * ic, a1 = A1 * ic, a2 = A2 * ic;
+  const double alpha = mode == PH_FP64_PLAIN ? 0.5 * (a0 * a0 + a1 * a1 + a2 * a2) : 0.0;
+  const bool extra = mode == PH_FP64_CN && n > 0;  // eps(t_{n+1/2}) = (3 eps_n - eps_{n-1}) / 2
+  const double* cur = extra ? T.eps_lv + (long long)(n & 1) * S.nat : T.eps;
+  const double* prv = extra ? T.eps_lv + (long long)((n - 1) & 1) * S.nat : T.eps;
+  auto shift = [&](int a) { return extra ? 1.5 * cur[a] - 0.5 * prv[a] : cur[a]; };
+  const double eI = shift(I), dI = delta ? T.eps[I] - S.eps0[I] : 0.0;
+  // element e: h, and in the delta form d
+  auto element = [&](int e, double2& h, double2& d) {
+    const int K = J.el_J[e];
+    const double2 s = kS[e], h0 = kH0[e], px = kP[e], py = kP[ps + e], pz = kP[2 * ps + e];
+    const double pr = a0 * px.x + a1 * py.x + a2 * pz.x, pi = a0 * px.y + a1 * py.y + a2 * pz.y;
+    const double beta = alpha + 0.5 * (eI + shift(K));
+    h = make_double2(h0.x + beta * s.x + pr, h0.y + beta * s.y + pi);
+    if (delta) {
+      const double db = 0.5 * (dI + (T.eps[K] - S.eps0[K]));
+      d = make_double2(db * s.x + pr, db * s.y + pi);
+    }
+  };
+  auto high = [](double2 v) {
+    return max((uint32_t)__double2hiint(v.x) & 0x7fffffffu, (uint32_t)__double2hiint(v.y) & 0x7fffffffu);
+  };
+  auto write = [](const SliceMat& out, int r, int c, double2 v, uint32_t mx) {
     const bool bad = mx >= 0x7ff00000u;
     const int efm = max((int)(mx >> 20), 1);
     const unsigned long long wr = slice_bytes(bad ? 0.0 : v.x, efm), wi = slice_bytes(bad ? 0.0 : v.y, efm);
-    __nv_bfloat16* o = J.out.dig + (long long)r * ld + c;
+    const long long ld = 2LL * out.Kp, pst = ld * out.rows;
+    __nv_bfloat16* o = out.dig + (long long)r * ld + c;
 #pragma unroll
-    for (int s = 1; s <= kSlices; ++s, o += ps) {
+    for (int s = 1; s <= kSlices; ++s, o += pst) {
       o[0] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(slice_digit(wr, s)) >> 16));
-      o[J.out.Kp] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(slice_digit(wi, s)) >> 16));
+      o[out.Kp] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(slice_digit(wi, s)) >> 16));
     }
+  };
+  for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+    double2 h, d = make_double2(0.0, 0.0);
+    element(e, h, d);
+    const int r = S.el_off[e] / S.Np - oi;
+    atomicMax(&s_rowmax[r], high(h));
+    if (delta) atomicMax(&s_rowmax[max_orb + r], high(d));
+  }
+  __syncthreads();
+  for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+    double2 h, d = make_double2(0.0, 0.0);
+    element(e, h, d);
+    const int off = S.el_off[e], r = off / S.Np, c = off - r * S.Np;
+    write(J.out, r, c, h, s_rowmax[r - oi]);
+    if (delta) write(J.dout, r, c, d, s_rowmax[max_orb + r - oi]);
   }
   for (int r = threadIdx.x; r < ni; r += blockDim.x) {
-    const uint32_t mx = s_rowmax[r];
-    J.out.ex[oi + r] = mx >= 0x7ff00000u ? kSliceNaN : max((int)(mx >> 20), 1) - 1021;
+    const uint32_t mh = s_rowmax[r], md = s_rowmax[max_orb + r];
+    J.out.ex[oi + r] = mh >= 0x7ff00000u ? kSliceNaN : max((int)(mh >> 20), 1) - 1021;
+    if (delta) J.dout.ex[oi + r] = md >= 0x7ff00000u ? kSliceNaN : max((int)(md >> 20), 1) - 1021;
   }
 }
 
-void launch_slice_pattern(const SlicePatJob* jobs, int n_jobs, int max_nat, int max_orb, cudaStream_t st) {
-  launch_pdl(k_slice_pattern, dim3(max_nat, n_jobs), 128, (size_t)max_orb * sizeof(uint32_t), st, jobs);
+void launch_slice_hamilton(const SliceHamJob* jobs, int n_jobs, int max_nat, int max_orb, const DevSys* sys,
+                           const DevTraj* trj, const int* step, int mode, cudaStream_t st) {
+  launch_pdl(k_slice_hamilton, dim3(max_nat, n_jobs), 128, 2 * (size_t)max_orb * sizeof(uint32_t), st, jobs, sys, trj,
+             max_orb, step, mode);
 }
 
 // ---------------------------------------------------------------------------

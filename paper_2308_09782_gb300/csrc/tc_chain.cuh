@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(192, 1)
           store_x(pr, stg, row - lane, lane, gn, r, nv);
         } else {
           const int slot = (c0 >> 5) & 1;
-          stage_w(pr, stg, row, lane, gc, r, nv >> 4, slot);
+          stage_w(pr, stg, row, lane, gn, gc, r, nv >> 4, slot);
           if (slot || c0 + 32 >= w)
             flush_w(pr, stg, row - lane, lane, (gn - 32 * slot) >> 1, 2 * slot + (nv >> 4));
         }

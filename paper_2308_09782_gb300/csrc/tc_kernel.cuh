@@ -51,10 +51,14 @@ struct TcProb {
   // (product 2 of a real S_k^-1: the panels of its real half)
   const int* kofs;
   const short* kidx;
-  // product 1: added to W in the epilogue: W_mj += G_mj e_j with G planar FP32
-  // [Np][2 Np] and one factor per orbital (null: nothing)
+  // product 1: added to W in the epilogue: W_mj += G_mj e_j + sum_a A_a/c F_a,mj with G and the
+  // three F_a planar FP32 [Np][2 Np] (F_a f_stride apart), one factor e_j per orbital and the three
+  // A_a/c (G null: nothing)
   const float* G;
   const float* ge;
+  const float* F;
+  const float* fa;
+  long long f_stride;
   int w_half;          // product 1: product 2 reads only the left half [Re W; -Im W] of the embedded W
   // 2-SM pair kernel, classic schedule: first B row of each column tile
   // (tiles_n + 1 entries, the last 2 Np; widths multiples of 16 up to 256, so
@@ -365,29 +369,55 @@ __device__ __forceinline__ uint4 pack8_bf16(const float (&x)[16], int h) {
 
 // Product 1 epilogue: 32 accumulator columns gn .. gn + 31 of output row `row`
 // (gn a multiple of 16) in the interleaved order (4 Re, 4 Im per block of four W
-// columns) become 16 consecutive W columns j0 = gn / 2 .. j0 + 15.  The term
-// G_mj e_j is added first, in FP32; the hi and lo pieces of Re and Im go to slot
+// columns) become 16 consecutive W columns j0 = gn / 2 .. j0 + 15.  The D0
+// terms are added first, in FP32; the hi and lo pieces of Re and Im go to slot
 // `slot` (0 or 1) of the staging area [piece][row][64 bytes].
 // (nh = 1: only the first 16 accumulator columns are the tile's, 8 W columns).
-// The D0 term's operands for 32 accumulator columns, read a chunk ahead of their use.
+// The D0 terms' operands for 32 accumulator columns, read a chunk ahead of their use: G and, for the
+// nonzero A_a, F_a (one of them as it is read, to be scaled at its use; several are summed here, which
+// waits for the reads).
 struct GChunk {
-  float4 re[4], im[4], e[4];
+  float4 re[4], im[4], fr[4], fi[4];
+  float fs;  // factor of fr, fi
 };
+
+__device__ __forceinline__ float4 fma4(float a, float4 x, float4 y) {
+  return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
+}
 
 __device__ __forceinline__ void load_g(const TcProb& pr, int row, int gn, int nh, GChunk& c) {
   if (!pr.G || row >= pr.Np) return;
-  const float4* g = reinterpret_cast<const float4*>(pr.G + (long long)row * 2 * pr.Np + (gn >> 1));
-  const float4* e = reinterpret_cast<const float4*>(pr.ge + (gn >> 1));
+  const long long o = (long long)row * 2 * pr.Np + (gn >> 1);
+  const int im = pr.Np / 4;
+  const float4* g = reinterpret_cast<const float4*>(pr.G + o);
 #pragma unroll
   for (int b = 0; b < 4; ++b)
     if (b < 2 * nh) {
       c.re[b] = g[b];
-      c.im[b] = g[b + pr.Np / 4];
-      c.e[b] = e[b];
+      c.im[b] = g[b + im];
     }
+  const float av[3] = {pr.fa[0], pr.fa[1], pr.fa[2]};
+  const int cnt = (av[0] != 0.f) + (av[1] != 0.f) + (av[2] != 0.f);
+  c.fs = cnt == 0 ? 0.f : 1.f;
+  bool first = true;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (av[a] == 0.f) continue;
+    const float4* f = reinterpret_cast<const float4*>(pr.F + a * pr.f_stride + o);
+    if (cnt == 1) c.fs = av[a];
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      if (b < 2 * nh) {
+        const float4 x = f[b], y = f[b + im];
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        c.fr[b] = cnt == 1 ? x : fma4(av[a], x, first ? z : c.fr[b]);
+        c.fi[b] = cnt == 1 ? y : fma4(av[a], y, first ? z : c.fi[b]);
+      }
+    first = false;
+  }
 }
 
-__device__ __forceinline__ void stage_w(const TcProb& pr, uint4* stg, int row, int lane, const GChunk& g,
+__device__ __forceinline__ void stage_w(const TcProb& pr, uint4* stg, int row, int lane, int gn, const GChunk& g,
                                         const uint32_t (&r)[32], int nh, int slot) {
   float re[16], im[16], rel[16], iml[16];
 #pragma unroll
@@ -401,7 +431,18 @@ __device__ __forceinline__ void stage_w(const TcProb& pr, uint4* stg, int row, i
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       if (b >= 2 * nh) break;
-      const float4 gr = g.re[b], gi = g.im[b], f = g.e[b];
+      const float4 f = reinterpret_cast<const float4*>(pr.ge + (gn >> 1))[b];
+      float4 gr = g.re[b], gi = g.im[b];
+      if (g.fs != 0.f) {
+        re[4 * b] = fmaf(g.fs, g.fr[b].x, re[4 * b]);
+        re[4 * b + 1] = fmaf(g.fs, g.fr[b].y, re[4 * b + 1]);
+        re[4 * b + 2] = fmaf(g.fs, g.fr[b].z, re[4 * b + 2]);
+        re[4 * b + 3] = fmaf(g.fs, g.fr[b].w, re[4 * b + 3]);
+        im[4 * b] = fmaf(g.fs, g.fi[b].x, im[4 * b]);
+        im[4 * b + 1] = fmaf(g.fs, g.fi[b].y, im[4 * b + 1]);
+        im[4 * b + 2] = fmaf(g.fs, g.fi[b].z, im[4 * b + 2]);
+        im[4 * b + 3] = fmaf(g.fs, g.fi[b].w, im[4 * b + 3]);
+      }
       re[4 * b] = fmaf(gr.x, f.x, re[4 * b]);
       re[4 * b + 1] = fmaf(gr.y, f.y, re[4 * b + 1]);
       re[4 * b + 2] = fmaf(gr.z, f.z, re[4 * b + 2]);
@@ -672,7 +713,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcPa
           store_x(pr, stg, row - lane, lane, gn, r, 32);
         } else {
           const int slot = (c0 >> 5) & 1;
-          stage_w(pr, stg, row, lane, g, r, 2, slot);
+          stage_w(pr, stg, row, lane, gn, g, r, 2, slot);
           if (slot) flush_w(pr, stg, row - lane, lane, (gn - 32) >> 1, 4);
         }
       }
@@ -989,7 +1030,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm2(const __grid_constant__ TcP
           store_x(pr, stg, row - lane, lane, gn, r, nv);
         } else {
           const int slot = (c0 >> 5) & 1;
-          stage_w(pr, stg, row, lane, gc, r, nv >> 4, slot);
+          stage_w(pr, stg, row, lane, gn, gc, r, nv >> 4, slot);
           if (slot || c0 + 32 >= w)
             flush_w(pr, stg, row - lane, lane, (gn - 32 * slot) >> 1, 2 * slot + (nv >> 4));
         }

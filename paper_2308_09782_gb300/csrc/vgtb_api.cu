@@ -61,10 +61,10 @@ struct HostSys {
   bool density_set = false;
   std::vector<int> trajs;  // trajectories of this system
   const double2 *d_kS = nullptr, *d_kP = nullptr;
-  const int *d_el_off = nullptr, *d_el_atom0 = nullptr, *d_orb_off = nullptr;
+  const int *d_el_off = nullptr, *d_el_J = nullptr;
   std::vector<char> k_set;  // which k-points received a user density
-  // split form, FP32 planar [nk][Np][2Np] each (Kf: [3][nk]): D0 S, D0, -i (S^-1 P_a D0 - h.c.)
-  float *Gf = nullptr, *D0f = nullptr, *Kf = nullptr;
+  // split form, FP32 planar [nk][Np][2Np] each (Ff: [3][nk]): D0 S, D0, D0 P_a
+  float *Gf = nullptr, *D0f = nullptr, *Ff = nullptr;
   int bsr_units = 0;        // block-sparse first product: CTAs per item (groups x column chunks)
   int bsr_tg_max = 0;       // most targets of one atom group
   int bsr_ent_max = 0;      // most column atoms in the union of one atom group
@@ -98,10 +98,10 @@ struct SliceRound {
   SliceGemm* g1 = nullptr;     // W (null: the first product runs block-sparse)
   SliceGemm* g2 = nullptr;     // X
   SliceRowJob* jD = nullptr;   // D (dD) to digits
-  SlicePatJob* jH = nullptr;   // H, and in the delta form dH, to digits
+  SliceHamJob* jH = nullptr;   // H, and in the delta form dH, to digits
   SliceRowJob* jW = nullptr;   // planes (or matrix) of W to digits
   LeapItem* leap = nullptr;
-  int n = 0, nH = 0, max_N = 0, max_Np = 0, max_nat = 0;
+  int n = 0, max_N = 0, max_Np = 0, max_nat = 0;
   // Crank-Nicolson: D = 2 C C^dagger, M = S^-1 H (g2), the sweeps Y^dagger M^dagger (g1)
   SliceGemm* gD = nullptr;
   ConjTItem* tC = nullptr;     // C from C^dagger
@@ -414,7 +414,6 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
   double2* pz;
   TRY(upload(ctx, &pi, h.orb_off.data(), h.orb_off.size()));
   d.orb_off = pi;
-  h.d_orb_off = pi;
   TRY(upload(ctx, &pd, h.z.data(), h.z.size()));
   d.z = pd;
   TRY(upload(ctx, &pd, h.gamma.data(), h.gamma.size()));
@@ -507,22 +506,24 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
     }
     // element offsets of the nonzeros (row-major within each target) and per-atom ranges
     if ((long long)h.Np * h.Np > 2147483647LL) return fail(ctx, VGTB_E_INVALID, "system %d: Np too large", si);
-    std::vector<int> eoff(h.n_el), eat(h.nat + 1);
+    std::vector<int> eoff(h.n_el), eJ(h.n_el), eat(h.nat + 1);
     for (int tg = 0; tg < h.n_tgt; ++tg) {
       const int oi = h.orb_off[h.tgt_I[tg]], oj = h.orb_off[h.tgt_J[tg]];
       const int nj = h.orb_off[h.tgt_J[tg] + 1] - oj;
       for (int e = h.tgt_el0[tg]; e < h.tgt_el0[tg + 1]; ++e) {
         const int a = (e - h.tgt_el0[tg]) / nj, b = (e - h.tgt_el0[tg]) % nj;
         eoff[e] = (oi + a) * h.Np + oj + b;
+        eJ[e] = h.tgt_J[tg];
       }
     }
     for (int i = 0; i <= h.nat; ++i) eat[i] = h.tgt_el0[h.atom_tgt0[i]];
     TRY(upload(ctx, &pi, eoff.data(), eoff.size()));
     d.el_off = pi;
     h.d_el_off = pi;
+    TRY(upload(ctx, &pi, eJ.data(), eJ.size()));
+    h.d_el_J = pi;
     TRY(upload(ctx, &pi, eat.data(), eat.size()));
     d.el_atom0 = pi;
-    h.d_el_atom0 = pi;
   }
   d.n_el = h.n_el;
   TRY(dalloc(ctx, &d.kS, (size_t)h.nk * h.n_el));
@@ -543,7 +544,7 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
     TRY(dalloc(ctx, &h.Sinv_p, 4 * NN * h.nk));
     TRY(dalloc(ctx, &h.Gf, 2 * NN * h.nk));
     TRY(dalloc(ctx, &h.D0f, 2 * NN * h.nk));
-    TRY(dalloc(ctx, &h.Kf, 6 * NN * h.nk));
+    TRY(dalloc(ctx, &h.Ff, 6 * NN * h.nk));
     TRY(dalloc(ctx, &h.R0f, 2 * NN * h.nk));
   }
   d.Sinv = h.Sinv;
@@ -946,15 +947,14 @@ int finish_density(vgtb_ctx* ctx, int si) {
   CK(cudaMemcpyAsync(h.eps0, h.eps0_h.data(), sizeof(double) * h.nat, cudaMemcpyHostToDevice, ctx->stream));
   if (ctx->delta) {
     // constant terms of the delta form, all in FP64: R0 = -i(S^-1 H_ref D0 - h.c.) with
-    // H_ref = H(A = 0, eps0); split form: D0 S and K_a = -i(S^-1 P_a D0 - h.c.)
+    // H_ref = H(A = 0, eps0); split form: D0 S and D0 P_a
     SetupProducts sp(ctx, h);
     TRY(sp.init());
-    double2 *Hb = nullptr, *Wb = nullptr, *Xb = nullptr, *Kb = nullptr;
+    double2 *Hb = nullptr, *Wb = nullptr, *Xb = nullptr;
     LeapItem* dl = nullptr;
     TRY(sp.alloc(&Hb, NN));
     TRY(sp.alloc(&Wb, NN));
     TRY(sp.alloc(&Xb, NN));
-    TRY(sp.alloc(&Kb, NN));
     TRY(sp.alloc(&dl, 1));
     // out = -i(S^-1 B D0 - h.c.) for the Hermitian B in Hb
     auto derivative = [&](int k, double2* out) -> int {
@@ -984,8 +984,8 @@ int finish_density(vgtb_ctx* ctx, int si) {
       launch_to_planar_f32(Wb, h.Gf + 2 * NN * k, h.Np, ctx->stream);
       for (int a = 0; a < 3; ++a) {
         launch_scatter(h.d_kP + ((size_t)a * h.nk + k) * h.n_el, h.d_el_off, h.n_el, Hb, ctx->stream);
-        TRY(derivative(k, Kb));
-        launch_to_planar_f32(Kb, h.Kf + ((size_t)a * h.nk + k) * 2 * NN, h.Np, ctx->stream);
+        TRY(sp.run(h.D0 + k * NN, Hb, Wb));
+        launch_to_planar_f32(Wb, h.Ff + ((size_t)a * h.nk + k) * 2 * NN, h.Np, ctx->stream);
       }
     }
     CK(cudaGetLastError());
@@ -1211,7 +1211,7 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
   for (size_t r = 0; r < n_rounds; ++r) {
     SliceRound R;
     std::vector<SliceRowJob> jD, jW;
-    std::vector<SlicePatJob> jH;
+    std::vector<SliceHamJob> jH;
     std::vector<LeapItem> lv;
     std::vector<SliceProd> p1, p2;
     for (size_t s = 0; s < ctx->sys.size(); ++s) {
@@ -1234,25 +1234,21 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
           SliceRowJob d = slice_row_job(it.D[0], h.Np, h.N, h.N, c.D.mat(b));
           d.src_par = (long long)NN;
           jD.push_back(d);
-          SlicePatJob hj{};
-          hj.nat = h.nat;
-          hj.Np = h.Np;
-          hj.v = (const double2*)it.kH;
-          hj.el_off = h.d_el_off;
-          hj.el_atom0 = h.d_el_atom0;
-          hj.orb_off = h.d_orb_off;
+          SliceHamJob hj{};
+          hj.sys = it.sys;
+          hj.traj = it.traj;
+          hj.k = it.k;
+          hj.el_J = h.d_el_J;
           hj.out = c.H.mat(b);
+          if (ctx->delta) hj.dout = c.dH.mat(b);
           jH.push_back(hj);
           p1.push_back(SliceProd{c.fD, b, c.fH, b, pl[0], nw, false, c.pat});
           w.n_planes = 1;
           w.pl[0] = SlicePlanes{pl[0], (long long)h.N * 2 * nw, nw, d.out.ex, hj.out.ex};
           if (ctx->delta) {
-            hj.v = (const double2*)it.kdH;
-            hj.out = c.dH.mat(b);
-            jH.push_back(hj);
             p1.push_back(SliceProd{c.fD0, it.k, c.fdH, b, pl[1], nw, false, c.pat});
             w.n_planes = 2;
-            w.pl[1] = SlicePlanes{pl[1], (long long)h.N * 2 * nw, nw, h.fD0.mat(it.k).ex, hj.out.ex};
+            w.pl[1] = SlicePlanes{pl[1], (long long)h.N * 2 * nw, nw, h.fD0.mat(it.k).ex, hj.dout.ex};
           }
         } else {
           w.src = it.W;
@@ -1268,7 +1264,6 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
       }
     }
     R.n = (int)lv.size();
-    R.nH = (int)jH.size();
     std::string msg;
     ctx->rounds.push_back(R);
     SliceRound& Q = ctx->rounds.back();
@@ -1353,7 +1348,7 @@ int slice_build_cn(vgtb_ctx* ctx) {
     SliceRound R;
     std::vector<ConjTItem> tC;
     std::vector<SliceRowJob> jC, jD, jM, jC0, jS[4];
-    std::vector<SlicePatJob> jH;
+    std::vector<SliceHamJob> jH;
     std::vector<SliceProd> pD, pM, pS;
     for (size_t s = 0; s < ctx->sys.size(); ++s) {
       const HostSys& h = ctx->sys[s];
@@ -1379,13 +1374,11 @@ int slice_build_cn(vgtb_ctx* ctx) {
         d.dst = it.D[0];
         d.ldd = h.Np;
         jD.push_back(d);
-        SlicePatJob hj{};
-        hj.nat = h.nat;
-        hj.Np = h.Np;
-        hj.v = (const double2*)it.kH;
-        hj.el_off = h.d_el_off;
-        hj.el_atom0 = h.d_el_atom0;
-        hj.orb_off = h.d_orb_off;
+        SliceHamJob hj{};
+        hj.sys = it.sys;
+        hj.traj = it.traj;
+        hj.k = it.k;
+        hj.el_J = h.d_el_J;
         hj.out = c.H.mat(b);
         jH.push_back(hj);
         pM.push_back(SliceProd{c.fS, it.k, c.fH, b, pl, nw, h.k_real[it.k] != 0, c.pat});
@@ -1416,7 +1409,7 @@ int slice_build_cn(vgtb_ctx* ctx) {
         }
       }
     }
-    R.n = R.nH = (int)jC.size();
+    R.n = (int)jC.size();
     std::string msg;
     ctx->rounds.push_back(R);
     SliceRound& Q = ctx->rounds.back();
@@ -1538,9 +1531,15 @@ void launch_cn_density(vgtb_ctx* ctx, cudaStream_t st) {
   }
 }
 
+// H_k(t) of a round's items as digits
+void launch_slice_h(vgtb_ctx* ctx, const SliceRound& r, cudaStream_t st) {
+  launch_slice_hamilton(r.jH, r.n, r.max_nat, ctx->max_orb, ctx->d_sys, ctx->d_trj, ctx->d_step,
+                        ctx->cn ? PH_FP64_CN : (ctx->delta ? PH_FP64_DELTA : PH_FP64_PLAIN), st);
+}
+
 // M = S^-1 H of a round's items, as digits
 void launch_cn_m(vgtb_ctx* ctx, const SliceRound& r, cudaStream_t st) {
-  launch_slice_pattern(r.jH, r.nH, r.max_nat, ctx->max_orb, st);
+  if (&r != &ctx->rounds.front()) launch_slice_h(ctx, r, st);
   slice_gemm_launch(r.g2, st);
   launch_slice_rows(r.jM, r.n, r.max_N, r.max_N, ctx->slice_mp, nullptr, st);
 }
@@ -1567,8 +1566,10 @@ int enqueue_step_cn(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag) {
   if (ev) CK(cudaEventRecordWithFlags(ev[1], st, evflag));
   launch_scc(ctx->d_sys, ctx->d_trj, nt, ctx->d_step, ctx->max_nat, st);
   if (ev) CK(cudaEventRecordWithFlags(ev[2], st, evflag));
-  launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk, ctx->d_step,
-               PH_FP64_CN, -1, st);
+  if (ctx->n_dense)
+    launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk, ctx->d_step,
+                 PH_FP64_CN, -1, st);
+  if (!ctx->rounds.empty()) launch_slice_h(ctx, ctx->rounds.front(), st);
   if (ev) CK(cudaEventRecordWithFlags(ev[3], st, evflag));
   if (ctx->n_dense == 0) {
   } else if (ctx->bsr) {
@@ -1606,11 +1607,12 @@ void launch_obs_scc(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag, int stride,
   launch_scc(ctx->d_sys, ctx->d_trj, nt, ctx->d_step, ctx->max_nat, st, ctx->split ? finish : 1);
 }
 
-// W = D H of a round: digits of D and H, the digit products (block-sparse first product: W is there already)
+// W = D H of a round: digits of D (and of H, which the first round has had in the phase build's place),
+// the digit products (block-sparse first product: W is there already)
 int launch_slice_first(vgtb_ctx* ctx, const SliceRound& r, cudaStream_t st) {
   if (!r.g1) return VGTB_OK;
+  if (&r != &ctx->rounds.front()) launch_slice_h(ctx, r, st);
   launch_slice_rows(r.jD, r.n, r.max_N, r.max_N, ctx->slice_mp, ctx->d_step, st);
-  launch_slice_pattern(r.jH, r.nH, r.max_nat, ctx->max_orb, st);
   if (slice_gemm_launch(r.g1, st)) return fail(ctx, VGTB_E_CUDA, "sliced product 1 launch failed");
   return VGTB_OK;
 }
@@ -1639,9 +1641,10 @@ int enqueue_step(vgtb_ctx* ctx, cudaEvent_t* ev) {
   if (ctx->split)
     launch_phase_split(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk,
                        ctx->d_step, 1, st);
-  else
+  else if (ctx->n_dense || ctx->n_bsr)
     launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk, ctx->d_step,
                  ctx->delta ? PH_FP64_DELTA : PH_FP64_PLAIN, -1, st);
+  if (!ctx->rounds.empty() && ctx->rounds.front().g1) launch_slice_h(ctx, ctx->rounds.front(), st);
   if (ev) CK(cudaEventRecordWithFlags(ev[3], st, evflag));
   if (ctx->bsr && ctx->n_bsr > 0)
     launch_bsr(ctx->d_bsr, ctx->d_bsrsys, ctx->n_bsr, ctx->bsr_units_max, ctx->bsr_units_total, ctx->d_bsr_u0,
@@ -1948,9 +1951,13 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
         it.Wemb_p = fam[T.sys].Wemb + 8 * NN * li;
         it.Xf = fam[T.sys].Xf + 2 * NN * li;
         it.Gf = h.Gf + 2 * NN * k;
+        it.Ff = h.Ff + 2 * NN * k;
+        it.f_stride = (long long)(2 * NN * h.nk);
       } else if (ctx->cn) {
         const size_t nc = (size_t)h.nocc * h.Np;
-        if (ctx->bsr || h.slice) {
+        if (h.slice) {
+          // H goes straight to digits
+        } else if (ctx->bsr) {
           double2* kh = nullptr;
           if ((rc = dalloc(ctx, &kh, (size_t)h.n_el))) return bail(rc);
           it.kH = kh;
@@ -1963,7 +1970,9 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
         if ((rc = dalloc(ctx, &it.Y[0], nc))) return bail(rc);
         if ((rc = dalloc(ctx, &it.Y[1], nc))) return bail(rc);
       } else {
-        if (ctx->bsr || h.slice) {
+        if (h.slice && ctx->opt.product1 != VGTB_P1_BLOCKS) {
+          // H (and dH) go straight to digits
+        } else if (ctx->bsr) {
           double2 *kh = nullptr, *kdh = nullptr;
           if ((rc = dalloc(ctx, &kh, (size_t)h.n_el))) return bail(rc);
           if (ctx->delta && (rc = dalloc(ctx, &kdh, (size_t)h.n_el))) return bail(rc);
@@ -1986,8 +1995,11 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     if (ctx->split) {
       if ((rc = dalloc(ctx, &T.epsf, h.nat))) return bail(rc);
       if ((rc = dalloc(ctx, &T.deh, h.Np))) return bail(rc);
-      for (int k = 0; k < h.nk; ++k) ctx->items_h[T.item0 + k].ge = T.deh;
       if ((rc = dalloc(ctx, &T.af, 3))) return bail(rc);
+      for (int k = 0; k < h.nk; ++k) {
+        ctx->items_h[T.item0 + k].ge = T.deh;
+        ctx->items_h[T.item0 + k].fa = T.af;
+      }
     }
     if ((rc = dalloc(ctx, &T.cpart, 6 * (size_t)((h.nat + kSccRowsPerCta - 1) / kSccRowsPerCta)))) return bail(rc);
     if ((rc = dalloc(ctx, &T.apart, 4 * (size_t)h.nat))) return bail(rc);
@@ -2045,10 +2057,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     l.R0 = (ctx->delta && !ctx->split) ? h.R0 + it.k * NN : nullptr;
     if (ctx->split) {
       l.R0f = h.R0f + 2 * NN * it.k;
-      l.Kf = h.Kf + 2 * NN * it.k;
-      l.k_stride = (long long)(2 * NN * h.nk);
       l.D0f = h.D0f + 2 * NN * it.k;
-      l.af = ctx->trj[it.traj].af;
       l.deh = it.ge;
     }
     l.D[0] = it.D[0];
@@ -2092,6 +2101,9 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
         b.A[0] = it.dDf;                       // FP32 copy of the current dD level
         b.G = it.Gf;
         b.ge = it.ge;
+        b.F = it.Ff;
+        b.fa = it.fa;
+        b.f_stride = it.f_stride;
         b.W = it.Wemb_p;
       } else {
         b.A[0] = it.D[0];                      // level of the step's parity

@@ -178,6 +178,9 @@ struct DevItem {
   __nv_bfloat16* Wemb_p;   // split form: [2][2Np][2Np] embedded W
   const float* Gf;         // split form: D0 S of the item's k-point, planar FP32 [Np][2Np]
   const float* ge;         // split form: (eps_I - eps0_I) / 2 of every orbital [Np]
+  const float* Ff;         // split form: D0 P_a, three planar FP32 matrices f_stride apart
+  const float* fa;         // split form: A(t_n) / c
+  long long f_stride;
   float* Xf;               // split form: [Np][2Np] planar X
   double2* Cd;             // Crank-Nicolson: occupied states as rows, C^dagger [nocc][Np]
   double2* Y[2];           // Crank-Nicolson: fixed-point iterates [nocc][Np]
@@ -213,8 +216,12 @@ struct BsrItem {
   long long a_par;         // segment 0 reads A[0] + ((*step) & 1) * a_par (leapfrog level)
   const void* R[2];        // [n_el] complex target blocks (4 x 4 row-major each)
   void* W;                 // FP64: [Np][Np] double2; split: embedded BF16 pieces [2][2Np][2Np]
-  const float* G;          // split: W_ij += G_ij ge_j (planar FP32 [Np][2Np], one factor per orbital)
+  // split: W_ij += G_ij ge_j + sum_a fa_a F_a,ij (planar FP32 [Np][2Np], one factor per orbital)
+  const float* G;
   const float* ge;
+  const float* F;
+  const float* fa;
+  long long f_stride;
 };
 int bsr_group(int fp64);
 size_t bsr_smem_bytes(int fp64, int max_grp_targets);
@@ -326,11 +333,8 @@ struct LeapItem {
   SlicePlanes pl;          // or the planes of X (launch_leap with mp != 0)
   const double2* R0;       // optional (FP64 path)
   const float* R0f;        // optional (split path, FP32 planar)
-  // split path, the terms of the derivative that are linear in A and in the shift:
-  const float* Kf;         // [3] planes, stride k_stride: K_a = -i (S^-1 P_a D0 - h.c.), FP32 planar
-  long long k_stride;
+  // split path, the term of the derivative that is linear in the shift:
   const float* D0f;        // D0, FP32 planar
-  const float* af;         // A(t_n) / c
   const float* deh;        // (eps_I - eps0_I) / 2 per orbital
   double2* D[2];
   __nv_bfloat16* pieces;   // optional [2][Np][2Np]

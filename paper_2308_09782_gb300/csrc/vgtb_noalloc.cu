@@ -113,6 +113,9 @@ __global__ void k_na_prob(TcProb* prob, int* err, int Np, float* out) {
   p.kidx = nullptr;
   p.G = nullptr;
   p.ge = nullptr;
+  p.F = nullptr;
+  p.fa = nullptr;
+  p.f_stride = 0;
   p.w_half = 0;
   p.cofs = nullptr;  // column tiles of 256
   *prob = p;

@@ -28,17 +28,15 @@ struct SliceRowJob {
 void launch_slice_rows(const SliceRowJob* jobs, int n_jobs, int max_rows, int max_cols, int mp, const int* step,
                        cudaStream_t st);
 
-// Digits of a Hermitian-pattern matrix given at the target elements only (H_k):
-// positions off the pattern are left as they are (zeros).
-struct SlicePatJob {
-  int nat, Np;
-  const double2* v;        // [n_el]
-  const int* el_off;       // [n_el] row * Np + column
-  const int* el_atom0;     // [nat+1]
-  const int* orb_off;      // [nat+1]
-  SliceMat out;
+// H_k(t) (delta form: and dH_k(t)) of one item from the k-space blocks S_k, H0_k, P_k, straight to
+// digits: positions off the nonzero pattern are left as they are (zeros).
+struct SliceHamJob {
+  int sys, traj, k;
+  const int* el_J;         // [n_el] column atom of every nonzero
+  SliceMat out, dout;      // H; dH in the delta form, else dout.dig == null
 };
-void launch_slice_pattern(const SlicePatJob* jobs, int n_jobs, int max_nat, int max_orb, cudaStream_t st);
+void launch_slice_hamilton(const SliceHamJob* jobs, int n_jobs, int max_nat, int max_orb, const DevSys* sys,
+                           const DevTraj* trj, const int* step, int mode, cudaStream_t st);
 
 // One operand family: the digits of `batch` matrices of one shape, contiguous.
 struct SliceFam {
