@@ -399,21 +399,31 @@ __device__ __forceinline__ void load_g(const TcProb& pr, int row, int gn, int nh
   const float av[3] = {pr.fa[0], pr.fa[1], pr.fa[2]};
   const int cnt = (av[0] != 0.f) + (av[1] != 0.f) + (av[2] != 0.f);
   c.fs = cnt == 0 ? 0.f : 1.f;
-  bool first = true;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    if (av[a] == 0.f) continue;
+  if (cnt == 1) {
+    const int a = av[0] != 0.f ? 0 : (av[1] != 0.f ? 1 : 2);
     const float4* f = reinterpret_cast<const float4*>(pr.F + a * pr.f_stride + o);
-    if (cnt == 1) c.fs = av[a];
+    c.fs = a == 0 ? av[0] : (a == 1 ? av[1] : av[2]);
 #pragma unroll
     for (int b = 0; b < 4; ++b)
       if (b < 2 * nh) {
-        const float4 x = f[b], y = f[b + im];
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        c.fr[b] = cnt == 1 ? x : fma4(av[a], x, first ? z : c.fr[b]);
-        c.fi[b] = cnt == 1 ? y : fma4(av[a], y, first ? z : c.fi[b]);
+        c.fr[b] = f[b];
+        c.fi[b] = f[b + im];
       }
-    first = false;
+  } else if (cnt > 1) {
+    bool first = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      if (av[a] == 0.f) continue;
+      const float4* f = reinterpret_cast<const float4*>(pr.F + a * pr.f_stride + o);
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (b < 2 * nh) {
+          const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+          c.fr[b] = fma4(av[a], f[b], first ? z : c.fr[b]);
+          c.fi[b] = fma4(av[a], f[b + im], first ? z : c.fi[b]);
+        }
+      first = false;
+    }
   }
 }
 
