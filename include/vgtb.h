@@ -121,7 +121,7 @@ typedef struct {
                                a tile's rows of H_k are zero, or below 97 orbitals runs it
                                block-sparse (below), as does the Crank-Nicolson integrator its
                                product M = S^-1 H; the split form runs the tcgen05 GEMM and skips the 64-wide k-panels in
-                               which a tile's rows of H_k and dH_k are zero;
+                               which a tile's rows of H_k are zero;
                                DENSE: a dense product over all of H_k (8 N^3 flops, no panel
                                skipped); BLOCKS: block-sparse over the
                                nonzero atom blocks of H_k on the CUDA cores (8 nnz(H) N flops;
@@ -264,11 +264,11 @@ int vgtb_kernel_stats(vgtb_ctx* ctx, long long* launches, double* ms, int n);
 /* Text of the last error on this context (or of the last failed create when
  * ctx is NULL).  Valid until the next call on the same context. */
 /* Split-precision contexts: the tile variant each tcgen05 product runs with
- * (product 1 = [dD|D0][H|dH]^dagger, product 2 = S^-1 W^dagger), chosen at
+ * (product 1 = dD H^dagger, product 2 = S^-1 W^dagger), chosen at
  * create (variant 0, or the autotuner's fastest).  cfg[4] = {tile width,
  * pipeline stages, schedule (0 classic, 1 stream-K, 2 whole waves classic and
  * stream-K over the rest; + 4: the k-panels skipped in which the tile's rows
- * of H_k and dH_k are zero (product 1), or the imaginary half of a real S_k^-1 (product 2); + 8: classic over column tiles of
+ * of H_k are zero (product 1), or the imaginary half of a real S_k^-1 (product 2); + 8: classic over column tiles of
  * planned widths, multiples of 16, the tile width being the widest; + 16: both
  * products run as one launch, VGTB_CHAIN_*), 1 if the tile spans a 2-SM CTA pair}.  When the first product runs block-sparse
  * (VGTB_P1_BLOCKS), product 1 reports {atoms per group, output rows per CTA, 3, 0}.

@@ -1,13 +1,16 @@
 // Dense FP64 kernels:
-//   k_gemm_f64 - C = sum_seg A_seg R_seg^dagger (complex128, row-major), the two
-//                commutator products of Eq. 6 in FP64:
+//   k_gemm_f64,
+//   k_gemm_f64_small - C = sum_seg A_seg R_seg^dagger (complex128, row-major) on the FP64
+//                pipe: the two commutator products of Eq. 6 up to kGemmSmall orbitals
 //                  W = D H (= (H D)^dagger),  X = S^-1 W^dagger = S^-1 H D
+//                (larger ones run as digit products on the tensor cores, k_slice.cu),
+//                set-up products, and whatever the sliced products have no room for
 //   k_leap     - dD/dt = R0 - i (X - X^dagger) (Eq. 6 with X = S^-1 H D) and the
 //                leapfrog update of Eq. 13; tile (bi, bj) and (bj, bi) are handled by
 //                one CTA so X^dagger is read from shared memory, and each D level is
 //                read and written exactly once.
 //   helpers    - Hermitian fill, eigenvector transpose, BF16 hi/lo splitting.
-// GB300 has no FP64 tensor-core kind, so the FP64 path runs on DFMA.
+// GB300 has no FP64 tensor-core kind, so these kernels run on DFMA.
 #include <algorithm>
 
 #include "slice.cuh"
