@@ -2549,6 +2549,11 @@ int vgtb_set_state(vgtb_ctx* ctx, const void* buf, long long bytes) {
       CK(cudaMemcpyAsync(t.eps_lv, p, b, cudaMemcpyHostToDevice, ctx->stream));
       p += b;
     }
+  // the state holds C^dagger; D of the restored level is what vgtb_get_density reads
+  if (ctx->cn) {
+    launch_cn_density(ctx, ctx->stream);
+    CK(cudaGetLastError());
+  }
   CK(cudaMemcpyAsync(ctx->d_step, &n, sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemsetAsync(ctx->d_counter, 0, sizeof(int), ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));

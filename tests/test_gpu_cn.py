@@ -192,3 +192,35 @@ def test_cn_argument_errors():
             c.set_density(0, 0, gs["D"][0])
         with pytest.raises(vgtb.VgtbError):
             c.set_coefficients(0, 0, gs["C"][0][:, :-1])
+
+
+@pytest.mark.parametrize("atoms", [8, 64])
+def test_cn_density_after_set_state_is_the_restored_level(atoms):
+    """get_density reads D_k(t_n) = 2 C C^dagger of the restored states, in the context that saved them
+    and in a fresh one, before any further step.  Both sides round sums of n_occ products of entries
+    below 1: 1e-13 absolute."""
+    if atoms == 8:
+        s, _, gs = si8d()
+    else:
+        s, gs = system("si64_pulse")[0], oracle_ground("si64_pulse")[1]
+    n, n_occ = 12, gs["C"][0].shape[1]
+    A = inputs.pulse_field(n, s["dt"], 0.05, 0.3)
+
+    def check(c):
+        for k in (0, len(gs["C"]) - 1):
+            C = c.get_coefficients(0, k, n_occ)
+            assert np.abs(C).max() < 1.0
+            assert np.abs(c.get_density(0, k) - 2.0 * (C @ C.conj().T)).max() <= 1e-13
+
+    with _cn_ctx(s, gs["C"]) as c, _cn_ctx(s, gs["C"]) as fresh:
+        c.set_field(0, A)
+        c.propagate(5)
+        state, D5 = c.get_state(), c.get_density(0, 0)
+        c.propagate(n - 5)
+        assert np.abs(c.get_density(0, 0) - D5).max() > 1e-6
+        c.set_state(state)
+        check(c)
+        assert np.array_equal(c.get_density(0, 0), D5)
+        fresh.set_field(0, A)
+        fresh.set_state(state)
+        check(fresh)
