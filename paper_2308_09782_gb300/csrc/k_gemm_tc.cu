@@ -292,8 +292,10 @@ static std::vector<int> plan_columns(const TcSysView& v, bool skip, int full, in
   return even_split(total, score[0].second);
 }
 
+// The tables go up on `stream`, on which the products run: it may be a non-blocking stream, which
+// copies on the legacy stream are not ordered with.
 static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevItem>& items, int epi, int variant,
-                     long long timeout_ns, TcPlan* plan, std::string* msg) {
+                     long long timeout_ns, cudaStream_t stream, TcPlan* plan, std::string* msg) {
   const Variant& var = kVariants[variant];
   const int BNv = var.bn;
   const bool pair = var.pair != 0;
@@ -381,8 +383,8 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
       *msg = "cudaMalloc failed for the k-panel lists";
       return -1;
     }
-    cudaMemcpy(plan->d_kofs, all_kofs.data(), sizeof(int) * all_kofs.size(), cudaMemcpyHostToDevice);
-    cudaMemcpy(plan->d_kidx, all_kidx.data(), sizeof(short) * all_kidx.size(), cudaMemcpyHostToDevice);
+    cudaMemcpyAsync(plan->d_kofs, all_kofs.data(), sizeof(int) * all_kofs.size(), cudaMemcpyHostToDevice, stream);
+    cudaMemcpyAsync(plan->d_kidx, all_kidx.data(), sizeof(short) * all_kidx.size(), cudaMemcpyHostToDevice, stream);
     plan->skip = true;
   }
   if (var.widths || narrow) {
@@ -394,7 +396,7 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
       *msg = "cudaMalloc failed for the column tiles";
       return -1;
     }
-    cudaMemcpy(plan->d_cofs, all_cofs.data(), sizeof(int) * all_cofs.size(), cudaMemcpyHostToDevice);
+    cudaMemcpyAsync(plan->d_cofs, all_cofs.data(), sizeof(int) * all_cofs.size(), cudaMemcpyHostToDevice, stream);
   }
   std::vector<TcProb> probs;
   std::vector<int> local(sys.size(), 0);
@@ -447,8 +449,8 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
     *msg = "cudaMalloc failed for the product plan";
     return -1;
   }
-  cudaMemcpy(plan->d_probs, probs.data(), sizeof(TcProb) * probs.size(), cudaMemcpyHostToDevice);
-  cudaMemset(plan->d_err, 0, sizeof(int));
+  cudaMemcpyAsync(plan->d_probs, probs.data(), sizeof(TcProb) * probs.size(), cudaMemcpyHostToDevice, stream);
+  cudaMemsetAsync(plan->d_err, 0, sizeof(int), stream);
   plan->probs_h = probs;
   plan->starts_h = starts;
   plan->cost_h = tile_cost;
@@ -468,7 +470,7 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
       *msg = "cudaMalloc failed for the tile order";
       return -1;
     }
-    cudaMemcpy(plan->d_tord, tord.data(), sizeof(int) * tord.size(), cudaMemcpyHostToDevice);
+    cudaMemcpyAsync(plan->d_tord, tord.data(), sizeof(int) * tord.size(), cudaMemcpyHostToDevice, stream);
     plan->P.tord = plan->d_tord;
     plan->P.n_tord = (int)tord.size();
   }
@@ -501,9 +503,14 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
       *msg = "cudaMalloc failed for the stream-K workspace";
       return -1;
     }
-    cudaMemset(plan->d_flags, 0, sizeof(int) * nsm);
+    cudaMemsetAsync(plan->d_flags, 0, sizeof(int) * nsm, stream);
     plan->P.ws = plan->d_ws;
     plan->P.flags = plan->d_flags;
+  }
+  // the host tables leave scope
+  if (cudaStreamSynchronize(stream) != cudaSuccess) {
+    *msg = "upload of the product plan failed";
+    return -1;
   }
   return 0;
 }
@@ -571,7 +578,7 @@ int tc_build_plans(const std::vector<TcSysView>& sys, const std::vector<DevItem>
     const int nv = fv >= 0 ? first + 1 : (autotune ? kNumVariants : first + 1);
     for (int v = first; v < nv; ++v) {
       TcPlan* p = new TcPlan();
-      if (build_one(sys, items, epi, v, timeout_ns, p, msg)) {
+      if (build_one(sys, items, epi, v, timeout_ns, st, p, msg)) {
         tc_destroy_plan(p);
         for (auto& r : ran) tc_destroy_plan(r.first);
         return -1;
@@ -580,7 +587,8 @@ int tc_build_plans(const std::vector<TcSysView>& sys, const std::vector<DevItem>
       if (nv - first > 1) {
         ms = time_plan(p, st);
         int err = 0;
-        cudaMemcpy(&err, p->d_err, sizeof(int), cudaMemcpyDeviceToHost);
+        cudaMemcpyAsync(&err, p->d_err, sizeof(int), cudaMemcpyDeviceToHost, st);
+        cudaStreamSynchronize(st);
         if (cudaGetLastError() != cudaSuccess || err) {
           tc_destroy_plan(p);
           continue;
@@ -601,11 +609,11 @@ int tc_build_plans(const std::vector<TcSysView>& sys, const std::vector<DevItem>
     const bool keep_alt = alt && bestc >= 0 && bestc != best;
     for (int i = 0; i < (int)ran.size(); ++i)
       if (i != best && !(keep_alt && i == bestc)) tc_destroy_plan(ran[i].first);
-    cudaMemset(ran[best].first->d_err, 0, sizeof(int));
+    tc_clear_error(ran[best].first, st);
     (epi == 0 ? *p1 : *p2) = ran[best].first;
     if (ms_best) ms_best[epi] = ran[best].second;
     if (keep_alt) {
-      cudaMemset(ran[bestc].first->d_err, 0, sizeof(int));
+      tc_clear_error(ran[bestc].first, st);
       *alt = ran[bestc].first;
     }
   }
@@ -640,8 +648,8 @@ void tc_destroy_plan(TcPlan* p) {
 
 int tc_plan_variant(const TcPlan* p) { return p ? p->variant : -1; }
 
-void tc_clear_error(TcPlan* p) {
-  if (p) cudaMemset(p->d_err, 0, sizeof(int));
+void tc_clear_error(TcPlan* p, cudaStream_t st) {
+  if (p) cudaMemsetAsync(p->d_err, 0, sizeof(int), st);
 }
 
 int tc_plan_info(const TcPlan* p, int* out4) {
@@ -739,7 +747,7 @@ static std::vector<int> chain_order(const TcPlan* p1, const TcPlan* p2, int G, d
   return ord;
 }
 
-int tc_build_chain(const TcPlan* p1, const TcPlan* p2, TcChain** out, std::string* msg) {
+int tc_build_chain(const TcPlan* p1, const TcPlan* p2, cudaStream_t st, TcChain** out, std::string* msg) {
   *out = nullptr;
   if (!tc_chainable(p1, p2)) {
     *msg = "the two products cannot be chained (2-SM pair, classic schedule and 64-column stages needed)";
@@ -790,10 +798,14 @@ int tc_build_chain(const TcPlan* p1, const TcPlan* p2, TcChain** out, std::strin
     *msg = "cudaMalloc failed for the chained schedule";
     return -1;
   }
-  cudaMemcpy(c->d_ord, ord.data(), sizeof(int) * ord.size(), cudaMemcpyHostToDevice);
-  cudaMemcpy(c->d_blk0, blk0.data(), sizeof(int) * blk0.size(), cudaMemcpyHostToDevice);
-  cudaMemset(c->d_ready, 0, sizeof(unsigned long long) * nblk);
-  cudaMemset(c->d_epoch, 0, 2 * sizeof(unsigned long long));
+  cudaMemcpyAsync(c->d_ord, ord.data(), sizeof(int) * ord.size(), cudaMemcpyHostToDevice, st);
+  cudaMemcpyAsync(c->d_blk0, blk0.data(), sizeof(int) * blk0.size(), cudaMemcpyHostToDevice, st);
+  tc_reset_chain(c, st);
+  if (cudaStreamSynchronize(st) != cudaSuccess) {  // the host tables leave scope
+    tc_destroy_chain(c);
+    *msg = "upload of the chained schedule failed";
+    return -1;
+  }
   c->X.ord = c->d_ord;
   c->X.n_ord = (int)ord.size();
   c->X.t1 = p1->P.total_tiles;
@@ -858,8 +870,9 @@ int tc_time_chain(TcChain* c, TcPlan* p1, TcPlan* p2, cudaStream_t st, double* m
   *ms_chain = a[R / 2];
   *ms_sep = b[R / 2];
   int err = 0, errc = 0;
-  cudaMemcpy(&err, p1->d_err, sizeof(int), cudaMemcpyDeviceToHost);
-  cudaMemcpy(&errc, c->p1->d_err, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaMemcpyAsync(&err, p1->d_err, sizeof(int), cudaMemcpyDeviceToHost, st);
+  cudaMemcpyAsync(&errc, c->p1->d_err, sizeof(int), cudaMemcpyDeviceToHost, st);
+  cudaStreamSynchronize(st);
   if (cudaGetLastError() != cudaSuccess || err || errc) return -1;
   return 0;
 }

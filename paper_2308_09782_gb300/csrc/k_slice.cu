@@ -626,13 +626,16 @@ bool slice_map(CUtensorMap* m, const SliceFam& f, int box_rows, std::string* msg
   return true;
 }
 
+// On the stream of the launches: k_slice_gemm reads its units before it waits for the kernel ahead
+// of it, and the stream may be a non-blocking one, which copies on the legacy stream are not ordered
+// with.
 template <class T>
-bool slice_upload(SliceGemm* g, const T** dst, const std::vector<T>& v) {
+bool slice_upload(SliceGemm* g, const T** dst, const std::vector<T>& v, cudaStream_t st) {
   void* p = nullptr;
   if (cudaMalloc(&p, std::max<size_t>(v.size(), 1) * sizeof(T)) != cudaSuccess) return false;
   g->mem.push_back(p);
   *dst = (const T*)p;
-  return cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice) == cudaSuccess;
+  return cudaMemcpyAsync(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, st) == cudaSuccess;
 }
 
 // 64-wide column panels of the R rows of every 128-row tile that hold a nonzero of the pattern
@@ -675,8 +678,8 @@ void slice_panels(const SlicePattern* pat, int N, int Kp, std::vector<int>& kofs
 }  // namespace
 
 int slice_gemm_create(const std::vector<SliceFam>& fams, const std::vector<SliceProd>& prods,
-                      const std::vector<SlicePattern>& patterns, int mp, long long timeout_ns, int* err, SliceGemm** out,
-                      std::string* msg) {
+                      const std::vector<SlicePattern>& patterns, int mp, long long timeout_ns, int* err,
+                      cudaStream_t st, SliceGemm** out, std::string* msg) {
   *out = nullptr;
   SliceGemm* g = new SliceGemm();
   auto bail = [&](const char* m) {
@@ -779,8 +782,10 @@ int slice_gemm_create(const std::vector<SliceFam>& fams, const std::vector<Slice
   const CUtensorMap* d_maps;
   const SliceUnit* d_units;
   const short* d_kidx;
-  if (!slice_upload(g, &d_maps, maps) || !slice_upload(g, &d_units, order) || !slice_upload(g, &d_kidx, all_kidx))
-    return bail("cudaMalloc failed");
+  const bool up = slice_upload(g, &d_maps, maps, st) && slice_upload(g, &d_units, order, st) &&
+                  slice_upload(g, &d_kidx, all_kidx, st);
+  if (cudaStreamSynchronize(st) != cudaSuccess || !up)  // the host tables leave scope
+    return bail("upload of the sliced product's tables failed");
   g->P.maps = d_maps;
   g->P.units = d_units;
   g->P.kidx = d_kidx;

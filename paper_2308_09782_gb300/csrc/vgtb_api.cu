@@ -866,8 +866,8 @@ class SetupProducts {
     std::string msg;
     if (alloc(&fa.dig, dig) || alloc(&fr.dig, dig) || alloc(&fa.ex, h.N) || alloc(&fr.ex, h.N) ||
         alloc(&planes, (size_t)slice_num_planes(mp) * h.N * 2 * nw) || alloc(&dj, 3) || alloc(&err, 1) ||
-        slice_gemm_create({fa, fr}, {SliceProd{0, 0, 1, 0, planes, nw, false, -1}}, {}, mp, 2000000000LL, err, &g,
-                          &msg)) {
+        slice_gemm_create({fa, fr}, {SliceProd{0, 0, 1, 0, planes, nw, false, -1}}, {}, mp, 2000000000LL, err,
+                          ctx->stream, &g, &msg)) {
       // no room for the digits: the FP64 pipe
       slice_gemm_destroy(g);
       g = nullptr;
@@ -1267,8 +1267,8 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
     std::string msg;
     ctx->rounds.push_back(R);
     SliceRound& Q = ctx->rounds.back();
-    if ((first && slice_gemm_create(fams, p1, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.g1, &msg)) ||
-        slice_gemm_create(fams, p2, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.g2, &msg))
+    if ((first && slice_gemm_create(fams, p1, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g1, &msg)) ||
+        slice_gemm_create(fams, p2, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g2, &msg))
       return fail(ctx, VGTB_E_CUDA, "sliced product plan: %s", msg.c_str());
     if (first) TRY(upload(ctx, &Q.jD, jD.data(), jD.size()));
     if (first) TRY(upload(ctx, &Q.jH, jH.data(), jH.size()));
@@ -1413,9 +1413,9 @@ int slice_build_cn(vgtb_ctx* ctx) {
     std::string msg;
     ctx->rounds.push_back(R);
     SliceRound& Q = ctx->rounds.back();
-    if (slice_gemm_create(fams, pD, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.gD, &msg) ||
-        slice_gemm_create(fams, pM, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.g2, &msg) ||
-        slice_gemm_create(fams, pS, pats, ctx->slice_mp, tmo, ctx->d_slice_err, &Q.g1, &msg))
+    if (slice_gemm_create(fams, pD, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.gD, &msg) ||
+        slice_gemm_create(fams, pM, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g2, &msg) ||
+        slice_gemm_create(fams, pS, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g1, &msg))
       return fail(ctx, VGTB_E_CUDA, "sliced product plan: %s", msg.c_str());
     TRY(upload(ctx, &Q.tC, tC.data(), tC.size()));
     TRY(upload(ctx, &Q.jC, jC.data(), jC.size()));
@@ -2167,7 +2167,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     TcPlan* c1 = (alt1 && !tc_chainable(ctx->tc1, ctx->tc1)) ? alt1 : ctx->tc1;
     TcPlan* c2 = (alt2 && !tc_chainable(ctx->tc2, ctx->tc2)) ? alt2 : ctx->tc2;
     if (ctx->opt.chain != VGTB_CHAIN_OFF && tc_chainable(c1, c2)) {
-      if (tc_build_chain(c1, c2, &ctx->tcc, &msg)) {
+      if (tc_build_chain(c1, c2, ctx->stream, &ctx->tcc, &msg)) {
         if (alt1) tc_destroy_plan(alt1);
         if (alt2) tc_destroy_plan(alt2);
         return bail(fail(ctx, VGTB_E_CUDA, "tcgen05 chained plan: %s", msg.c_str()));
@@ -2183,10 +2183,10 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
         if (tr) {
           cudaStreamSynchronize(ctx->stream);
           cudaGetLastError();
-          tc_clear_error(ctx->tc1);
-          tc_clear_error(ctx->tc2);
-          tc_clear_error(c1);
-          tc_clear_error(c2);
+          tc_clear_error(ctx->tc1, ctx->stream);
+          tc_clear_error(ctx->tc2, ctx->stream);
+          tc_clear_error(c1, ctx->stream);
+          tc_clear_error(c2, ctx->stream);
         }
       }
     }

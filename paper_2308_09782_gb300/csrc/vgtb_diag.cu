@@ -240,7 +240,8 @@ extern "C" int vgtb_diag_slice_product(int m, int n, int k, const double* a, con
     return VGTB_E_CUDA;
   SliceGemm* g = nullptr;
   std::string msg;
-  if (slice_gemm_create({fa, fr}, {SliceProd{0, 0, 1, 0, pl, nw, a_real != 0, -1}}, {}, mp, 2000000000LL, err, &g, &msg))
+  if (slice_gemm_create({fa, fr}, {SliceProd{0, 0, 1, 0, pl, nw, a_real != 0, -1}}, {}, mp, 2000000000LL, err, 0, &g,
+                        &msg))
     return VGTB_E_CUDA;
   launch_slice_rows(dj, 2, std::max(m, n), k, mp, nullptr, 0);
   int rc = slice_gemm_launch(g, 0) ? VGTB_E_CUDA : VGTB_OK;

@@ -75,8 +75,9 @@ struct SliceGemm;
 int slice_pairs_per_plane(long long tiles);  // 7, or 2 when 7 planes of work leave the chip idle
 int slice_tiles(int M, int N);
 int slice_gemm_create(const std::vector<SliceFam>& fams, const std::vector<SliceProd>& prods,
-                      const std::vector<SlicePattern>& patterns, int mp, long long timeout_ns, int* err, SliceGemm** out,
-                      std::string* msg);  // err: device word that an expired wait sets
+                      const std::vector<SlicePattern>& patterns, int mp, long long timeout_ns, int* err,
+                      cudaStream_t st, SliceGemm** out,
+                      std::string* msg);  // err: device word that an expired wait sets; st: the stream of the launches
 int slice_gemm_launch(SliceGemm* g, cudaStream_t st);
 void slice_gemm_destroy(SliceGemm* g);
 inline int slice_kp(int K) { return (K + 63) / 64 * 64; }
