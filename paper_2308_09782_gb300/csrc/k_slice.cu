@@ -449,11 +449,10 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_slice_gemm(const __grid_const
       bool ok = true, issued = false;
       for (; ok && u.code; u = *++up) {
         const int total = unit_cnt(u) * u.npan;
-        const int run = unit_g(u) >= 8 ? total : SG_RUN;
         const bool a_real = unit_real(u);
-        for (int done = 0; ok && done < total; done += run, ++f) {
+        for (int done = 0; ok && done < total; done += SG_RUN, ++f) {
           const int ab = f & 1, ph = f >> 1;
-          const int n = min(run, total - done);
+          const int n = min(SG_RUN, total - done);
           if (!mbar_wait(acce0 + 8 * ab, (ph & 1) ^ 1, P.timeout_ns, abort_flag, P.err)) {
             ok = false;
             break;
@@ -517,11 +516,10 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_slice_gemm(const __grid_const
     while (ok && u.code) {
       const SliceUnit nx = *++up;
       const int total = unit_cnt(u) * u.npan;
-      const int run = unit_g(u) >= 8 ? total : SG_RUN;
       int acc[SG_N];
 #pragma unroll
       for (int c = 0; c < SG_N; ++c) acc[c] = 0;
-      for (int done = 0; done < total; done += run, ++f) {
+      for (int done = 0; done < total; done += SG_RUN, ++f) {
         const int ab = f & 1, ph = f >> 1;
         if (leader) s_epi_ok[f & 1] = mbar_wait(accf0 + 8 * ab, ph & 1, P.timeout_ns, abort_flag, P.err) ? 1 : 0;
         asm volatile("bar.sync 1, 256;" ::: "memory");

@@ -19,8 +19,7 @@
 // Exactness: a digit product is at most 2^14, so a run of 512 complex (1024
 //   real) k keeps every partial sum at or below 2^24, which FP32 holds exactly;
 //   the kernel takes the accumulator out after each run and adds the runs as
-//   32-bit integers.  Groups 8 and 9 have weights 2^-64 and 2^-72 and are not cut
-//   into runs: FP32 rounding of their sums stays at the level of the pairs left out.
+//   32-bit integers.
 // Integer sums do not depend on their order: results are the same for every
 // tiling, batch composition and schedule.
 //

@@ -114,3 +114,19 @@ def test_uneven_orbitals_match_oracle(form, kgrid):
                 X = np.stack([c.get_density(t, k) for k in range(len(C))])
                 R = np.stack(ref["D"])
                 assert np.linalg.norm(X - R) / np.linalg.norm(R) <= (1e-4 if split else 1e-10)
+
+
+@pytest.mark.parametrize("planes", [8, 19])
+def test_group_sums_are_exact_where_digits_correlate(planes):
+    """[x | x] [x | -x]^dagger is zero.  Built from digits in [-127, 127], x has these digits and -x their
+    negatives, so every group sum is zero too and the result has to be exactly zero.  The squares of
+    equal digits (the pair (4, 4)) add up to 2 x 2048 x 127 x 128 / 3 = 2.2e7 > 2^24 half way through
+    k = 4096, which FP32 does not hold unless the sums are taken out in time."""
+    rng = np.random.default_rng(17)
+    d = rng.integers(-127, 128, (2, 7, 40, 2048))
+    d[:, 0] = rng.integers(64, 121, (2, 40, 2048))       # row maxima in [1/4, 1/2): every scale is 1
+    d[:, 6] = 4 * rng.integers(-31, 32, (2, 40, 2048))   # 53 bits
+    x = sum(d[:, s].astype(float) * 2.0 ** (-8 * (s + 1)) for s in range(7))
+    x = x[0] + 1j * x[1]
+    c = vgtb.diag_slice_product(np.hstack([x, x]), np.hstack([x, -x]), planes=planes)
+    assert not np.any(c)
