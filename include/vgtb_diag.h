@@ -52,7 +52,8 @@ int vgtb_diag_bounded_wait(long long limit_ns, int which);
 /* The sliced FP64 product of the FP64 propagation: c = a r^dagger for host
  * matrices a [m][k], r [n][k], c [m][n] (complex interleaved), as exact digit
  * products on the tensor cores.  a_real = 1: a's imaginary parts are zero and
- * not read.  planes: 8 or 19 integer planes (the result is the same).
+ * not read.  planes: 8 = one integer plane per group of digit pairs,
+ * 19 = planes of at most two pairs (the result is the same).
  * Errors: E_INVALID, E_NOMEM, E_UNSUPPORTED, E_TIMEOUT, E_CUDA. */
 int vgtb_diag_slice_product(int m, int n, int k, const double* a, const double* r, int a_real, int planes, double* c);
 

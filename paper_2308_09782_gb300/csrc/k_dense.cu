@@ -227,7 +227,7 @@ __device__ __forceinline__ void split_bf16_d(double x, __nv_bfloat16& hi, __nv_b
   lo = __double2bfloat16(x - (double)__bfloat162float(hi));
 }
 
-// MP = 0: X is a matrix; MP = 7 or 2: X is put together from the integer planes of the sliced
+// MP = 0: X is a matrix; MP = 8 or 2: X is put together from the integer planes of the sliced
 // product (slice.cuh), which saves writing and reading X once (134 MB at N = 2048).
 // 16 rows of threads: two elements of each tile per thread, so that few are handled one after the
 // other where the grid leaves room.
@@ -330,8 +330,8 @@ void launch_leap(const LeapItem* items, int n_items, int Np_max, int mp, const i
   const int nt = Np_max / LT;
   dim3 grid(nt * (nt + 1) / 2, n_items);
   dim3 block(LT, LY);
-  if (mp == 7)
-    launch_pdl(k_leap<7>, grid, block, 0, st, items, step, dt, counter, step_rw);
+  if (mp == kSlicePairs)
+    launch_pdl(k_leap<kSlicePairs>, grid, block, 0, st, items, step, dt, counter, step_rw);
   else if (mp == 2)
     launch_pdl(k_leap<2>, grid, block, 0, st, items, step, dt, counter, step_rw);
   else

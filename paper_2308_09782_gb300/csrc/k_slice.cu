@@ -12,13 +12,13 @@ namespace vgtb {
 
 namespace {
 
-// digits of one real number as bytes: byte 8 (7 - s) of the result is d_s + 128 for s = 2..7,
-// the bits from 48 up are d_1 + 128.  efm: exponent field of the row's largest part (at least 1).
+// digits of one real number as bytes: byte 8 - s of the result is d_s + 128 for s = 2..8, and the
+// first byte d_1 itself.  efm: exponent field of the row's scale (slice_field).
 __device__ __forceinline__ unsigned long long slice_bytes(double x, int efm) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int f = (int)((b >> 52) & 0x7ffu);
   unsigned long long m = (b & 0xfffffffffffffull) | (f ? 0x10000000000000ull : 0ull);
-  const int sh = efm - (f ? f : 1) - 2;  // x 2^(56 - e) = m 2^-sh
+  const int sh = efm - (f ? f : 1) - 10;  // x 2^(64 - e) = m 2^-sh, below 2^63 - 2^56
   if (sh <= 0)
     m <<= -sh;
   else
@@ -29,7 +29,7 @@ __device__ __forceinline__ unsigned long long slice_bytes(double x, int efm) {
 
 // float with the value of digit s (1-based) of slice_bytes' result: an exact integer
 __device__ __forceinline__ float slice_digit(unsigned long long w, int s) {
-  const uint32_t b = s == 1 ? (uint32_t)(w >> 48) : (uint32_t)(w >> (8 * (7 - s))) & 0xffu;
+  const uint32_t b = s == 1 ? (uint32_t)(w >> 56) ^ 0x80u : (uint32_t)(w >> (8 * (kSlices - s))) & 0xffu;
   return __uint_as_float(0x4b000000u | b) - 8388736.0f;  // 2^23 + 128
 }
 
@@ -65,7 +65,7 @@ __device__ __forceinline__ void slice_load4(const SlicePlanes& S, long long row,
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int er = col + j < cols ? S.exR[col + j] : 0;
-    k[j] = (ea == kSliceNaN || er == kSliceNaN) ? kSliceNaN : ea + er - 72;
+    k[j] = (ea == kSliceNaN || er == kSliceNaN) ? kSliceNaN : ea + er - kSliceShift;
   }
   double r[4], i[4];
   slice_part4<MP>(p, S.stride, k, r);
@@ -82,7 +82,7 @@ __device__ __forceinline__ void slice_load4(const SlicePlanes& S, long long row,
 
 // One row per TPR threads, four adjacent columns per thread and iteration (IT iterations), the row
 // kept in registers between the search for its largest part and the cut.  Memory bound: at
-// N = 2048 it reads 67 MB (a matrix) or 268 MB (planes) and writes 117 MB of digits.  One
+// N = 2048 it reads 67 MB (a matrix) or 302 MB (planes) and writes 134 MB of digits.  One
 // iteration per thread wherever a CTA can hold the row: with four, 128 threads a row, the 130 to
 // 150 registers left 16 warps an SM and the loads waited (planes, N = 2048: 123 us, now 98).
 template <int TPR, int IT, int MP>
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(TPR > 128 ? TPR : 128)
   }
   if (!live) return;
   const bool bad = mx >= 0x7ff00000u;
-  const int efm = max((int)(mx >> 20), 1);
+  const int efm = slice_field(mx);
   if (t == 0) J.out.ex[row] = bad ? kSliceNaN : efm - 1021;
   const long long ld = 2LL * J.out.Kp, ps = ld * J.out.rows;
 #pragma unroll
@@ -199,8 +199,8 @@ static void launch_rows_mp(const SliceRowJob* jobs, int n_jobs, int max_rows, in
 
 void launch_slice_rows(const SliceRowJob* jobs, int n_jobs, int max_rows, int max_cols, int mp, const int* step,
                        cudaStream_t st) {
-  if (mp == 7)
-    launch_rows_mp<7>(jobs, n_jobs, max_rows, max_cols, step, st);
+  if (mp == kSlicePairs)
+    launch_rows_mp<kSlicePairs>(jobs, n_jobs, max_rows, max_cols, step, st);
   else
     launch_rows_mp<2>(jobs, n_jobs, max_rows, max_cols, step, st);
 }
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(128) k_slice_hamilton(const SliceHamJob* __res
   };
   auto write = [](const SliceMat& out, int r, int c, double2 v, uint32_t mx) {
     const bool bad = mx >= 0x7ff00000u;
-    const int efm = max((int)(mx >> 20), 1);
+    const int efm = slice_field(mx);
     const unsigned long long wr = slice_bytes(bad ? 0.0 : v.x, efm), wi = slice_bytes(bad ? 0.0 : v.y, efm);
     const long long ld = 2LL * out.Kp, pst = ld * out.rows;
     __nv_bfloat16* o = out.dig + (long long)r * ld + c;
@@ -291,8 +291,8 @@ __global__ void __launch_bounds__(128) k_slice_hamilton(const SliceHamJob* __res
   }
   for (int r = threadIdx.x; r < ni; r += blockDim.x) {
     const uint32_t mh = s_rowmax[r], md = s_rowmax[max_orb + r];
-    J.out.ex[oi + r] = mh >= 0x7ff00000u ? kSliceNaN : max((int)(mh >> 20), 1) - 1021;
-    if (delta) J.dout.ex[oi + r] = md >= 0x7ff00000u ? kSliceNaN : max((int)(md >> 20), 1) - 1021;
+    J.out.ex[oi + r] = mh >= 0x7ff00000u ? kSliceNaN : slice_field(mh) - 1021;
+    if (delta) J.dout.ex[oi + r] = md >= 0x7ff00000u ? kSliceNaN : slice_field(md) - 1021;
   }
 }
 
@@ -588,12 +588,15 @@ struct SliceGemm {
 
 int slice_tiles(int M, int N) { return ((M + 2 * BM - 1) / (2 * BM)) * ((N + SG_N - 1) / SG_N); }
 
-// A plane of up to 7 pairs is the longest unit.  With few tiles the 34 pairs of a tile are spread
-// over 19 planes of at most 2 pairs, so that more pairs of SMs get work and no unit is long; the
-// integers to read back grow from 8 to 19 per real part.  Product and read-back with 7 | 2 pairs a
-// plane: 2 tiles (N = 256) 41 | 29 us, 8 tiles (N = 468) 61 | 49 us, 15 tiles (N = 640) 79 | 90 us,
-// 16 tiles (8 x N = 256) 53 | 63 us.
-int slice_pairs_per_plane(long long tiles) { return tiles >= 12 ? 7 : 2; }
+// A plane of a whole group (up to 8 pairs) is the longest unit.  With few tiles the 43 pairs of a tile
+// are spread over 24 planes of at most 2 pairs, so that more pairs of SMs get work and no unit is
+// long; the integers to read back grow from 9 to 24 per real part.  `tiles` counts the tiles of a
+// product, twice where more is read back: delta form (two products make W), Crank-Nicolson (twelve
+// sweeps).  Products and read-back of a step with 8 | 2 pairs a plane, in us: leapfrog 1 tile
+// (N = 116) 70 | 62, 2 (256) 89 | 69, 8 (468) 131 | 121, 8 (512) 121 | 117, 15 (576) 168 | 200,
+// 16 (8 x 256) 137 | 182; delta form 2 x 2 (256) 94 | 79, 2 x 6 (384) 116 | 123, 2 x 8 (512)
+// 140 | 160; Crank-Nicolson 2 x 2 (256) 485 | 315, 2 x 4 (512) 825 | 564, 2 x 8 (8 x 128) 435 | 481.
+int slice_pairs_per_plane(long long tiles) { return tiles >= 12 ? kSlicePairs : 2; }
 
 namespace {
 

@@ -7,15 +7,22 @@
 // Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59, 2012) with a fixed number
 // of slices.
 //
-// Operand row:  x[k] = 2^e sum_{s=1..7} d_s[k] 2^{-8s},  |d_1| <= 128,
-//   d_s in [-128, 127] for s > 1, e from the row's largest part so that
-//   max |x| 2^-e is in [1/4, 1/2): the row is held to 2^-57 of 2^e, 2^-55 of its
-//   largest entry at worst.
-// Product:      C = A R^dagger, C[m][n] = 2^{eA[m] + eR[n]} sum_{g=2..9} 2^{-8g} P_g[m][n],
-//   P_g = sum_{s+t=g} A_s R_t^dagger.  Pairs with s + t > 9 are left out: a term of
-//   theirs is below 2^-66 of 2^{eA + eR}.  (Without group 9, 28 instead of 34 pairs,
-//   products of matrices that decay away from the diagonal came out 1.3e-15 off in the
-//   2-norm at N = 128, against 3.6e-16 for FP64 multiply-adds.)
+// Operand row:  x[k] = 2^e sum_{s=1..8} d_s[k] 2^{-8s},  d_s in [-128, 127],
+//   e from the row's largest part so that max |x| 2^-e is in [1/4, 1/2): the row
+//   is held to 2^-65 of 2^e.  Every entry down to 2^-10 of the row's largest
+//   keeps all of its 53 bits.
+// Product:      C = A R^dagger, C[m][n] = 2^{eA[m] + eR[n]} sum_{g=2..10} 2^{-8g} P_g[m][n],
+//   P_g = sum_{s+t=g} A_s R_t^dagger.  Pairs with s + t > 10 are left out: a term of
+//   theirs is at most 2^-74 of 2^{eA + eR}.
+// Error against 64-bit results, relative in the Frobenius norm | largest over the
+//   elements relative to (|A| |R|)_mn, of the products of 512 silicon atoms:
+//                          D H                    S^-1 W
+//   FP64 multiply-adds     2.3e-16 | 1.0e-15      5.7e-16 | 1.7e-15
+//   7 digits, s + t <= 9   3.7e-16 | 4.1e-14      1.3e-15 | 5.2e-13    (34 pairs)
+//   8 digits, s + t <= 9   5.5e-17 | 1.7e-15      2.6e-16 | 1.3e-13    (36)
+//   8 digits, s + t <= 10  5.2e-17 | 1.5e-16      4.2e-17 | 2.1e-15    (43, this form)
+//   Rows that decay much faster (e^{-0.2 |m - k|} and more over a hundred orbitals) keep
+//   the norm, but not the elements far below their row's scale.
 // Exactness: a digit product is at most 2^14, so a run of 512 complex (1024
 //   real) k keeps every partial sum at or below 2^24, which FP32 holds exactly;
 //   the kernel takes the accumulator out after each run and adds the runs as
@@ -23,17 +30,21 @@
 // Integer sums do not depend on their order: results are the same for every
 // tiling, batch composition and schedule.
 //
-// What bounds it: 34 digit products of 8 N^3 BF16 flops stand in for one FP64
-// product, 34 / 1750 TFLOP/s against 1 / 1.2 TFLOP/s on the FP64 pipe.
+// What bounds it: 43 digit products of 8 N^3 BF16 flops stand in for one FP64
+// product, 43 / 1750 TFLOP/s against 1 / 1.2 TFLOP/s on the FP64 pipe.
 #pragma once
 #include "vgtb_internal.h"
 
 namespace vgtb {
 
-constexpr int kSlices = 7;
-constexpr int kSliceGroups = 8;            // s + t = 2 .. 9
+constexpr int kSlices = 8;
+constexpr int kSliceGroups = 9;            // s + t = 2 .. 10
+constexpr int kSliceShift = 8 * (kSliceGroups + 1);  // the last group's weight is 2^-kSliceShift
+constexpr int kSlicePairs = 8;             // most pairs of a group
 constexpr int kSliceNaN = 1 << 24;         // row exponent of a row with a non-finite entry
-constexpr int kSliceMaxN = 8192;           // 32-bit group sums: 7 pairs x 2 N x 2^14 < 2^31
+// 32-bit group sums: 8 pairs x 2 N x 2^14 = 2^31, which would take 128 for the magnitude of every
+// digit, i.e. -128, and so |x| 2^-e above 1/2
+constexpr int kSliceMaxN = 8192;
 
 // digits of `rows` rows of K complex numbers: dig[s][row][2 Kp], planar [Re | Im], Kp = K rounded up to 64
 struct SliceMat {
@@ -62,41 +73,43 @@ static __device__ __noinline__ double slice_scaled(double m, int k, int q) {
   return k >= kSliceNaN / 2 ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(m, q);
 }
 
-// 2^k (sum over groups of G[g - 2] 2^{72 - 8g}) correctly rounded to FP64 (NaN for k = kSliceNaN)
+// exponent field of a row's scale from the largest high word of its parts: e = field - 1021.  A
+// largest part within 1/64 of the next power of two takes that power's scale, so that the first digit
+// never rounds up to 128.
+__device__ __forceinline__ int slice_field(uint32_t high) { return max((int)((high + 0x4000u) >> 20), 1); }
+
+// 2^k (sum over groups of G[g - 2] 2^{80 - 8g}) correctly rounded to FP64 (NaN for k = kSliceNaN)
 // with integer operations (the FP64 pipe runs at a small fraction of the integer rate).
 __device__ __forceinline__ double slice_value(const int (&G)[kSliceGroups], int k) {
-  // weights relative to the last group: 2^56, 2^48, ..., 2^0
-  long long hi = ((long long)G[0] << 24) + ((long long)G[1] << 16) + ((long long)G[2] << 8) + G[3];  // x 2^32
-  long long lo = ((long long)G[4] << 24) + ((long long)G[5] << 16) + ((long long)G[6] << 8) + G[7];
-  hi += lo >> 32;
-  uint32_t l = (uint32_t)lo;
+  // weights relative to the last group: 2^64, 2^56, ..., 2^0.  The sum as a 128-bit number hi : lo
+  // (|G[4]| has 5 pairs: the second part stays below 2^63)
+  const long long a = ((long long)G[0] << 24) + ((long long)G[1] << 16) + ((long long)G[2] << 8) + G[3];  // x 2^40
+  const long long b = ((long long)G[4] << 32) + ((long long)G[5] << 24) + ((long long)G[6] << 16) +
+                      ((long long)G[7] << 8) + G[8];
+  unsigned long long lo = ((unsigned long long)a << 40) + (unsigned long long)b;
+  long long hi = (a >> 24) + (b >> 63) + (lo < (unsigned long long)b ? 1 : 0);
   const bool neg = hi < 0;
-  if (neg) {  // magnitude of the 96-bit number
-    l = 0u - l;
-    hi = ~hi + (l == 0u ? 1 : 0);
+  if (neg) {  // magnitude
+    lo = 0ull - lo;
+    hi = ~hi + (lo == 0ull ? 1 : 0);
   }
-  unsigned long long top;
-  uint32_t rest = 0;
+  unsigned long long top = lo, rest = 0;
   int len;  // bits of the magnitude
   if (hi == 0) {
-    if (l == 0u) return k >= kSliceNaN / 2 ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
-    const int z = __clz((int)l);
-    top = (unsigned long long)l << (32 + z);
-    len = 32 - z;
+    if (lo == 0ull) return k >= kSliceNaN / 2 ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
+    const int z = __clzll((long long)lo);
+    top = lo << z;
+    len = 64 - z;
   } else {
-    const int z = __clzll(hi);
-    len = 96 - z;
-    if (z < 32) {
-      top = ((unsigned long long)hi << z) | ((unsigned long long)l >> (32 - z));
-      rest = l << z;
-    } else {
-      top = ((unsigned long long)hi << z) | ((unsigned long long)l << (z - 32));
-    }
+    const int z = __clzll(hi);  // hi is below 2^30
+    top = ((unsigned long long)hi << z) | (lo >> (64 - z));
+    rest = lo << z;
+    len = 128 - z;
   }
   // top has its first bit set: value = top 2^(len - 64) (plus the sticky rest)
   unsigned long long m = top >> 11;
   const uint32_t r = ((uint32_t)top & 0x7ffu);
-  const bool up = r > 0x400u || (r == 0x400u && (rest != 0u || (m & 1ull)));
+  const bool up = r > 0x400u || (r == 0x400u && (rest != 0ull || (m & 1ull)));
   m += up ? 1ull : 0ull;  // a carry out of the 53 bits raises the exponent below
   const int ef = 1023 + len - 1 + k;
   if (ef > 0 && ef < 2046) {
@@ -124,7 +137,7 @@ __device__ __forceinline__ double2 slice_load(const SlicePlanes& S, long long ro
     gi[g - 2] = b;
   }
   const int ea = S.exA[row], er = S.exR[col];
-  const int k = (ea == kSliceNaN || er == kSliceNaN) ? kSliceNaN : ea + er - 72;
+  const int k = (ea == kSliceNaN || er == kSliceNaN) ? kSliceNaN : ea + er - kSliceShift;
   return make_double2(slice_value(gr, k), slice_value(gi, k));
 }
 

@@ -33,7 +33,7 @@ namespace {
 
 thread_local std::string g_create_error;
 
-// From kSliceMinN orbitals up the 34 exact digit products on the tensor cores take less time than
+// From kSliceMinN orbitals up the 43 exact digit products on the tensor cores take less time than
 // one product on the FP64 pipe (N = 256, 8 k-points: 1.06 ms for one product on the FP64 pipe);
 // below, a product is a few microseconds of FP64 work and the extra launches cost more.
 constexpr int kSliceMinN = 97;
@@ -145,7 +145,7 @@ struct vgtb_ctx {
   int n_dense = 0;                 // items of the lists above (the others take the sliced products)
   int max_dense = 0, max_dense_occ = 0;  // their largest matrix size and count of occupied states
   std::vector<SliceRound> rounds;  // sliced FP64 products
-  int slice_mp = 7, max_orb = 1;
+  int slice_mp = kSlicePairs, max_orb = 1;
   int* d_slice_err = nullptr;
   // tcgen05 plans
   TcPlan* tc1 = nullptr;
@@ -923,7 +923,7 @@ class SetupProducts {
   vgtb_ctx* ctx;
   const HostSys& h;
   SliceFam fa, fr;
-  int *planes = nullptr, *err = nullptr, mp = 7, nw = 0;
+  int *planes = nullptr, *err = nullptr, mp = kSlicePairs, nw = 0;
   SliceRowJob* dj = nullptr;
   GemmF64Item* dg = nullptr;
   SliceGemm* g = nullptr;
@@ -992,7 +992,7 @@ int finish_density(vgtb_ctx* ctx, int si) {
     TRY(sp.finish());
   }
   if (h.d_jD0) {
-    launch_slice_rows(h.d_jD0, h.nk, h.N, h.N, 7, nullptr, ctx->stream);
+    launch_slice_rows(h.d_jD0, h.nk, h.N, h.N, kSlicePairs, nullptr, ctx->stream);
     CK(cudaGetLastError());
   }
   h.density_set = true;
@@ -1116,7 +1116,7 @@ int slice_sinv(vgtb_ctx* ctx, HostSys& h) {
   for (int k = 0; k < h.nk; ++k) js[k] = slice_row_job(h.Sinv + (size_t)k * h.Np * h.Np, h.Np, h.N, h.N, h.fSinv.mat(k));
   SliceRowJob* dj = nullptr;
   TRY(upload(ctx, &dj, js.data(), js.size()));
-  launch_slice_rows(dj, h.nk, h.N, h.N, 7, nullptr, ctx->stream);
+  launch_slice_rows(dj, h.nk, h.N, h.N, kSlicePairs, nullptr, ctx->stream);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(ctx->stream));  // js leaves scope
   return VGTB_OK;
@@ -1161,7 +1161,7 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
     tiles += (long long)c.cap * slice_tiles(h.N, h.N);
     for (int I = 0; I < h.nat; ++I) ctx->max_orb = std::max(ctx->max_orb, h.orb_off[I + 1] - h.orb_off[I]);
   }
-  ctx->slice_mp = slice_pairs_per_plane(tiles);
+  ctx->slice_mp = slice_pairs_per_plane(ctx->delta ? 2 * tiles : tiles);
   const int np = slice_num_planes(ctx->slice_mp);
   const bool first = ctx->opt.product1 != VGTB_P1_BLOCKS;  // the first product is sliced too
   for (size_t s = 0; s < ctx->sys.size(); ++s) {
@@ -1311,7 +1311,7 @@ int slice_build_cn(vgtb_ctx* ctx) {
     tiles += (long long)c.cap * slice_tiles(h.nocc, h.N);
     for (int I = 0; I < h.nat; ++I) ctx->max_orb = std::max(ctx->max_orb, h.orb_off[I + 1] - h.orb_off[I]);
   }
-  ctx->slice_mp = slice_pairs_per_plane(tiles);
+  ctx->slice_mp = slice_pairs_per_plane(2 * tiles);
   const int np = slice_num_planes(ctx->slice_mp);
   for (size_t s = 0; s < ctx->sys.size(); ++s) {
     if (items[s].empty()) continue;

@@ -195,10 +195,10 @@ extern "C" int vgtb_diag_bounded_wait(long long limit_ns, int which) {
 extern "C" int vgtb_diag_slice_product(int m, int n, int k, const double* a, const double* r, int a_real, int planes,
                                        double* c) {
   if (m < 1 || n < 1 || k < 1 || std::max(m, std::max(n, k)) > kSliceMaxN || !a || !r || !c ||
-      (planes != slice_num_planes(7) && planes != slice_num_planes(2)))
+      (planes != 8 && planes != 19))
     return VGTB_E_INVALID;
   if (!tc_gemm_supported()) return VGTB_E_UNSUPPORTED;
-  const int mp = planes == slice_num_planes(7) ? 7 : 2, nw = slice_nw(n), kp = slice_kp(k);
+  const int mp = planes == 8 ? kSlicePairs : 2, np = slice_num_planes(mp), nw = slice_nw(n), kp = slice_kp(k);
   Scratch sc;
   double2* ad = sc.get<double2>((size_t)m * k);
   double2* rd = sc.get<double2>((size_t)n * k);
@@ -213,7 +213,7 @@ extern "C" int vgtb_diag_slice_product(int m, int n, int k, const double* a, con
   fr.dig = sc.get<__nv_bfloat16>((size_t)kSlices * n * 2 * kp);
   fa.ex = sc.get<int>(m);
   fr.ex = sc.get<int>(n);
-  int* pl = sc.get<int>((size_t)planes * m * 2 * nw);
+  int* pl = sc.get<int>((size_t)np * m * 2 * nw);
   int* err = sc.get<int>(1);
   SliceRowJob* dj = sc.get<SliceRowJob>(3);
   if (!ad || !rd || !cd || !fa.dig || !fr.dig || !fa.ex || !fr.ex || !pl || !err || !dj) return VGTB_E_NOMEM;

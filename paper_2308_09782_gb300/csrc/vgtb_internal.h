@@ -343,7 +343,7 @@ struct LeapItem {
   int mode;                // 0 = leapfrog, 1 = write the derivative only into out
   double2* out;            // mode 1 target
 };
-// mp: 0 = X is a matrix, else X comes from planes of at most mp pairs (7 or 2);
+// mp: 0 = X is a matrix, else X comes from planes of at most mp pairs (8 or 2);
 // counter may be null: the step counter is then left alone
 void launch_leap(const LeapItem* items, int n_items, int Np_max, int mp, const int* step, double dt,
                  int* counter, int* step_rw, cudaStream_t st);

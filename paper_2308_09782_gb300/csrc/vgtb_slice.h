@@ -24,7 +24,7 @@ struct SliceRowJob {
   int ldd;
   SliceMat out;            // digits wanted when out.dig != null
 };
-// mp: pairs per plane of the sources (7 or 2)
+// mp: pairs per plane of the sources (8 or 2)
 void launch_slice_rows(const SliceRowJob* jobs, int n_jobs, int max_rows, int max_cols, int mp, const int* step,
                        cudaStream_t st);
 
@@ -72,7 +72,7 @@ struct SliceProd {
 };
 
 struct SliceGemm;
-int slice_pairs_per_plane(long long tiles);  // 7, or 2 when 7 planes of work leave the chip idle
+int slice_pairs_per_plane(long long tiles);  // 8, or 2 when few units of whole groups leave the chip idle
 int slice_tiles(int M, int N);
 int slice_gemm_create(const std::vector<SliceFam>& fams, const std::vector<SliceProd>& prods,
                       const std::vector<SlicePattern>& patterns, int mp, long long timeout_ns, int* err,
@@ -82,6 +82,6 @@ int slice_gemm_launch(SliceGemm* g, cudaStream_t st);
 void slice_gemm_destroy(SliceGemm* g);
 inline int slice_kp(int K) { return (K + 63) / 64 * 64; }
 inline int slice_nw(int N) { return (N + 31) / 32 * 32; }
-inline int slice_num_planes(int mp) { return mp == 7 ? slice_planes<7>() : slice_planes<2>(); }
+inline int slice_num_planes(int mp) { return mp == kSlicePairs ? slice_planes<kSlicePairs>() : slice_planes<2>(); }
 
 }  // namespace vgtb

@@ -130,3 +130,25 @@ def test_group_sums_are_exact_where_digits_correlate(planes):
     x = x[0] + 1j * x[1]
     c = vgtb.diag_slice_product(np.hstack([x, x]), np.hstack([x, -x]), planes=planes)
     assert not np.any(c)
+
+
+@pytest.mark.parametrize("shape", [(40, 33, 96), (257, 129, 513)])
+@pytest.mark.parametrize("fall", [0.0, 0.05])
+def test_slice_product_holds_more_than_fp64_rows(shape, fall):
+    """Eight digits: with 2^e <= 4.07 of the row's largest part (slice_field) an entry is off by at most
+    2^-65 2^e, a real product by 1.02 x 2^-62 of the row maxima, and the pairs left out (s + t > 10, at
+    most 6.1 x 2^14 2^-88 of 2^eA 2^eR) add 2^-67: |error| <= 2^-53 |c| + 2 k 1.1 x 2^-62 max|a_row| max|r_row|,
+    also for the elements that rows falling off from the diagonal make small."""
+    if np.finfo(np.longdouble).nmant < 100:
+        pytest.skip("the reference needs a 128-bit long double")
+    m, n, k = shape
+    rng = np.random.default_rng(m + k)
+    a, r = ((rng.normal(size=(q, k)) + 1j * rng.normal(size=(q, k)))
+            * np.exp(-fall * np.abs(np.arange(q)[:, None] - np.arange(k)[None])) for q in (m, n))
+    e = a.astype(np.clongdouble) @ r.conj().T.astype(np.clongdouble)
+    part = lambda x: np.maximum(np.abs(x.real), np.abs(x.imag))  # noqa: E731
+    scale = part(a).max(1)[:, None] * part(r).max(1)[None]
+    for planes in (8, 19):
+        d = vgtb.diag_slice_product(a, r, planes=planes).astype(np.clongdouble) - e
+        for got, val in ((d.real, e.real), (d.imag, e.imag)):
+            assert np.all(np.abs(got) <= 2.0 ** -53 * np.abs(val) * (1 + 2.0 ** -40) + 2.2 * k * 2.0 ** -62 * scale)
