@@ -54,8 +54,11 @@ extern "C" {
 
 /* precision forms of the commutator products */
 #define VGTB_FP64          0   /* complex FP64 everywhere (Eq. 6 evaluated directly); from 97 orbitals
-                                  up the products run as exact digit products on the tensor cores,
-                                  no further off than FP64 multiply-adds in the norm of a product */
+                                  up the products run as exact digit products on the tensor cores, whose
+                                  operands are held to 2^-62 of their row's largest entry: closer to the
+                                  64-bit result than FP64 multiply-adds in the norm of a product.  With
+                                  product1 = DENSE or BLOCKS every product is made of FP64 multiply-adds,
+                                  which hold every entry to its own scale */
 #define VGTB_SPLIT_BF16X3  1   /* delta form, tcgen05 BF16 hi/lo 3-product GEMMs, FP32 accumulate */
 
 #define VGTB_INIT_GROUND   0   /* create() computes the SCC ground state D_k(0) */
@@ -117,17 +120,20 @@ typedef struct {
   int tile_variant[2];      /* split form: tile variant of product 1 / product 2 (see
                                vgtb_tile_config; -1 = variant 0, or the autotuner's choice) */
   int product1;             /* form of the first product W = D H of Eq. 6 (VGTB_P1_*):
-                               AUTO (0, default): the FP64 path skips the 64-wide k-panels in which
-                               a tile's rows of H_k are zero, or below 97 orbitals runs it
-                               block-sparse (below), as does the Crank-Nicolson integrator its
-                               product M = S^-1 H; the split form runs the tcgen05 GEMM and skips the 64-wide k-panels in
-                               which a tile's rows of H_k are zero;
+                               AUTO (0, default): the FP64 path and the Crank-Nicolson integrator (whose
+                               M = S^-1 H this option names) run digit products on the tensor cores from
+                               97 orbitals up and skip the 64-wide k-panels in which a tile's rows of
+                               H_k are zero; up to 96 orbitals FP64 multiply-adds over all of H_k; where
+                               the digits do not fit in a quarter of the free device memory (32 GB at
+                               most), or above 8192 orbitals, block-sparse FP64 (below) if every atom
+                               carries 4 orbitals, else dense.  The split form runs the tcgen05 GEMM and
+                               skips the k-panels in the same way;
                                DENSE: a dense product over all of H_k (8 N^3 flops, no panel
-                               skipped); BLOCKS: block-sparse over the
-                               nonzero atom blocks of H_k on the CUDA cores (8 nnz(H) N flops;
-                               FP64, or FP32 in the split form), which needs every atom to carry
-                               4 orbitals (the FP64 AUTO falls back to DENSE otherwise, BLOCKS
-                               fails with E_UNSUPPORTED) */
+                               skipped), in FP64 with multiply-adds in both products; BLOCKS:
+                               block-sparse over the nonzero atom blocks of H_k on the CUDA cores
+                               (8 nnz(H) N flops; FP64, with the second product in FP64
+                               multiply-adds too, or FP32 in the split form), which needs every atom
+                               to carry 4 orbitals (else E_UNSUPPORTED) */
   int scc;                  /* VGTB_SCC_ON (0, default): the shift eps = gamma dq of Eq. 10 follows
                                the charges at every step; VGTB_SCC_FROZEN: H keeps the shift of
                                D_k(0) at every step (non-self-consistent propagation); charges,

@@ -95,11 +95,11 @@ struct HostTraj {
 
 // One round of the sliced FP64 products: as many items as share the digit and plane scratch.
 struct SliceRound {
-  SliceGemm* g1 = nullptr;     // W (null: the first product runs block-sparse)
+  SliceGemm* g1 = nullptr;     // W
   SliceGemm* g2 = nullptr;     // X
   SliceRowJob* jD = nullptr;   // D (dD) to digits
   SliceHamJob* jH = nullptr;   // H, and in the delta form dH, to digits
-  SliceRowJob* jW = nullptr;   // planes (or matrix) of W to digits
+  SliceRowJob* jW = nullptr;   // planes of W to digits
   LeapItem* leap = nullptr;
   int n = 0, max_N = 0, max_Np = 0, max_nat = 0;
   // Crank-Nicolson: D = 2 C C^dagger, M = S^-1 H (g2), the sweeps Y^dagger M^dagger (g1)
@@ -855,6 +855,7 @@ class SetupProducts {
   int init() {
     TRY(alloc(&dg, 1));
     if (h.N < kSliceMinN || h.N > kSliceMaxN || !tc_gemm_supported()) return VGTB_OK;
+    if (!ctx->split && ctx->opt.product1 != VGTB_P1_AUTO) return VGTB_OK;  // as slice_choose
     const size_t held = mem.size();
     fa.rows = fa.K = h.N;
     fa.Kp = slice_kp(h.N);
@@ -1084,11 +1085,11 @@ double slice_budget() {
   return std::min(0.25 * (double)fr, 32e9);
 }
 
-// Which systems take the sliced products: FP64 leapfrog, enough orbitals, and room for the
-// scratch of one item of every such system within the budget.
+// Which systems take the sliced products: FP64, enough orbitals, and room for the scratch of one item
+// of every such system within the budget.  An explicit product1 keeps both products on the FP64 pipe:
+// the digit products hold an operand to its row's scale, multiply-adds hold every entry to its own.
 void slice_choose(vgtb_ctx* ctx) {
-  // an explicit block-sparse product keeps its kernel (Crank-Nicolson: and all that goes with it)
-  if (ctx->split || !tc_gemm_supported() || (ctx->cn && ctx->opt.product1 == VGTB_P1_BLOCKS)) return;
+  if (ctx->split || ctx->opt.product1 != VGTB_P1_AUTO || !tc_gemm_supported()) return;
   const double budget = slice_budget();
   double one = 0.0;
   for (auto& h : ctx->sys) {
@@ -1163,14 +1164,13 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
   }
   ctx->slice_mp = slice_pairs_per_plane(ctx->delta ? 2 * tiles : tiles);
   const int np = slice_num_planes(ctx->slice_mp);
-  const bool first = ctx->opt.product1 != VGTB_P1_BLOCKS;  // the first product is sliced too
   for (size_t s = 0; s < ctx->sys.size(); ++s) {
     if (items[s].empty()) continue;
     HostSys& h = ctx->sys[s];
     SysScratch& c = sc[s];
     const int nw = slice_nw(h.N);
     TRY(slice_sinv(ctx, h));
-    if (ctx->delta && first) {
+    if (ctx->delta) {
       TRY(slice_family(ctx, h.fD0, h.N, h.N, h.nk));
       std::vector<SliceRowJob> j0(h.nk);
       for (int k = 0; k < h.nk; ++k) j0[k] = slice_row_job(h.D0 + (size_t)k * h.Np * h.Np, h.Np, h.N, h.N, h.fD0.mat(k));
@@ -1179,33 +1179,29 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
     }
     TRY(slice_family(ctx, c.D, h.N, h.N, c.cap));
     TRY(dalloc(ctx, &c.exW, (size_t)c.cap * h.N));
-    if (first) TRY(slice_family(ctx, c.H, h.N, h.N, c.cap));
-    if (first && ctx->delta) TRY(slice_family(ctx, c.dH, h.N, h.N, c.cap));
+    TRY(slice_family(ctx, c.H, h.N, h.N, c.cap));
+    if (ctx->delta) TRY(slice_family(ctx, c.dH, h.N, h.N, c.cap));
     const size_t psz = (size_t)c.cap * np * h.N * 2 * nw;
     TRY(dalloc(ctx, &c.planes[0], psz));
-    if (first && ctx->delta) TRY(dalloc(ctx, &c.planes[1], psz));
+    if (ctx->delta) TRY(dalloc(ctx, &c.planes[1], psz));
     c.fS = (int)fams.size();
     fams.push_back(h.fSinv);
     c.fW = (int)fams.size();  // the digits of W take the place of D's (dead once W is known)
     SliceFam w = c.D;
     w.ex = c.exW;
     fams.push_back(w);
-    if (first) {
-      c.fD = (int)fams.size();
-      fams.push_back(c.D);
-      c.fH = (int)fams.size();
-      fams.push_back(c.H);
-      if (ctx->delta) {
-        c.fD0 = (int)fams.size();
-        fams.push_back(h.fD0);
-        c.fdH = (int)fams.size();
-        fams.push_back(c.dH);
-      }
-      if (ctx->opt.product1 != VGTB_P1_DENSE) {
-        c.pat = (int)pats.size();
-        pats.push_back(slice_pattern(h));
-      }
+    c.fD = (int)fams.size();
+    fams.push_back(c.D);
+    c.fH = (int)fams.size();
+    fams.push_back(c.H);
+    if (ctx->delta) {
+      c.fD0 = (int)fams.size();
+      fams.push_back(h.fD0);
+      c.fdH = (int)fams.size();
+      fams.push_back(c.dH);
     }
+    c.pat = (int)pats.size();
+    pats.push_back(slice_pattern(h));
   }
   const long long tmo = std::max(ctx->opt.timeout_ns, 2000000000LL);
   for (size_t r = 0; r < n_rounds; ++r) {
@@ -1230,29 +1226,24 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
         for (int q = 0; q < 2; ++q) pl[q] = c.planes[q] ? c.planes[q] + (size_t)b * np * h.N * 2 * nw : nullptr;
         SliceRowJob w{};
         w.rows = w.cols = h.N;
-        if (first) {
-          SliceRowJob d = slice_row_job(it.D[0], h.Np, h.N, h.N, c.D.mat(b));
-          d.src_par = (long long)NN;
-          jD.push_back(d);
-          SliceHamJob hj{};
-          hj.sys = it.sys;
-          hj.traj = it.traj;
-          hj.k = it.k;
-          hj.el_J = h.d_el_J;
-          hj.out = c.H.mat(b);
-          if (ctx->delta) hj.dout = c.dH.mat(b);
-          jH.push_back(hj);
-          p1.push_back(SliceProd{c.fD, b, c.fH, b, pl[0], nw, false, c.pat});
-          w.n_planes = 1;
-          w.pl[0] = SlicePlanes{pl[0], (long long)h.N * 2 * nw, nw, d.out.ex, hj.out.ex};
-          if (ctx->delta) {
-            p1.push_back(SliceProd{c.fD0, it.k, c.fdH, b, pl[1], nw, false, c.pat});
-            w.n_planes = 2;
-            w.pl[1] = SlicePlanes{pl[1], (long long)h.N * 2 * nw, nw, h.fD0.mat(it.k).ex, hj.dout.ex};
-          }
-        } else {
-          w.src = it.W;
-          w.lds = h.Np;
+        SliceRowJob d = slice_row_job(it.D[0], h.Np, h.N, h.N, c.D.mat(b));
+        d.src_par = (long long)NN;
+        jD.push_back(d);
+        SliceHamJob hj{};
+        hj.sys = it.sys;
+        hj.traj = it.traj;
+        hj.k = it.k;
+        hj.el_J = h.d_el_J;
+        hj.out = c.H.mat(b);
+        if (ctx->delta) hj.dout = c.dH.mat(b);
+        jH.push_back(hj);
+        p1.push_back(SliceProd{c.fD, b, c.fH, b, pl[0], nw, false, c.pat});
+        w.n_planes = 1;
+        w.pl[0] = SlicePlanes{pl[0], (long long)h.N * 2 * nw, nw, d.out.ex, hj.out.ex};
+        if (ctx->delta) {
+          p1.push_back(SliceProd{c.fD0, it.k, c.fdH, b, pl[1], nw, false, c.pat});
+          w.n_planes = 2;
+          w.pl[1] = SlicePlanes{pl[1], (long long)h.N * 2 * nw, nw, h.fD0.mat(it.k).ex, hj.dout.ex};
         }
         w.out = c.D.mat(b);
         w.out.ex = c.exW + (size_t)b * h.N;
@@ -1267,11 +1258,11 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
     std::string msg;
     ctx->rounds.push_back(R);
     SliceRound& Q = ctx->rounds.back();
-    if ((first && slice_gemm_create(fams, p1, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g1, &msg)) ||
+    if (slice_gemm_create(fams, p1, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g1, &msg) ||
         slice_gemm_create(fams, p2, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g2, &msg))
       return fail(ctx, VGTB_E_CUDA, "sliced product plan: %s", msg.c_str());
-    if (first) TRY(upload(ctx, &Q.jD, jD.data(), jD.size()));
-    if (first) TRY(upload(ctx, &Q.jH, jH.data(), jH.size()));
+    TRY(upload(ctx, &Q.jD, jD.data(), jD.size()));
+    TRY(upload(ctx, &Q.jH, jH.data(), jH.size()));
     TRY(upload(ctx, &Q.jW, jW.data(), jW.size()));
     TRY(upload(ctx, &Q.leap, lv.data(), lv.size()));
     CK(cudaStreamSynchronize(ctx->stream));  // the lists leave scope
@@ -1338,10 +1329,8 @@ int slice_build_cn(vgtb_ctx* ctx) {
       *p.first = (int)fams.size();
       fams.push_back(*p.second);
     }
-    if (ctx->opt.product1 != VGTB_P1_DENSE) {
-      c.pat = (int)pats.size();
-      pats.push_back(slice_pattern(h));
-    }
+    c.pat = (int)pats.size();
+    pats.push_back(slice_pattern(h));
   }
   const long long tmo = std::max(ctx->opt.timeout_ns, 2000000000LL);
   for (size_t r = 0; r < n_rounds; ++r) {
@@ -1608,9 +1597,8 @@ void launch_obs_scc(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag, int stride,
 }
 
 // W = D H of a round: digits of D (and of H, which the first round has had in the phase build's place),
-// the digit products (block-sparse first product: W is there already)
+// the digit products
 int launch_slice_first(vgtb_ctx* ctx, const SliceRound& r, cudaStream_t st) {
-  if (!r.g1) return VGTB_OK;
   if (&r != &ctx->rounds.front()) launch_slice_h(ctx, r, st);
   launch_slice_rows(r.jD, r.n, r.max_N, r.max_N, ctx->slice_mp, ctx->d_step, st);
   if (slice_gemm_launch(r.g1, st)) return fail(ctx, VGTB_E_CUDA, "sliced product 1 launch failed");
@@ -1644,7 +1632,7 @@ int enqueue_step(vgtb_ctx* ctx, cudaEvent_t* ev) {
   else if (ctx->n_dense || ctx->n_bsr)
     launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk, ctx->d_step,
                  ctx->delta ? PH_FP64_DELTA : PH_FP64_PLAIN, -1, st);
-  if (!ctx->rounds.empty() && ctx->rounds.front().g1) launch_slice_h(ctx, ctx->rounds.front(), st);
+  if (!ctx->rounds.empty()) launch_slice_h(ctx, ctx->rounds.front(), st);
   if (ev) CK(cudaEventRecordWithFlags(ev[3], st, evflag));
   if (ctx->bsr && ctx->n_bsr > 0)
     launch_bsr(ctx->d_bsr, ctx->d_bsrsys, ctx->n_bsr, ctx->bsr_units_max, ctx->bsr_units_total, ctx->d_bsr_u0,
@@ -1970,7 +1958,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
         if ((rc = dalloc(ctx, &it.Y[0], nc))) return bail(rc);
         if ((rc = dalloc(ctx, &it.Y[1], nc))) return bail(rc);
       } else {
-        if (h.slice && ctx->opt.product1 != VGTB_P1_BLOCKS) {
+        if (h.slice) {
           // H (and dH) go straight to digits
         } else if (ctx->bsr) {
           double2 *kh = nullptr, *kdh = nullptr;
@@ -1982,10 +1970,10 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
           if ((rc = dalloc(ctx, &it.H, NN))) return bail(rc);
           if (ctx->delta && (rc = dalloc(ctx, &it.dH, NN))) return bail(rc);
         }
-        if (!h.slice || ctx->opt.product1 == VGTB_P1_BLOCKS)
+        if (!h.slice) {
           if ((rc = dalloc(ctx, &it.W, NN))) return bail(rc);
-        if (!h.slice)
           if ((rc = dalloc(ctx, &it.X, NN))) return bail(rc);
+        }
       }
       ctx->items_h.push_back(it);
     }
@@ -2085,7 +2073,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     std::vector<int> u0(1, 0);
     for (int i = 0; i < ctx->n_items; ++i) {
       const DevItem& it = ctx->items_h[i];
-      if (ctx->sys[it.sys].slice && (ctx->cn || ctx->opt.product1 != VGTB_P1_BLOCKS)) continue;
+      if (ctx->sys[it.sys].slice) continue;
       const HostSys& h = ctx->sys[it.sys];
       const size_t NN = (size_t)h.Np * h.Np;
       BsrItem b{};

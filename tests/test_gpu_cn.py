@@ -224,3 +224,18 @@ def test_cn_density_after_set_state_is_the_restored_level(atoms):
         fresh.set_field(0, A)
         fresh.set_state(state)
         check(fresh)
+
+
+@pytest.mark.parametrize("name,n", [("si8_pulse", 60), ("si64_pulse", 20)])
+def test_cn_block_sparse_m_matches_oracle(name, n):
+    """product1 = BLOCKS: M = S^-1 H over H's nonzero atom blocks and D at H's pattern, in FP64."""
+    from paper_2308_09782_gb300 import vgtb
+    sysd, A, _ = system(name)
+    ctx, gs = oracle_ground(name)
+    ref = cn.propagate_cn(sysd, A[:n + 1], n, gs["C"], ctx=ctx)
+    with _cn_ctx(sysd, gs["C"], product1=vgtb.P1_BLOCKS) as c:
+        c.set_field(0, A[:n + 1])
+        c.propagate(n)
+        _, _, _, Cs = _compare(c, ref, sysd, gs["C"][0].shape[1])
+        # the read-out forms the whole D
+        assert np.abs(c.get_density(0, 1) - 2.0 * (Cs[1] @ Cs[1].conj().T)).max() <= 1e-13

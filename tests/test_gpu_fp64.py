@@ -237,3 +237,44 @@ def test_frozen_scc_shift_matches_oracle(precision):
         assert np.abs(q - ref["q"]).max() <= 1e-10
     else:
         assert err_j <= 1e-4
+
+
+@pytest.mark.parametrize("product1", [1, 2])
+def test_explicit_product_forms_hold_every_element_to_its_own_scale(product1):
+    """product1 = DENSE or BLOCKS runs FP64 multiply-adds in both products.  Atoms coupled by blocks of
+    1e-30 and S = 1: the density between atoms is of that size, in rows whose diagonal is of order one.
+    Every element is a sum of a few terms of like size, so it agrees with the oracle to 1e-12 of itself
+    (elements that cancel: to 1e-44, 1e-14 of the coupling)."""
+    sysd, _, _ = system("si64_pulse")
+    off, ijl = np.asarray(sysd["orb_offset"]), np.asarray(sysd["blk_ijl"])
+    onsite = np.repeat((ijl[:, 0] == ijl[:, 1]) & ~ijl[:, 2:].any(1), 16)
+    one = np.tile(np.eye(4).ravel(), len(ijl)) * onsite
+    weak = {**sysd, "s": one, "h0": np.where(onsite, sysd["h0"], 1e-30 * np.asarray(sysd["h0"])),
+            "ds": np.zeros_like(sysd["ds"]), "gamma": np.zeros_like(sysd["gamma"]), "kpt": np.zeros((1, 3)),
+            "wk": np.ones(1)}
+    n, N = 3, off[-1]
+    D0 = np.diag(np.tile([2.0, 2 / 3, 2 / 3, 2 / 3], 64)).astype(complex)
+    A = np.zeros((n + 1, 3))
+    ref = O.propagate(weak, A, n, [D0], ctx=O.setup(weak))["D"][0]
+    from paper_2308_09782_gb300 import vgtb
+    with vgtb.Context(weak, precision=vgtb.FP64, init=vgtb.INIT_USER, product1=product1) as c:
+        c.set_density(0, 0, D0)
+        c.set_field(0, A)
+        c.propagate(n)
+        D = c.get_density(0, 0)
+    small = np.abs(ref)[~np.eye(N, dtype=bool)]
+    assert 1e-34 < small.max() < 1e-28
+    assert np.all(np.abs(D - ref) <= 1e-12 * np.abs(ref) + 1e-44)
+
+
+@pytest.mark.parametrize("delta", [0, 1])
+@pytest.mark.parametrize("name,nsteps", [("si8_pulse", 100), ("si64_pulse", 60)])
+def test_block_sparse_fp64_product_matches_oracle(name, nsteps, delta):
+    """product1 = BLOCKS: W = D H (delta form: dD H + D0 dH) over H's nonzero atom blocks in FP64."""
+    ref = oracle_run(name, nsteps)
+    with gpu_run(name, nsteps, product1=2, delta_form=delta) as c:
+        J, E, q = c.observables(0)
+        D = [c.get_density(0, k) for k in range(8)]
+    assert rel_fro(D, ref["D"]) <= 1e-10
+    assert rel_fro([J], [ref["J"]]) <= 1e-8
+    assert np.abs(q - ref["q"]).max() <= 1e-10
