@@ -31,24 +31,28 @@ __global__ void __launch_bounds__(kSpecThreads) k_conductivity(const double* __r
                                                                double* eps) {
   // Level m = n - n0 = 256 a + b: e^{iwt} e^{-t/tau0} is the product of a factor of b, kept by thread
   // b, and one of a, made for 256 rows at a time, so a level costs four multiplications instead of a
-  // sincos and an exp on the FP64 pipe, which bound this kernel (1201 levels: 5 + 5 calls a thread,
-  // now 2 + 2; 5001 levels: 20 + 20, now 2 + 2).
+  // sincos and an exp on the FP64 pipe, which bound this kernel (400 frequencies, 1201 levels, both
+  // read-out calls of a pass: 166 us with 5 + 5 calls a thread, 127 with 2 + 2).  256 levels share a
+  // factor and with it the rounding of its phase, so the phase is taken without: the remainders of
+  // m dt and of w t turn the sine and cosine by what the two products rounded off.
   __shared__ double sh[kSpecThreads];
   __shared__ double2 sf[kSpecThreads];
   const double w = omega[blockIdx.x];
-  auto factor = [&](double t) {
+  auto factor = [&](double m) {
+    const double t = m * dt, p = w * t;
+    const double r = fma(w, fma(m, dt, -t), fma(w, t, -p));
     double s, c;
-    sincos(w * t, &s, &c);
+    sincos(p, &s, &c);
     const double f = exp(-t / tau0);
-    return make_double2(f * c, f * s);
+    return make_double2(f * fma(-r, s, c), f * fma(r, c, s));
   };
-  const double2 fb = factor(threadIdx.x * dt);
+  const double2 fb = factor((double)threadIdx.x);
   double acc[6] = {0, 0, 0, 0, 0, 0};  // (re, im) for x, y, z
   const int rows = (n1 - n0) / kSpecThreads + 1;
   for (int m = threadIdx.x, a = 0; a < rows; m += kSpecThreads, ++a) {
     if (a % kSpecThreads == 0) {
       __syncthreads();
-      if (a + threadIdx.x < rows) sf[threadIdx.x] = factor((double)(a + threadIdx.x) * kSpecThreads * dt);
+      if (a + threadIdx.x < rows) sf[threadIdx.x] = factor((double)(a + threadIdx.x) * kSpecThreads);
       __syncthreads();
     }
     const int n = n0 + m;

@@ -99,3 +99,34 @@ def test_laser_sweep_coordination_charge_transfer_matches_oracle():
         assert np.abs(got[tr] - ref).max() <= 1e-10
         moved.append(np.abs(ref).max())
     assert min(moved) > 1e-7                          # every pulse moved charge
+
+
+def test_spectrum_takes_the_phases_without_rounding():
+    """Every level's weight is e^{i w t} e^{-t/tau0} at the exact product w n dt.  Against the same sum over the
+    device's own J with phases reduced in rational arithmetic: a sine or cosine is off by at most 2 ulp and
+    an exp by 1 in either factor (12 x 2^-53), their product and those with J and the trapezoid weight round
+    6 times, and 5 + 5 + 8 additions follow; here the reduced phase, cosine, exp and products make at most
+    12: below 48 x 2^-53 of the sum of |terms|, 64 allowed.  (Phases rounded as w t are off by up to
+    1e6 x 2^-53 at the highest frequency.)"""
+    from fractions import Fraction
+    from paper_2308_09782_gb300 import vgtb
+    sysd, _, _ = system("si8_pulse")
+    _, gs = oracle_ground("si8_pulse")
+    n, a0, tau0 = 1200, 0.001, 200.0
+    w = [0.05, 0.4, 373.0, 1207.0, 4001.0]
+    with vgtb.Context(sysd, init=vgtb.INIT_USER) as c:
+        for k, D in enumerate(gs["D"]):
+            c.set_density(0, k, D)
+        c.set_field(0, inputs.kick_field(n, a0))
+        c.propagate(n)
+        J, _, _ = c.observables(0)
+        s, _ = c.spectrum(0, 1.0, np.array(w), tau0=tau0)
+    turn = Fraction("6.283185307179586476925286766559005768394338798750211641949889")
+    f = np.full(n + 1, sysd["dt"])
+    f[[0, -1]] *= 0.5
+    term = (f * np.exp(-np.arange(n + 1) * sysd["dt"] / tau0))[:, None] * J
+    size = 64 * 2.0 ** -53 * np.abs(term).sum(0)
+    for i, wi in enumerate(w):
+        x = np.array([float(Fraction(wi) * Fraction(float(sysd["dt"])) * m % turn) for m in range(n + 1)])[:, None]
+        assert np.all(np.abs(s[i].real - (np.cos(x) * term).astype(np.longdouble).sum(0)) <= size), wi
+        assert np.all(np.abs(s[i].imag - (np.sin(x) * term).astype(np.longdouble).sum(0)) <= size), wi
