@@ -106,7 +106,9 @@ typedef struct {
                                dD/dt = R0 - i[S^-1(H dD + dH D0) - h.c.] (same result as Eq. 6) */
   int init;                 /* VGTB_INIT_GROUND or VGTB_INIT_USER */
   void* cuda_stream;        /* cudaStream_t to enqueue on; NULL = the context creates one */
-  long long timeout_ns;     /* limit of every device-side wait (0 = 2e9 ns) */
+  long long timeout_ns;     /* limit of every device-side wait (0 = 2e9 ns): E_TIMEOUT from
+                               vgtb_propagate until a field, a start or a state is set; a set-up product
+                               that runs into it is made with FP64 multiply-adds instead */
   int obs_stride;           /* charges q(t_n) are stored every obs_stride steps (0 = 1) */
   int graph_steps;          /* steps captured per CUDA graph replay (0 = 32; 1 = no graph) */
   int autotune;             /* 1 = time the GEMM tile candidates at create and keep the fastest */

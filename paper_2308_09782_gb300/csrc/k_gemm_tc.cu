@@ -505,6 +505,7 @@ static int build_one(const std::vector<TcSysView>& sys, const std::vector<DevIte
     }
     cudaMemsetAsync(plan->d_flags, 0, sizeof(int) * nsm, stream);
     plan->P.ws = plan->d_ws;
+    plan->n_flags = nsm;
     plan->P.flags = plan->d_flags;
   }
   // the host tables leave scope
@@ -649,7 +650,9 @@ void tc_destroy_plan(TcPlan* p) {
 int tc_plan_variant(const TcPlan* p) { return p ? p->variant : -1; }
 
 void tc_clear_error(TcPlan* p, cudaStream_t st) {
-  if (p) cudaMemsetAsync(p->d_err, 0, sizeof(int), st);
+  if (!p) return;
+  cudaMemsetAsync(p->d_err, 0, sizeof(int), st);
+  if (p->d_flags) cudaMemsetAsync(p->d_flags, 0, sizeof(int) * p->n_flags, st);
 }
 
 int tc_plan_info(const TcPlan* p, int* out4) {

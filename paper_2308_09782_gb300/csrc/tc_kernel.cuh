@@ -102,7 +102,7 @@ struct TcPlan {
   short* d_kidx = nullptr;
   int* d_tord = nullptr;
   int* d_cofs = nullptr;    // planned column tiles of every system
-  int grid = 0, smem = 0, variant = 0, epi = 0, wmax = 0;
+  int grid = 0, smem = 0, variant = 0, epi = 0, wmax = 0, n_flags = 0;
   bool skip = false;
   // host copies for the chained schedule: the problem table, every system's
   // column-tile starts and the modelled time of every tile

@@ -147,6 +147,7 @@ struct vgtb_ctx {
   std::vector<SliceRound> rounds;  // sliced FP64 products
   int slice_mp = kSlicePairs, max_orb = 1;
   int* d_slice_err = nullptr;
+  bool expired = false;            // a product's wait ran out: its error words are still set
   // tcgen05 plans
   TcPlan* tc1 = nullptr;
   TcPlan* tc2 = nullptr;
@@ -867,8 +868,8 @@ class SetupProducts {
     std::string msg;
     if (alloc(&fa.dig, dig) || alloc(&fr.dig, dig) || alloc(&fa.ex, h.N) || alloc(&fr.ex, h.N) ||
         alloc(&planes, (size_t)slice_num_planes(mp) * h.N * 2 * nw) || alloc(&dj, 3) || alloc(&err, 1) ||
-        slice_gemm_create({fa, fr}, {SliceProd{0, 0, 1, 0, planes, nw, false, -1}}, {}, mp, 2000000000LL, err,
-                          ctx->stream, &g, &msg)) {
+        slice_gemm_create({fa, fr}, {SliceProd{0, 0, 1, 0, planes, nw, false, -1}}, {}, mp, ctx->opt.timeout_ns,
+                          err, ctx->stream, &g, &msg)) {
       // no room for the digits: the FP64 pipe
       slice_gemm_destroy(g);
       g = nullptr;
@@ -899,25 +900,26 @@ class SetupProducts {
       launch_slice_rows(dj, 2, h.N, h.N, mp, nullptr, ctx->stream);
       if (slice_gemm_launch(g, ctx->stream)) return fail(ctx, VGTB_E_CUDA, "sliced set-up product launch failed");
       launch_slice_rows(dj + 2, 1, h.N, h.N, mp, nullptr, ctx->stream);
-    } else {
-      GemmF64Item t{};
-      t.A[0] = A;
-      t.R[0] = R;
-      t.K[0] = t.M = t.N = h.N;
-      t.lda[0] = t.ldr[0] = t.ldc = h.Np;
-      t.nseg = 1;
-      t.C = C;
-      CK(cudaMemcpyAsync(dg, &t, sizeof(t), cudaMemcpyHostToDevice, ctx->stream));
-      launch_gemm_f64(dg, 1, h.N, h.N, nullptr, ctx->stream);
+      int e = 0;
+      CK(cudaGetLastError());
+      CK(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+      CK(cudaStreamSynchronize(ctx->stream));
+      if (!e) return VGTB_OK;
+      // the wait limit ran out: the FP64 pipe, which waits for nothing, from here on
+      slice_gemm_destroy(g);
+      g = nullptr;
     }
+    GemmF64Item t{};
+    t.A[0] = A;
+    t.R[0] = R;
+    t.K[0] = t.M = t.N = h.N;
+    t.lda[0] = t.ldr[0] = t.ldc = h.Np;
+    t.nseg = 1;
+    t.C = C;
+    CK(cudaMemcpyAsync(dg, &t, sizeof(t), cudaMemcpyHostToDevice, ctx->stream));
+    launch_gemm_f64(dg, 1, h.N, h.N, nullptr, ctx->stream);
     CK(cudaGetLastError());
     return VGTB_OK;
-  }
-  int finish() {
-    int e = 0;
-    if (g) CK(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    return e ? fail(ctx, VGTB_E_TIMEOUT, "sliced set-up product reported status %d", e) : VGTB_OK;
   }
 
  private:
@@ -990,7 +992,6 @@ int finish_density(vgtb_ctx* ctx, int si) {
       }
     }
     CK(cudaGetLastError());
-    TRY(sp.finish());
   }
   if (h.d_jD0) {
     launch_slice_rows(h.d_jD0, h.nk, h.N, h.N, kSlicePairs, nullptr, ctx->stream);
@@ -998,6 +999,17 @@ int finish_density(vgtb_ctx* ctx, int si) {
   }
   h.density_set = true;
   CK(cudaStreamSynchronize(ctx->stream));
+  return VGTB_OK;
+}
+
+// error words of a product whose wait ran out, at a restart
+int clear_expired(vgtb_ctx* ctx) {
+  if (!ctx->expired) return VGTB_OK;
+  if (ctx->d_slice_err) CK(cudaMemsetAsync(ctx->d_slice_err, 0, sizeof(int), ctx->stream));
+  tc_clear_error(ctx->tc1, ctx->stream);
+  tc_clear_error(ctx->tc2, ctx->stream);
+  CK(cudaGetLastError());
+  ctx->expired = false;
   return VGTB_OK;
 }
 
@@ -1017,6 +1029,7 @@ int reset_all(vgtb_ctx* ctx) {
     if (it.dDf) CK(cudaMemsetAsync(it.dDf, 0, NN * sizeof(float2), ctx->stream));
   }
   for (auto& t : ctx->trj) CK(cudaMemsetAsync(t.status, 0, sizeof(int), ctx->stream));
+  TRY(clear_expired(ctx));
   CK(cudaMemsetAsync(ctx->d_step, 0, sizeof(int), ctx->stream));
   CK(cudaMemsetAsync(ctx->d_counter, 0, sizeof(int), ctx->stream));
   ctx->n_done = 0;
@@ -1203,7 +1216,6 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
     c.pat = (int)pats.size();
     pats.push_back(slice_pattern(h));
   }
-  const long long tmo = std::max(ctx->opt.timeout_ns, 2000000000LL);
   for (size_t r = 0; r < n_rounds; ++r) {
     SliceRound R;
     std::vector<SliceRowJob> jD, jW;
@@ -1258,8 +1270,8 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
     std::string msg;
     ctx->rounds.push_back(R);
     SliceRound& Q = ctx->rounds.back();
-    if (slice_gemm_create(fams, p1, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g1, &msg) ||
-        slice_gemm_create(fams, p2, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g2, &msg))
+    if (slice_gemm_create(fams, p1, pats, ctx->slice_mp, ctx->opt.timeout_ns, ctx->d_slice_err, ctx->stream, &Q.g1, &msg) ||
+        slice_gemm_create(fams, p2, pats, ctx->slice_mp, ctx->opt.timeout_ns, ctx->d_slice_err, ctx->stream, &Q.g2, &msg))
       return fail(ctx, VGTB_E_CUDA, "sliced product plan: %s", msg.c_str());
     TRY(upload(ctx, &Q.jD, jD.data(), jD.size()));
     TRY(upload(ctx, &Q.jH, jH.data(), jH.size()));
@@ -1332,7 +1344,6 @@ int slice_build_cn(vgtb_ctx* ctx) {
     c.pat = (int)pats.size();
     pats.push_back(slice_pattern(h));
   }
-  const long long tmo = std::max(ctx->opt.timeout_ns, 2000000000LL);
   for (size_t r = 0; r < n_rounds; ++r) {
     SliceRound R;
     std::vector<ConjTItem> tC;
@@ -1402,9 +1413,9 @@ int slice_build_cn(vgtb_ctx* ctx) {
     std::string msg;
     ctx->rounds.push_back(R);
     SliceRound& Q = ctx->rounds.back();
-    if (slice_gemm_create(fams, pD, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.gD, &msg) ||
-        slice_gemm_create(fams, pM, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g2, &msg) ||
-        slice_gemm_create(fams, pS, pats, ctx->slice_mp, tmo, ctx->d_slice_err, ctx->stream, &Q.g1, &msg))
+    if (slice_gemm_create(fams, pD, pats, ctx->slice_mp, ctx->opt.timeout_ns, ctx->d_slice_err, ctx->stream, &Q.gD, &msg) ||
+        slice_gemm_create(fams, pM, pats, ctx->slice_mp, ctx->opt.timeout_ns, ctx->d_slice_err, ctx->stream, &Q.g2, &msg) ||
+        slice_gemm_create(fams, pS, pats, ctx->slice_mp, ctx->opt.timeout_ns, ctx->d_slice_err, ctx->stream, &Q.g1, &msg))
       return fail(ctx, VGTB_E_CUDA, "sliced product plan: %s", msg.c_str());
     TRY(upload(ctx, &Q.tC, tC.data(), tC.size()));
     TRY(upload(ctx, &Q.jC, jC.data(), jC.size()));
@@ -1723,7 +1734,26 @@ int build_graph(vgtb_ctx* ctx, int G) {
   return VGTB_OK;
 }
 
+int slice_status(vgtb_ctx* ctx) {
+  if (!ctx->d_slice_err) return VGTB_OK;
+  int err = 0;
+  CK(cudaMemcpyAsync(&err, ctx->d_slice_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  if (!err) return VGTB_OK;
+  ctx->expired = true;
+  return fail(ctx, VGTB_E_TIMEOUT, "sliced product reported status %d (bounded wait expired)", err);
+}
+
 int check_status(vgtb_ctx* ctx) {
+  // an expired wait in a product is the cause of whatever the observables show after it
+  TRY(slice_status(ctx));
+  const int tc = ctx->split ? tc_status(ctx->tc1, ctx->stream) | tc_status(ctx->tc2, ctx->stream) : 0;
+  if (tc) {
+    // an aborted chained launch left its block counts short: start them again
+    if (ctx->tcc) tc_reset_chain(ctx->tcc, ctx->stream);
+    ctx->expired = true;
+    return fail(ctx, VGTB_E_TIMEOUT, "tcgen05 product reported status %d (bounded wait expired)", tc);
+  }
   for (size_t t = 0; t < ctx->trj.size(); ++t) {
     int st = 0;
     CK(cudaMemcpyAsync(&st, ctx->trj[t].status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1735,19 +1765,6 @@ int check_status(vgtb_ctx* ctx) {
                   "trajectory %zu: Crank-Nicolson fixed point not converged (raise cn_iter or lower dt)", t);
     if (st & ST_NONFINITE) return fail(ctx, VGTB_E_UNSTABLE, "trajectory %zu: non-finite observables", t);
     if (st & ST_DRIFT) return fail(ctx, VGTB_E_UNSTABLE, "trajectory %zu: electron count drifted", t);
-  }
-  if (ctx->d_slice_err) {
-    int err = 0;
-    CK(cudaMemcpyAsync(&err, ctx->d_slice_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    if (err) return fail(ctx, VGTB_E_TIMEOUT, "sliced product reported status %d (bounded wait expired)", err);
-  }
-  if (!ctx->split) return VGTB_OK;
-  const int tc = tc_status(ctx->tc1, ctx->stream) | tc_status(ctx->tc2, ctx->stream);
-  if (tc) {
-    // an aborted chained launch left its block counts short: start them again
-    if (ctx->tcc) tc_reset_chain(ctx->tcc, ctx->stream);
-    return fail(ctx, VGTB_E_TIMEOUT, "tcgen05 product reported status %d (bounded wait expired)", tc);
   }
   return VGTB_OK;
 }
@@ -2517,6 +2534,7 @@ int vgtb_set_state(vgtb_ctx* ctx, const void* buf, long long bytes) {
   const int n = (int)hd[1];
   for (auto& t : ctx->trj)
     if (t.n_times < n + 1) return fail(ctx, VGTB_E_STATE, "field table shorter than the saved step");
+  TRY(clear_expired(ctx));
   const char* p = (const char*)buf + 4 * sizeof(long long);
   for (auto& it : ctx->items_h) {
     const HostSys& h = ctx->sys[it.sys];
@@ -2546,7 +2564,7 @@ int vgtb_set_state(vgtb_ctx* ctx, const void* buf, long long bytes) {
   CK(cudaMemsetAsync(ctx->d_counter, 0, sizeof(int), ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   ctx->n_done = n;
-  return VGTB_OK;
+  return slice_status(ctx);  // of the density
 }
 
 int vgtb_profile(vgtb_ctx* ctx, int enable) {

@@ -51,7 +51,7 @@ int tc_launch(TcPlan* p, cudaStream_t st);
 int tc_status(TcPlan* p, cudaStream_t st);  // 0 or the plan's device error word
 void tc_destroy_plan(TcPlan* p);
 int tc_plan_variant(const TcPlan* p);  // index of the tile variant the plan uses
-void tc_clear_error(TcPlan* p, cudaStream_t st);  // zero the plan's device error word
+void tc_clear_error(TcPlan* p, cudaStream_t st);  // zero the device error word and the stream-K flags
 
 // Chained schedule: both products in one launch (tc_chain.cuh), over the
 // tables of two plans that it does not own (2-SM pair, classic schedule,

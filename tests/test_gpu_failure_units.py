@@ -90,3 +90,41 @@ def test_bit_conversions_match_cuda():
     assert np.all(fb == 0.0) and np.array_equal(np.signbit(fb), np.signbit(tiny))
     assert np.all(db == 0.0) and np.array_equal(np.signbit(db), np.signbit(tiny_f))
     assert np.any(fr != 0.0)  # CUDA itself rounds to subnormals here
+
+
+@pytest.mark.parametrize("form", ["fp64", "fp64_delta", "cn", "split"])
+def test_wait_limit_is_honoured_and_its_error_ends_with_a_reset(form):
+    """A 1 ns limit runs out inside the products of 256 orbitals: E_TIMEOUT (-8) from vgtb_propagate, in
+    every form.  Set-up products that run into it are made without waits, so setting the density works,
+    and the restart by vgtb_set_field clears the error: level 0 reads as in a context with the usual limit."""
+    from paper_2308_09782_gb300 import vgtb
+    from tests._gpu_util import oracle_ground
+    sysd, A, _ = system("si64_pulse")
+    _, gs = oracle_ground("si64_pulse")
+    opt = {"precision": vgtb.SPLIT_BF16X3 if form == "split" else vgtb.FP64, "init": vgtb.INIT_USER,
+           "delta_form": int(form == "fp64_delta"), "graph_steps": 1,
+           "integrator": vgtb.CRANK_NICOLSON if form == "cn" else vgtb.LEAPFROG}
+
+    def start(**more):
+        c = vgtb.Context(sysd, **opt, **more)
+        for k in range(8):
+            (c.set_coefficients if form == "cn" else c.set_density)(0, k, (gs["C"] if form == "cn" else gs["D"])[k])
+        c.set_field(0, A[:4])
+        return c
+
+    with start(timeout_ns=1) as c, start() as ok:
+        with pytest.raises(vgtb.VgtbError) as e:
+            c.propagate(1)
+        assert e.value.code == -8
+        c.set_field(0, A[:4])
+        ok.propagate(0)
+        if form == "cn":  # its start density is a digit product too
+            with pytest.raises(vgtb.VgtbError) as e:
+                c.propagate(0)
+            assert e.value.code == -8
+        else:
+            c.propagate(0)
+            for a, b in zip(c.observables(0), ok.observables(0)):
+                assert np.allclose(a, b, rtol=0, atol=1e-12)
+        ok.propagate(3)
+        assert np.all(np.isfinite(ok.observables(0)[0]))
