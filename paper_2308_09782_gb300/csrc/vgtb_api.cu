@@ -539,7 +539,7 @@ int prepare_system(vgtb_ctx* ctx, int si, const vgtb_system& s, HostSys& h, DevS
   TRY(dalloc(ctx, &h.D0, NN * h.nk));
   TRY(dalloc(ctx, &h.dq0, h.nat));
   TRY(dalloc(ctx, &h.eps0, h.nat));
-  if (ctx->delta) TRY(dalloc(ctx, &h.R0, NN * h.nk));
+  if (ctx->delta && !ctx->split) TRY(dalloc(ctx, &h.R0, NN * h.nk));
   if (ctx->cn) TRY(dalloc(ctx, &h.C0d, (size_t)h.nk * h.nocc * h.Np));
   if (ctx->split) {
     TRY(dalloc(ctx, &h.Sinv_p, 4 * NN * h.nk));
@@ -977,9 +977,12 @@ int finish_density(vgtb_ctx* ctx, int si) {
     for (int k = 0; k < h.nk; ++k) {
       CK(cudaMemsetAsync(Hb, 0, NN * sizeof(double2), ctx->stream));
       launch_bloch_setup(ctx->d_sys, si, h.n_tgt, k, 1, h.eps0, Hb, ctx->stream);
-      TRY(derivative(k, h.R0 + k * NN));
-      if (!ctx->split) continue;
-      launch_to_planar_f32(h.R0 + k * NN, h.R0f + 2 * NN * k, h.Np, ctx->stream);
+      if (!ctx->split) {
+        TRY(derivative(k, h.R0 + k * NN));
+        continue;
+      }
+      TRY(derivative(k, Wb));  // W is done with; the split form keeps R0 in FP32 only
+      launch_to_planar_f32(Wb, h.R0f + 2 * NN * k, h.Np, ctx->stream);
       launch_to_planar_f32(h.D0 + k * NN, h.D0f + 2 * NN * k, h.Np, ctx->stream);
       launch_split_planar(h.Sinv + k * NN, h.Sinv_p + 4 * NN * k, h.N, h.Np, ctx->stream);
       launch_scatter(h.d_kS + (size_t)k * h.n_el, h.d_el_off, h.n_el, Hb, ctx->stream);
@@ -2059,7 +2062,7 @@ int vgtb_create_batch(vgtb_ctx** out, int n_sys, const vgtb_system* sys, int n_t
     }
     LeapItem l{};
     l.X = ctx->split ? (const void*)it.Xf : (const void*)it.X;
-    l.R0 = (ctx->delta && !ctx->split) ? h.R0 + it.k * NN : nullptr;
+    l.R0 = h.R0 ? h.R0 + it.k * NN : nullptr;
     if (ctx->split) {
       l.R0f = h.R0f + 2 * NN * it.k;
       l.D0f = h.D0f + 2 * NN * it.k;

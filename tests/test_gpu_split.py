@@ -179,3 +179,23 @@ def test_split_rerun_bitwise_and_autotuned_variants_agree():
         assert np.array_equal(a.get_density(0, 5), b.get_density(0, 5))
     ref = oracle_run(name, nsteps)
     assert rel_fro([Jc], [ref["J"]]) <= 1e-4
+
+
+def test_split_context_memory_per_matrix():
+    """A k-point more of one system and trajectory takes 168 Np^2 bytes of matrices: FP64 S^-1, D0 and two levels
+    of dD (64), pieces of S^-1, dD, H and W (48), FP32 X, R0, D0, D0 S and three D0 P_a (56), and 80 bytes for
+    each of H's nonzeros (S, H0, P).  16 MB for tables and the granularity of allocations; one matrix more
+    would be 67 MB."""
+    import torch
+    from paper_2308_09782_gb300 import vgtb
+    sysd, _, _ = system("si512_kick")
+    pairs = len(np.unique(np.asarray(sysd["blk_ijl"])[:, :2], axis=0))
+    used = []
+    for nk in (2, 1, 2):  # the first one loads kernels and library handles
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        kpt = {"kpt": np.array([[0.0, 0.0, 0.0], [0.5, 0.0, 0.0]])[:nk], "wk": np.full(nk, 1.0 / nk)}
+        with vgtb.Context({**sysd, **kpt}, precision=vgtb.SPLIT_BF16X3, init=vgtb.INIT_USER):
+            used.append(free - torch.cuda.mem_get_info()[0])
+    want = 168 * 2048 ** 2 + 80 * 16 * pairs
+    assert want <= used[2] - used[1] + (16 << 20) and used[2] - used[1] <= want + (16 << 20), used
