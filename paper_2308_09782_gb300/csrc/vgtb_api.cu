@@ -172,8 +172,7 @@ struct vgtb_ctx {
   long long prof_launch[VGTB_K_COUNT] = {0};
   double prof_ms[VGTB_K_COUNT] = {0};
   cusolverDnHandle_t solver = nullptr;
-  // read-out buffer of the density, spectrum and charge calls: grows to the largest call's need
-  // (densities: kReadBytes), lives as long as the context
+  // read-out buffer of the density, spectrum and charge calls (read_buffer)
   void* read_dev = nullptr;
   size_t read_bytes = 0;
 };
@@ -222,15 +221,31 @@ void touch_pages(double* p, size_t n) {
   for (size_t o = 0; o < n; o += 512) p[o] = 0.0;
 }
 
+// The read-out buffer: up to kReadBytes stay with the context, a larger call's is given back at its end.
 constexpr size_t kReadBytes = 32u << 20;
+
+void read_free(vgtb_ctx* ctx) {
+  if (ctx->read_dev) cudaFree(ctx->read_dev);
+  ctx->read_dev = nullptr;
+  ctx->read_bytes = 0;
+}
 
 int read_buffer(vgtb_ctx* ctx, size_t bytes) {
   if (bytes <= ctx->read_bytes) return VGTB_OK;
-  void* q = nullptr;
-  CK(cudaMalloc(&q, bytes));
-  if (ctx->read_dev) cudaFree(ctx->read_dev);
-  ctx->read_dev = q;
+  read_free(ctx);
+  if (cudaMalloc(&ctx->read_dev, bytes) != cudaSuccess) {
+    ctx->read_dev = nullptr;
+    cudaGetLastError();
+    return fail(ctx, VGTB_E_NOMEM, "cudaMalloc of %zu bytes failed", bytes);
+  }
   ctx->read_bytes = bytes;
+  return VGTB_OK;
+}
+
+// the end of a read-out call
+int read_done(vgtb_ctx* ctx) {
+  CK(cudaStreamSynchronize(ctx->stream));
+  if (ctx->read_bytes > kReadBytes) read_free(ctx);
   return VGTB_OK;
 }
 
@@ -2443,8 +2458,7 @@ int vgtb_spectrum(vgtb_ctx* ctx, int t, int n0, int n1, double e0, double tau0, 
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(sigma, dw + nw, sizeof(double) * 6 * nw, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaMemcpyAsync(eps, dw + 7 * nw, sizeof(double) * 6 * nw, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
-  return VGTB_OK;
+  return read_done(ctx);
 }
 
 int vgtb_group_charges(vgtb_ctx* ctx, int t, int n_groups, const int* group, double* out) {
@@ -2465,8 +2479,7 @@ int vgtb_group_charges(vgtb_ctx* ctx, int t, int n_groups, const int* group, dou
   launch_group_charge(T.q, nat, dg, n_groups, nlev, dout, ctx->stream);
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(out, dout, out_bytes, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
-  return VGTB_OK;
+  return read_done(ctx);
 }
 
 int vgtb_get_initial_density(vgtb_ctx* ctx, int s, int k, double* d_out) {
@@ -2620,7 +2633,7 @@ void vgtb_destroy(vgtb_ctx* ctx) {
   tc_destroy_plan(ctx->tc1);
   tc_destroy_plan(ctx->tc2);
   for (void* p : ctx->allocs) cudaFree(p);
-  if (ctx->read_dev) cudaFree(ctx->read_dev);
+  read_free(ctx);
   if (ctx->solver) cusolverDnDestroy(ctx->solver);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
   delete ctx;

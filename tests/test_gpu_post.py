@@ -130,3 +130,25 @@ def test_spectrum_takes_the_phases_without_rounding():
         x = np.array([float(Fraction(wi) * Fraction(float(sysd["dt"])) * m % turn) for m in range(n + 1)])[:, None]
         assert np.all(np.abs(s[i].real - (np.cos(x) * term).astype(np.longdouble).sum(0)) <= size), wi
         assert np.all(np.abs(s[i].imag - (np.sin(x) * term).astype(np.longdouble).sum(0)) <= size), wi
+
+
+def test_a_large_read_out_gives_its_buffer_back():
+    """Charges of 2001 levels by 8192 groups are 131 MB on the device: as much is free after the call as before
+    (an allocation's granularity of 2 MB aside), and a small call still answers."""
+    import torch
+    from paper_2308_09782_gb300 import vgtb
+    sysd, _, _ = system("si8_pulse")
+    _, gs = oracle_ground("si8_pulse")
+    n = 2000
+    with vgtb.Context(sysd, init=vgtb.INIT_USER) as c:
+        for k, D in enumerate(gs["D"]):
+            c.set_density(0, k, D)
+        c.set_field(0, inputs.kick_field(n, 0.01))
+        c.propagate(n)
+        small = c.group_charges(0, np.arange(8, dtype=np.int32) % 2, 2)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        big = c.group_charges(0, np.arange(8, dtype=np.int32) % 2, 8192)
+        assert torch.cuda.mem_get_info()[0] >= free - (2 << 20)
+        assert np.array_equal(big[:, :2], small) and not big[:, 2:].any()
+        assert np.array_equal(c.group_charges(0, np.arange(8, dtype=np.int32) % 2, 2), small)
