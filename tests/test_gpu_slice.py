@@ -152,3 +152,34 @@ def test_slice_product_holds_more_than_fp64_rows(shape, fall):
         d = vgtb.diag_slice_product(a, r, planes=planes).astype(np.clongdouble) - e
         for got, val in ((d.real, e.real), (d.imag, e.imag)):
             assert np.all(np.abs(got) <= 2.0 ** -53 * np.abs(val) * (1 + 2.0 ** -40) + 2.2 * k * 2.0 ** -62 * scale)
+
+
+@pytest.mark.parametrize("form", ["fp64", "fp64_delta", "cn"])
+def test_rounds_that_share_scratch_equal_single_runs(form):
+    """The digits and planes of a step's items take at most 32 GB (a quarter of the free memory): 512 atoms at
+    134 MB of digits a matrix and 805 MB of planes need more than one round from 30 (16, 24) trajectories
+    on.  Every trajectory equals its own single run bit for bit, whichever round holds it."""
+    from paper_2308_09782_gb300 import inputs
+    from tests._gpu_util import oracle_ground, system
+    sysd, _, _ = system("si512_kick")
+    _, gs = oracle_ground("si512_kick")
+    dig, planes = 2 * 8 * 2048 * 2 * 2048, 4 * 24 * 2048 * 2 * 2048
+    n_traj = int(32e9 / {"fp64": 2 * dig + planes, "fp64_delta": 3 * dig + 2 * planes, "cn": 4 * dig + planes}[form]) + 2
+    n = 2
+    fields = [inputs.kick_field(n, 0.001 * (1.0 + 0.1 * t), np.array([1.0, 0.1 * t, 0.0])) for t in range(n_traj)]
+
+    def run(which):
+        c = vgtb.Context([sysd], traj_sys=[0] * len(which), init=vgtb.INIT_USER, delta_form=int(form == "fp64_delta"),
+                         integrator=vgtb.CRANK_NICOLSON if form == "cn" else vgtb.LEAPFROG, graph_steps=1)
+        (c.set_coefficients if form == "cn" else c.set_density)(0, 0, (gs["C"] if form == "cn" else gs["D"])[0])
+        for i, t in enumerate(which):
+            c.set_field(i, fields[t])
+        c.propagate(n)
+        return c
+
+    with run(range(n_traj)) as many:
+        for t in (0, n_traj - 3, n_traj - 1):
+            with run([t]) as one:
+                for a, b in zip(many.observables(t), one.observables(0)):
+                    assert np.array_equal(a, b)
+                assert np.array_equal(many.get_density(t, 0), one.get_density(0, 0))
