@@ -208,6 +208,37 @@ def fp32_alu_peak(peaks):
                                              "(derived from unit counts and the maximum SM clock)")
 
 
+def kept_panels(sysd, tile_n, uniform):
+    """Fraction of product 1's 64-wide k-panels that run: those in which a column tile of tile_n B rows (tile_n / 2
+    rows of H, real and imaginary interleaved) meets an atom block of H; stream-K pads every tile to the longest list."""
+    off = np.asarray(sysd["orb_offset"])
+    Np = (int(off[-1]) + 127) // 128 * 128
+    pairs = np.unique(np.asarray(sysd["blk_ijl"])[:, :2], axis=0)
+    first, last = off[pairs[:, 1]] // 64, (off[pairs[:, 1] + 1] - 1) // 64
+    kept = []
+    for r0 in range(0, Np, tile_n // 2):
+        sel = (off[pairs[:, 0]] < r0 + tile_n // 2) & (off[pairs[:, 0] + 1] > r0)
+        kept.append(max(1, len(set(first[sel]) | set(last[sel]))))
+    return (max(kept) if uniform else sum(kept) / len(kept)) / (Np // 64)
+
+
+def executed_flops(systems, n_items, tiles):
+    """BF16 flops that the two split products execute per launch (padded sizes): product 1 over the k-panels it keeps
+    (None over planned column widths, which the library does not report), product 2 over the real half of its panels
+    at the k-points where every Bloch phase is real."""
+    f1, f2 = 0.0, 0.0
+    sched, tn = tiles["product1"].get("schedule", ""), tiles["product1"].get("tile_n")
+    for s, n_it in zip(systems, n_items):
+        full = n_it * 24.0 * float((int(s["orb_offset"][-1]) + 127) // 128 * 128) ** 3
+        real = np.mean([float(np.all(2 * np.asarray(k) == np.round(2 * np.asarray(k)))) for k in s.get("kpt", [[0.1] * 3])])
+        f2 += full * (1.0 - 0.5 * real)
+        if tn is None or "planned" in sched:
+            f1 = None
+        elif f1 is not None:
+            f1 += full * (kept_panels(s, tn, "stream-K" in sched) if "skipped" in sched else 1.0)
+    return f1, f2
+
+
 def split_product_rooflines(systems, n_items, stats, tiles, peaks):
     """Roofline of both commutator products of the split form, in algorithmic flops.
 
@@ -215,7 +246,8 @@ def split_product_rooflines(systems, n_items, stats, tiles, peaks):
     atom blocks, 8 nnz(H) N FP32 flops per item, against the FP32 ALU peak.  Product 1, dense tcgen05
     (the split form's default): 3 split terms x 8 N^3 = 24 N^3 per item.  Product 2 (tcgen05
     BF16x3): 24 N^3 per item (unpadded N; the kernel executes 24 Np^3).  Both
-    tensor figures are against the measured sustained BF16 peak."""
+    tensor figures are against the measured sustained BF16 peak; executed_frac counts the flops that run
+    (zero k-panels and the imaginary half of a real S^-1 left out), so frac may exceed one and it may not."""
     sust = peaks.get("bf16_tflops_sustained")
     sust_kind = "measured sustained bf16 (MEASURED_PEAKS.json)"
     if sust is None:
@@ -223,6 +255,7 @@ def split_product_rooflines(systems, n_items, stats, tiles, peaks):
     burst = peaks.get("bf16_tflops", 1900.0)
     g1 = stats["gemm1"][1] / max(stats["gemm1"][0], 1)
     g2 = stats["gemm2"][1] / max(stats["gemm2"][0], 1)
+    e1, e2 = executed_flops(systems, n_items, tiles)
     n3 = sum(n_it * float(int(s["orb_offset"][-1])) ** 3 for s, n_it in zip(systems, n_items))
     np3 = sum(n_it * float((int(s["orb_offset"][-1]) + 127) // 128 * 128) ** 3 for s, n_it in zip(systems, n_items))
     if "one launch" in tiles["product1"].get("schedule", ""):
@@ -262,13 +295,16 @@ def split_product_rooflines(systems, n_items, stats, tiles, peaks):
                                                     "before zero k-panels are skipped)",
               "executed_tflops_upper": round(24 * np3 / (g1 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g1, 4),
               "traffic": kernel_traffic("tc_gemm1", float(sum(n_items)), tiles["product1"])}
+        if e1 is not None:
+            p1.update(executed_flops=e1, executed_frac=round(e1 / (g1 * 1e-3) / 1e12 / sust, 4))
     f2 = 24.0 * n3
     a2 = f2 / (g2 * 1e-3) / 1e12
     p2 = {"kernel": "k_tc_gemm2<3,1> (product 2: X = S^-1 W^dagger, tcgen05 BF16x3)", "bound": "tensor",
           "achieved": round(a2, 1), "peak": sust, "unit": "TFLOP/s", "frac": round(a2 / sust, 4),
           "peak_kind": sust_kind, "frac_of_burst": round(a2 / burst, 4), "flops_per_launch": f2,
           "flops_note": "3 split terms x 8 N^3 (algorithmic, unpadded N); half of it is skipped where S^-1 is real",
-          "executed_tflops_upper": round(24 * np3 / (g2 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g2, 4),
+          "executed_flops": e2, "executed_frac": round(e2 / (g2 * 1e-3) / 1e12 / sust, 4),
+          "avg_launch_ms": round(g2, 4),
           "traffic": kernel_traffic("tc_gemm2", float(sum(n_items)), tiles["product2"])}
     return p1, p2
 
@@ -598,8 +634,7 @@ def native(args):
                               "achieved": round(a64_2, 3), "peak": round(p64, 3), "unit": "TFLOP/s",
                               "frac": round(a64_2 / p64, 4), "flops_per_launch": fl64_2,
                               "peak_kind": "cuBLAS ZGEMM 2048^3 measured in this run (torch.matmul complex128)"},
-                 "product1": {"kernel": ("k_slice_rows, k_slice_pattern, k_slice_gemm (W = D H, zero k-panels skipped)" if fp64_sparse
-                                         else "k_gemm_f64 (W = D H, dense)"),
+                 "product1": {"kernel": "k_slice_rows, k_slice_hamilton, k_slice_gemm (W = D H, zero k-panels skipped)",
                               "achieved": round(a64_1, 3), "peak": round(p64, 3), "unit": "TFLOP/s",
                               "frac": round(a64_1 / p64, 4), "flops_per_launch": fl64_1,
                               "avg_launch_ms": round(f64_1, 3)}},
