@@ -474,8 +474,7 @@ int scc_configure(int max_nat) {
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_phase(const DevSys* __restrict__ sysv, const DevTraj* __restrict__ trj,
                                                const DevItem* __restrict__ items, const int* __restrict__ wpre,
-                                               int n_traj, int total, const int* __restrict__ step, int mode,
-                                               int fixed_step) {
+                                               int n_traj, int total, const int* __restrict__ step, int mode) {
   pdl_wait();
   pdl_trigger();
   const Unit U = unit_of(wpre, n_traj, total);
@@ -483,7 +482,7 @@ __global__ void __launch_bounds__(256) k_phase(const DevSys* __restrict__ sysv, 
   const int lane = threadIdx.x & 15;
   const DevTraj& T = trj[U.t];
   const DevSys& S = sysv[T.sys];
-  const int n = fixed_step >= 0 ? fixed_step : *step;
+  const int n = *step;
   double A0 = 0.0, A1 = 0.0, A2 = 0.0;
   if (T.A) {
     A0 = T.A[3 * n];
@@ -547,12 +546,11 @@ __global__ void __launch_bounds__(256) k_phase(const DevSys* __restrict__ sysv, 
 }
 
 void launch_phase(const DevSys* sys, const DevTraj* trj, const DevItem* items, const int* warp_prefix,
-                  int n_traj, int total_units, int max_nk, const int* step, int mode, int fixed_step,
-                  cudaStream_t st) {
+                  int n_traj, int total_units, int max_nk, const int* step, int mode, cudaStream_t st) {
   const int threads = 128;
   const int blocks = (total_units * 16 + threads - 1) / threads;
-  launch_pdl(k_phase, dim3(blocks, max_nk), threads, 0, st, sys, trj, items, warp_prefix, n_traj, total_units, step, mode,
-             fixed_step);
+  launch_pdl(k_phase, dim3(blocks, max_nk), threads, 0, st, sys, trj, items, warp_prefix, n_traj, total_units, step,
+             mode);
 }
 
 // ---------------------------------------------------------------------------

@@ -84,7 +84,8 @@ __device__ __forceinline__ void slice_load4(const SlicePlanes& S, long long row,
 // kept in registers between the search for its largest part and the cut.  Memory bound: at
 // N = 2048 it reads 67 MB (a matrix) or 302 MB (planes) and writes 134 MB of digits.  One
 // iteration per thread wherever a CTA can hold the row: with four, 128 threads a row, the 130 to
-// 150 registers left 16 warps an SM and the loads waited (planes, N = 2048: 123 us, now 98).
+// 150 registers left 16 warps an SM and the loads waited (planes of seven digits, N = 2048: 123 us
+// against 98).  Eight digits: a matrix 54 us, planes 116.
 template <int TPR, int IT, int MP>
 __global__ void __launch_bounds__(TPR > 128 ? TPR : 128)
     k_slice_rows(const SliceRowJob* __restrict__ jobs, const int* __restrict__ step) {

@@ -33,9 +33,11 @@ namespace {
 
 thread_local std::string g_create_error;
 
-// From kSliceMinN orbitals up the 43 exact digit products on the tensor cores take less time than
-// one product on the FP64 pipe (N = 256, 8 k-points: 1.06 ms for one product on the FP64 pipe);
-// below, a product is a few microseconds of FP64 work and the extra launches cost more.
+// From kSliceMinN orbitals up the 43 exact digit products on the tensor cores take no longer than
+// FP64 multiply-adds in 8 x 8 tiles; below, the extra launches cost more.  Phase build, both products
+// and leapfrog of a step, multiply-adds | digits, in us: one item of 64 orbitals 60 | 68, 92 orbitals
+// 72 | 74, 116 orbitals 83 | 75, 156 orbitals 110 | 78; 8 items of 64 orbitals 77 | 87, 92 orbitals
+// 147 | 101, 128 orbitals 287 | 108 (several items would put the line lower, at about 70).
 constexpr int kSliceMinN = 97;
 static_assert(kSliceMinN == kGemmSmall + 1, "every FP64 size has its kernel");
 
@@ -1586,7 +1588,7 @@ int enqueue_step_cn(vgtb_ctx* ctx, cudaEvent_t* ev, unsigned evflag) {
   if (ev) CK(cudaEventRecordWithFlags(ev[2], st, evflag));
   if (ctx->n_dense)
     launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk, ctx->d_step,
-                 PH_FP64_CN, -1, st);
+                 PH_FP64_CN, st);
   if (!ctx->rounds.empty()) launch_slice_h(ctx, ctx->rounds.front(), st);
   if (ev) CK(cudaEventRecordWithFlags(ev[3], st, evflag));
   if (ctx->n_dense == 0) {
@@ -1660,7 +1662,7 @@ int enqueue_step(vgtb_ctx* ctx, cudaEvent_t* ev) {
                        ctx->d_step, 1, st);
   else if (ctx->n_dense || ctx->n_bsr)
     launch_phase(ctx->d_sys, ctx->d_trj, ctx->d_items, ctx->d_wpre, nt, ctx->total_warps, ctx->max_nk, ctx->d_step,
-                 ctx->delta ? PH_FP64_DELTA : PH_FP64_PLAIN, -1, st);
+                 ctx->delta ? PH_FP64_DELTA : PH_FP64_PLAIN, st);
   if (!ctx->rounds.empty()) launch_slice_h(ctx, ctx->rounds.front(), st);
   if (ev) CK(cudaEventRecordWithFlags(ev[3], st, evflag));
   if (ctx->bsr && ctx->n_bsr > 0)

@@ -291,7 +291,7 @@ void launch_phase_split(const DevSys* sys, DevTraj* trj, const DevItem* items, c
 void launch_to_planar_f32(const double2* src, float* dst, int Np, cudaStream_t st);
 // grid rows = max_nk, as launch_phase_split
 void launch_phase(const DevSys* sys, const DevTraj* trj, const DevItem* items, const int* warp_prefix,
-                  int n_traj, int total_warps, int max_nk, const int* step, int mode, int fixed_step, cudaStream_t st);
+                  int n_traj, int total_warps, int max_nk, const int* step, int mode, cudaStream_t st);
 int scc_configure(int max_nat);
 void launch_kblocks(const DevSys* sys, int s_idx, int n_tgt, int k, cudaStream_t st);
 void launch_obs0(const DevSys* sys, int s_idx, int n_tgt, int nat, cudaStream_t st);
