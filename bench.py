@@ -273,7 +273,7 @@ def split_product_rooflines(systems, n_items, stats, tiles, peaks):
                             f"at most {48 * np3:.3e} BF16 flops (both with K' = 2 Np, before product 1's zero k-panels "
                             "and the imaginary half of a real S^-1 are skipped)",
               "executed_tflops_upper": round(48 * np3 / (g1 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g1, 4),
-              "schedule": kept, "traffic": kernel_traffic("tc_chain", float(sum(n_items)), tiles["product1"])}
+              "schedule": kept, "traffic": kernel_traffic("tc_chain", float(sum(n_items)), tiles["product1"]) if len(systems) == 1 else None}
         return pc, None
     if tiles["product1"].get("schedule") == "block-sparse":
         f1 = sum(n_it * 8.0 * nonzeros(s) * int(s["orb_offset"][-1]) for s, n_it in zip(systems, n_items))
@@ -283,7 +283,7 @@ def split_product_rooflines(systems, n_items, stats, tiles, peaks):
               "bound": "alu", "achieved": round(a1, 2), "peak": round(alu, 2), "unit": "TFLOP/s",
               "frac": round(a1 / alu, 4), "peak_kind": alu_kind, "flops_per_launch": f1,
               "flops_note": "8 nnz(H) N (the minimum of Eq. 6)",
-              "avg_launch_ms": round(g1, 4), "traffic": kernel_traffic("bsr_f32", float(sum(n_items)))}
+              "avg_launch_ms": round(g1, 4), "traffic": kernel_traffic("bsr_f32", float(sum(n_items))) if len(systems) == 1 else None}
     else:
         f1 = 24.0 * n3
         a1 = f1 / (g1 * 1e-3) / 1e12
@@ -294,7 +294,7 @@ def split_product_rooflines(systems, n_items, stats, tiles, peaks):
                                                     f"at most {24 * np3:.3e} BF16 flops (K' = 2 Np, padded, "
                                                     "before zero k-panels are skipped)",
               "executed_tflops_upper": round(24 * np3 / (g1 * 1e-3) / 1e12, 1), "avg_launch_ms": round(g1, 4),
-              "traffic": kernel_traffic("tc_gemm1", float(sum(n_items)), tiles["product1"])}
+              "traffic": kernel_traffic("tc_gemm1", float(sum(n_items)), tiles["product1"]) if len(systems) == 1 else None}
         if e1 is not None:
             p1.update(executed_flops=e1, executed_frac=round(e1 / (g1 * 1e-3) / 1e12 / sust, 4))
     f2 = 24.0 * n3
@@ -305,7 +305,7 @@ def split_product_rooflines(systems, n_items, stats, tiles, peaks):
           "flops_note": "3 split terms x 8 N^3 (algorithmic, unpadded N); half of it is skipped where S^-1 is real",
           "executed_flops": e2, "executed_frac": round(e2 / (g2 * 1e-3) / 1e12 / sust, 4),
           "avg_launch_ms": round(g2, 4),
-          "traffic": kernel_traffic("tc_gemm2", float(sum(n_items)), tiles["product2"])}
+          "traffic": kernel_traffic("tc_gemm2", float(sum(n_items)), tiles["product2"]) if len(systems) == 1 else None}
     return p1, p2
 
 
