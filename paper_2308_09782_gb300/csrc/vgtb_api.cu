@@ -1104,11 +1104,19 @@ int slice_family(vgtb_ctx* ctx, SliceFam& f, int rows, int K, int batch) {
   return dalloc(ctx, &f.ex, (size_t)batch * rows);
 }
 
+// tiles of system h that count for the choice of the planes (slice_pairs_per_plane)
+long long slice_plane_tiles(const vgtb_ctx* ctx, const HostSys& h) {
+  if (ctx->cn) return 2LL * slice_tiles(h.nocc, h.N);
+  return (ctx->delta ? 2LL : 1LL) * slice_tiles(h.N, h.N);
+}
+
 // bytes of scratch that one item of system h takes: digits of D (later of W) and of H, planes
-// (delta form: digits of dH and a second set of planes)
+// (delta form: digits of dH and a second set of planes).  The planes are those that the system takes by
+// itself; others beside it only make them fewer.
 double slice_item_bytes(const vgtb_ctx* ctx, const HostSys& h) {
   // (Crank-Nicolson: digits of C, C^dagger or Y, H and M take no more than four full matrices)
-  const double dig = 2.0 * kSlices * h.N * 2.0 * slice_kp(h.N), pl = 4.0 * slice_num_planes(2) * h.N * 2.0 * slice_nw(h.N);
+  const int np = slice_num_planes(slice_pairs_per_plane(slice_plane_tiles(ctx, h)));
+  const double dig = 2.0 * kSlices * h.N * 2.0 * slice_kp(h.N), pl = 4.0 * np * h.N * 2.0 * slice_nw(h.N);
   return ctx->cn ? 4.0 * dig + pl : (ctx->delta ? 3.0 * dig + 2.0 * pl : 2.0 * dig + pl);
 }
 
@@ -1192,10 +1200,10 @@ int slice_build(vgtb_ctx* ctx, const std::vector<LeapItem>& leap) {
     SysScratch& c = sc[s];
     c.cap = std::max(1, std::min((int)items[s].size(), (int)(budget / n_sliced / slice_item_bytes(ctx, h))));
     n_rounds = std::max(n_rounds, (items[s].size() + c.cap - 1) / c.cap);
-    tiles += (long long)c.cap * slice_tiles(h.N, h.N);
+    tiles += c.cap * slice_plane_tiles(ctx, h);
     for (int I = 0; I < h.nat; ++I) ctx->max_orb = std::max(ctx->max_orb, h.orb_off[I + 1] - h.orb_off[I]);
   }
-  ctx->slice_mp = slice_pairs_per_plane(ctx->delta ? 2 * tiles : tiles);
+  ctx->slice_mp = slice_pairs_per_plane(tiles);
   const int np = slice_num_planes(ctx->slice_mp);
   for (size_t s = 0; s < ctx->sys.size(); ++s) {
     if (items[s].empty()) continue;
@@ -1331,10 +1339,10 @@ int slice_build_cn(vgtb_ctx* ctx) {
     SysScratch& c = sc[s];
     c.cap = std::max(1, std::min((int)items[s].size(), (int)(budget / n_sliced / slice_item_bytes(ctx, h))));
     n_rounds = std::max(n_rounds, (items[s].size() + c.cap - 1) / c.cap);
-    tiles += (long long)c.cap * slice_tiles(h.nocc, h.N);
+    tiles += c.cap * slice_plane_tiles(ctx, h);
     for (int I = 0; I < h.nat; ++I) ctx->max_orb = std::max(ctx->max_orb, h.orb_off[I + 1] - h.orb_off[I]);
   }
-  ctx->slice_mp = slice_pairs_per_plane(2 * tiles);
+  ctx->slice_mp = slice_pairs_per_plane(tiles);
   const int np = slice_num_planes(ctx->slice_mp);
   for (size_t s = 0; s < ctx->sys.size(); ++s) {
     if (items[s].empty()) continue;

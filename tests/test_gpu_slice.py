@@ -157,13 +157,13 @@ def test_slice_product_holds_more_than_fp64_rows(shape, fall):
 @pytest.mark.parametrize("form", ["fp64", "fp64_delta", "cn"])
 def test_rounds_that_share_scratch_equal_single_runs(form):
     """The digits and planes of a step's items take at most 32 GB (a quarter of the free memory): 512 atoms at
-    134 MB of digits a matrix and 805 MB of planes need more than one round from 30 (16, 24) trajectories
+    134 MB of digits a matrix and 302 MB of planes need more than one round from 57 (32, 39) trajectories
     on.  Every trajectory equals its own single run bit for bit, whichever round holds it."""
     from paper_2308_09782_gb300 import inputs
     from tests._gpu_util import oracle_ground, system
     sysd, _, _ = system("si512_kick")
     _, gs = oracle_ground("si512_kick")
-    dig, planes = 2 * 8 * 2048 * 2 * 2048, 4 * 24 * 2048 * 2 * 2048
+    dig, planes = 2 * 8 * 2048 * 2 * 2048, 4 * 9 * 2048 * 2 * 2048
     n_traj = int(32e9 / {"fp64": 2 * dig + planes, "fp64_delta": 3 * dig + 2 * planes, "cn": 4 * dig + planes}[form]) + 2
     n = 2
     fields = [inputs.kick_field(n, 0.001 * (1.0 + 0.1 * t), np.array([1.0, 0.1 * t, 0.0])) for t in range(n_traj)]
@@ -183,3 +183,15 @@ def test_rounds_that_share_scratch_equal_single_runs(form):
                 for a, b in zip(many.observables(t), one.observables(0)):
                     assert np.array_equal(a, b)
                 assert np.array_equal(many.get_density(t, 0), one.get_density(0, 0))
+
+
+def test_group_sums_fit_at_the_largest_size():
+    """k = 8192, the most that 32-bit group sums hold, with digits -128 wherever the row's scale allows it (the
+    first one -125): every sum has one sign, and 2 k x^2 comes out to its last bit but one."""
+    from fractions import Fraction
+    x = sum(d * 2.0 ** (-8 * (s + 1)) for s, d in enumerate([-125] + [-128] * 6))
+    a = np.full((3, 8192), x * (1 + 1j))
+    want = float(2 * 8192 * Fraction(x) ** 2)
+    for planes in (8, 19):
+        c = vgtb.diag_slice_product(a, a, planes=planes)
+        assert np.all(np.abs(c.real - want) <= 2.0 ** -52 * want) and not np.any(c.imag)
